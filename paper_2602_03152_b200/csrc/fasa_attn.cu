@@ -21,6 +21,7 @@
 
 #include "fasa_cluster_merge.cuh"
 #include "fasa_common.cuh"
+#include "fasa_launch.cuh"
 #include "fasa_score_core.cuh"
 
 namespace cg = cooperative_groups;
@@ -346,38 +347,6 @@ struct MmaSmem {
   uint16_t p_hi[kMmaWarps][8][16];                  // P^T: [head][row]
   uint16_t p_lo[kMmaWarps][8][16];
 };
-
-// Programmatic dependent launch: these kernels may be scheduled while the kernel before them
-// on the stream is still draining (their launch latency then overlaps its tail).  They wait
-// here until that kernel has completed and its writes are visible, and let their own
-// successor be scheduled early in turn.  Launched the ordinary way, both are no-ops.
-__device__ __forceinline__ void pdl_wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// cluster_x > 0: the CTAs of a grid row form one thread-block cluster of that size.
-template <typename Kernel, typename... Args>
-cudaError_t launch_after_predecessor(Kernel kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                     int cluster_x, Args... args) {
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.numAttrs = 1;
-  if (cluster_x > 0) {
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)cluster_x;
-    attr[1].val.clusterDim.y = 1;
-    attr[1].val.clusterDim.z = 1;
-    cfg.numAttrs = 2;
-  }
-  cfg.attrs = attr;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
 
 // CLUSTER: the splits of a unit are the CTAs of one cluster (grid.x = cluster size) and merge
 // in the same launch; otherwise each split writes its partial result for the merge kernel.

@@ -359,7 +359,7 @@ extern "C" int32_t fasa_topk_batched(fasa_ctx_t* ctx, const float* scores, const
   if (q_len < 1 || q_len > FASA_MAX_QLEN) return FASA_ERR_UNSUPPORTED;
   if (!(ctx->fused_cs > 0)) return FASA_ERR_UNSUPPORTED;            // needs the cluster kernel's selection phases
   if ((long long)ctx->cfg.batch * q_len * ctx->n_sets > 65535) return FASA_ERR_UNSUPPORTED;
-  return fasa_fused_topk_rows(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, q_len * ctx->n_sets,
+  return fasa_topk_row_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, q_len * ctx->n_sets,
                               ctx->cfg.n_sink, ctx->cfg.n_recent, (cudaStream_t)stream, q_len);
 }
 

@@ -171,7 +171,7 @@ extern "C" int32_t fasa_calib_accumulate(fasa_ctx_t* ctx, const void* q, const v
       (const uint16_t*)q, (const uint16_t*)k_cache, seq_lens, scores, ctx->d_status, c.n_q_heads, c.n_kv_heads,
       c.max_len, c.rope_pairing, c.k_stride_b, c.k_stride_h, c.k_stride_t, fasa_page_map(ctx));
   FASA_LAUNCH_CHECK(ctx);
-  const int32_t st = fasa_fused_topk_rows(ctx, scores, seq_lens, top_k, top_k, idx, n_sel, c.n_q_heads * kRows,
+  const int32_t st = fasa_topk_row_launch(ctx, scores, seq_lens, top_k, top_k, idx, n_sel, c.n_q_heads * kRows,
                                           0, 0, s);
   if (st != FASA_OK) return st;
   calib_intersect_kernel<<<samples, 256, (size_t)top_k * sizeof(int32_t), s>>>(

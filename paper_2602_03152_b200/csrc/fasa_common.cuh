@@ -39,7 +39,6 @@ struct fasa_ctx {
   size_t step_smem;
   int step_resident;      // clusters of the step's shape that the device holds at once
   int use_fused;          // fasa_decode_step takes the one-launch kernel when it is available
-  int topk_rows;          // fasa_topk by the one-CTA-per-row kernel whatever the number of rows (fasa_set_step_mode 2)
   // host-buffer step: the last host pointers seen and what the device can use in their place
   // (null: not page-locked + mapped), so that a decode loop with fixed buffers asks the driver once
   const void* host_seen[4];
@@ -136,19 +135,12 @@ int32_t fasa_attn_split_keys(fasa_ctx* ctx, const void* q, const void* k_nondom,
 bool fasa_on_host(fasa_ctx* ctx, const void* p);
 
 bool fasa_topk_row_ok(const fasa_ctx* ctx);
+// TopK-I over rows_per_seq score rows per sequence (row r of the buffer belongs to sequence
+// r / rows_per_seq), with the given forced positions.  q_len > 1: the rows of a sequence are (query, set)
+// pairs, query-major, and query t of the block sees seq_lens[b] - (q_len - 1 - t) positions.
 int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget,
                              int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
-                             int n_recent, cudaStream_t stream, int q_len);
-int32_t fasa_fused_topk_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens,
-                               int32_t budget, int32_t n_sel_max, int32_t* idx, int32_t* n_sel,
-                               cudaStream_t stream);
-
-// q_len > 1: the rows of a sequence are (query, set) pairs, query-major, and query t of the
-// block sees seq_lens[b] - (q_len - 1 - t) positions.
-int32_t fasa_fused_topk_rows(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens,
-                             int32_t budget, int32_t n_sel_max, int32_t* idx, int32_t* n_sel,
-                             int rows_per_seq, int n_sink, int n_recent, cudaStream_t stream, int q_len = 1);
-
+                             int n_recent, cudaStream_t stream, int q_len = 1);
 // Paged caches: how a (sequence, token) pair finds its page.  All zero = contiguous caches.
 struct PageMap {
   const int32_t* table;   // [batch][pages_per_seq]: physical page of each logical page

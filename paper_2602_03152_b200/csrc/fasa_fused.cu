@@ -120,8 +120,6 @@ struct FusedParams {
   int32_t* status;
   int n_q_heads, n_kv_heads, n_sets, group, max_len, chunks, n_sink, n_recent, budget, n_sel_max;   // group: query heads of a unit
   int max_reduce;          // score of a KV head = max over its query heads instead of their sum
-  int q_len;               // select-only form over blocks of queries: rows per sequence are (query, set) pairs,
-                           // query t sees q_len - 1 - t fewer positions (0 or 1: plain rows)
   int64_t ksb, ksh, kst, vsb, vsh, vst;
   float scale_log2;        // softmax_scale * log2(e)
   PageMap pm;              // paged caches (all zero: contiguous)
@@ -165,14 +163,12 @@ __device__ __forceinline__ bool warp_find_kth(uint32_t v, uint32_t kth, int lane
 
 // A tile's 16-channel blocks are taken NG groups of KB at a time (KB = 1, 2, 4; NG = 2 only with
 // KB = 4, for more than 4 blocks), which bounds the registers the loads in flight need.
-// MODE 0: the whole step.  MODE 1: TopK-I alone (fasa_topk): the keys come from a score buffer
-// instead of the proxy stream, and the kernel ends after the index list is written.  MODE 2:
-// the step without its attention phase (large selections are attended by the split-K
-// tensor-core kernel instead).
+// ATTEND: the whole step; otherwise the step without its attention phase (large selections are
+// attended by the split-K tensor-core kernel instead).
 // PAGED: K, V and the proxy are page pools behind a block table (compiled separately, so that
 // the contiguous form keeps its plain address arithmetic within 64 registers).
 // NT: threads per CTA: 512 (two CTAs per SM) or 1024 (one CTA per SM with twice the slice).
-template <int KB, int NG, int MODE, bool PAGED = false, int NT = 512>
+template <int KB, int NG, bool ATTEND, bool PAGED = false, int NT = 512>
 __global__ void __launch_bounds__(NT, NT == 512 ? 2 : 1)
 fused_decode_kernel(const FusedParams p) {
   constexpr int kFT = NT;                  // (shadow the file-level constants inside this kernel)
@@ -211,18 +207,14 @@ fused_decode_kernel(const FusedParams p) {
   // length, this thread's 16 bytes of the unit's query rows and its entry of the channel table.
   // The scoring operand (query values at the dominant channels) is gathered from the staged
   // copies in shared memory after the set-up barrier: no load waits on another load's result.
-  const bool append = MODE != 1 && p.k_new != nullptr;
+  const bool append = p.k_new != nullptr;
   int len_raw = 0;
   if (!append || tid == 0) len_raw = p.seq_lens[b];
   uint4 q_stage = make_uint4(0u, 0u, 0u, 0u);
-  if (MODE != 1 && tid < FASA_MAX_GROUP * (FASA_HEAD_DIM / 8) && tid / (FASA_HEAD_DIM / 8) < p.group)
+  if (tid < FASA_MAX_GROUP * (FASA_HEAD_DIM / 8) && tid / (FASA_HEAD_DIM / 8) < p.group)
     q_stage = *reinterpret_cast<const uint4*>(p.q + su.q0 * FASA_HEAD_DIM + tid * 8);
   int16_t chan_stage = -1;
-  if (MODE != 1 && tid < p.chunks * 8) chan_stage = p.chan[h * p.chunks * 8 + tid];
-  if (MODE == 1 && p.q_len > 1) {
-    const int t = (u % p.n_sets) / (p.n_sets / p.q_len);        // the query of this row
-    if (len_raw >= 0 && len_raw <= p.max_len) len_raw = max(0, len_raw - (p.q_len - 1 - t));   // (a bad length is left for clamp_len to flag)
-  }
+  if (tid < p.chunks * 8) chan_stage = p.chan[h * p.chunks * 8 + tid];
   int len_old;
   if (append) {
     if (tid == 0) s_len_old = clamp_len(len_raw, p.max_len, p.status);
@@ -254,7 +246,7 @@ fused_decode_kernel(const FusedParams p) {
   // the two halves of the machine out of phase for the rest of the launch: one half streams while
   // the other selects.  Measured: batch 16 at 64-128 K 177.9 -> 167.9 us, batch 32 at 64 K
   // 225.9 -> 189.2 us.  The wait is a sleep bounded by the clock; nothing is waited for.
-  if (MODE != 1 && p.shift_ctas > 0 && (int)blockIdx.y < p.shift_clusters && (blockIdx.y & 1)) {
+  if (p.shift_ctas > 0 && (int)blockIdx.y < p.shift_clusters && (blockIdx.y & 1)) {
     const float ns = 0.45f * (float)p.shift_ctas * (float)nloc * (float)(p.chunks * 16) * (1.0f / 6400.0f);
     const unsigned long long want = (unsigned long long)fminf(ns, 200000.0f);
     unsigned long long t0, t1;
@@ -318,8 +310,8 @@ fused_decode_kernel(const FusedParams p) {
   int T = ((crank * per) >> 4) + warp * TPI;                  // slices start on a tile boundary
   const bool own_new = grows && c0 <= len_old && len_old < c1;
   uint4 a[TPI][KB];
-  if (MODE != 1) locate(tp, T);
-  if (MODE != 1 && !own_new) fetch(a, T, 0);
+  locate(tp, T);
+  if (!own_new) fetch(a, T, 0);
 
   if (own_new) {
     // this CTA's slice holds the new row: K and V copies (16 lanes each) and the packed
@@ -364,11 +356,11 @@ fused_decode_kernel(const FusedParams p) {
   for (int i = tid; i < 3 * 2 * kGroups; i += kFT) (&s_gsum[0][0][0])[i] = 0u;
   for (int i = tid; i < 3 * 2 * 32; i += kFT) (&s_fine[0][0][0])[i] = 0u;
   if (tid == 0) { s_ncand = 0u; s_cgt = 0u; s_ceq = 0u; }
-  if (MODE != 1 && tid < GP * (FASA_HEAD_DIM / 8))
+  if (tid < GP * (FASA_HEAD_DIM / 8))
     *reinterpret_cast<uint4*>(&s_qraw[tid / (FASA_HEAD_DIM / 8)][(tid % (FASA_HEAD_DIM / 8)) * 8]) = q_stage;
-  if (MODE != 1 && tid < p.chunks * 8) s_chan[tid] = chan_stage;
+  if (tid < p.chunks * 8) s_chan[tid] = chan_stage;
   // query, scaled into the base-2 logit domain, for the attention phase
-  if (MODE == 0 && tid < GP * (FASA_HEAD_DIM / 8)) {
+  if (ATTEND && tid < GP * (FASA_HEAD_DIM / 8)) {
     const int g = tid / (FASA_HEAD_DIM / 8), c = (tid % (FASA_HEAD_DIM / 8)) * 8;
     const uint4 w = q_stage;
     const float2 f0 = bf16x2_to_f32x2(w.x), f1 = bf16x2_to_f32x2(w.y), f2 = bf16x2_to_f32x2(w.z), f3 = bf16x2_to_f32x2(w.w);
@@ -381,37 +373,12 @@ fused_decode_kernel(const FusedParams p) {
   // waits for the others' arrival only when it is about to touch them, after its stream.
   cluster_arrive();
   ScoreFrag<KB> f[NG];
-  if constexpr (MODE != 1) {
 #pragma unroll
-    for (int grp = 0; grp < NG; ++grp)
-      load_score_b<KB>(f[grp], &s_qraw[0][0], s_chan, p.chunks, p.group, lane, grp * KB);
-  }
+  for (int grp = 0; grp < NG; ++grp)
+    load_score_b<KB>(f[grp], &s_qraw[0][0], s_chan, p.chunks, p.group, lane, grp * KB);
 
   // ---- 1. scoring stream -> keys + first histogram ------------------------------------------
-  if constexpr (MODE == 1) {
-    // keys from the caller's score buffer, four consecutive tokens per thread
-    const float* sin = p.scores + (int64_t)u * p.max_len;
-    const bool vec_ok = ((reinterpret_cast<uintptr_t>(sin) & 15) == 0);
-    for (int i = c0 + tid * 4; i < c1; i += kFT * 4) {
-      float sv[4] = {0.f, 0.f, 0.f, 0.f};
-      if (vec_ok && i + 3 < c1) {
-        const float4 v4 = *reinterpret_cast<const float4*>(sin + i);
-        sv[0] = v4.x; sv[1] = v4.y; sv[2] = v4.z; sv[3] = v4.w;
-      } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if (i + e < c1) sv[e] = sin[i + e];
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        if (i + e < c1) {
-          const uint32_t key = fasa_item_key(sv[e], i + e, len, p.n_sink, p.n_recent);
-          atomicAdd(&hist0[key >> 21], 1u);
-          keys[i + e - c0] = key;
-        }
-      }
-    }
-  } else {
+  {
     if (own_new) fetch(a, T, 0);                              // (the new row is in place now)
     locate(tp_next, T + step);
     // The loop exists twice.  When the head's dominant channels fill whole 16-channel blocks and
@@ -813,7 +780,7 @@ fused_decode_kernel(const FusedParams p) {
     }
     if (crank == 0 && tid == 0) p.n_sel[u] = (int32_t)ktot;
   }
-  if constexpr (MODE != 0) return;   // (no peer reads this CTA's memory after the selection's last barrier)
+  if constexpr (!ATTEND) return;   // (no peer reads this CTA's memory after the selection's last barrier)
 
   // ---- 4. attention over this CTA's share of the selected rows -----------------------------
   // Register-lean form (64 registers per thread): four query heads per pass (two passes for
@@ -985,36 +952,34 @@ size_t fused_smem_bytes(int cap) { return (size_t)fused_smem_layout(cap).total; 
 
 using FusedFn = void (*)(const FusedParams);
 
-template <int MODE, bool PAGED>
+template <bool ATTEND, bool PAGED>
 FusedFn fused_variant(int chunks) {
   const int nb = (chunks + 1) / 2;      // 16-channel blocks per tile, the 8-channel one included
-  if (nb <= 1) return fused_decode_kernel<1, 1, MODE, PAGED>;
-  if (nb <= 2) return fused_decode_kernel<2, 1, MODE, PAGED>;
-  if (nb <= 4) return fused_decode_kernel<4, 1, MODE, PAGED>;
-  return fused_decode_kernel<4, 2, MODE, PAGED>;
+  if (nb <= 1) return fused_decode_kernel<1, 1, ATTEND, PAGED>;
+  if (nb <= 2) return fused_decode_kernel<2, 1, ATTEND, PAGED>;
+  if (nb <= 4) return fused_decode_kernel<4, 1, ATTEND, PAGED>;
+  return fused_decode_kernel<4, 2, ATTEND, PAGED>;
 }
 
 FusedFn fused_fn(int chunks, bool paged = false) {
-  return paged ? fused_variant<0, true>(chunks) : fused_variant<0, false>(chunks);
+  return paged ? fused_variant<true, true>(chunks) : fused_variant<true, false>(chunks);
 }
-
-FusedFn topk_fn() { return fused_decode_kernel<1, 1, 1>; }
 
 // The wide form of the step: 1024 threads, one CTA per SM.
-template <int MODE, bool PAGED>
+template <bool ATTEND, bool PAGED>
 FusedFn wide_variant(int chunks) {
   const int nb = (chunks + 1) / 2;
-  if (nb <= 1) return fused_decode_kernel<1, 1, MODE, PAGED, 1024>;
-  if (nb <= 2) return fused_decode_kernel<2, 1, MODE, PAGED, 1024>;
-  if (nb <= 4) return fused_decode_kernel<4, 1, MODE, PAGED, 1024>;
-  return fused_decode_kernel<4, 2, MODE, PAGED, 1024>;
+  if (nb <= 1) return fused_decode_kernel<1, 1, ATTEND, PAGED, 1024>;
+  if (nb <= 2) return fused_decode_kernel<2, 1, ATTEND, PAGED, 1024>;
+  if (nb <= 4) return fused_decode_kernel<4, 1, ATTEND, PAGED, 1024>;
+  return fused_decode_kernel<4, 2, ATTEND, PAGED, 1024>;
 }
-FusedFn wide_fn(int chunks, bool paged) { return paged ? wide_variant<0, true>(chunks) : wide_variant<0, false>(chunks); }
-FusedFn wide_select_fn(int chunks, bool paged) { return paged ? wide_variant<2, true>(chunks) : wide_variant<2, false>(chunks); }
+FusedFn wide_fn(int chunks, bool paged) { return paged ? wide_variant<true, true>(chunks) : wide_variant<true, false>(chunks); }
+FusedFn wide_select_fn(int chunks, bool paged) { return paged ? wide_variant<false, true>(chunks) : wide_variant<false, false>(chunks); }
 constexpr int kCapWide = 40960;        // keys a 1024-thread CTA can hold (one CTA per SM)
 
 FusedFn select_fn(int chunks, bool paged = false) {         // the step without attention
-  return paged ? fused_variant<2, true>(chunks) : fused_variant<2, false>(chunks);
+  return paged ? fused_variant<false, true>(chunks) : fused_variant<false, false>(chunks);
 }
 
 }  // namespace
@@ -1069,11 +1034,9 @@ int fasa_fused_plan(fasa_ctx* ctx) {
       cudaGetLastError();
       continue;
     }
-    // the select-only forms of the kernel run with the same cluster shape
-    if (cudaFuncSetAttribute((const void*)topk_fn(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit) != cudaSuccess ||
-        cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit) != cudaSuccess ||
-        (cs > 8 && (cudaFuncSetAttribute((const void*)topk_fn(), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-                    cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess))) {
+    // the form without attention runs with the same cluster shape
+    if (cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit) != cudaSuccess ||
+        (cs > 8 && cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
       cudaGetLastError();
       continue;
     }
@@ -1144,7 +1107,6 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
   p.chunks = ctx->chunks; p.n_sink = c.n_sink; p.n_recent = c.n_recent; p.budget = budget;
   p.n_sel_max = n_sel_max;
   p.max_reduce = c.group_reduce;
-  p.q_len = 1;
   p.ksb = c.k_stride_b; p.ksh = c.k_stride_h; p.kst = c.k_stride_t;
   p.vsb = c.v_stride_b; p.vsh = c.v_stride_h; p.vst = c.v_stride_t;
   p.scale_log2 = c.softmax_scale * 1.4426950408889634f;
@@ -1177,66 +1139,6 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cudaError_t e = cudaLaunchKernelEx(&cfg, fn, p);
-  ctx->launches += 1;
-  FASA_CUDA_TRY(ctx, e);
-  return FASA_OK;
-}
-
-// TopK-I alone with the cluster kernel's selection phases (fasa_topk).
-int32_t fasa_fused_topk_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens,
-                               int32_t budget, int32_t n_sel_max, int32_t* idx, int32_t* n_sel,
-                               cudaStream_t stream) {
-  return fasa_fused_topk_rows(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, ctx->n_sets,
-                              ctx->cfg.n_sink, ctx->cfg.n_recent, stream);
-}
-
-// TopK-I over rows_per_seq score rows per sequence (row r of the buffer belongs to sequence
-// r / rows_per_seq), with the given forced positions instead of the context's.
-int32_t fasa_fused_topk_rows(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens,
-                             int32_t budget, int32_t n_sel_max, int32_t* idx, int32_t* n_sel,
-                             int rows_per_seq, int n_sink, int n_recent, cudaStream_t stream, int q_len) {
-  const fasa_config_t& c = ctx->cfg;
-  // Many long rows (batch 16 at 64-128 K, blocks of queries, calibration): clusters would run in
-  // rounds, each paying the whole chain of cluster barriers; one CTA per row is faster there (128 rows
-  // of 64-128 K: 64 -> 53 us; calibration of 512 samples at 64-128 K: 18.5 -> 11.6 ms; eight queries
-  // per sequence at batch 8, 64 K: 133 -> 105 us).  For few rows and for short ones the cluster form
-  // wins (64 rows of 64 K: 21 against 31 us; 8 rows of 32 K: 16 against 23 us; 2080 rows of 32 K: 387
-  // against 420 us).
-  if (fasa_topk_row_ok(ctx) &&
-      (((long long)c.batch * rows_per_seq >= ctx->n_sm * 3 / 4 && c.max_len >= 65536) || ctx->topk_rows))
-    return fasa_topk_row_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, rows_per_seq, n_sink, n_recent, stream, q_len);
-  FusedParams p;
-  memset(&p, 0, sizeof(p));
-  p.seq_lens = seq_lens; p.scores = const_cast<float*>(scores); p.idx = idx; p.n_sel = n_sel;
-  p.status = ctx->d_status;
-  // (the select-only form uses the unit index for its score row and its sequence alone)
-  p.n_q_heads = rows_per_seq; p.n_kv_heads = 1; p.n_sets = rows_per_seq; p.group = 1; p.max_len = c.max_len;
-  p.chunks = ctx->chunks; p.n_sink = n_sink; p.n_recent = n_recent; p.budget = budget;
-  p.n_sel_max = n_sel_max;
-  p.q_len = q_len;
-  // The context's cluster size suits its own number of rows (few rows: wide clusters, so the
-  // whole GPU works on them).  A launch with many more rows takes the narrowest cluster that
-  // holds a row's keys: more rows are then resident at once.
-  int cs = ctx->fused_cs;
-  auto cap_of = [&](int n) { return (((c.max_len + n - 1) / n) + 31) & ~31; };
-  if (rows_per_seq > ctx->n_sets) {
-    cs = 1;
-    while (cs < ctx->fused_cs && cap_of(cs) > kCapPair) cs *= 2;
-  }
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)cs, (unsigned)(c.batch * rows_per_seq), 1);
-  cfg.blockDim = dim3(kFT, 1, 1);
-  cfg.dynamicSmemBytes = cs == ctx->fused_cs ? ctx->fused_smem : fused_smem_bytes(cap_of(cs));
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)cs;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, topk_fn(), p);
   ctx->launches += 1;
   FASA_CUDA_TRY(ctx, e);
   return FASA_OK;

@@ -1,0 +1,404 @@
+// TopK-I (Sec. 4.1) of one score row by one thread block: the k best positions of a row in
+// ascending order, equal scores lowest index first (= a stable sort).
+//
+// A row of L scores is not sorted or histogrammed as a whole.  It is cut into groups of 8 or 32
+// consecutive positions whose maxima bound the k-th largest score from below: at least k groups have a
+// maximum at or above the k-th largest maximum, so at least k scores do, and a group whose maximum lies
+// below it holds none of the k best.  With k well below the number of groups only those k groups are
+// looked at again (k = 256 of 65536 positions: 2100 of them); otherwise the row is taken whole.
+//   1. the k-th largest group maximum, to the resolution of one histogram of 1024 bins spread evenly
+//      over the range of the maxima (values, not their bit patterns: real scores crowd into a few
+//      exponents, which makes the atomics of a radix histogram collide and its bins useless);
+//   2. the list of the groups at or above that bin, ascending;
+//   3. one more such histogram, over the scores of these groups from the bound up, gives the bin of the
+//      k-th largest score; its few members are ranked against each other by (score, index), which
+//      settles which of them are taken;
+//   4. the bit masks of the selected positions become ranks (a block-wide prefix sum).
+// What bounds this is instructions and block barriers (seven), not bytes: a pass touches a score with
+// a dozen instructions per 32 of them, so the fewer positions a pass visits the better.  Bins are
+// monotone in the score, whatever the rounding, so the result is exact; scores that even bins cannot
+// spread (infinities and NaNs, hundreds of equal scores at the threshold) are settled by an
+// 11 / 11 / 10-bit radix select on order-preserving keys instead.
+#pragma once
+
+#include "fasa_common.cuh"
+#include "fasa_score_core.cuh"
+
+#ifdef __CUDACC__
+
+constexpr int kSelBins = 1024;
+constexpr int kSelRank = 256;            // members of the threshold's bin that are ranked against each other
+constexpr int kSelRadixBins = 2048;
+
+struct SelShared {
+  uint32_t hist[2][kSelBins];            // group maxima; scores.  Together: the bins of a radix pass
+  uint32_t ckey[kSelRank], cpos[kSelRank];
+  uint32_t wlo[32], whi[32], wcnt[32];
+  uint32_t n_cand;
+};
+static_assert(2 * kSelBins == kSelRadixBins, "the radix passes use both histograms");
+
+// A block's dynamic shared memory for a row: the maxima of the groups (float; later their bins) and, once the
+// groups are listed, the bins of the positions looked at in their place; the list of groups; one bit per position
+// looked at.
+struct SelLayout {
+  int gm_cap, uni_cap, word_cap;         // group maxima (and list entries) / positions' bins / mask words that fit
+  __host__ __device__ int list_off() const { return ((gm_cap * 4 > uni_cap * 2 ? gm_cap * 4 : uni_cap * 2) + 15) & ~15; }
+  __host__ __device__ int word_off() const { return list_off() + ((gm_cap * 2 + 15) & ~15); }
+  __host__ __device__ int bytes() const { return word_off() + word_cap * 4; }
+};
+
+// max and min that keep NaNs, so that one in the row is noticed
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
+__device__ __forceinline__ float sel_key_value(uint32_t k) {       // inverse of fasa_order_key
+  return __uint_as_float((k & 0x80000000u) ? k ^ 0x80000000u : ~k);
+}
+
+// Evenly spread bins 1 .. kSelBins - 1 from `lo` up; 0 is what lies below.
+struct SelBinning {
+  float lo, scale;
+  __device__ __forceinline__ int bin(float x) const {              // non-decreasing in x
+    return min(kSelBins - 1, max(0, __float2int_rz(fmaf(x - lo, scale, 1.0f))));
+  }
+};
+__device__ __forceinline__ SelBinning sel_binning(float lo, float hi) {
+  SelBinning b;
+  b.lo = lo;
+  b.scale = (float)(kSelBins - 1) / (hi - lo);                      // hi == lo, or a range past the largest float: one bin
+  if (!(b.scale < 3.0e38f)) b.scale = 0.f;
+  return b;
+}
+
+__device__ __forceinline__ uint32_t sel_scan(uint32_t v, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  return v;
+}
+
+// One warp: the bin of hist[0 .. NB) that holds the kth largest entry (counted from the highest bin
+// down; kth <= entries), its rank inside the bin and the bin's count.
+template <int NB>
+__device__ __forceinline__ void sel_find(const uint32_t* hist, uint32_t kth, int lane, int* bin, uint32_t* rank, uint32_t* count) {
+  constexpr int PER = NB / 32;
+  uint32_t v = 0;
+#pragma unroll
+  for (int j = 0; j < PER / 4; ++j) {
+    // (the start of a lane's run rotates with the lane, so that the lanes' 16-byte reads spread over the banks)
+    const uint4 q = *reinterpret_cast<const uint4*>(hist + NB - PER * (lane + 1) + 4 * ((j + lane) & (PER / 4 - 1)));
+    v += q.x + q.y + q.z + q.w;
+  }
+  const uint32_t incl = sel_scan(v, lane);
+  const uint32_t hits = __ballot_sync(0xffffffffu, incl >= kth);
+  const int hit = hits ? __ffs(hits) - 1 : 31;
+  uint32_t left = kth - __shfl_sync(0xffffffffu, incl - v, hit);
+  int top = NB - PER * hit;                                         // one past the run's highest bin
+#pragma unroll
+  for (int part = 0; part < PER; part += 32) {
+    const uint32_t c = hist[top - 1 - lane];
+    const uint32_t ci = sel_scan(c, lane);
+    const uint32_t h2 = __ballot_sync(0xffffffffu, ci >= left);
+    if (h2 || part + 32 >= PER) {
+      const int first = h2 ? __ffs(h2) - 1 : 31;
+      *bin = top - 1 - first;
+      *rank = left - __shfl_sync(0xffffffffu, ci - c, first);
+      *count = __shfl_sync(0xffffffffu, c, first);
+      return;
+    }
+    left -= __shfl_sync(0xffffffffu, ci, 31);
+    top -= 32;
+  }
+}
+
+// Block-wide min and max of the threads' values (one barrier); false when one of them is not finite.
+template <int NT>
+__device__ __forceinline__ bool sel_minmax(SelShared& sm, float& lo, float& hi, int warp, int lane) {
+  const uint32_t kl = __reduce_min_sync(0xffffffffu, fasa_order_key(lo)), kh = __reduce_max_sync(0xffffffffu, fasa_order_key(hi));
+  if (lane == 0) { sm.wlo[warp] = kl; sm.whi[warp] = kh; }
+  __syncthreads();
+  lo = sel_key_value(__reduce_min_sync(0xffffffffu, lane < NT / 32 ? sm.wlo[lane] : 0xffffffffu));
+  hi = sel_key_value(__reduce_max_sync(0xffffffffu, lane < NT / 32 ? sm.whi[lane] : 0u));
+  return hi - lo < 3.0e38f;                                         // (false for NaN)
+}
+
+// Block-wide exclusive prefix of v over the threads and the total (one barrier; sm.wcnt is used).
+template <int NT>
+__device__ __forceinline__ uint32_t sel_block_prefix(SelShared& sm, uint32_t v, int warp, int lane, uint32_t* total) {
+  const uint32_t incl = sel_scan(v, lane);
+  if (lane == 31) sm.wcnt[warp] = incl;
+  __syncthreads();
+  const uint32_t w = lane < NT / 32 ? sm.wcnt[lane] : 0u, wi = sel_scan(w, lane);
+  *total = __shfl_sync(0xffffffffu, wi, 31);
+  return __shfl_sync(0xffffffffu, wi - w, warp) + incl - v;
+}
+
+// The positions a row may be selected from, and how many of them are.
+struct SelRow {
+  const float* scores;
+  int lo, hi;                            // positions [lo, hi) compete (the others are forced or past the end)
+  int k;                                 // 0 <= k <= hi - lo
+};
+
+// Before a row: clears what the row's histograms add to (a barrier must follow).
+template <int NT>
+__device__ __forceinline__ void sel_begin(SelShared& sm) {
+  for (int i = threadIdx.x; i < kSelRadixBins / 4; i += NT) reinterpret_cast<uint4*>(&sm.hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (threadIdx.x == 0) sm.n_cand = 0u;
+}
+
+// Groups of 1 << shift positions narrow a row of n positions down; 0: take the row whole.  Groups of 8 leave
+// the fewest positions to look at, those of 32 have the fewest maxima: with about 1.5 instructions per 32
+// maxima and pass and 5 per 32 positions the larger ones pay below k = n / 1024.
+__host__ __device__ __forceinline__ int sel_group_shift(int n, int k, int gm_cap) {
+  const bool by8 = (long long)k * 12 <= n && (n >> 3) + 2 <= gm_cap;
+  const bool by32 = (long long)k * 43 <= n && (n >> 5) + 2 <= gm_cap;
+  if (by32 && ((long long)k * 1024 <= n || !by8)) return 5;
+  return by8 ? 3 : 0;
+}
+
+// Calls emit(r, position) for the r-th selected position in ascending order, r = 0 .. k - 1.
+// gs > 0: dyn starts with the maxima (float) of the groups (r.lo >> gs) .. ((r.hi - 1) >> gs), positions
+// outside [lo, hi) left out, and gm_lo / gm_hi are the least and the largest of those that this thread
+// has written.  sel_begin comes before; all threads call.
+template <int NT, typename Emit>
+__device__ __forceinline__ void sel_row(const SelRow& r, int gs, float gm_lo, float gm_hi, SelShared& sm, unsigned char* dyn,
+                                        const SelLayout& lay, Emit emit) {
+  constexpr int NW = NT / 32;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  if (r.k <= 0) return;                                             // (uniform)
+  if (r.k == r.hi - r.lo) {
+    for (int i = tid; i < r.k; i += NT) emit(i, r.lo + i);
+    return;
+  }
+  float* gm = reinterpret_cast<float*>(dyn);
+  uint16_t* list = reinterpret_cast<uint16_t*>(dyn + lay.list_off());
+  uint16_t* bins16 = reinterpret_cast<uint16_t*>(dyn);
+  uint32_t* words = reinterpret_cast<uint32_t*>(dyn + lay.word_off());
+  const uint32_t below = (1u << lane) - 1u;
+
+  bool radix = false;                    // the even bins do not apply
+  int n_list = 0;
+  float bound = 0.f;
+  int g0 = 0;
+  if (gs > 0) {
+    // ---- 1, 2: the groups that can hold one of the k best -------------------------------------
+    g0 = r.lo >> gs;
+    const int n_groups = ((r.hi - 1) >> gs) + 1 - g0;
+    if (!sel_minmax<NT>(sm, gm_lo, gm_hi, warp, lane)) {            // (the maxima are complete after its barrier)
+      radix = true;
+      gs = 0;
+    } else {
+      const SelBinning first = sel_binning(gm_lo, gm_hi);
+      for (int i = tid; i < n_groups; i += NT) {
+        const int bin = first.bin(gm[i]);
+        atomicAdd(&sm.hist[0][bin], 1u);
+        gm[i] = __int_as_float(bin);
+      }
+      __syncthreads();
+      int b0;
+      uint32_t rank, count;
+      sel_find<kSelBins>(sm.hist[0], (uint32_t)r.k, lane, &b0, &rank, &count);
+      const int per = ((n_groups + NW - 1) / NW + 31) & ~31;        // a warp takes a run of groups
+      const int s0 = min(n_groups, warp * per), s1 = min(n_groups, s0 + per);
+      uint32_t mine = 0;
+      for (int i = s0 + lane; i < s1; i += 32) mine += __float_as_int(gm[i]) >= b0 ? 1u : 0u;
+      mine = __reduce_add_sync(0xffffffffu, mine);
+      if (lane == 0) sm.wcnt[warp] = mine;
+      __syncthreads();
+      const uint32_t w = lane < NW ? sm.wcnt[lane] : 0u, incl = sel_scan(w, lane);
+      n_list = (int)__shfl_sync(0xffffffffu, incl, 31);
+      uint32_t at = __shfl_sync(0xffffffffu, incl - w, warp);
+      for (int i = s0; i < s1; i += 32) {                           // uniform over the warp
+        const bool in = i + lane < s1 && __float_as_int(gm[i + lane]) >= b0;
+        const uint32_t m = __ballot_sync(0xffffffffu, in);
+        if (in) list[at + __popc(m & below)] = (uint16_t)(i + lane);
+        at += __popc(m);
+      }
+      // (a little below the bin's edge, so that rounding leaves none of the listed maxima under it)
+      bound = first.scale > 0.f ? first.lo + ((float)b0 - 1.0625f) / first.scale : first.lo;
+      __syncthreads();
+    }
+  }
+  // The universe: positions base + 0, 1, ... or those of the listed groups, 32 to a chunk; a warp owns a
+  // run of chunks throughout.
+  const bool listed = gs > 0;
+  const int base = listed ? g0 << gs : r.lo & ~31;
+  const int n_uni = listed ? n_list << gs : r.hi - base;
+  const int n_chunks = (n_uni + 31) >> 5;
+  const int cper = (n_chunks + NW - 1) / NW;
+  const int c0 = min(n_chunks, warp * cper), c1 = min(n_chunks, c0 + cper);
+  const bool held = n_chunks * 32 <= lay.uni_cap;
+  auto pos_at = [&](int c, int l) -> int {                          // position l of chunk c (it may not compete)
+    if (!listed) return base + 32 * c + l;
+    const int e = (c << (5 - gs)) + (l >> gs);
+    return e < n_list ? base + ((int)list[e] << gs) + (l & ((1 << gs) - 1)) : -1;
+  };
+  constexpr int UNR = 4;
+  // visits this warp's chunks, UNR loads in flight: f(chunk, competes, score)
+  auto visit = [&](auto f) {
+    for (int c = c0; c < c1; c += UNR) {                            // uniform over the warp
+      float x[UNR];
+      bool ok[UNR];
+#pragma unroll
+      for (int j = 0; j < UNR; ++j) {
+        const int p = pos_at(c + j, lane);
+        ok[j] = c + j < c1 && p >= r.lo && p < r.hi;
+        x[j] = ok[j] ? __ldg(r.scores + p) : -INFINITY;
+      }
+#pragma unroll
+      for (int j = 0; j < UNR; ++j)
+        if (c + j < c1) f(c + j, ok[j], x[j]);
+    }
+  };
+  SelBinning second{0.f, 0.f};
+  if (listed) {
+    second = sel_binning(bound, gm_hi);
+  } else if (!radix) {
+    float lo = INFINITY, hi = -INFINITY;
+    visit([&](int, bool ok, float x) {
+      if (ok) { lo = fminf(lo, x); hi = max_nan(hi, x); }           // (a NaN shows in hi)
+    });
+    if (!sel_minmax<NT>(sm, lo, hi, warp, lane)) radix = true;
+    else second = sel_binning(lo, hi);
+  }
+  uint32_t rank = 0, count = 0;
+  int b1 = 0;
+  if (!radix) {
+    visit([&](int c, bool ok, float x) {
+      const int bin = ok ? second.bin(x) : 0;
+      if (bin > 0) atomicAdd(&sm.hist[1][bin], 1u);
+      if (held) bins16[c * 32 + lane] = (uint16_t)bin;
+    });
+    __syncthreads();
+    sel_find<kSelBins>(sm.hist[1], (uint32_t)r.k, lane, &b1, &rank, &count);
+    if (count > (uint32_t)kSelRank || b1 == 0) {
+      radix = true;
+      __syncthreads();                   // (every warp has read the histogram)
+    }
+  }
+
+  // ---- 3: one bit per position of the universe: selected or not ----------------------------------
+  if (!radix) {
+    auto classify = [&](int c, int bin) {
+      const uint32_t ma = __ballot_sync(0xffffffffu, bin > b1), mc = __ballot_sync(0xffffffffu, bin == b1);
+      if (lane == 0) words[c] = ma;
+      if (mc) {
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(&sm.n_cand, (uint32_t)__popc(mc));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(mc & below);
+        if (bin == b1 && at < (uint32_t)kSelRank) {
+          sm.cpos[at] = (uint32_t)(c * 32 + lane);
+          sm.ckey[at] = fasa_order_key(__ldg(r.scores + pos_at(c, lane)));
+        }
+      }
+    };
+    if (held) {
+#pragma unroll 4
+      for (int c = c0; c < c1; ++c) classify(c, bins16[c * 32 + lane]);
+    } else {
+      visit([&](int c, bool ok, float x) { classify(c, ok ? second.bin(x) : 0); });
+    }
+    __syncthreads();
+    // four threads to a member, each comparing it with a quarter of the others
+    for (int i = tid >> 2; i < (int)count; i += NT / 4) {           // (uniform over the four)
+      const uint32_t key = sm.ckey[i], pos = sm.cpos[i];
+      uint32_t ahead = 0;
+      for (int j = tid & 3; j < (int)count; j += 4) {
+        const uint32_t kj = sm.ckey[j];
+        ahead += kj > key || (kj == key && sm.cpos[j] < pos) ? 1u : 0u;
+      }
+      const uint32_t quad = 0xfu << (lane & ~3);
+      ahead += __shfl_xor_sync(quad, ahead, 1);
+      ahead += __shfl_xor_sync(quad, ahead, 2);
+      if ((tid & 3) == 0 && ahead < rank) atomicOr(&words[pos >> 5], 1u << (pos & 31));
+    }
+  } else {
+    uint32_t* bins = &sm.hist[0][0];
+    uint32_t prefix = 0, kth = (uint32_t)r.k;
+    int shift = 32;
+#pragma unroll 1
+    for (int level = 0; level < 3; ++level) {
+      const int bits = level == 2 ? 10 : 11, above = shift;
+      for (int i = tid; i < kSelRadixBins; i += NT) bins[i] = 0u;
+      __syncthreads();
+      shift -= bits;
+      visit([&](int, bool ok, float x) {
+        const uint32_t key = fasa_order_key(x);
+        if (ok && (level == 0 || (key >> above) == prefix)) atomicAdd(&bins[(key >> shift) & ((1u << bits) - 1u)], 1u);
+      });
+      __syncthreads();
+      int bin;
+      uint32_t in_bin;
+      sel_find<kSelRadixBins>(bins, kth, lane, &bin, &kth, &in_bin);
+      prefix = (prefix << bits) | (uint32_t)bin;
+      __syncthreads();
+    }
+    // prefix = the threshold, kth = how many of the scores equal to it are taken, lowest index first
+    uint32_t equal = 0;
+    visit([&](int, bool ok, float x) { equal += __popc(__ballot_sync(0xffffffffu, ok && fasa_order_key(x) == prefix)); });
+    uint32_t total, e_run = sel_block_prefix<NT>(sm, lane == 0 ? equal : 0u, warp, lane, &total);
+    e_run = __shfl_sync(0xffffffffu, e_run, 0);
+    visit([&](int c, bool ok, float x) {
+      const uint32_t key = fasa_order_key(x);
+      const uint32_t me = __ballot_sync(0xffffffffu, ok && key == prefix);
+      const bool in = ok && (key > prefix || (key == prefix && e_run + __popc(me & below) < kth));
+      const uint32_t m = __ballot_sync(0xffffffffu, in);
+      if (lane == 0) words[c] = m;
+      e_run += __popc(me);
+    });
+  }
+  __syncthreads();
+
+  // ---- 4: ranks in ascending order ---------------------------------------------------------------
+  const int wpt = (n_chunks + NT - 1) / NT;
+  const int w0 = min(n_chunks, tid * wpt), w1 = min(n_chunks, w0 + wpt);
+  uint32_t mine = 0;
+  for (int c = w0; c < w1; ++c) mine += __popc(words[c]);
+  uint32_t total, at = sel_block_prefix<NT>(sm, mine, warp, lane, &total);
+  for (int c = w0; c < w1; ++c) {
+    uint32_t m = words[c];
+    while (m) {
+      const int j = __ffs(m) - 1;
+      m &= m - 1;
+      emit((int)at, pos_at(c, j));
+      ++at;
+    }
+  }
+}
+
+// The selection of a row of `len` positions with forced ones: how the budget, the forced positions and
+// the size of the list combine (the forced ones are taken first, in ascending order).
+struct SelPlan {
+  int ktot;                              // positions selected
+  int sink, n_forced;
+  int lo, hi, k;                         // the free positions and how many of them are taken
+  bool clamped;                          // the list was too small
+};
+__device__ __forceinline__ SelPlan sel_plan(int len, int budget, int n_sink, int n_recent, int n_sel_max) {
+  SelPlan s;
+  const long long kb = budget > 0 ? (long long)budget : ((long long)(-budget) * len + 999) / 1000;
+  s.sink = min(len, n_sink);
+  s.lo = s.sink;
+  s.hi = len - min(n_recent, len - s.sink);
+  s.n_forced = len - (s.hi - s.lo);
+  long long kt = min((long long)len, (long long)s.n_forced + kb);
+  s.clamped = kt > n_sel_max;
+  if (s.clamped) kt = n_sel_max;
+  s.ktot = (int)kt;
+  s.k = max(0, s.ktot - s.n_forced);
+  return s;
+}
+// Rank of the i-th forced position (ascending) in the list, and the position itself.
+__device__ __forceinline__ void sel_forced(const SelPlan& s, int i, int* rank, int* pos) {
+  *rank = i < s.sink ? i : i + s.k;
+  *pos = i < s.sink ? i : s.hi + (i - s.sink);
+}
+
+#endif  // __CUDACC__

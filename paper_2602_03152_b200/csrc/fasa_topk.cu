@@ -215,11 +215,11 @@ extern "C" int32_t fasa_topk(fasa_ctx_t* ctx, const float* scores, const int32_t
   if (budget < -1000) return FASA_ERR_INVALID_ARG;
   const fasa_config_t& c = ctx->cfg;
   const int units = c.batch * ctx->n_sets;
-  // The cluster kernel's selection phases (keys in shared memory, one barrier per radix pass,
-  // mask compaction) serve wherever a cluster shape exists for this context; the
-  // register-resident kernel below remains for the rest (max_len beyond 16 x 22528).
-  if (ctx->use_fused && ctx->fused_cs > 0)
-    return fasa_fused_topk_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, (cudaStream_t)stream);
+  // One CTA per row from the maxima of the row's groups; the register-resident cluster kernel below
+  // remains for longer rows and as mode 0.
+  if (ctx->use_fused && fasa_topk_row_ok(ctx))
+    return fasa_topk_row_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, ctx->n_sets, c.n_sink, c.n_recent,
+                                (cudaStream_t)stream);
 
   // Cluster size: enough CTAs to hold max_len scores in registers, more when few units
   // would leave SMs idle (down to 2048 scores per CTA).

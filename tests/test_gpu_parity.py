@@ -1376,6 +1376,25 @@ def test_topk_exact_on_special_values():
         _assert_topk_exact(sc, [4096], budget)
 
 
+@pytest.mark.parametrize("L,budget", [
+    (1, 1), (31, 2), (33, 32), (97, 8), (98, 8), (383, 32), (385, 32),           # whole rows / groups of 8 (12 k <= L)
+    (12289, 12), (12289, 13), (20001, 19), (20001, 20), (20001, 1666), (20001, 1667),   # groups of 32 (1024 k <= L) / 8 / whole rows
+    (65553, 64), (70001, 1627), (70001, 1628),                                   # beyond 65536: groups of 32 (43 k <= L) / whole rows
+])
+@pytest.mark.parametrize("n_sink,n_recent", [(0, 0), (5, 70)])
+def test_topk_exact_at_the_edges_of_its_groups(L, budget, n_sink, n_recent):
+    # every form of the one-CTA-per-row selection (groups of 8, of 32, whole rows) next to the size where the next
+    # one starts; odd row lengths misalign all rows but the first; one row rises with the position, so that the
+    # groups that matter sit at its end, one has its largest scores in a single group, one has a run of equal scores
+    g = torch.Generator().manual_seed(L + budget)
+    sc = torch.randn(1, 5, L, generator=g)
+    sc[0, 1] = torch.arange(L, dtype=torch.float32) * 0.5 + sc[0, 1]
+    sc[0, 2, L // 2:L // 2 + 32] += 1e3
+    sc[0, 3, L // 3:L // 3 + max(1, budget)] = 2.5
+    sc[0, 4] = sc[0, 4].abs() ** 9
+    _assert_topk_exact(sc, [L], budget, n_sink=n_sink, n_recent=n_recent)
+
+
 @pytest.mark.parametrize("L,B,H", [(32768, 1, 8), (131072, 2, 2), (140001, 1, 2), (20000, 3, 5)])
 def test_topk_exact_at_scale(L, B, H):
     # 131072 fills the register-resident capacity of an 8-CTA cluster; 140001 takes the
