@@ -31,7 +31,7 @@ constexpr int kSelRank = 256;            // members of the threshold's bin that 
 constexpr int kSelRadixBins = 2048;
 
 struct SelShared {
-  uint32_t hist[2][kSelBins];            // group maxima; scores.  Together: the bins of a radix pass
+  alignas(16) uint32_t hist[2][kSelBins];   // (read 16 bytes at a time) group maxima; scores.  Together: the bins of a radix pass
   uint32_t ckey[kSelRank], cpos[kSelRank];
   uint32_t wlo[32], whi[32], wcnt[32];
   uint32_t n_cand;
