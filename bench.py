@@ -611,9 +611,9 @@ def run_calib(args):
     us = float(np.mean(ts))
     samples = int(sum(1 for l in t["seq_lens"].tolist() if l > top_k)) * w.n_q_heads
     tokens = int(sum(t["seq_lens"].tolist()))
-    # K rows once per KV head (query heads of a group re-read them from L2), 65 fp32 score rows
-    # per sample written and read once, 65 index lists written and read once
-    by = tokens * w.n_kv_heads * 256 + 2 * tokens * w.n_q_heads * 65 * 4 + 2 * samples * 65 * top_k * 4
+    # K rows once per KV head, its channel pairs (as many bytes) written and read once (the query heads
+    # of a group re-read them from L2), the full head's fp32 scores per sample and 65 index lists likewise
+    by = 3 * tokens * w.n_kv_heads * 256 + 2 * tokens * w.n_q_heads * 4 + 2 * samples * 65 * top_k * 4
     peak, peak_src = _peaks()
     # the oracle on one sample (sequence 0, query head 0), as it stands
     q0 = t["q"][0, 0].double().cpu().numpy()

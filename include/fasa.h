@@ -461,8 +461,8 @@ int32_t fasa_decode_step_host(fasa_ctx_t* ctx, const void* q_host, const void* k
  * q: bf16 [batch][n_q_heads][128]; k_cache as everywhere; ca_counts: int64
  * [n_q_heads][64] and n_used: int64 [n_q_heads], device, 8-byte aligned, zeroed by the
  * caller before the first call and carried from call to call (Stage 1 of Algorithm 1).
- * workspace: fasa_calib_workspace_bytes(ctx, top_k) bytes = batch * n_q_heads * 65 *
- * (max_len + top_k + 1) * 4 plus padding, 256-byte aligned.  The context's n_dom, sinks,
+ * workspace: fasa_calib_workspace_bytes(ctx, top_k) bytes = batch * (n_kv_heads * 64 * max_len +
+ * n_q_heads * (max_len + 65 * (top_k + 1))) * 4 plus padding, 256-byte aligned.  The context's n_dom, sinks,
  * budget and select_heads play no part.  Three kernels on `stream`, no synchronisation.
  * UNSUPPORTED: top_k outside 1..min(max_len, 8192), batch * n_q_heads * 65 > 65535, or a
  * max_len the cluster kernel cannot take (fasa_step_cluster_size() == 0). */

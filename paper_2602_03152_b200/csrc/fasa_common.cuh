@@ -135,12 +135,20 @@ int32_t fasa_attn_split_keys(fasa_ctx* ctx, const void* q, const void* k_nondom,
 bool fasa_on_host(fasa_ctx* ctx, const void* p);
 
 bool fasa_topk_row_ok(const fasa_ctx* ctx);
+// Calibration: the single-FC rows of a (sequence, query head) are not stored, they are computed from the KV head's
+// channel pairs: pairs [batch * n_kv_heads][64][stride], two bf16 values per position.
+struct fasa_calib_rows {
+  const uint32_t* pairs;
+  const uint16_t* q;        // [samples][128]
+  int64_t stride;           // positions per row, a multiple of 4 (also of the full-head score rows)
+  int group, pairing;       // query heads per KV head; rope_pairing
+};
 // TopK-I over rows_per_seq score rows per sequence (row r of the buffer belongs to sequence
 // r / rows_per_seq), with the given forced positions.  q_len > 1: the rows of a sequence are (query, set)
 // pairs, query-major, and query t of the block sees seq_lens[b] - (q_len - 1 - t) positions.
 int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget,
                              int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
-                             int n_recent, cudaStream_t stream, int q_len = 1);
+                             int n_recent, cudaStream_t stream, int q_len = 1, const struct fasa_calib_rows* calib = nullptr);
 // Paged caches: how a (sequence, token) pair finds its page.  All zero = contiguous caches.
 struct PageMap {
   const int32_t* table;   // [batch][pages_per_seq]: physical page of each logical page

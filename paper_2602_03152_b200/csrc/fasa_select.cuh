@@ -55,6 +55,12 @@ __device__ __forceinline__ float max_nan(float a, float b) {
   return r;
 }
 
+__device__ __forceinline__ float max_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 __device__ __forceinline__ float sel_key_value(uint32_t k) {       // inverse of fasa_order_key
   return __uint_as_float((k & 0x80000000u) ? k ^ 0x80000000u : ~k);
 }
@@ -139,9 +145,33 @@ __device__ __forceinline__ uint32_t sel_block_prefix(SelShared& sm, uint32_t v, 
   return __shfl_sync(0xffffffffu, wi - w, warp) + incl - v;
 }
 
+// Where the scores of a row come from: a buffer, or (calibration) the channel pairs of one FC, two bf16 values to a
+// position, with the query's values at these two channels: fl(q0 k0 + q1 k1), the products of bf16 values being exact.
+struct SelScores {
+  const float* p;
+  __device__ __forceinline__ float operator()(int i) const { return p[i]; }
+  __device__ __forceinline__ float4 four(int i) const { return *reinterpret_cast<const float4*>(p + i); }
+  __device__ __forceinline__ bool aligned() const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+};
+struct SelPairs {
+  const uint32_t* p;
+  float q0, q1;
+  __device__ __forceinline__ float score(uint32_t w) const {
+    const float2 k = bf16x2_to_f32x2(w);
+    return fmaf(q0, k.x, q1 * k.y) + 0.0f;                          // (-0 becomes +0)
+  }
+  __device__ __forceinline__ float operator()(int i) const { return score(p[i]); }
+  __device__ __forceinline__ float4 four(int i) const {
+    const uint4 w = *reinterpret_cast<const uint4*>(p + i);
+    return make_float4(score(w.x), score(w.y), score(w.z), score(w.w));
+  }
+  __device__ __forceinline__ bool aligned() const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+};
+
 // The positions a row may be selected from, and how many of them are.
+template <typename Src>
 struct SelRow {
-  const float* scores;
+  Src src;
   int lo, hi;                            // positions [lo, hi) compete (the others are forced or past the end)
   int k;                                 // 0 <= k <= hi - lo
 };
@@ -167,8 +197,8 @@ __host__ __device__ __forceinline__ int sel_group_shift(int n, int k, int gm_cap
 // gs > 0: dyn starts with the maxima (float) of the groups (r.lo >> gs) .. ((r.hi - 1) >> gs), positions
 // outside [lo, hi) left out, and gm_lo / gm_hi are the least and the largest of those that this thread
 // has written.  sel_begin comes before; all threads call.
-template <int NT, typename Emit>
-__device__ __forceinline__ void sel_row(const SelRow& r, int gs, float gm_lo, float gm_hi, SelShared& sm, unsigned char* dyn,
+template <int NT, typename Src, typename Emit>
+__device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, float gm_lo, float gm_hi, SelShared& sm, unsigned char* dyn,
                                         const SelLayout& lay, Emit emit) {
   constexpr int NW = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -250,7 +280,7 @@ __device__ __forceinline__ void sel_row(const SelRow& r, int gs, float gm_lo, fl
       for (int j = 0; j < UNR; ++j) {
         const int p = pos_at(c + j, lane);
         ok[j] = c + j < c1 && p >= r.lo && p < r.hi;
-        x[j] = ok[j] ? __ldg(r.scores + p) : -INFINITY;
+        x[j] = ok[j] ? r.src(p) : -INFINITY;
       }
 #pragma unroll
       for (int j = 0; j < UNR; ++j)
@@ -295,7 +325,7 @@ __device__ __forceinline__ void sel_row(const SelRow& r, int gs, float gm_lo, fl
         at = __shfl_sync(0xffffffffu, at, 0) + __popc(mc & below);
         if (bin == b1 && at < (uint32_t)kSelRank) {
           sm.cpos[at] = (uint32_t)(c * 32 + lane);
-          sm.ckey[at] = fasa_order_key(__ldg(r.scores + pos_at(c, lane)));
+          sm.ckey[at] = fasa_order_key(r.src(pos_at(c, lane)));
         }
       }
     };

@@ -3,8 +3,8 @@
 //
 // The pass is a stream of 16-byte loads with one max per score; what follows works on a few thousand
 // values and costs instructions and block barriers.  Measured (ncu), against a select that histograms
-// every key: 320 rows of 40-65 K positions, 512 of each: 67 -> 38 us; 2080 rows of 24 K, 256 of each:
-// 200 -> 93 us (53 M warp instructions, a quarter of what the histogram form issued).
+// every key: 320 rows of 40-65 K positions, 512 of each: 67 -> 34 us; 2080 rows of 24 K, 256 of each:
+// 200 -> 72 us (44 M warp instructions, a fifth of what the histogram form issued).
 #include "fasa_common.cuh"
 #include "fasa_launch.cuh"
 #include "fasa_score_core.cuh"
@@ -13,7 +13,8 @@
 namespace {
 
 struct RowParams {
-  const float* scores;                  // [rows][max_len]
+  const float* scores;                  // [rows][max_len]; CALIB: [samples][stride], the full-head scores
+  fasa_calib_rows calib;                // (CALIB) the other 64 rows of a sample
   const int32_t* seq_lens;
   int32_t* idx;
   int32_t* n_sel;
@@ -22,16 +23,10 @@ struct RowParams {
   SelLayout lay;
 };
 
-template <int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT)
-topk_row_kernel(const RowParams p) {
-  extern __shared__ __align__(16) unsigned char rsm[];
-  __shared__ SelShared sm;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int u = blockIdx.x, b = u / p.rows_per_seq;
-  sel_begin<NT>(sm);
-  pdl_wait_for_predecessor();
-  pdl_release_successor();
+// One row: unit u = blockIdx.x of sequence b.
+template <int NT, typename Src>
+__device__ __forceinline__ void topk_row(const RowParams& p, const Src& src, int b, SelShared& sm, unsigned char* rsm) {
+  const int tid = threadIdx.x, lane = tid & 31, u = blockIdx.x;
   int len_raw = p.seq_lens[b];
   if (p.q_len > 1) {                                // rows of a block of queries: query t sees q_len - 1 - t fewer positions
     const int t = (u % p.rows_per_seq) / (p.rows_per_seq / p.q_len);
@@ -43,56 +38,55 @@ topk_row_kernel(const RowParams p) {
     if (plan.clamped) atomicOr(p.status, FASA_DEV_NSEL_CLAMPED);
     p.n_sel[u] = plan.ktot;
   }
-  SelRow row;
-  row.scores = p.scores + (int64_t)u * p.max_len;
+  SelRow<Src> row;
+  row.src = src;
   row.lo = plan.lo;
   row.hi = plan.hi;
   row.k = plan.k;
   const int gs = row.k > 0 && row.k < row.hi - row.lo ? sel_group_shift(row.hi - row.lo, row.k, p.lay.gm_cap) : 0;
   float gm_lo = INFINITY, gm_hi = -INFINITY;
   if (gs > 0) {
-    // a warp takes 128 consecutive positions at a time, a lane four of them
+    // A thread takes eight consecutive positions: their maximum needs no other lane (groups of 32: two shuffles).
     float* gm = reinterpret_cast<float*>(rsm);
-    const int g0 = row.lo >> gs, first = (g0 << gs) & ~127;
-    const bool vec_ok = (reinterpret_cast<uintptr_t>(row.scores) & 15) == 0;
-    constexpr int UNR = 4, STEP = NT * 4;
-    auto group = [&](float4 v, int i) {
-      float m = max_nan(max_nan(v.x, v.y), max_nan(v.z, v.w));
-      m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 1));
-      if (gs == 5) {
-        m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 2));
-        m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 4));
-      }
-      const int g = (i >> gs) - g0;
-      if ((i & ((1 << gs) - 1)) == 0 && g >= 0 && i < row.hi) {
-        gm[g] = m;
-        gm_lo = fminf(gm_lo, m);
-        gm_hi = max_nan(gm_hi, m);
-      }
-    };
-    for (int w0 = first + (tid - lane) * 4; w0 < row.hi; w0 += STEP * UNR) {       // uniform over the warp
-      const int i0 = w0 + lane * 4;
-      float4 v[UNR];
-      if (vec_ok && w0 >= row.lo && w0 + STEP * (UNR - 1) + 128 <= row.hi) {        // whole blocks of plain positions
+    const int g0 = row.lo >> gs, first = g0 << gs;
+    const bool vec_ok = src.aligned();
+    constexpr int UNR = 2, STEP = NT * 8;
+    for (int w0 = first + (tid - lane) * 8; w0 < row.hi; w0 += STEP * UNR) {       // uniform over the warp
+      const int i0 = w0 + lane * 8;
+      float m[UNR];
+      if (vec_ok && w0 >= row.lo && w0 + STEP * (UNR - 1) + 256 <= row.hi) {        // plain positions only
+        float4 v[UNR][2];
 #pragma unroll
-        for (int j = 0; j < UNR; ++j) v[j] = __ldg(reinterpret_cast<const float4*>(row.scores + i0 + j * STEP));
+        for (int j = 0; j < UNR; ++j) {
+          v[j][0] = src.four(i0 + j * STEP);
+          v[j][1] = src.four(i0 + j * STEP + 4);
+        }
+#pragma unroll
+        for (int j = 0; j < UNR; ++j)
+          m[j] = max_nan(max_nan(v[j][0].x, v[j][0].y, v[j][0].z), max_nan(v[j][0].w, v[j][1].x, v[j][1].y), max_nan(v[j][1].z, v[j][1].w));
       } else {
 #pragma unroll
         for (int j = 0; j < UNR; ++j) {
-          const int i = i0 + j * STEP;
-          v[j] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-          if (vec_ok && i >= row.lo && i + 3 < row.hi) {
-            v[j] = __ldg(reinterpret_cast<const float4*>(row.scores + i));
-          } else {
-            if (i >= row.lo && i < row.hi) v[j].x = __ldg(row.scores + i);
-            if (i + 1 >= row.lo && i + 1 < row.hi) v[j].y = __ldg(row.scores + i + 1);
-            if (i + 2 >= row.lo && i + 2 < row.hi) v[j].z = __ldg(row.scores + i + 2);
-            if (i + 3 >= row.lo && i + 3 < row.hi) v[j].w = __ldg(row.scores + i + 3);
+          m[j] = -INFINITY;
+          for (int e = 0; e < 8; ++e) {
+            const int i = i0 + j * STEP + e;
+            if (i >= row.lo && i < row.hi) m[j] = max_nan(m[j], src(i));
           }
         }
       }
 #pragma unroll
-      for (int j = 0; j < UNR; ++j) group(v[j], i0 + j * STEP);
+      for (int j = 0; j < UNR; ++j) {
+        const int i = i0 + j * STEP;
+        if (gs == 5) {
+          m[j] = max_nan(m[j], __shfl_xor_sync(0xffffffffu, m[j], 1));
+          m[j] = max_nan(m[j], __shfl_xor_sync(0xffffffffu, m[j], 2));
+        }
+        if (i < row.hi && (gs == 3 || (lane & 3) == 0)) {
+          gm[(i >> gs) - g0] = m[j];
+          gm_lo = fminf(gm_lo, m[j]);
+          gm_hi = max_nan(gm_hi, m[j]);
+        }
+      }
     }
   }
   __syncthreads();
@@ -105,6 +99,36 @@ topk_row_kernel(const RowParams p) {
   sel_row<NT>(row, gs, gm_lo, gm_hi, sm, rsm, p.lay, [&](int r, int pos) { out[plan.sink + r] = pos; });
 }
 
+// CALIB: row r < 64 of a sample (sequence, query head) is FC r alone, computed from the channel pairs as it is read, row
+// 64 the full head: the 64 rows of the four to eight query heads of a KV head share 4 bytes per position and FC
+// instead of having 4 bytes each.
+template <int NT, bool CALIB>
+__global__ void __launch_bounds__(NT, 1024 / NT)
+topk_row_kernel(const RowParams p) {
+  extern __shared__ __align__(16) unsigned char rsm[];
+  __shared__ SelShared sm;
+  sel_begin<NT>(sm);
+  pdl_wait_for_predecessor();
+  pdl_release_successor();
+  const int b = blockIdx.x / p.rows_per_seq;
+  if constexpr (CALIB) {
+    const int sample = blockIdx.x / 65, fc = blockIdx.x - 65 * sample;
+    if (fc < 64) {
+      const int kv = sample / p.calib.group;        // (sequence, KV head)
+      const uint16_t* q = p.calib.q + (int64_t)sample * FASA_HEAD_DIM;
+      SelPairs src;
+      src.p = p.calib.pairs + ((int64_t)kv * 64 + fc) * p.calib.stride;
+      src.q0 = bf16_bits_to_f32(q[p.calib.pairing == 0 ? fc : 2 * fc]);
+      src.q1 = bf16_bits_to_f32(q[p.calib.pairing == 0 ? fc + 64 : 2 * fc + 1]);
+      topk_row<NT>(p, src, b, sm, rsm);
+    } else {
+      topk_row<NT>(p, SelScores{p.scores + (int64_t)sample * p.calib.stride}, b, sm, rsm);
+    }
+  } else {
+    topk_row<NT>(p, SelScores{p.scores + (int64_t)blockIdx.x * p.max_len}, b, sm, rsm);
+  }
+}
+
 }  // namespace
 
 // Longest row the kernel takes: its group maxima and their list must fit in shared memory.
@@ -114,12 +138,13 @@ bool fasa_topk_row_ok(const fasa_ctx* ctx) { return ctx->cfg.max_len <= kTopkRow
 
 int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget,
                              int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
-                             int n_recent, cudaStream_t stream, int q_len) {
+                             int n_recent, cudaStream_t stream, int q_len, const fasa_calib_rows* calib) {
   const fasa_config_t& c = ctx->cfg;
   RowParams p;
   p.scores = scores; p.seq_lens = seq_lens; p.idx = idx; p.n_sel = n_sel; p.status = ctx->d_status;
   p.rows_per_seq = rows_per_seq; p.max_len = c.max_len; p.n_sink = n_sink; p.n_recent = n_recent;
   p.budget = budget; p.n_sel_max = n_sel_max; p.q_len = q_len;
+  p.calib = calib ? *calib : fasa_calib_rows{};
   // Groups of 8 up to 65536 positions, groups of 32 beyond (16 KB + 8 KB to 64 KB + 32 KB of shared memory).
   const int by32 = (c.max_len >> 5) + 2, by8 = (c.max_len >> 3) + 2;
   p.lay.gm_cap = by32 > 8194 ? by32 : (by8 < 8194 ? by8 : 8194);
@@ -136,7 +161,8 @@ int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* 
   // Threads: a lone row ends soonest with many, a launch of many rows issues fewest instructions with few (every
   // warp scans the histograms) and needs all of them resident: 320 rows of 64 K took two rounds of 512 threads,
   // 38 us, and fit in one round of 256.
-  if (rows <= ctx->n_sm && c.max_len > 16384) return go(topk_row_kernel<1024>, 1024);
-  if (rows <= 2 * ctx->n_sm) return go(topk_row_kernel<512>, 512);
-  return go(topk_row_kernel<256>, 256);
+  if (calib) return go(topk_row_kernel<256, true>, 256);
+  if (rows <= ctx->n_sm && c.max_len > 16384) return go(topk_row_kernel<1024, false>, 1024);
+  if (rows <= 2 * ctx->n_sm) return go(topk_row_kernel<512, false>, 512);
+  return go(topk_row_kernel<256, false>, 256);
 }
