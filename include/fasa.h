@@ -279,6 +279,8 @@ int32_t fasa_sparse_decode_attn_static(fasa_ctx_t* ctx, const void* q, const voi
  * same hand-over happens, whatever the selection size, when the caches are page-locked host
  * memory and an index set serves more than four query heads (the cluster kernel would fetch
  * every row twice over the host link).
+ * A set per query head (select_heads = 1) with a workspace, rows of at least 2048 positions and many sets runs as two
+ * launches instead: one stream of the proxy that scores all heads of a KV head, then selection and attention.
  * Mode 0, and every configuration mode 1 cannot take: fasa_fc_score -> fasa_topk ->
  * fasa_sparse_decode_attn; scores and workspace are then required (INVALID_ARG if NULL).
  * Both modes select identical index sets; outputs agree to fp32 rounding.

@@ -4,6 +4,8 @@
 #include <vector>
 
 #include "fasa_common.cuh"
+#include "fasa_select.cuh"
+#include "fasa_stream.cuh"
 
 namespace {
 
@@ -235,15 +237,66 @@ fasa_split_plan fasa_plan_splits(const fasa_ctx* ctx, int n_upper, int units) {
   return p;
 }
 
-// The partial-result area is sized for the largest split count any call can use
-// (the bound at max_len for the fewest units a launch can have, one per KV head), so it does
-// not depend on the selection size.
+// Workspace: split-K partial results, then (sets per query head) what the two-launch step passes from its first half to
+// its second, a score row and a row of group maxima per index set.  The partial-result area is sized for the largest
+// split count any call can use (the bound at max_len for the fewest units a launch can have, one per KV head), so
+// nothing here depends on the selection size.
+static bool set_per_head(const fasa_ctx* ctx) { return ctx->sel_heads == 1 && ctx->group > 1; }
+struct fasa_ws {
+  size_t scores, gm, total;
+};
+static fasa_ws ws_layout(const fasa_ctx* ctx) {
+  const fasa_config_t& c = ctx->cfg;
+  const int n = split_count_bound(ctx, c.max_len, c.batch * c.n_kv_heads);
+  const size_t per_split = (size_t)c.batch * c.n_q_heads * (FASA_HEAD_DIM + 2) * sizeof(float), rows = set_per_head(ctx) ? (size_t)c.batch * ctx->n_sets : 0;
+  fasa_ws w;
+  w.scores = fasa_align_up(per_split * (size_t)n, 256) + 256;
+  w.gm = w.scores + fasa_align_up(rows * (size_t)c.max_len * sizeof(float), 256);
+  w.total = w.gm + fasa_align_up(rows * (size_t)fasa_stream_gm_stride(ctx) * sizeof(float), 256);
+  return w;
+}
 extern "C" int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max, size_t* out_bytes) {
   if (!ctx || !out_bytes || n_sel_max < 0) return FASA_ERR_INVALID_ARG;
-  const int n = split_count_bound(ctx, ctx->cfg.max_len, ctx->cfg.batch * ctx->cfg.n_kv_heads);
-  size_t per_split = (size_t)ctx->cfg.batch * ctx->cfg.n_q_heads * (FASA_HEAD_DIM + 2) * sizeof(float);
-  *out_bytes = fasa_align_up(per_split * (size_t)n, 256) + 256;
+  *out_bytes = ws_layout(ctx).total;
   return FASA_OK;
+}
+
+// Whether a step over index sets per query head runs as two launches (score stream, then selection and attention)
+// instead of the cluster kernel, which streams a KV head's proxy once per set.  Measured (32 / 8 heads): batch 4 at
+// 50 K 92 -> 43 us with 128 rows a set, 99 -> 58 us with 1024; batch 16 at 16 K 123 -> 66 and 153 -> 121 us; batch 4 at
+// 4 K 24 -> 19 us; 28 / 4 heads, batch 4 at 50 K 89 -> 33 us.  Few sets with long lists stay with the cluster kernel, whose
+// CTAs share one selection (batch 1 at 16 K, 1024 rows a set: 24 against 28 us), as do groups of two or three, where the
+// stream saves less (16 / 8 heads, batch 4 at 50 K: 40 against 42 us; batch 16 at 16 K: 71 -> 50 us), and rows shorter
+// than 2048, which are one launch whatever the batch.
+static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, const void* workspace) {
+  const fasa_config_t& c = ctx->cfg;
+  if (workspace == nullptr || !set_per_head(ctx) || c.max_len < 2048 || !fasa_select_attend_ok(ctx, n_sel_max)) return false;
+  const long long sets = (long long)c.batch * ctx->n_sets;
+  if (ctx->group < 4 ? sets < 192 : sets < 96 && n_sel_max > 512) return false;
+  return !(c.page_size == 0 && fasa_on_host(ctx, k_cache));
+}
+
+// The groups whose maxima the first half takes: those that suit a row of max_len.
+static int stream_group_shift(const fasa_ctx* ctx, int budget) {
+  const long long n = ctx->cfg.max_len, k = budget > 0 ? budget : ((long long)-budget * n + 999) / 1000;
+  return sel_group_shift((int)n, (int)(k < n ? k : n), 16386);
+}
+
+static int32_t two_launch_step(fasa_ctx* ctx, const void* q, const void* k_new, const void* v_new, void* k_cache, void* v_cache,
+                               void* proxy_k, const int32_t* seq_lens, int32_t budget, int32_t n_sel_max, float* scores,
+                               int32_t* idx, int32_t* n_sel, float* out, float* lse, void* workspace, float* out_mirror,
+                               cudaStream_t stream) {
+  const fasa_ws w = ws_layout(ctx);
+  fasa_stream_args a;
+  a.q = q; a.proxy_k = proxy_k; a.seq_lens = seq_lens;
+  a.scores = scores ? scores : (float*)((char*)workspace + w.scores);
+  a.gm = (float*)((char*)workspace + w.gm);
+  a.gs = stream_group_shift(ctx, budget);
+  a.k_new = k_new; a.v_new = v_new; a.k_cache = k_cache; a.v_cache = v_cache;
+  int32_t st = fasa_stream_launch(ctx, a, stream);
+  if (st != FASA_OK) return st;
+  return fasa_select_attend_launch(ctx, q, k_cache, v_cache, a.scores, a.gm, a.gs, seq_lens, budget, n_sel_max, idx, n_sel, out, lse,
+                                   out_mirror, k_new != nullptr, stream);
 }
 
 // The cluster kernel attends to groups of more than four query heads in two passes over the
@@ -277,6 +330,11 @@ extern "C" int32_t fasa_decode_step(fasa_ctx_t* ctx, const void* q, const void* 
         ((uintptr_t)v_cache & 15) || (scores && ((uintptr_t)scores & 3)))
       return FASA_ERR_INVALID_ARG;
     if (!fasa_pages_ready(ctx)) return FASA_ERR_INVALID_ARG;
+    if (two_launches(ctx, k_cache, n_sel_max, workspace)) {
+      if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;
+      return two_launch_step(ctx, q, nullptr, nullptr, const_cast<void*>(k_cache), const_cast<void*>(v_cache), const_cast<void*>(proxy_k),
+                             seq_lens, budget, n_sel_max, scores, idx, n_sel, out, lse, workspace, nullptr, (cudaStream_t)stream);
+    }
     if (fasa_attend_separately(ctx, n_sel_max, workspace) || fasa_host_rows_twice(ctx, k_cache, workspace)) {
       if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;   // (what the second launch would refuse)
       int32_t st2 = fasa_fused_launch(ctx, q, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores,
@@ -315,6 +373,12 @@ static int32_t append_decode_step_impl(fasa_ctx_t* ctx, const void* q, const voi
         (scores && ((uintptr_t)scores & 3)))
       return FASA_ERR_INVALID_ARG;
     if (!fasa_pages_ready(ctx)) return FASA_ERR_INVALID_ARG;
+    if (two_launches(ctx, k_cache, n_sel_max, workspace)) {
+      if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;
+      *mirrored = out_mirror != nullptr;
+      return two_launch_step(ctx, q, k_new, v_new, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores, idx, n_sel,
+                             out, lse, workspace, out_mirror, (cudaStream_t)stream);
+    }
     if (fasa_attend_separately(ctx, n_sel_max, workspace) || fasa_host_rows_twice(ctx, k_cache, workspace)) {
       if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;   // (what the second launch would refuse)
       int32_t st2 = fasa_fused_launch(ctx, q, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores,

@@ -19,6 +19,7 @@
 // launch: no partial result touches HBM, no second launch, no workspace.
 #include <mutex>
 
+#include "fasa_attn_core.cuh"
 #include "fasa_cluster_merge.cuh"
 #include "fasa_common.cuh"
 #include "fasa_launch.cuh"
@@ -284,69 +285,9 @@ decode_attn_kernel(const AttnParams p) {
 }
 
 // ---------------------------------------------------------------------------------------------
-// Tensor-core form.  With a GQA group of G query heads the two products of a decode step are
-// [rows x 128] . [128 x G] (logits) and [128 x rows] . [rows x G] (output, transposed): G <= 8
-// is exactly the N = 8 of mma.m16n8k16.  The scalar kernel above spends ~60 instructions per
-// K/V row per four heads and is bound by instruction issue (0.67 of the copy bandwidth at
-// G = 4, 0.3 at G = 7); here a warp handles 16 rows with 8 + 16 MMAs.
-//   - K and V rows go to shared memory with 16-byte cp.async copies (row stride padded by 16
-//     bytes, so ldmatrix reads them without bank conflicts);
-//   - logits: A = K tile via ldmatrix.x4, B = q (bf16, exact) in registers; the softmax scale
-//     is applied to the fp32 result;
-//   - online softmax per head on the accumulator fragment (a thread owns heads 2t, 2t+1 of
-//     rows g, g+8; row maxima and sums by xor-shuffles over g);
-//   - output: A = V^T via ldmatrix.x4.trans, B = P^T.  P is split into two bf16 terms
-//     (p = hi + lo, error 2^-17 p) because one bf16 term would cost up to 2^-9 |v| of the
-//     2e-3 tolerance; two MMAs per block.
+// Tensor-core form: see fasa_attn_core.cuh.
 constexpr int kMmaThreads = 128;
 constexpr int kMmaWarps = kMmaThreads / 32;
-constexpr int kRowPad = FASA_HEAD_DIM + 8;          // bf16 elements per staged row (272 bytes)
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-// The same through L1 ("cache all levels"): rows that live in page-locked HOST memory cross the
-// host link in full 128-byte requests this way, at twice the rate of the L2-only form (measured:
-// 50 vs 25 GB/s of a 55 GB/s link); for rows in HBM the L2-only form above is the faster one.
-__device__ __forceinline__ void cp_async16_ca(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// waits until at most N of this thread's committed groups are still in flight
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const void* row) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(row)));
-}
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], const void* row) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_addr(row)));
-}
-__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// round-to-nearest-even fp32 -> bf16 bits (finite inputs)
-__device__ __forceinline__ uint32_t f32_to_bf16_bits(float f) {
-  const uint32_t u = __float_as_uint(f);
-  return (u + 0x7fffu + ((u >> 16) & 1u)) >> 16;
-}
-
-struct MmaSmem {
-  uint16_t k[kMmaWarps][16][kRowPad];
-  uint16_t v[kMmaWarps][16][kRowPad];
-  uint16_t p_hi[kMmaWarps][8][16];                  // P^T: [head][row]
-  uint16_t p_lo[kMmaWarps][8][16];
-};
 
 // CLUSTER: the splits of a unit are the CTAs of one cluster (grid.x = cluster size) and merge
 // in the same launch; otherwise each split writes its partial result for the merge kernel.
@@ -356,15 +297,15 @@ struct MmaSmem {
 // link) followed by its dominant channels in proxy order (from the GPU-resident proxy); the
 // query operand is loaded in the same channel order, so the logits are the same dot products
 // summed in another order.
+// (CTAs per SM: six is what the 37 KB of staging memory per CTA allow; fewer where the registers do not)
 template <bool SPARSE, bool PAGED, bool CLUSTER, bool HOSTMEM = false, bool KSPLIT = false>
-__global__ void __launch_bounds__(kMmaThreads)
+__global__ void __launch_bounds__(kMmaThreads, KSPLIT || PAGED ? 4 : (CLUSTER || SPARSE ? 5 : 6))
 decode_attn_mma_kernel(const AttnParams p) {
   __shared__ ClusterMergeSmem s_merge;              // (CLUSTER only: written by the peers)
   pdl_wait_for_predecessor();
   pdl_release_successor();
   const int u = blockIdx.y;
   const SelUnit su = sel_unit(u, p.n_sets, p.group, p.n_q_heads, p.n_kv_heads);
-  const int h = su.h;
   const int b = su.b;
   int n;
   if (SPARSE) {
@@ -387,46 +328,15 @@ decode_attn_mma_kernel(const AttnParams p) {
   const int r1 = min(n, r0 + chunk);
 
   const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int g = lane >> 2, t = lane & 3;
-
   extern __shared__ __align__(16) unsigned char attn_smem_raw[];
-  MmaSmem& sm = *reinterpret_cast<MmaSmem*>(attn_smem_raw);
-
-  // B operand of the logits: q[head g][channels], bf16 as stored, for the 8 blocks of 16 channels
   uint32_t qb[8][2];
-  {
-    const uint16_t* qh = p.q + (su.q0 + (g < p.group ? g : 0)) * FASA_HEAD_DIM;
-    // position c of an assembled key row holds channel ndchan[c] (c < nd) or chan[c - nd]
-    auto q_at = [&](int c) -> uint32_t {
-      const int ch = c < p.ks.nd ? p.ks.ndchan[h * p.ks.nd + c] : p.ks.chan[h * p.ks.chunks * 8 + c - p.ks.nd];
-      return qh[ch];
-    };
-#pragma unroll
-    for (int kb = 0; kb < 8; ++kb) {
-      uint32_t w0, w1;
-      if constexpr (KSPLIT) {
-        w0 = q_at(kb * 16 + 2 * t) | (q_at(kb * 16 + 2 * t + 1) << 16);
-        w1 = q_at(kb * 16 + 2 * t + 8) | (q_at(kb * 16 + 2 * t + 9) << 16);
-      } else {
-        w0 = *reinterpret_cast<const uint32_t*>(qh + kb * 16 + 2 * t);
-        w1 = *reinterpret_cast<const uint32_t*>(qh + kb * 16 + 2 * t + 8);
-      }
-      qb[kb][0] = g < p.group ? w0 : 0u;
-      qb[kb][1] = g < p.group ? w1 : 0u;
-    }
-  }
-
-  float acc[8][4];                                  // out^T: [16-channel block][frag], heads 2t, 2t+1
-#pragma unroll
-  for (int cb = 0; cb < 8; ++cb) acc[cb][0] = acc[cb][1] = acc[cb][2] = acc[cb][3] = 0.f;
-  float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};
+  attn_load_query<KSPLIT>(qb, p, su, lane);
 
   const int32_t* irow = SPARSE ? p.idx + (int64_t)u * p.n_sel_max : nullptr;
 
   // The CTA's slice of the index list goes to shared memory in one coalesced read (checked
   // once): a tile then costs one memory round trip (its rows), not two (its indices first).
-  int32_t* s_idx = reinterpret_cast<int32_t*>(attn_smem_raw + sizeof(MmaSmem));
+  int32_t* s_idx = reinterpret_cast<int32_t*>(attn_smem_raw + sizeof(MmaSmem<kMmaWarps>));
   if (SPARSE) {
     for (int i = threadIdx.x; i < r1 - r0; i += kMmaThreads) {
       int tok = __ldg(irow + r0 + i);
@@ -446,196 +356,10 @@ decode_attn_mma_kernel(const AttnParams p) {
     __syncthreads();
   }
 
-  // Staging of a tile's 16 K rows (or V rows): lane l copies chunk (l % 16) of rows 2j + l / 16.
-  // The K and the V buffer of a warp are two pipeline stages: the next tile's K rows are
-  // requested as soon as this tile's logits are done (they travel during the output
-  // product), its V rows as soon as the output product is done (they travel during the next
-  // logits), so memory stays busy while the warp computes.  One cp.async group per buffer
-  // fill, an empty group when there is no next tile, so "all but the newest group" always
-  // names the buffer that is needed next.
-  const int bc = b / p.q_len;                       // the sequence whose cache this unit reads
-  const uint16_t* kunit = PAGED ? p.k : p.k + bc * p.ksb + h * p.ksh;
-  const uint16_t* vunit = PAGED ? p.v : p.v + bc * p.vsb + h * p.vsh;
-  auto stage = [&](uint16_t (*dst)[kRowPad], const uint16_t* unit, int64_t sb, int64_t sh, int64_t st, int base) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      const int row = 2 * j + (lane >> 4);
-      const int r = min(base + row, r1 - 1);        // rows past the end repeat the last one (masked below)
-      const int tok = SPARSE ? s_idx[r - r0] : r;
-      const int c8 = (lane & 15) * 8;
-      // (contiguous caches keep the plain address arithmetic: the page map costs registers)
-      if constexpr (PAGED) cp_async16(&dst[row][c8], unit + cache_row(p.pm, bc, h, tok, sb, sh, st, p.status) + c8);
-      else if constexpr (HOSTMEM) cp_async16_ca(&dst[row][c8], unit + (int64_t)tok * st + c8);
-      else cp_async16(&dst[row][c8], unit + (int64_t)tok * st + c8);
-    }
-  };
-  // Combine: the 16 key rows of a tile from their two homes
-  const ProxyGeom ks_pg = proxy_geom(KSPLIT ? p.ks.chunks : 1);
-  const unsigned char* ks_proxy = KSPLIT ? p.ks.proxy + (int64_t)su.kv * ((p.max_len + 15) >> 4) * ks_pg.tile_bytes : nullptr;
-  const uint16_t* res_rows = KSPLIT && p.ks.res.tags ? p.ks.res.rows + (int64_t)su.kv * p.ks.res.slots * 2 * FASA_HEAD_DIM : nullptr;
-  auto stage_split_k = [&](uint16_t (*dst)[kRowPad], int base) {
-    const int nd_chunks = p.ks.nd >> 3, words = 4 * p.ks.chunks;
-    for (int c = lane; c < 16 * nd_chunks; c += 32) {                 // the part that crosses the link
-      const int row = c / nd_chunks, ch = c % nd_chunks;
-      const int tok = s_idx[min(base + row, r1 - 1) - r0];
-      if (tok >= 0) cp_async16_ca(&dst[row][ch * 8], kunit + (int64_t)tok * p.kst + ch * 8);
-    }
-    for (int c = lane; c < 16 * words; c += 32) {                     // the dominant pairs, from the proxy
-      const int row = c / words, w = c % words;
-      const int tok = s_idx[min(base + row, r1 - 1) - r0];
-      if (tok >= 0) cp_async4(&dst[row][p.ks.nd + 2 * w], ks_proxy + proxy_word_offset(ks_pg, tok, w));
-    }
-    if (res_rows != nullptr) {                                        // resident rows: whole assembled key rows
-      for (int c = lane; c < 16 * 16; c += 32) {
-        const int row = c >> 4, ch = c & 15;
-        const int tok = s_idx[min(base + row, r1 - 1) - r0];
-        if (tok < 0) cp_async16(&dst[row][ch * 8], res_rows + (int64_t)(-1 - tok) * 2 * FASA_HEAD_DIM + ch * 8);
-      }
-    }
-  };
-  // value rows of a tile with a split key cache: from the host, or from the resident rows
-  auto stage_split_v = [&](uint16_t (*dst)[kRowPad], int base) {
-    for (int c = lane; c < 16 * 16; c += 32) {
-      const int row = c >> 4, ch = c & 15;
-      const int tok = s_idx[min(base + row, r1 - 1) - r0];
-      if (tok >= 0) cp_async16_ca(&dst[row][ch * 8], vunit + (int64_t)tok * p.vst + ch * 8);
-      else cp_async16(&dst[row][ch * 8], res_rows + (int64_t)(-1 - tok) * 2 * FASA_HEAD_DIM + FASA_HEAD_DIM + ch * 8);
-    }
-  };
-  auto stage_v = [&](int base) {
-    if constexpr (KSPLIT) stage_split_v(sm.v[warp], base);
-    else stage(sm.v[warp], vunit, p.vsb, p.vsh, p.vst, base);
-  };
-  auto stage_k = [&](int base) {
-    if constexpr (KSPLIT) stage_split_k(sm.k[warp], base);
-    else stage(sm.k[warp], kunit, p.ksb, p.ksh, p.kst, base);
-  };
-  constexpr int kTileStep = kMmaWarps * 16;
-  if (r0 + warp * 16 < r1) stage_k(r0 + warp * 16);
-  cp_async_commit();
-  if (r0 + warp * 16 < r1) stage_v(r0 + warp * 16);
-  cp_async_commit();
-
-  for (int base = r0 + warp * 16; base < r1; base += kTileStep) {   // uniform over the warp
-    const bool more = base + kTileStep < r1;
-    cp_async_wait<1>();                             // this tile's K rows have landed
-    __syncwarp();
-
-    // ---- logits: D[16 rows x 8 heads] ---------------------------------------------------------
-    float c[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-    for (int kb = 0; kb < 8; ++kb) {
-      uint32_t a[4];
-      // matrices: (rows 0-7, ch 0-7), (rows 8-15, ch 0-7), (rows 0-7, ch 8-15), (rows 8-15, ch 8-15)
-      ldmatrix_x4(a, &sm.k[warp][(lane & 7) + 8 * ((lane >> 3) & 1)][kb * 16 + 8 * (lane >> 4)]);
-      mma16816(c, a, qb[kb][0], qb[kb][1]);
-    }
-    // thread: c0, c1 = row g, heads 2t, 2t+1; c2, c3 = row g + 8
-    const bool ok_lo = base + g < r1, ok_hi = base + g + 8 < r1;
-    float lg[4];
-    lg[0] = ok_lo ? c[0] * p.scale_log2 : -INFINITY;
-    lg[1] = ok_lo ? c[1] * p.scale_log2 : -INFINITY;
-    lg[2] = ok_hi ? c[2] * p.scale_log2 : -INFINITY;
-    lg[3] = ok_hi ? c[3] * p.scale_log2 : -INFINITY;
-    float alpha[2];
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      float bm = fmaxf(lg[e], lg[2 + e]);
-      bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 4));
-      bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 8));
-      bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, 16));
-      const float m_new = fmaxf(m_run[e], bm);
-      const float m_safe = m_new == -INFINITY ? 0.f : m_new;
-      alpha[e] = exp2f(m_run[e] - m_safe);
-      lg[e] = exp2f(lg[e] - m_safe);
-      lg[2 + e] = exp2f(lg[2 + e] - m_safe);
-      l_run[e] = l_run[e] * alpha[e] + lg[e] + lg[2 + e];   // this thread's rows; the g lanes are added at the end
-      m_run[e] = m_new;
-    }
-    // P^T[head][row] as two bf16 terms
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int head = 2 * t + (e & 1), row = g + 8 * (e >> 1);
-      const uint32_t hi = f32_to_bf16_bits(lg[e]);
-      const float rest = lg[e] - __uint_as_float(hi << 16);
-      sm.p_hi[warp][head][row] = (uint16_t)hi;
-      sm.p_lo[warp][head][row] = (uint16_t)f32_to_bf16_bits(rest);
-    }
-    __syncwarp();                                   // P is visible; every lane is done with the K buffer
-    if (more) stage_k(base + kTileStep);
-    cp_async_commit();
-    cp_async_wait<1>();                             // this tile's V rows have landed
-    __syncwarp();
-    // B operand of the output product: B[k = row][n = head g]: rows 2t, 2t+1 and 2t+8, 2t+9
-    const uint32_t ph0 = *reinterpret_cast<const uint32_t*>(&sm.p_hi[warp][g][2 * t]);
-    const uint32_t ph1 = *reinterpret_cast<const uint32_t*>(&sm.p_hi[warp][g][2 * t + 8]);
-    const uint32_t pl0 = *reinterpret_cast<const uint32_t*>(&sm.p_lo[warp][g][2 * t]);
-    const uint32_t pl1 = *reinterpret_cast<const uint32_t*>(&sm.p_lo[warp][g][2 * t + 8]);
-
-    // ---- output: out^T[16 ch x 8 heads] += V^T[16 ch x 16 rows] . P^T[16 rows x 8 heads] ------
-#pragma unroll
-    for (int cb = 0; cb < 8; ++cb) {
-      acc[cb][0] *= alpha[0]; acc[cb][1] *= alpha[1]; acc[cb][2] *= alpha[0]; acc[cb][3] *= alpha[1];
-      uint32_t a[4];
-      // source blocks (token rows x channels), transposed on load:
-      // (rows 0-7, ch 0-7), (rows 0-7, ch 8-15), (rows 8-15, ch 0-7), (rows 8-15, ch 8-15)
-      ldmatrix_x4_trans(a, &sm.v[warp][(lane & 7) + 8 * (lane >> 4)][cb * 16 + 8 * ((lane >> 3) & 1)]);
-      mma16816(acc[cb], a, ph0, ph1);
-      mma16816(acc[cb], a, pl0, pl1);
-    }
-    __syncwarp();                                   // every lane is done with the V buffer
-    if (more) stage_v(base + kTileStep);
-    cp_async_commit();
-  }
-  cp_async_wait<0>();
-
-  // ---- this warp's (m, l, acc) per head; the g lanes add their sums -------------------------------
-#pragma unroll
-  for (int e = 0; e < 2; ++e) {
-    l_run[e] += __shfl_xor_sync(0xffffffffu, l_run[e], 4);
-    l_run[e] += __shfl_xor_sync(0xffffffffu, l_run[e], 8);
-    l_run[e] += __shfl_xor_sync(0xffffffffu, l_run[e], 16);
-  }
-  __syncthreads();                                  // staging memory becomes the combine area
-  float* s_acc = reinterpret_cast<float*>(attn_smem_raw);                 // [warps][8 heads][128]
-  float* s_ml = s_acc + kMmaWarps * 8 * FASA_HEAD_DIM;                    // [warps][8 heads][2]
-#pragma unroll
-  for (int cb = 0; cb < 8; ++cb) {
-    s_acc[(warp * 8 + 2 * t) * FASA_HEAD_DIM + cb * 16 + g] = acc[cb][0];
-    s_acc[(warp * 8 + 2 * t + 1) * FASA_HEAD_DIM + cb * 16 + g] = acc[cb][1];
-    s_acc[(warp * 8 + 2 * t) * FASA_HEAD_DIM + cb * 16 + g + 8] = acc[cb][2];
-    s_acc[(warp * 8 + 2 * t + 1) * FASA_HEAD_DIM + cb * 16 + g + 8] = acc[cb][3];
-  }
-  if (g == 0) {
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      s_ml[(warp * 8 + 2 * t + e) * 2 + 0] = m_run[e];
-      s_ml[(warp * 8 + 2 * t + e) * 2 + 1] = l_run[e];
-    }
-  }
-  __syncthreads();
-  const int cch = threadIdx.x;                      // one channel per thread
-  // (CLUSTER: this CTA's partial per head goes to shared memory behind the combine area)
-  float (*s_part)[kMergePartStride] = reinterpret_cast<float (*)[kMergePartStride]>(s_ml + kMmaWarps * 8 * 2);
-  for (int gl = 0; gl < p.group; ++gl) {
-    float mx = -INFINITY;
-#pragma unroll
-    for (int w = 0; w < kMmaWarps; ++w) mx = fmaxf(mx, s_ml[(w * 8 + gl) * 2]);
-    float a = 0.f, l = 0.f;
-#pragma unroll
-    for (int w = 0; w < kMmaWarps; ++w) {
-      const float ms = s_ml[(w * 8 + gl) * 2];
-      const float wt = ms == -INFINITY ? 0.f : exp2f(ms - mx);
-      a += wt * s_acc[(w * 8 + gl) * FASA_HEAD_DIM + cch];
-      l += wt * s_ml[(w * 8 + gl) * 2 + 1];
-    }
-    float* dst = CLUSTER ? &s_part[gl][0] : p.partial + ((su.q0 + gl) * p.n_splits + split) * kPartialStride;
-    dst[2 + cch] = a;
-    if (cch == 0) {
-      dst[0] = mx;
-      dst[1] = l;
-    }
-  }
+  float (*s_part)[kMergePartStride] = mma_part<kMmaWarps>(attn_smem_raw);
+  attn_rows<kMmaWarps, SPARSE, PAGED, HOSTMEM, KSPLIT>(p, su, b / p.q_len, qb, r0, r1, s_idx, attn_smem_raw, [&](int gl) {
+    return CLUSTER ? &s_part[gl][0] : p.partial + ((su.q0 + gl) * p.n_splits + split) * kPartialStride;
+  });
   if constexpr (CLUSTER) {
     __syncthreads();
     cg::cluster_group cluster = cg::this_cluster();
@@ -733,9 +457,7 @@ int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
   p.scale_log2 = c.softmax_scale * 1.4426950408889634f;
   dim3 grid((unsigned)plan.n_splits, (unsigned)(n_seq * n_sets));
   if (ctx->use_fused) {   // default: the tensor-core kernel (mode 0 keeps the scalar one)
-    static_assert(sizeof(MmaSmem) >= ((size_t)kMmaWarps * 8 * (FASA_HEAD_DIM + 2) + 8 * kMergePartStride) * sizeof(float),
-                  "combine area");
-    const int max_smem = (int)(sizeof(MmaSmem) + 2080 * sizeof(int32_t));
+    const int max_smem = (int)(sizeof(MmaSmem<kMmaWarps>) + 2080 * sizeof(int32_t));
     // One launch where the splits of a unit fit a portable cluster: the split count becomes a
     // power of two <= 8 (the nearest to the planned one) and the cluster merges by itself.
     int cs = 1;
@@ -748,7 +470,7 @@ int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
       auto fn = c.page_size > 0 ? decode_attn_mma_kernel<SPARSE, true, true> : decode_attn_mma_kernel<SPARSE, false, true>;
       if (host) fn = decode_attn_mma_kernel<SPARSE, false, true, true>;
       if constexpr (SPARSE) { if (ksplit) fn = decode_attn_mma_kernel<true, false, true, true, true>; }
-      const size_t smem = sizeof(MmaSmem) + (SPARSE ? (size_t)cchunk * sizeof(int32_t) : 0);
+      const size_t smem = sizeof(MmaSmem<kMmaWarps>) + (SPARSE ? (size_t)cchunk * sizeof(int32_t) : 0);
       FASA_CUDA_TRY(ctx, cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
       FASA_CUDA_TRY(ctx, launch_after_predecessor(fn, dim3((unsigned)cs, grid.y), dim3(kMmaThreads), smem, s, cs, p));
       FASA_LAUNCH_CHECK(ctx);
@@ -758,7 +480,7 @@ int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
     if (host) fn = decode_attn_mma_kernel<SPARSE, false, false, true>;
     if constexpr (SPARSE) { if (ksplit) fn = decode_attn_mma_kernel<true, false, false, true, true>; }
     // (+ the slice of the index list: chunk <= 2048 rows)
-    const size_t smem = sizeof(MmaSmem) + (SPARSE ? (size_t)plan.chunk * sizeof(int32_t) : 0);
+    const size_t smem = sizeof(MmaSmem<kMmaWarps>) + (SPARSE ? (size_t)plan.chunk * sizeof(int32_t) : 0);
     FASA_CUDA_TRY(ctx, cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
     FASA_CUDA_TRY(ctx, launch_after_predecessor(fn, grid, dim3(kMmaThreads), smem, s, 0, p));
   } else if (G == 1) decode_attn_kernel<1, 1, SPARSE><<<grid, kAttnThreads, 0, s>>>(p);

@@ -2,11 +2,10 @@
 // flash decoding: m* = max_s m_s, out = sum_s 2^(m_s - m*) acc_s / sum_s 2^(m_s - m*) l_s),
 // shared by the one-launch decode step and by the split-K attention kernel.
 //
-// CTA r of the cluster finishes outputs [r * per_o, (r + 1) * per_o) of the unit's
-// group * 128 outputs.  Every CTA PUSHES its partial values for those outputs into r's shared
-// memory (consecutive threads write consecutive words of one peer, so the distributed-shared-
-// memory traffic is a few wide transactions); after ONE cluster barrier r combines from local
-// memory only: no CTA reads a peer afterwards, so none has to wait for the others to leave.
+// CTA r of a cluster of cs finishes channels [r, r + 1) * 128 / cs of every head.  Every CTA PUSHES its partial
+// values for those into r's shared memory (consecutive threads write runs of consecutive words of one
+// peer, so the distributed-shared-memory traffic is a few wide transactions); after ONE cluster barrier r
+// combines from local memory only: no CTA reads a peer afterwards, so none has to wait for the others to leave.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -20,7 +19,7 @@ constexpr int kMergeMaxCs = 16;                        // CTAs per cluster at mo
 // when the first peer finishes its part.
 struct ClusterMergeSmem {
   float racc[FASA_MAX_GROUP * FASA_HEAD_DIM + kMergeMaxCs];   // [rank][per_o]: accumulators of this CTA's outputs
-  float rml[kMergeMaxCs][FASA_MAX_GROUP][2];                 // every CTA's (m, l) per head
+  alignas(8) float rml[kMergeMaxCs][FASA_MAX_GROUP][2];                 // every CTA's (m, l) per head
 };
 
 // part[g] = (m, l, acc[128]) of head g of this CTA, base-2 logit domain, complete and visible to
@@ -36,26 +35,34 @@ __device__ __forceinline__ void cluster_merge_store(cooperative_groups::cluster_
   const int tid = threadIdx.x;
   constexpr int GP = FASA_MAX_GROUP;
   const int n_out = group * FASA_HEAD_DIM;
-  const int per_o = (n_out + cs - 1) / cs;
+  if (cs == 1) {                              // nothing to merge
+    for (int o = tid; o < n_out; o += NT) {
+      const int g = o / FASA_HEAD_DIM, c = o % FASA_HEAD_DIM;
+      const float l = part[g][1], ov = l > 0.f ? part[g][2 + c] / l : 0.f;
+      out[q0 * FASA_HEAD_DIM + o] = ov;
+      if (out_mirror) out_mirror[q0 * FASA_HEAD_DIM + o] = ov;
+      if (lse && c == 0) lse[q0 + g] = l > 0.f ? (part[g][0] + log2f(l)) * 0.6931471805599453f : -INFINITY;
+    }
+    return;
+  }
+  const int lc = 31 - __clz(cs), lw = 7 - lc, cw = 1 << lw;   // channels of a head that a CTA finishes: 128 / cs = 1 << lw
+  const int per_o = group << lw;
   for (int o = tid; o < n_out; o += NT) {
-    const int r = o / per_o, ol = o % per_o;
-    float* dst = cluster.map_shared_rank(&sm.racc[0], r);
-    dst[crank * per_o + ol] = part[o / FASA_HEAD_DIM][2 + o % FASA_HEAD_DIM];
+    const int c = o % FASA_HEAD_DIM, g = o / FASA_HEAD_DIM;
+    float* dst = cluster.map_shared_rank(&sm.racc[0], c >> lw);
+    dst[crank * per_o + (g << lw) + (c & (cw - 1))] = part[g][2 + c];
   }
   for (int i = tid; i < cs * GP; i += NT) {
     const int r = i / GP, g = i % GP;
-    float* dst = cluster.map_shared_rank(&sm.rml[0][0][0], r);
-    dst[(crank * GP + g) * 2 + 0] = part[g][0];
-    dst[(crank * GP + g) * 2 + 1] = part[g][1];
+    if (g < group) *reinterpret_cast<float2*>(cluster.map_shared_rank(&sm.rml[crank][g][0], r)) = make_float2(part[g][0], part[g][1]);
   }
   cluster.sync();   // the merge barrier: every CTA's partial results have arrived
-  const int opp = NT / cs;                   // outputs per pass
-  const int r = tid % cs, tl = tid / cs;
+  const int opp = NT >> lc;                  // outputs per pass
+  const int r = tid & (cs - 1), tl = tid >> lc;
   for (int t0 = 0; t0 < per_o; t0 += opp) {  // uniform trip count
     const int t = t0 + tl;
-    const int o = crank * per_o + t;
-    const bool ok = t < per_o && o < n_out;
-    const int g = ok ? o / FASA_HEAD_DIM : 0;
+    const bool ok = t < per_o;
+    const int g = ok ? t >> lw : 0;
     const float ms = sm.rml[r][g][0], ls = sm.rml[r][g][1];
     const float as = ok ? sm.racc[r * per_o + t] : 0.f;
     float mx = ms;
@@ -67,7 +74,7 @@ __device__ __forceinline__ void cluster_merge_store(cooperative_groups::cluster_
       l += __shfl_xor_sync(0xffffffffu, l, off);
     }
     if (ok && r == 0) {
-      const int c = o % FASA_HEAD_DIM;
+      const int c = (crank << lw) + (t & (cw - 1));
       const int64_t hq = q0 + g;
       const float ov = l > 0.f ? av / l : 0.f;
       out[hq * FASA_HEAD_DIM + c] = ov;

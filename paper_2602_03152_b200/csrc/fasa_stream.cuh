@@ -1,0 +1,33 @@
+// The two halves of the two-launch decode step, for index sets per query head.
+#pragma once
+
+#include <type_traits>
+
+#include "fasa_common.cuh"
+
+// Floats per score row of the group-maxima buffer (groups of 8).
+int fasa_stream_gm_stride(const fasa_ctx* ctx);
+
+// First half: scores [batch][n_q_heads][max_len] (and maxima of groups of 1 << gs positions, gs > 0) of every cached
+// token; k_new != null: the appended token first.
+struct fasa_stream_args {
+  const void* q;
+  const void* proxy_k;
+  const int32_t* seq_lens;
+  float* scores;
+  float* gm;
+  int gs;
+  const void* k_new;
+  const void* v_new;
+  void* k_cache;
+  void* v_cache;
+};
+int32_t fasa_stream_launch(fasa_ctx* ctx, const fasa_stream_args& a, cudaStream_t stream);
+
+// Second half: selection and attention (append: of the grown sequences, whose lengths it stores); n_sel_max beyond
+// fasa_select_attend_ok is not taken.
+bool fasa_select_attend_ok(const fasa_ctx* ctx, int n_sel_max);
+int32_t fasa_select_attend_launch(fasa_ctx* ctx, const void* q, const void* k_cache, const void* v_cache, const float* scores,
+                                  const float* gm, int gs, const int32_t* seq_lens, int32_t budget, int32_t n_sel_max,
+                                  int32_t* idx, int32_t* n_sel, float* out, float* lse, float* out_mirror, bool append,
+                                  cudaStream_t stream);

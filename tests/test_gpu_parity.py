@@ -492,6 +492,59 @@ def test_index_sets_per_query_head_append_form(mode):
                       what="append+step, sets per head", **b.oracle_kwargs())
 
 
+@pytest.mark.parametrize("kw", [
+    dict(batch=3, max_len=2111, len_lo=70, len_hi=2110, budget=40, n_sink=3, n_recent=33),         # groups of 8, last pair of one tile
+    dict(batch=2, max_len=5000, len_lo=4990, len_hi=5000, budget=4),                               # groups of 32; a full sequence
+    dict(batch=3, max_len=3000, len_lo=900, len_hi=2990, budget=900, n_dom=3),                     # rows taken whole; an 8-channel block
+    dict(batch=2, n_q_heads=28, n_kv_heads=4, max_len=2500, len_lo=1, len_hi=2500, budget=-100, n_dom=13, pairing=1),   # group of 7
+    dict(batch=12, n_q_heads=16, n_kv_heads=8, max_len=2100, len_lo=1000, len_hi=2100, budget=64, n_dom=64),             # group of 2, 8 blocks
+    dict(batch=1, max_len=2048, len_lo=1500, len_hi=1500, budget=64, n_dom=32),
+])
+@pytest.mark.parametrize("page", [0, 32])
+def test_index_sets_per_query_head_in_two_launches(kw, page):
+    # the score stream + the select-and-attend kernel against the oracle, as a plain step and with an appended token; ragged
+    # lengths leave warps with shares that start and end inside a (sequence, KV head)
+    w = C["c1"].replace(**dict(dict(n_sink=0, n_recent=0, sel_heads=1), **kw))
+    t = synth.make_inputs(w, "cpu")
+    if page:
+        r, f, kp, vp, tab, table, need = _paged_twin(w, t, page, extra_tokens=1)
+        proxy = f.alloc_proxy()
+        f.proxy_build(kp, proxy, r.seq_lens)
+    else:
+        r = Run(w, t)
+        f, kp, vp = r.fasa, r.k, r.v
+        r.build_proxy()
+        proxy = r.proxy
+    n0 = f.launch_count()
+    f.decode_step(r.q, kp, vp, proxy, r.seq_lens, w.budget, r.scores, r.idx, r.n_sel, r.out, r.ws, r.lse)
+    torch.cuda.synchronize()
+    assert f.launch_count() - n0 == 2 and f.device_status() == 0
+    h = r.host()
+    parity.check_step(h["q"], h["k"], h["v"], h["seq_lens"], h["dom"], scores=h["scores"], idx=h["idx"], n_sel=h["n_sel"],
+                      out=h["out"], what="two launches", **r.oracle_kwargs())
+    for b, L in enumerate(h["seq_lens"].tolist()):
+        assert np.all(h["scores"][b, :, L:] == SENTINEL)
+    # the appended token: scored from its source, stored for the next step; a full sequence drops it
+    full = int((r.seq_lens >= w.max_len).sum()) > 0
+    lens = torch.clamp(r.seq_lens + 1, max=w.max_len).cpu()
+    s = synth.make_step_inputs(w, 3, "cuda")
+    r.reset_outputs()
+    f.append_decode_step(s["q"], s["k_new"], s["v_new"], kp, vp, proxy, r.seq_lens, w.budget, None, r.idx, r.n_sel, r.out, r.ws)
+    torch.cuda.synchronize()
+    assert torch.equal(r.seq_lens.cpu(), lens)
+    assert (f.device_status() & binding.DEV_APPEND_FULL != 0) == full
+    kl = _logical(kp, table, need, page, w.max_len) if page else kp
+    vl = _logical(vp, table, need, page, w.max_len) if page else vp
+    parity.check_step(s["q"].cpu().double().numpy(), kl.cpu().double().numpy(), vl.cpu().double().numpy(), lens.numpy(), h["dom"],
+                      idx=r.idx.cpu().numpy(), n_sel=r.n_sel.cpu().numpy(), out=r.out.cpu().numpy(), what="two launches, appended",
+                      **r.oracle_kwargs())
+    ref = f.alloc_proxy()
+    f.proxy_build(kp, ref, r.seq_lens)
+    px = [_logical(x.view(f.n_pages, w.n_kv_heads, page // 16, -1), table, need, page // 16, (w.max_len + 15) // 16) if page else x for x in (proxy, ref)]
+    for b, L in enumerate(lens.tolist()):
+        assert torch.equal(px[0][b, :, :L // 16], px[1][b, :, :L // 16])
+
+
 def test_index_sets_per_query_head_large_selection_and_static_scratch():
     # one head per set: the split route starts at n_sel_max >= 2048; the no-workspace variant agrees
     w = C["c1"].replace(batch=1, n_q_heads=8, n_kv_heads=2, max_len=6000, len_lo=5000, len_hi=6000, budget=2500,
