@@ -1034,6 +1034,11 @@ int fasa_fused_plan(fasa_ctx* ctx) {
       cudaGetLastError();
       continue;
     }
+    // A grid meant for one wave whose clusters do not all fit at once (a cluster lives on one GPC, so wide ones leave
+    // SMs over) would run a second round for the last few: half the cluster size instead.  Likewise the wide form below is
+    // taken only if it holds every unit or the narrow one does not either.  16 units at 25 K (wide clusters of 8, 14 or 15
+    // of them at once): 41.9 -> 22.8 us with 512-thread CTAs; at 60 K 50 -> 30 us; 36 units at 6 K 48 -> 26 us.
+    if (n_clusters < units && (long long)units * cs <= slots && cs > 1 && cap_of(cs / 2) <= kCapPair) continue;
     // the form without attention runs with the same cluster shape
     if (cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit) != cudaSuccess ||
         (cs > 8 && cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
@@ -1074,7 +1079,8 @@ int fasa_fused_plan(fasa_ctx* ctx) {
       int n_w = 0;
       if (cudaFuncSetAttribute((const void*)fw, cudaFuncAttributeMaxDynamicSharedMemorySize, limit_w) == cudaSuccess &&
           cudaFuncSetAttribute((const void*)fs, cudaFuncAttributeMaxDynamicSharedMemorySize, limit_w) == cudaSuccess &&
-          cudaOccupancyMaxActiveClusters(&n_w, (const void*)fw, &cw) == cudaSuccess && n_w >= 1) {
+          cudaOccupancyMaxActiveClusters(&n_w, (const void*)fw, &cw) == cudaSuccess && n_w >= 1 &&
+          (n_w >= units || n_clusters < units)) {
         ctx->step_threads = 1024;
         ctx->step_cs = cs_w;
         ctx->step_smem = smem_w;
