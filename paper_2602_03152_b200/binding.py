@@ -2,12 +2,15 @@
 
 Argument marshalling only: every step of the decode path runs in the library's
 kernels.  Tensors are torch CUDA tensors used as device memory; their data
-pointers are passed through unchanged.  There is no CPU fallback: if the shared
-object is missing or a call fails, an exception is raised.
+pointers are passed through unchanged.  Calls on the decode path go through the
+extension module `_marshal.so`, which checks and converts their arguments
+natively.  There is no CPU fallback: if a shared object is missing or a call
+fails, an exception is raised.
 """
 from __future__ import annotations
 
 import ctypes
+import importlib.util
 import os
 from typing import Optional
 
@@ -15,6 +18,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libfasa.so")
+MARSHAL_PATH = os.path.join(_PKG, "_marshal.so")
 
 OK, ERR_INVALID_ARG, ERR_UNSUPPORTED, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT = 0, -1, -2, -3, -4, -5
 DEV_LEN_CLAMPED, DEV_APPEND_FULL, DEV_IDX_CLAMPED, DEV_NSEL_CLAMPED, DEV_PAGE_CLAMPED, DEV_TIMEOUT = 1, 2, 4, 8, 16, 32
@@ -53,6 +57,8 @@ class FasaConfig(ctypes.Structure):
 
 
 _lib = None
+_invoke = None
+_address = {}          # entry point -> address
 
 
 def load_library() -> ctypes.CDLL:
@@ -110,8 +116,22 @@ def load_library() -> ctypes.CDLL:
     for name, (res, args) in sig.items():
         fn = getattr(lib, name)
         fn.restype, fn.argtypes = res, args
+        _address[name] = ctypes.cast(fn, ctypes.c_void_p).value
     _lib = lib
     return lib
+
+
+def _load_marshal():
+    """The extension module's call(function address, context address, kinds, *arguments)."""
+    global _invoke
+    if _invoke is None:
+        if not os.path.exists(MARSHAL_PATH):
+            raise FileNotFoundError(f"{MARSHAL_PATH} is missing: build it with `python -m paper_2602_03152_b200.build`")
+        spec = importlib.util.spec_from_file_location("_marshal", MARSHAL_PATH)
+        module = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(module)
+        _invoke = module.invoke
+    return _invoke
 
 
 def _dp(t: Optional[torch.Tensor], dtype=None) -> Optional[int]:
@@ -142,6 +162,7 @@ class Fasa:
                  group_reduce=0, n_sink=0, n_recent=0, softmax_scale=0.0, k_strides=(0, 0, 0),
                  v_strides=(0, 0, 0), select_heads=0, page_size=0, n_pages=0):
         self._lib = load_library()
+        _load_marshal()
         self._h = ctypes.c_void_p()
         dom = torch.as_tensor(dom, dtype=torch.int32).contiguous().cpu()
         n_dom = dom.shape[-1] if dom.dim() == 2 else 0
@@ -185,6 +206,13 @@ class Fasa:
             if st == ERR_CUDA:
                 detail += ": " + self._lib.fasa_last_cuda_error(self._h).decode()
             raise FasaError(st, where, detail)
+
+    def _call(self, name: str, kinds: str, *args):
+        """name(context, *args, current stream).  kinds, a letter per argument: n integer, p any tensor's pointer, u a
+        contiguous CUDA tensor, b / f / i / l one of bf16 / fp32 / int32 / int64; None is a null pointer."""
+        st = _invoke(_address[name], self._h.value, kinds, *args)
+        if st != OK:
+            self._check(st, name)
 
     # -- sizes ---------------------------------------------------------------
     def workspace_bytes(self, n_sel_max: int) -> int:
@@ -248,75 +276,44 @@ class Fasa:
 
     # -- the calls of include/fasa.h --------------------------------------------
     def kv_append(self, k_cache, v_cache, proxy_k, seq_lens, k_new, v_new):
-        n_new = k_new.shape[2]
-        self._check(self._lib.fasa_kv_append(self._h, k_cache.data_ptr(), v_cache.data_ptr(), _dp(proxy_k),
-                                             _dp(seq_lens, torch.int32), _dp(k_new, torch.bfloat16),
-                                             _dp(v_new, torch.bfloat16), n_new, _stream()), "fasa_kv_append")
+        self._call("fasa_kv_append", "ppuibbn", k_cache, v_cache, proxy_k, seq_lens, k_new, v_new, k_new.size(2))
 
     def proxy_build(self, k_cache, proxy_k, seq_lens):
-        self._check(self._lib.fasa_proxy_build(self._h, k_cache.data_ptr(), _dp(proxy_k),
-                                               _dp(seq_lens, torch.int32), _stream()), "fasa_proxy_build")
+        self._call("fasa_proxy_build", "pui", k_cache, proxy_k, seq_lens)
 
     def fc_score(self, q, proxy_k, seq_lens, scores):
-        self._check(self._lib.fasa_fc_score(self._h, _dp(q, torch.bfloat16), _dp(proxy_k),
-                                            _dp(seq_lens, torch.int32), _dp(scores, torch.float32), _stream()),
-                    "fasa_fc_score")
+        self._call("fasa_fc_score", "buif", q, proxy_k, seq_lens, scores)
 
     def topk(self, scores, seq_lens, budget, idx, n_sel, workspace=None):
-        n_sel_max = idx.shape[-1]
-        self._check(self._lib.fasa_topk(self._h, _dp(scores, torch.float32), _dp(seq_lens, torch.int32), budget,
-                                        n_sel_max, _dp(idx, torch.int32), _dp(n_sel, torch.int32), _dp(workspace),
-                                        _stream()), "fasa_topk")
+        self._call("fasa_topk", "finniiu", scores, seq_lens, budget, idx.size(-1), idx, n_sel, workspace)
 
     def sparse_decode_attn(self, q, k_cache, v_cache, idx, n_sel, out, workspace, lse=None):
-        n_sel_max = idx.shape[-1]
-        self._check(self._lib.fasa_sparse_decode_attn(self._h, _dp(q, torch.bfloat16), k_cache.data_ptr(),
-                                                      v_cache.data_ptr(), _dp(idx, torch.int32),
-                                                      _dp(n_sel, torch.int32), n_sel_max, _dp(out, torch.float32),
-                                                      _dp(lse), _dp(workspace), _stream()), "fasa_sparse_decode_attn")
+        self._call("fasa_sparse_decode_attn", "bppiinfuu", q, k_cache, v_cache, idx, n_sel, idx.size(-1), out, lse, workspace)
 
     def sparse_decode_attn_static(self, q, k_cache, v_cache, idx, n_sel, out, lse=None):
         """fasa_sparse_decode_attn for callers that cannot provide a workspace: the split-K
         partials go to a fixed array inside the library (no allocation anywhere).  Calls share
         that array, so keep them ordered on one stream."""
-        n_sel_max = idx.shape[-1]
-        self._check(self._lib.fasa_sparse_decode_attn_static(
-            self._h, _dp(q, torch.bfloat16), k_cache.data_ptr(), v_cache.data_ptr(), _dp(idx, torch.int32),
-            _dp(n_sel, torch.int32), n_sel_max, _dp(out, torch.float32), _dp(lse), _stream()),
-            "fasa_sparse_decode_attn_static")
+        self._call("fasa_sparse_decode_attn_static", "bppiinfu", q, k_cache, v_cache, idx, n_sel, idx.size(-1), out, lse)
 
     def full_decode_attn(self, q, k_cache, v_cache, seq_lens, out, workspace, lse=None):
-        self._check(self._lib.fasa_full_decode_attn(self._h, _dp(q, torch.bfloat16), k_cache.data_ptr(),
-                                                    v_cache.data_ptr(), _dp(seq_lens, torch.int32),
-                                                    _dp(out, torch.float32), _dp(lse), _dp(workspace), _stream()),
-                    "fasa_full_decode_attn")
+        self._call("fasa_full_decode_attn", "bppifuu", q, k_cache, v_cache, seq_lens, out, lse, workspace)
 
     def decode_step(self, q, k_cache, v_cache, proxy_k, seq_lens, budget, scores, idx, n_sel, out, workspace=None,
                     lse=None):
-        n_sel_max = idx.shape[-1]
-        self._check(self._lib.fasa_decode_step(self._h, _dp(q, torch.bfloat16), k_cache.data_ptr(),
-                                               v_cache.data_ptr(), _dp(proxy_k), _dp(seq_lens, torch.int32), budget,
-                                               n_sel_max, _dp(scores, torch.float32), _dp(idx, torch.int32),
-                                               _dp(n_sel, torch.int32), _dp(out, torch.float32), _dp(lse),
-                                               _dp(workspace), _stream()), "fasa_decode_step")
+        self._call("fasa_decode_step", "bppuinnfiifuu", q, k_cache, v_cache, proxy_k, seq_lens, budget, idx.size(-1),
+                   scores, idx, n_sel, out, lse, workspace)
 
     def append_decode_step(self, q, k_new, v_new, k_cache, v_cache, proxy_k, seq_lens, budget, scores, idx, n_sel,
                            out, workspace=None, lse=None):
         """Append one token per sequence, then the decode step on the grown cache (one launch in mode 1)."""
-        n_sel_max = idx.shape[-1]
-        self._check(self._lib.fasa_append_decode_step(
-            self._h, _dp(q, torch.bfloat16), _dp(k_new, torch.bfloat16), _dp(v_new, torch.bfloat16),
-            k_cache.data_ptr(), v_cache.data_ptr(), _dp(proxy_k), _dp(seq_lens, torch.int32), budget, n_sel_max,
-            _dp(scores, torch.float32), _dp(idx, torch.int32), _dp(n_sel, torch.int32), _dp(out, torch.float32),
-            _dp(lse), _dp(workspace), _stream()), "fasa_append_decode_step")
+        self._call("fasa_append_decode_step", "bbbppuinnfiifuu", q, k_new, v_new, k_cache, v_cache, proxy_k, seq_lens,
+                   budget, idx.size(-1), scores, idx, n_sel, out, lse, workspace)
 
     def select_step(self, q, k_cache, v_cache, proxy_k, seq_lens, budget, scores, idx, n_sel, k_new=None, v_new=None):
         """Scoring and selection in one launch, no attention (appending form when k_new / v_new are given)."""
-        n_sel_max = idx.shape[-1]
-        self._check(self._lib.fasa_select_step(
-            self._h, _dp(q, torch.bfloat16), _dp(k_new, torch.bfloat16), _dp(v_new, torch.bfloat16),
-            k_cache.data_ptr(), v_cache.data_ptr(), _dp(proxy_k), _dp(seq_lens, torch.int32), budget, n_sel_max,
-            _dp(scores, torch.float32), _dp(idx, torch.int32), _dp(n_sel, torch.int32), _stream()), "fasa_select_step")
+        self._call("fasa_select_step", "bbbppuinnfii", q, k_new, v_new, k_cache, v_cache, proxy_k, seq_lens, budget,
+                   idx.size(-1), scores, idx, n_sel)
 
     # -- memory-optimised variant with a split key cache (Algorithm 2) -----------------
     def alloc_host_nondom(self) -> torch.Tensor:
@@ -328,27 +325,19 @@ class Fasa:
         return t
 
     def m_split(self, k_cache, k_nondom, seq_lens):
-        self._check(self._lib.fasa_m_split(self._h, k_cache.data_ptr(), k_nondom.data_ptr(), _dp(seq_lens, torch.int32), _stream()),
-                    "fasa_m_split")
+        self._call("fasa_m_split", "ppi", k_cache, k_nondom, seq_lens)
 
     def m_kv_append(self, k_nondom, v_cache, proxy_k, seq_lens, k_new, v_new):
-        self._check(self._lib.fasa_m_kv_append(self._h, k_nondom.data_ptr(), v_cache.data_ptr(), _dp(proxy_k), _dp(seq_lens, torch.int32),
-                                               _dp(k_new, torch.bfloat16), _dp(v_new, torch.bfloat16), k_new.shape[2], _stream()),
-                    "fasa_m_kv_append")
+        self._call("fasa_m_kv_append", "ppuibbn", k_nondom, v_cache, proxy_k, seq_lens, k_new, v_new, k_new.size(2))
 
     def m_sparse_decode_attn(self, q, k_nondom, v_cache, proxy_k, idx, n_sel, out, workspace, lse=None):
-        self._check(self._lib.fasa_m_sparse_decode_attn(self._h, _dp(q, torch.bfloat16), k_nondom.data_ptr(), v_cache.data_ptr(),
-                                                        _dp(proxy_k), _dp(idx, torch.int32), _dp(n_sel, torch.int32), idx.shape[-1],
-                                                        _dp(out, torch.float32), _dp(lse), _dp(workspace), _stream()),
-                    "fasa_m_sparse_decode_attn")
+        self._call("fasa_m_sparse_decode_attn", "bppuiinfuu", q, k_nondom, v_cache, proxy_k, idx, n_sel, idx.size(-1),
+                   out, lse, workspace)
 
     def m_decode_step(self, q, k_nondom, v_cache, proxy_k, seq_lens, budget, scores, idx, n_sel, out, workspace, lse=None,
                       k_new=None, v_new=None):
-        self._check(self._lib.fasa_m_decode_step(
-            self._h, _dp(q, torch.bfloat16), _dp(k_new, torch.bfloat16), _dp(v_new, torch.bfloat16), k_nondom.data_ptr(),
-            v_cache.data_ptr(), _dp(proxy_k), _dp(seq_lens, torch.int32), budget, idx.shape[-1], _dp(scores, torch.float32),
-            _dp(idx, torch.int32), _dp(n_sel, torch.int32), _dp(out, torch.float32), _dp(lse), _dp(workspace), _stream()),
-            "fasa_m_decode_step")
+        self._call("fasa_m_decode_step", "bbbppuinnfiifuu", q, k_new, v_new, k_nondom, v_cache, proxy_k, seq_lens, budget,
+                   idx.size(-1), scores, idx, n_sel, out, lse, workspace)
 
     def alloc_resident(self) -> torch.Tensor:
         """Device buffer for the GPU-resident sink / recent rows of the memory-optimised variant, registered."""
@@ -365,30 +354,22 @@ class Fasa:
         self._resident = buf                       # (kept by reference in the library)
 
     def m_resident_build(self, k_nondom, v_cache, proxy_k, seq_lens):
-        self._check(self._lib.fasa_m_resident_build(self._h, k_nondom.data_ptr(), v_cache.data_ptr(), _dp(proxy_k),
-                                                    _dp(seq_lens, torch.int32), _stream()), "fasa_m_resident_build")
+        self._call("fasa_m_resident_build", "ppui", k_nondom, v_cache, proxy_k, seq_lens)
 
     # -- blocks of query tokens: tensors carry a query axis after the batch axis ------
     def fc_score_batched(self, q, proxy_k, seq_lens, scores):
-        self._check(self._lib.fasa_fc_score_batched(self._h, _dp(q, torch.bfloat16), _dp(proxy_k), _dp(seq_lens, torch.int32),
-                                                    q.shape[1], _dp(scores, torch.float32), _stream()), "fasa_fc_score_batched")
+        self._call("fasa_fc_score_batched", "buinf", q, proxy_k, seq_lens, q.size(1), scores)
 
     def topk_batched(self, scores, seq_lens, budget, idx, n_sel):
-        self._check(self._lib.fasa_topk_batched(self._h, _dp(scores, torch.float32), _dp(seq_lens, torch.int32), scores.shape[1],
-                                                budget, idx.shape[-1], _dp(idx, torch.int32), _dp(n_sel, torch.int32), _stream()),
-                    "fasa_topk_batched")
+        self._call("fasa_topk_batched", "finnnii", scores, seq_lens, scores.size(1), budget, idx.size(-1), idx, n_sel)
 
     def sparse_decode_attn_batched(self, q, k_cache, v_cache, idx, n_sel, out, workspace, lse=None):
-        self._check(self._lib.fasa_sparse_decode_attn_batched(
-            self._h, _dp(q, torch.bfloat16), k_cache.data_ptr(), v_cache.data_ptr(), _dp(idx, torch.int32),
-            _dp(n_sel, torch.int32), q.shape[1], idx.shape[-1], _dp(out, torch.float32), _dp(lse), _dp(workspace), _stream()),
-            "fasa_sparse_decode_attn_batched")
+        self._call("fasa_sparse_decode_attn_batched", "bppiinnfuu", q, k_cache, v_cache, idx, n_sel, q.size(1), idx.size(-1),
+                   out, lse, workspace)
 
     def decode_step_batched(self, q, k_cache, v_cache, proxy_k, seq_lens, budget, scores, idx, n_sel, out, workspace, lse=None):
-        self._check(self._lib.fasa_decode_step_batched(
-            self._h, _dp(q, torch.bfloat16), k_cache.data_ptr(), v_cache.data_ptr(), _dp(proxy_k), _dp(seq_lens, torch.int32),
-            q.shape[1], budget, idx.shape[-1], _dp(scores, torch.float32), _dp(idx, torch.int32), _dp(n_sel, torch.int32),
-            _dp(out, torch.float32), _dp(lse), _dp(workspace), _stream()), "fasa_decode_step_batched")
+        self._call("fasa_decode_step_batched", "bppuinnnfiifuu", q, k_cache, v_cache, proxy_k, seq_lens, q.size(1), budget,
+                   idx.size(-1), scores, idx, n_sel, out, lse, workspace)
 
     # -- offline calibration (Algorithm 1) ---------------------------------------
     def calib_workspace_bytes(self, top_k: int) -> int:
@@ -399,10 +380,7 @@ class Fasa:
     def calib_accumulate(self, q, k_cache, seq_lens, top_k, ca_counts, n_used, workspace):
         """Adds this batch's top_k * CA sums (Eq. 4) to ca_counts [n_q_heads, 64] and the sample
         numbers to n_used [n_q_heads] (int64 CUDA tensors carried from call to call)."""
-        self._check(self._lib.fasa_calib_accumulate(self._h, _dp(q, torch.bfloat16), k_cache.data_ptr(),
-                                                    _dp(seq_lens, torch.int32), top_k, _dp(ca_counts, torch.int64),
-                                                    _dp(n_used, torch.int64), _dp(workspace), _stream()),
-                    "fasa_calib_accumulate")
+        self._call("fasa_calib_accumulate", "bpinllu", q, k_cache, seq_lens, top_k, ca_counts, n_used, workspace)
 
     def decode_step_host(self, q_host, k_new_host, v_new_host, dev_stage, k_cache, v_cache, proxy_k, seq_lens,
                          budget, scores, idx, n_sel, out, out_host, workspace):
