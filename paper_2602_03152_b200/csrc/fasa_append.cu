@@ -1,6 +1,7 @@
 // Cache update: K/V rows plus the packed dominant-FC proxy rows (Algorithm 2: Split,
 // UpdateCache), and the one-off proxy build from an existing key cache.
 #include "fasa_common.cuh"
+#include "fasa_launch.cuh"
 #include "fasa_score_core.cuh"
 
 namespace {
@@ -44,14 +45,18 @@ __device__ __forceinline__ RowDst row_dst(const PageMap& m, int b, int h, int n_
 // 128 threads per appended row: 16 copy the K row, 16 the V row (16 bytes each), up to 64
 // write the proxy words (one dominant FC = one 4-byte channel pair each) to their places in
 // the tiled proxy layout.
+// (The pointers that another kernel may have written carry no __restrict__ here and in the other kernels that wait for
+// their predecessor inside the kernel: a load through the read-only path could move ahead of that wait.)
 __global__ void __launch_bounds__(256)
-kv_append_kernel(uint16_t* __restrict__ k_cache, uint16_t* __restrict__ v_cache,
-                 unsigned char* __restrict__ proxy, const int32_t* seq_lens /* same memory as seq_lens_w */,
-                 const uint16_t* __restrict__ k_new, const uint16_t* __restrict__ v_new,
+kv_append_kernel(uint16_t* k_cache, uint16_t* v_cache,
+                 unsigned char* proxy, const int32_t* seq_lens /* same memory as seq_lens_w */,
+                 const uint16_t* k_new, const uint16_t* v_new,
                  const int16_t* __restrict__ chan, int32_t* __restrict__ status, int n_rows,
                  int n_new, int n_kv_heads, int max_len, int chunks, int64_t ksb, int64_t ksh,
                  int64_t kst, int64_t vsb, int64_t vsh, int64_t vst, int32_t* seq_lens_w,
                  int32_t* arrive, const PageMap pm) {
+  pdl_wait_for_predecessor();
+  pdl_release_successor();
   const int row = blockIdx.x * 2 + (threadIdx.x >> 7);
   const bool live = row < n_rows;
   const int t = threadIdx.x & 127;
@@ -109,12 +114,14 @@ kv_append_kernel(uint16_t* __restrict__ k_cache, uint16_t* __restrict__ v_cache,
 constexpr int kBulkRows = 16;
 template <bool APPEND, bool PAGED>
 __global__ void __launch_bounds__(256)
-bulk_rows_kernel(uint16_t* k_cache, uint16_t* __restrict__ v_cache, unsigned char* __restrict__ proxy,
-                 const int32_t* seq_lens /* same memory as seq_lens_w */, const uint16_t* __restrict__ k_new,
-                 const uint16_t* __restrict__ v_new, const int16_t* __restrict__ chan,
+bulk_rows_kernel(uint16_t* k_cache, uint16_t* v_cache, unsigned char* proxy,
+                 const int32_t* seq_lens /* same memory as seq_lens_w */, const uint16_t* k_new,
+                 const uint16_t* v_new, const int16_t* __restrict__ chan,
                  int32_t* __restrict__ status, int n_new, int n_kv_heads, int max_len, int chunks,
                  int64_t ksb, int64_t ksh, int64_t kst, int64_t vsb, int64_t vsh, int64_t vst,
                  int32_t* seq_lens_w, int32_t* arrive, const PageMap pm_arg) {
+  pdl_wait_for_predecessor();
+  pdl_release_successor();
   const PageMap pm = PAGED ? pm_arg : PageMap{nullptr, 0, 0, 0};   // contiguous: the translation folds away
   __shared__ __align__(16) uint16_t s_k[kBulkRows][FASA_HEAD_DIM];
   const int u = blockIdx.y;
@@ -148,9 +155,9 @@ bulk_rows_kernel(uint16_t* k_cache, uint16_t* __restrict__ v_cache, unsigned cha
       const uint16_t* ksrc = APPEND ? k_new + ((int64_t)u * n_new + n0 + r) * FASA_HEAD_DIM : k_cache + d.k;
       kx = *reinterpret_cast<const uint4*>(ksrc + c8);
       if (APPEND) {
+        const uint4 vx = *reinterpret_cast<const uint4*>(v_new + ((int64_t)u * n_new + n0 + r) * FASA_HEAD_DIM + c8);
         *reinterpret_cast<uint4*>(k_cache + d.k + c8) = kx;
-        *reinterpret_cast<uint4*>(v_cache + d.v + c8) =
-            *reinterpret_cast<const uint4*>(v_new + ((int64_t)u * n_new + n0 + r) * FASA_HEAD_DIM + c8);
+        *reinterpret_cast<uint4*>(v_cache + d.v + c8) = vx;
       }
     }
   }
@@ -189,17 +196,17 @@ extern "C" int32_t fasa_kv_append(fasa_ctx_t* ctx, void* k_cache, void* v_cache,
   if (n_new >= kBulkRows) {
     dim3 grid((unsigned)((n_new + kBulkRows - 1) / kBulkRows), (unsigned)(c.batch * c.n_kv_heads));
     auto bulk = c.page_size > 0 ? bulk_rows_kernel<true, true> : bulk_rows_kernel<true, false>;
-    bulk<<<grid, 256, 0, s>>>(
-        (uint16_t*)k_cache, (uint16_t*)v_cache, (unsigned char*)proxy_k, seq_lens, (const uint16_t*)k_new,
-        (const uint16_t*)v_new, ctx->d_chan, ctx->d_status, n_new, c.n_kv_heads, c.max_len, ctx->chunks,
+    FASA_CUDA_TRY(ctx, launch_after_predecessor(
+        bulk, grid, dim3(256), (size_t)0, s, 0, (uint16_t*)k_cache, (uint16_t*)v_cache, (unsigned char*)proxy_k, seq_lens, (const uint16_t*)k_new,
+        (const uint16_t*)v_new, (const int16_t*)ctx->d_chan, ctx->d_status, (int)n_new, (int)c.n_kv_heads, (int)c.max_len, ctx->chunks,
         c.k_stride_b, c.k_stride_h, c.k_stride_t, c.v_stride_b, c.v_stride_h, c.v_stride_t, seq_lens, ctx->d_arrive,
-        fasa_page_map(ctx));
+        fasa_page_map(ctx)));
   } else {
-    kv_append_kernel<<<(unsigned)((n_rows + 1) / 2), 256, 0, s>>>(
-        (uint16_t*)k_cache, (uint16_t*)v_cache, (unsigned char*)proxy_k, seq_lens, (const uint16_t*)k_new,
-        (const uint16_t*)v_new, ctx->d_chan, ctx->d_status, (int)n_rows, n_new, c.n_kv_heads,
-        c.max_len, ctx->chunks, c.k_stride_b, c.k_stride_h, c.k_stride_t, c.v_stride_b,
-        c.v_stride_h, c.v_stride_t, seq_lens, ctx->d_arrive, fasa_page_map(ctx));
+    FASA_CUDA_TRY(ctx, launch_after_predecessor(
+        kv_append_kernel, dim3((unsigned)((n_rows + 1) / 2)), dim3(256), (size_t)0, s, 0, (uint16_t*)k_cache, (uint16_t*)v_cache, (unsigned char*)proxy_k, seq_lens, (const uint16_t*)k_new,
+        (const uint16_t*)v_new, (const int16_t*)ctx->d_chan, ctx->d_status, (int)n_rows, (int)n_new, (int)c.n_kv_heads,
+        (int)c.max_len, ctx->chunks, c.k_stride_b, c.k_stride_h, c.k_stride_t, c.v_stride_b,
+        c.v_stride_h, c.v_stride_t, seq_lens, ctx->d_arrive, fasa_page_map(ctx)));
   }
   FASA_LAUNCH_CHECK(ctx);
   return FASA_OK;
@@ -212,10 +219,11 @@ extern "C" int32_t fasa_proxy_build(fasa_ctx_t* ctx, const void* k_cache, void* 
   const fasa_config_t& c = ctx->cfg;
   dim3 grid((unsigned)((c.max_len + kBulkRows - 1) / kBulkRows), (unsigned)(c.batch * c.n_kv_heads));
   auto build = c.page_size > 0 ? bulk_rows_kernel<false, true> : bulk_rows_kernel<false, false>;
-  build<<<grid, 256, 0, (cudaStream_t)stream>>>(
-      const_cast<uint16_t*>((const uint16_t*)k_cache), nullptr, (unsigned char*)proxy_k, seq_lens, nullptr, nullptr,
-      ctx->d_chan, ctx->d_status, 0, c.n_kv_heads, c.max_len, ctx->chunks, c.k_stride_b, c.k_stride_h,
-      c.k_stride_t, 0, 0, 0, nullptr, nullptr, fasa_page_map(ctx));
+  FASA_CUDA_TRY(ctx, launch_after_predecessor(
+      build, grid, dim3(256), (size_t)0, (cudaStream_t)stream, 0, const_cast<uint16_t*>((const uint16_t*)k_cache), (uint16_t*)nullptr,
+      (unsigned char*)proxy_k, seq_lens, (const uint16_t*)nullptr, (const uint16_t*)nullptr, (const int16_t*)ctx->d_chan, ctx->d_status, 0,
+      (int)c.n_kv_heads, (int)c.max_len, ctx->chunks, c.k_stride_b, c.k_stride_h, c.k_stride_t, (int64_t)0, (int64_t)0, (int64_t)0,
+      (int32_t*)nullptr, (int32_t*)nullptr, fasa_page_map(ctx)));
   FASA_LAUNCH_CHECK(ctx);
   return FASA_OK;
 }

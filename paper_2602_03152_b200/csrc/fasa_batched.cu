@@ -34,6 +34,7 @@
 #include <type_traits>
 
 #include "fasa_common.cuh"
+#include "fasa_launch.cuh"
 #include "fasa_score_core.cuh"
 
 namespace {
@@ -105,6 +106,8 @@ fc_score_batched_kernel(const BatchedParams p) {
   const SelUnit su = sel_unit(u, p.n_sets, p.group, p.n_q_heads, p.n_kv_heads);
   const int b = su.b, h = su.h;
   const int hs = u % p.n_sets;
+  pdl_wait_for_predecessor();
+  pdl_release_successor();
   const int len = clamp_len(p.seq_lens[b], p.max_len, p.status);
   const int mt0 = blockIdx.x * p.tiles_per_cta;
   const int mt1 = min(min((p.max_len + kBM - 1) / kBM, mt0 + p.tiles_per_cta), (len + kBM - 1) / kBM);
@@ -329,8 +332,7 @@ extern "C" int32_t fasa_fc_score_batched(fasa_ctx_t* ctx, const void* q, const v
   auto go = [&](auto fn) -> cudaError_t {
     cudaError_t e = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
     if (e != cudaSuccess) return e;
-    fn<<<grid, kBT, smem, (cudaStream_t)stream>>>(p);
-    return cudaGetLastError();
+    return launch_after_predecessor(fn, grid, dim3(kBT), smem, (cudaStream_t)stream, 0, p);
   };
   const bool mx = c.group_reduce != 0;
   const int kb_of = nb <= 1 ? 1 : (nb <= 2 ? 2 : (nb <= 4 ? 4 : 8));

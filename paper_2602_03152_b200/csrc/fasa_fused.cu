@@ -40,6 +40,7 @@
 
 #include "fasa_cluster_merge.cuh"
 #include "fasa_common.cuh"
+#include "fasa_launch.cuh"
 #include "fasa_score_core.cuh"
 
 namespace cg = cooperative_groups;
@@ -110,6 +111,7 @@ struct FusedParams {
   unsigned char* proxy_w;
   int32_t* seq_lens_w;
   int32_t* arrive;
+  int early;               // at most one CTA per SM, all resident at once: launched early, and lets its successor be
   int shift_clusters, shift_ctas;   // phase shift of grids that run in rounds: clusters / CTAs resident at once (0: none)
   float* scores;           // nullable
   int32_t* idx;
@@ -199,6 +201,20 @@ fused_decode_kernel(const FusedParams p) {
   __shared__ int16_t s_chan[8 * FASA_MAX_DOM / 4];               // the head's channel table
   __shared__ ClusterMergeSmem s_merge;                            // pushed by the cluster: the partial results this CTA finishes
 
+  const int cap = (((p.max_len + cs - 1) / cs) + 31) & ~31;
+  const FusedSmem sl = fused_smem_layout(cap, kFW);
+  uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw + sl.keys);
+  uint32_t* hist0 = reinterpret_cast<uint32_t*>(smem_raw + sl.hist0);
+  uint32_t* hist1 = reinterpret_cast<uint32_t*>(smem_raw + sl.hist1);
+  uint32_t* s_mask = reinterpret_cast<uint32_t*>(smem_raw + sl.mask);
+  for (int i = tid; i < kFBins; i += kFT) { hist0[i] = 0u; hist1[i] = 0u; }
+  for (int i = tid; i < 3 * kFinBins; i += kFT) (&s_fin[0][0])[i] = 0u;
+  for (int i = tid; i < 3 * 2 * kGroups; i += kFT) (&s_gsum[0][0][0])[i] = 0u;
+  for (int i = tid; i < 3 * 2 * 32; i += kFT) (&s_fine[0][0][0])[i] = 0u;
+  if (tid == 0) { s_ncand = 0u; s_cgt = 0u; s_ceq = 0u; }
+  // (all of this before the kernel ahead on the stream has ended: it touches this CTA's shared memory alone)
+  pdl_wait_for_predecessor();
+
   // ---- slices -------------------------------------------------------------------------
   // Append-then-step: one thread reads the length for the whole CTA, so that the CTA's arrival
   // (below) certifies that it no longer needs the old value; the last CTA of the sequence to
@@ -256,12 +272,6 @@ fused_decode_kernel(const FusedParams p) {
       asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
     } while (t1 - t0 < want);
   }
-  const int cap = (((p.max_len + cs - 1) / cs) + 31) & ~31;
-  const FusedSmem sl = fused_smem_layout(cap, kFW);
-  uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw + sl.keys);
-  uint32_t* hist0 = reinterpret_cast<uint32_t*>(smem_raw + sl.hist0);
-  uint32_t* hist1 = reinterpret_cast<uint32_t*>(smem_raw + sl.hist1);
-  uint32_t* s_mask = reinterpret_cast<uint32_t*>(smem_raw + sl.mask);
 
   const long long k_budget =
       p.budget > 0 ? (long long)p.budget : ((long long)(-p.budget) * len + 999) / 1000;
@@ -351,11 +361,6 @@ fused_decode_kernel(const FusedParams p) {
       *reinterpret_cast<uint32_t*>(p.proxy_w + poff + proxy_word_offset(pg, prow, w)) = lo | (hi << 16);
     }
   }
-  for (int i = tid; i < kFBins; i += kFT) { hist0[i] = 0u; hist1[i] = 0u; }
-  for (int i = tid; i < 3 * kFinBins; i += kFT) (&s_fin[0][0])[i] = 0u;
-  for (int i = tid; i < 3 * 2 * kGroups; i += kFT) (&s_gsum[0][0][0])[i] = 0u;
-  for (int i = tid; i < 3 * 2 * 32; i += kFT) (&s_fine[0][0][0])[i] = 0u;
-  if (tid == 0) { s_ncand = 0u; s_cgt = 0u; s_ceq = 0u; }
   if (tid < GP * (FASA_HEAD_DIM / 8))
     *reinterpret_cast<uint4*>(&s_qraw[tid / (FASA_HEAD_DIM / 8)][(tid % (FASA_HEAD_DIM / 8)) * 8]) = q_stage;
   if (tid < p.chunks * 8) s_chan[tid] = chan_stage;
@@ -454,6 +459,9 @@ fused_decode_kernel(const FusedParams p) {
     if (pg.n8 == 0 && pg.n16 == KB * NG) stream(std::true_type{});
     else stream(std::false_type{});
   }
+  // At most one CTA per SM: the next kernel's launch and set-up may overlap what follows, which leaves most of the SM idle.
+  // (With more rounds its CTAs would take the places of those still to come: 174 -> 203 us at batch 16, 64-128 K.)
+  if (ATTEND && p.early) pdl_release_successor();
   __syncthreads();
 
   // ---- 2. radix select of the ktot-th largest key ------------------------------------------
@@ -1126,25 +1134,18 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
   const int threads = wide ? 1024 : kFT, cs_l = wide ? ctx->step_cs : ctx->fused_cs;
   const size_t smem_l = wide ? ctx->step_smem : ctx->fused_smem;
 
+  p.early = (long long)c.batch * ctx->n_sets <= ctx->step_resident && (long long)c.batch * ctx->n_sets * cs_l <= ctx->n_sm;
   // (from one and a half rounds of CTAs on: see the kernel)
   if (ctx->step_resident > 0 && 2ll * c.batch * ctx->n_sets >= 3ll * ctx->step_resident) {
     p.shift_clusters = ctx->step_resident;
     p.shift_ctas = ctx->step_resident * cs_l;
   }
-  cudaLaunchConfig_t cfg;
-  memset(&cfg, 0, sizeof(cfg));
-  cfg.gridDim = dim3((unsigned)cs_l, (unsigned)(c.batch * ctx->n_sets), 1);
-  cfg.blockDim = dim3((unsigned)threads, 1, 1);
-  cfg.dynamicSmemBytes = smem_l;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = (unsigned)cs_l;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, fn, p);
+  // Only a grid of at most one CTA per SM is launched early, and gains the launch latency (steps back to back, batch 1 at
+  // 32 K: 24.9 -> 21.9 us, batch 8 at 64 K: 59.6 -> 56.3 us).  The clusters of a larger one would be placed around the CTAs
+  // of the kernel ahead, which leaves SMs with two CTAs beside SMs with none (96 units on pages: 67.7 -> 69.9 us) and,
+  // over several rounds, gaps that stay (batch 16 at 64-128 K: 177 -> 211 us).
+  const fasa_launch_shape shape{dim3((unsigned)cs_l, (unsigned)(c.batch * ctx->n_sets)), dim3((unsigned)threads), smem_l, cs_l, p.early != 0};
+  const cudaError_t e = fasa_launch(fn, shape, stream, p);
   ctx->launches += 1;
   FASA_CUDA_TRY(ctx, e);
   return FASA_OK;

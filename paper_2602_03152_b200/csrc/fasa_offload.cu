@@ -10,6 +10,7 @@
 // (the row is then a whole number of 16-byte chunks and the proxy row has no padding) and
 // contiguous caches.
 #include "fasa_common.cuh"
+#include "fasa_launch.cuh"
 #include "fasa_score_core.cuh"
 
 namespace {
@@ -23,13 +24,15 @@ constexpr int kSplitRows = 16;
 // through the K strides) and only k_nondom rows j < seq_lens[b] are written.
 template <bool APPEND>
 __global__ void __launch_bounds__(256)
-split_rows_kernel(const uint16_t* __restrict__ k_src, const uint16_t* __restrict__ v_src, uint16_t* __restrict__ k_nondom,
-                  uint16_t* __restrict__ v_cache, unsigned char* __restrict__ proxy, const int32_t* seq_lens,
-                  int32_t* seq_lens_w, int32_t* arrive, const int16_t* __restrict__ chan,
-                  const int16_t* __restrict__ ndchan, int32_t* __restrict__ status, int n_new, int n_kv_heads,
+split_rows_kernel(const uint16_t* k_src, const uint16_t* v_src, uint16_t* k_nondom,
+                  uint16_t* v_cache, unsigned char* proxy, const int32_t* seq_lens,
+                  int32_t* seq_lens_w, int32_t* arrive, const int16_t* chan,
+                  const int16_t* ndchan, int32_t* status, int n_new, int n_kv_heads,
                   int max_len, int chunks, int nd, int64_t ksb, int64_t ksh, int64_t kst, int64_t vsb, int64_t vsh,
                   int64_t vst, const fasa_resident res) {
   __shared__ __align__(16) uint16_t s_k[kSplitRows][FASA_HEAD_DIM];
+  pdl_wait_for_predecessor();
+  pdl_release_successor();
   const int u = blockIdx.y, h = u % n_kv_heads, b = u / n_kv_heads, tid = threadIdx.x;
   const int len = clamp_len(seq_lens[b], max_len, status);
   const int n0 = blockIdx.x * kSplitRows;
@@ -155,10 +158,11 @@ extern "C" int32_t fasa_m_split(fasa_ctx_t* ctx, const void* k_cache, void* k_no
   if (!split_ok(ctx)) return FASA_ERR_UNSUPPORTED;
   const fasa_config_t& c = ctx->cfg;
   dim3 grid((unsigned)((c.max_len + kSplitRows - 1) / kSplitRows), (unsigned)(c.batch * c.n_kv_heads));
-  split_rows_kernel<false><<<grid, 256, 0, (cudaStream_t)stream>>>(
-      (const uint16_t*)k_cache, nullptr, (uint16_t*)k_nondom, nullptr, nullptr, seq_lens, nullptr, nullptr, ctx->d_chan,
-      ctx->d_ndchan, ctx->d_status, 0, c.n_kv_heads, c.max_len, ctx->chunks, FASA_HEAD_DIM - 2 * c.n_dom, c.k_stride_b,
-      c.k_stride_h, c.k_stride_t, c.v_stride_b, c.v_stride_h, c.v_stride_t, fasa_resident{});
+  FASA_CUDA_TRY(ctx, launch_after_predecessor(
+      split_rows_kernel<false>, grid, dim3(256), (size_t)0, (cudaStream_t)stream, 0, (const uint16_t*)k_cache, (const uint16_t*)nullptr,
+      (uint16_t*)k_nondom, (uint16_t*)nullptr, (unsigned char*)nullptr, seq_lens, (int32_t*)nullptr, (int32_t*)nullptr,
+      (const int16_t*)ctx->d_chan, (const int16_t*)ctx->d_ndchan, ctx->d_status, 0, (int)c.n_kv_heads, (int)c.max_len, ctx->chunks,
+      (int)(FASA_HEAD_DIM - 2 * c.n_dom), c.k_stride_b, c.k_stride_h, c.k_stride_t, c.v_stride_b, c.v_stride_h, c.v_stride_t, fasa_resident{}));
   FASA_LAUNCH_CHECK(ctx);
   return FASA_OK;
 }
@@ -171,11 +175,12 @@ extern "C" int32_t fasa_m_kv_append(fasa_ctx_t* ctx, void* k_nondom, void* v_cac
   if (!split_ok(ctx)) return FASA_ERR_UNSUPPORTED;
   const fasa_config_t& c = ctx->cfg;
   dim3 grid((unsigned)((n_new + kSplitRows - 1) / kSplitRows), (unsigned)(c.batch * c.n_kv_heads));
-  split_rows_kernel<true><<<grid, 256, 0, (cudaStream_t)stream>>>(
-      (const uint16_t*)k_new, (const uint16_t*)v_new, (uint16_t*)k_nondom, (uint16_t*)v_cache, (unsigned char*)proxy_k,
-      seq_lens, seq_lens, ctx->d_arrive, ctx->d_chan, ctx->d_ndchan, ctx->d_status, n_new, c.n_kv_heads, c.max_len,
-      ctx->chunks, FASA_HEAD_DIM - 2 * c.n_dom, c.k_stride_b, c.k_stride_h, c.k_stride_t, c.v_stride_b, c.v_stride_h,
-      c.v_stride_t, fasa_resident_of(ctx));
+  FASA_CUDA_TRY(ctx, launch_after_predecessor(
+      split_rows_kernel<true>, grid, dim3(256), (size_t)0, (cudaStream_t)stream, 0, (const uint16_t*)k_new, (const uint16_t*)v_new,
+      (uint16_t*)k_nondom, (uint16_t*)v_cache, (unsigned char*)proxy_k, (const int32_t*)seq_lens, seq_lens, ctx->d_arrive,
+      (const int16_t*)ctx->d_chan, (const int16_t*)ctx->d_ndchan, ctx->d_status, (int)n_new, (int)c.n_kv_heads, (int)c.max_len, ctx->chunks,
+      (int)(FASA_HEAD_DIM - 2 * c.n_dom), c.k_stride_b, c.k_stride_h, c.k_stride_t, c.v_stride_b, c.v_stride_h, c.v_stride_t,
+      fasa_resident_of(ctx)));
   FASA_LAUNCH_CHECK(ctx);
   return FASA_OK;
 }

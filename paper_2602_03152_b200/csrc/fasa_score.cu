@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "fasa_common.cuh"
+#include "fasa_launch.cuh"
 #include "fasa_score_core.cuh"
 
 namespace {
@@ -23,11 +24,11 @@ struct TilesPerIter {
 // KB = 16-channel blocks per tile rounded up to a power of two (1, 2, 4, 8).
 template <int KB, bool MAXRED, bool PAGED>
 __global__ void __launch_bounds__(kScoreThreads)
-fc_score_kernel(const uint16_t* __restrict__ q, const unsigned char* __restrict__ proxy,
-                const int32_t* __restrict__ seq_lens, const int16_t* __restrict__ chan,
-                float* __restrict__ scores, int32_t* __restrict__ status, int n_q_heads,
+fc_score_kernel(const uint16_t* q, const unsigned char* proxy, const int32_t* seq_lens, const int16_t* chan, float* scores, int32_t* status, int n_q_heads,
                 int n_kv_heads, int n_sets, int group, int max_len, int chunks, int tiles_per_cta,
                 const PageMap pm) {
+  pdl_wait_for_predecessor();
+  pdl_release_successor();
   constexpr int TPI = TilesPerIter<KB>::value;
   const int u = blockIdx.y;
   const SelUnit su = sel_unit(u, n_sets, group, n_q_heads, n_kv_heads);
@@ -127,7 +128,7 @@ fc_score_kernel(const uint16_t* __restrict__ q, const unsigned char* __restrict_
 }
 
 template <int KB>
-void launch_score(fasa_ctx* ctx, const void* q, const void* proxy, const int32_t* seq_lens,
+cudaError_t launch_score(fasa_ctx* ctx, const void* q, const void* proxy, const int32_t* seq_lens,
                   float* scores, cudaStream_t s) {
   const fasa_config_t& c = ctx->cfg;
   const int units = c.batch * ctx->n_sets;
@@ -139,13 +140,14 @@ void launch_score(fasa_ctx* ctx, const void* q, const void* proxy, const int32_t
   per = (per + kStep - 1) / kStep * kStep;
   dim3 grid((unsigned)((tiles + per - 1) / per), (unsigned)units);
   auto go = [&](auto kernel) {
-    kernel<<<grid, kScoreThreads, 0, s>>>(
-        (const uint16_t*)q, (const unsigned char*)proxy, seq_lens, ctx->d_chan, scores, ctx->d_status,
-        c.n_q_heads, c.n_kv_heads, ctx->n_sets, ctx->sel_heads, c.max_len, ctx->chunks, per, fasa_page_map(ctx));
+    return launch_after_predecessor(
+        kernel, grid, dim3(kScoreThreads), (size_t)0, s, 0, (const uint16_t*)q, (const unsigned char*)proxy, seq_lens,
+        (const int16_t*)ctx->d_chan, scores, ctx->d_status, (int)c.n_q_heads, (int)c.n_kv_heads, ctx->n_sets, ctx->sel_heads, (int)c.max_len,
+        ctx->chunks, per, fasa_page_map(ctx));
   };
   const bool paged = c.page_size > 0;
-  if (c.group_reduce == 0) paged ? go(fc_score_kernel<KB, false, true>) : go(fc_score_kernel<KB, false, false>);
-  else paged ? go(fc_score_kernel<KB, true, true>) : go(fc_score_kernel<KB, true, false>);
+  if (c.group_reduce == 0) return paged ? go(fc_score_kernel<KB, false, true>) : go(fc_score_kernel<KB, false, false>);
+  return paged ? go(fc_score_kernel<KB, true, true>) : go(fc_score_kernel<KB, true, false>);
 }
 
 }  // namespace
@@ -157,10 +159,12 @@ extern "C" int32_t fasa_fc_score(fasa_ctx_t* ctx, const void* q, const void* pro
     return FASA_ERR_INVALID_ARG;
   cudaStream_t s = (cudaStream_t)stream;
   const int nb = (ctx->chunks + 1) / 2;      // 16-channel blocks per tile, the 8-channel one included
-  if (nb <= 1) launch_score<1>(ctx, q, proxy_k, seq_lens, scores, s);
-  else if (nb <= 2) launch_score<2>(ctx, q, proxy_k, seq_lens, scores, s);
-  else if (nb <= 4) launch_score<4>(ctx, q, proxy_k, seq_lens, scores, s);
-  else launch_score<8>(ctx, q, proxy_k, seq_lens, scores, s);
-  FASA_LAUNCH_CHECK(ctx);
+  cudaError_t e;
+  if (nb <= 1) e = launch_score<1>(ctx, q, proxy_k, seq_lens, scores, s);
+  else if (nb <= 2) e = launch_score<2>(ctx, q, proxy_k, seq_lens, scores, s);
+  else if (nb <= 4) e = launch_score<4>(ctx, q, proxy_k, seq_lens, scores, s);
+  else e = launch_score<8>(ctx, q, proxy_k, seq_lens, scores, s);
+  ctx->launches += 1;
+  FASA_CUDA_TRY(ctx, e);
   return FASA_OK;
 }
