@@ -250,7 +250,8 @@ static fasa_ws ws_layout(const fasa_ctx* ctx) {
   const int n = split_count_bound(ctx, c.max_len, c.batch * c.n_kv_heads);
   const size_t per_split = (size_t)c.batch * c.n_q_heads * (FASA_HEAD_DIM + 2) * sizeof(float), rows = set_per_head(ctx) ? (size_t)c.batch * ctx->n_sets : 0;
   fasa_ws w;
-  w.scores = fasa_align_up(per_split * (size_t)n, 256) + 256;
+  const size_t dense = ((size_t)fasa_dense_ctas(ctx) + (size_t)c.batch * c.n_kv_heads) * ctx->group * (FASA_HEAD_DIM + 2) * sizeof(float);
+  w.scores = fasa_align_up(std::max(per_split * (size_t)n, dense), 256) + 256;
   w.gm = w.scores + fasa_align_up(rows * (size_t)c.max_len * sizeof(float), 256);
   w.total = w.gm + fasa_align_up(rows * (size_t)fasa_stream_gm_stride(ctx) * sizeof(float), 256);
   return w;

@@ -297,9 +297,9 @@ constexpr int kMmaWarps = kMmaThreads / 32;
 // link) followed by its dominant channels in proxy order (from the GPU-resident proxy); the
 // query operand is loaded in the same channel order, so the logits are the same dot products
 // summed in another order.
-// (CTAs per SM: six is what the 37 KB of staging memory per CTA allow; fewer where the registers do not)
+// (CTAs per SM: as many as the registers allow)
 template <bool SPARSE, bool PAGED, bool CLUSTER, bool HOSTMEM = false, bool KSPLIT = false>
-__global__ void __launch_bounds__(kMmaThreads, KSPLIT || PAGED ? 4 : (CLUSTER || SPARSE ? 5 : 6))
+__global__ void __launch_bounds__(kMmaThreads, KSPLIT || PAGED ? 4 : 5)
 decode_attn_mma_kernel(const AttnParams p) {
   __shared__ ClusterMergeSmem s_merge;              // (CLUSTER only: written by the peers)
   pdl_wait_for_predecessor();
@@ -367,13 +367,70 @@ decode_attn_mma_kernel(const AttnParams p) {
   }
 }
 
-// Merge pass: one CTA per (batch, query head); thread (c, j) takes channel c of the splits
-// s = j, j + 4, ... so that four chains of dependent loads run side by side, then the four
-// partial merges are merged.
-constexpr int kMergeWays = 4;
+// Merge pass: one CTA per (batch, query head); thread (c, j) takes channels 2 c and 2 c + 1 of the splits s = j, j + 8, ...,
+// eight of them in flight at a time, then the eight partial merges are merged.  (Four ways and a channel per thread, the
+// maxima read in a pass of their own: 8 us at 32 splits against 5 us.)
+constexpr int kMergeWays = 8, kMergeThreads = FASA_HEAD_DIM / 2 * kMergeWays;
+// ns partial results (m, l, acc[128]), `stride` floats apart (an even number), to out[128] and *lse (nullable).
+__device__ __forceinline__ void merge_partials(const float* src, int64_t stride, int ns, float* out, float* lse) {
+  const int c = threadIdx.x % (FASA_HEAD_DIM / 2), j = threadIdx.x / (FASA_HEAD_DIM / 2);
+  __shared__ float s_m[kMergeWays], s_l[kMergeWays];
+  __shared__ float2 s_a[kMergeWays][FASA_HEAD_DIM / 2];
+  float mx = -INFINITY, l = 0.f;
+  float2 a = make_float2(0.f, 0.f);
+  for (int s0 = j; s0 < ns; s0 += 8 * kMergeWays) {
+    float2 ml[8], as[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int s = s0 + i * kMergeWays;
+      const float* row = src + (s < ns ? s : s0) * stride;
+      ml[i] = *reinterpret_cast<const float2*>(row);
+      as[i] = *reinterpret_cast<const float2*>(row + 2 + 2 * c);
+      if (s >= ns) ml[i].x = -INFINITY;
+    }
+    float mn = mx;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) mn = fmaxf(mn, ml[i].x);
+    const float keep = mx == -INFINITY ? 0.f : exp2f(mx - mn);
+    a.x *= keep;
+    a.y *= keep;
+    l *= keep;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float w = ml[i].x == -INFINITY ? 0.f : exp2f(ml[i].x - mn);
+      a.x += w * as[i].x;
+      a.y += w * as[i].y;
+      l += w * ml[i].y;
+    }
+    mx = mn;
+  }
+  s_a[j][c] = a;
+  if (c == 0) {
+    s_m[j] = mx;
+    s_l[j] = l;
+  }
+  __syncthreads();
+  if (j != 0) return;
+  float m_all = -INFINITY, l_all = 0.f;
+#pragma unroll
+  for (int k = 0; k < kMergeWays; ++k) m_all = fmaxf(m_all, s_m[k]);
+  float2 a_all = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int k = 0; k < kMergeWays; ++k) {
+    const float w = s_m[k] == -INFINITY ? 0.f : exp2f(s_m[k] - m_all);
+    a_all.x += w * s_a[k][c].x;
+    a_all.y += w * s_a[k][c].y;
+    l_all += w * s_l[k];
+  }
+  const bool any = ns > 0 && l_all > 0.f;
+  out[2 * c] = any ? a_all.x / l_all : 0.f;
+  out[2 * c + 1] = any ? a_all.y / l_all : 0.f;
+  if (lse && c == 0) *lse = any ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+}
+
 template <bool SPARSE>
-__global__ void __launch_bounds__(FASA_HEAD_DIM * kMergeWays)
-decode_attn_merge_kernel(const float* __restrict__ partial, const int32_t* __restrict__ n_rows,
+__global__ void __launch_bounds__(kMergeThreads)
+decode_attn_merge_kernel(const float* partial, const int32_t* n_rows,
                          float* __restrict__ out, float* __restrict__ lse,
                          int32_t* __restrict__ status, int n_q_heads, int n_sets, int group,
                          int max_len, int n_cap, int chunk, int n_splits) {
@@ -390,40 +447,115 @@ decode_attn_merge_kernel(const float* __restrict__ partial, const int32_t* __res
     n = n < 0 ? 0 : (n > max_len ? max_len : n);
   }
   const int ns = min(n_splits, (n + chunk - 1) / chunk);
-  const int c = threadIdx.x % FASA_HEAD_DIM;
-  const int j = threadIdx.x / FASA_HEAD_DIM;
-  const float* src = partial + (int64_t)bh * n_splits * kPartialStride;
-  __shared__ float s_m[kMergeWays], s_l[kMergeWays];
-  __shared__ float s_a[kMergeWays][FASA_HEAD_DIM];
-  float mx = -INFINITY;
-  for (int s = j; s < ns; s += kMergeWays) mx = fmaxf(mx, src[s * kPartialStride]);
-  float a = 0.f, l = 0.f;
-  for (int s = j; s < ns; s += kMergeWays) {
-    const float ms = src[s * kPartialStride];
-    const float w = ms == -INFINITY ? 0.f : exp2f(ms - mx);
-    a += w * src[s * kPartialStride + 2 + c];
-    l += w * src[s * kPartialStride + 1];
-  }
-  s_a[j][c] = a;
-  if (c == 0) {
-    s_m[j] = mx;
-    s_l[j] = l;
-  }
-  __syncthreads();
-  if (j != 0) return;
-  float m_all = -INFINITY;
+  merge_partials(partial + (int64_t)bh * n_splits * kPartialStride, kPartialStride, ns, out + (int64_t)bh * FASA_HEAD_DIM, lse ? lse + bh : nullptr);
+}
+
+// ---- dense pass over long contexts -----------------------------------------------------------------
+// As many CTAs as the device holds at once; the rows of all (sequence, KV head) units, laid end to end in tiles of 16, are
+// dealt out to them evenly by the lengths on the device, so ragged batches end together and no last wave is left over.
+// A CTA whose share spans several units writes a partial result for each; segment (CTA i, unit u) is number i + u of
+// the partial results (from one segment to the next exactly one of the two grows).  Bound by HBM.  Measured (back to back,
+// with the merge) against splits of a fixed size: batch 4 at 20-60 K 126 -> 119 us, batch 16 x 4 heads at 9-18 K 94 -> 88 us,
+// batch 1 at 30 K 34.3 -> 32 us; equal lengths that filled the last wave before: the same.
+struct DenseDeal {
+  long long total;         // tiles of all units
+  int n;                   // CTAs that take part: at least four tiles each
+  int mine;                // tiles of a KV head of sequence `lane`
+};
+// (Products of tiles and CTAs are formed in 32 bits where they fit: a 64-bit division costs more than the rest of the set-up.)
+__device__ __forceinline__ int dense_tiles(const int32_t* seq_lens, int b, int batch, int max_len, int32_t* status) {
+  return b < batch ? (clamp_len(seq_lens[b], max_len, status) + 15) >> 4 : 0;
+}
+// One warp.
+__device__ __forceinline__ DenseDeal dense_deal(const int32_t* seq_lens, int batch, int n_kv_heads, int max_len, int n_ctas, int lane, int32_t* status) {
+  DenseDeal d;
+  d.mine = dense_tiles(seq_lens, lane, batch, max_len, status);
+  d.total = __reduce_add_sync(0xffffffffu, d.mine);
+  for (int b0 = 32; b0 < batch; b0 += 32) d.total += __reduce_add_sync(0xffffffffu, dense_tiles(seq_lens, b0 + lane, batch, max_len, status));
+  d.total *= n_kv_heads;
+  d.n = (int)min((long long)n_ctas, max(1ll, d.total >> 2));
+  return d;
+}
+
+template <bool PAGED, bool HOSTMEM>
+__global__ void __launch_bounds__(kMmaThreads, PAGED ? 4 : 6)
+dense_attn_kernel(const AttnParams p) {
+  pdl_wait_for_predecessor();
+  pdl_release_successor();
+  const int lane = threadIdx.x & 31;
+  const int batch = p.n_cap;                        // (the launch's number of sequences)
+  const DenseDeal d = dense_deal(p.n_rows, batch, p.n_kv_heads, p.max_len, (int)gridDim.x, lane, p.status);
+  const int i = blockIdx.x;
+  if (i >= d.n) return;
+  long long x = d.total < (1 << 22) ? (uint32_t)d.total * (uint32_t)i / (uint32_t)d.n : d.total * i / d.n;
+  const long long end = d.total < (1 << 22) ? (uint32_t)d.total * (uint32_t)(i + 1) / (uint32_t)d.n : d.total * (i + 1) / d.n;
+  if (x >= end) return;
+  // the sequence that tile x lies in
+  int b = 0, tiles = 0;
+  long long before = 0;                             // tiles of the sequences ahead of it
+  for (int b0 = 0; b0 < batch; b0 += 32) {
+    const int mine = b0 == 0 ? d.mine : dense_tiles(p.n_rows, b0 + lane, batch, p.max_len, p.status);
+    int incl = mine;
 #pragma unroll
-  for (int k = 0; k < kMergeWays; ++k) m_all = fmaxf(m_all, s_m[k]);
-  float a_all = 0.f, l_all = 0.f;
-#pragma unroll
-  for (int k = 0; k < kMergeWays; ++k) {
-    const float w = s_m[k] == -INFINITY ? 0.f : exp2f(s_m[k] - m_all);
-    a_all += w * s_a[k][c];
-    l_all += w * s_l[k];
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += v;
+    }
+    const uint32_t hits = __ballot_sync(0xffffffffu, before + (long long)incl * p.n_kv_heads > x);
+    if (hits) {
+      const int l = __ffs(hits) - 1;
+      b = b0 + l;
+      tiles = __shfl_sync(0xffffffffu, mine, l);
+      before += (long long)(__shfl_sync(0xffffffffu, incl, l) - tiles) * p.n_kv_heads;
+      break;
+    }
+    before += (long long)__shfl_sync(0xffffffffu, incl, 31) * p.n_kv_heads;
   }
-  out[(int64_t)bh * FASA_HEAD_DIM + c] = (ns > 0 && l_all > 0.f) ? a_all / l_all : 0.f;
-  if (lse && c == 0)
-    lse[bh] = (ns > 0 && l_all > 0.f) ? (m_all + log2f(l_all)) * 0.6931471805599453f : -INFINITY;
+  extern __shared__ __align__(16) unsigned char attn_smem_raw[];
+  int h = (int)(x - before) / tiles, t0 = (int)(x - before) - h * tiles;      // (within a sequence: 32 bits)
+  while (x < end) {                                 // uniform over the CTA: a segment per unit
+    const int n = (int)min((long long)(tiles - t0), end - x);
+    const int len = clamp_len(p.n_rows[b], p.max_len, p.status);
+    const SelUnit su = sel_unit(b * p.n_kv_heads + h, p.n_kv_heads, p.group, p.n_q_heads, p.n_kv_heads);
+    uint32_t qb[8][2];
+    attn_load_query<false>(qb, p, su, lane);
+    float* const dst = p.partial + (int64_t)(i + b * p.n_kv_heads + h) * p.group * kPartialStride;
+    attn_rows<kMmaWarps, false, PAGED, HOSTMEM, false>(p, su, b, qb, t0 * 16, min(len, (t0 + n) * 16), nullptr, attn_smem_raw,
+                                                       [&](int gl) { return dst + gl * kPartialStride; });
+    x += n;
+    if (x < end) {
+      t0 = 0;
+      if (++h == p.n_kv_heads) {
+        h = 0;
+        do tiles = dense_tiles(p.n_rows, ++b, batch, p.max_len, p.status);
+        while (tiles == 0 && b + 1 < batch);
+      }
+      __syncthreads();                              // the next segment's rows take over the combine area
+    }
+  }
+}
+
+// Merge of the segments of every (sequence, query head): one CTA each, as decode_attn_merge_kernel.
+__global__ void __launch_bounds__(kMergeThreads)
+dense_merge_kernel(const AttnParams p, int n_ctas) {
+  pdl_wait_for_predecessor();
+  pdl_release_successor();
+  const int bh = blockIdx.x, b = bh / p.n_q_heads, hq = bh % p.n_q_heads, h = hq / p.group;
+  const int lane = threadIdx.x & 31, batch = p.n_cap;
+  const DenseDeal d = dense_deal(p.n_rows, batch, p.n_kv_heads, p.max_len, n_ctas, lane, p.status);
+  long long first = 0;                              // this unit's first tile
+  for (int b0 = 0; b0 < b; b0 += 32)
+    first += __reduce_add_sync(0xffffffffu, b0 + lane < b ? (b0 == 0 ? d.mine : dense_tiles(p.n_rows, b0 + lane, batch, p.max_len, p.status)) : 0);
+  const int tiles = b < 32 ? __shfl_sync(0xffffffffu, d.mine, b & 31) : dense_tiles(p.n_rows, b, batch, p.max_len, p.status);
+  first = first * p.n_kv_heads + (long long)h * tiles;
+  // tile x belongs to CTA ((x + 1) n - 1) / total
+  auto cta_of = [&](long long y) {                  // y = x + 1
+    return d.total < (1 << 22) ? (int)(((uint32_t)y * (uint32_t)d.n - 1u) / (uint32_t)d.total) : (int)((y * d.n - 1) / d.total);
+  };
+  const int i0 = tiles > 0 ? cta_of(first + 1) : 0;
+  const int ns = tiles > 0 ? cta_of(first + tiles) - i0 + 1 : 0;
+  merge_partials(p.partial + ((int64_t)(i0 + b * p.n_kv_heads + h) * p.group + hq % p.group) * kPartialStride, (int64_t)p.group * kPartialStride, ns,
+                 p.out + (int64_t)bh * FASA_HEAD_DIM, p.lse ? p.lse + bh : nullptr);
 }
 
 // out_mirror (nullable): a second destination of out; *mirrored tells whether it was written
@@ -476,13 +608,27 @@ int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
       FASA_LAUNCH_CHECK(ctx);
       return FASA_OK;
     }
-    auto fn = c.page_size > 0 ? decode_attn_mma_kernel<SPARSE, true, false> : decode_attn_mma_kernel<SPARSE, false, false>;
-    if (host) fn = decode_attn_mma_kernel<SPARSE, false, false, true>;
-    if constexpr (SPARSE) { if (ksplit) fn = decode_attn_mma_kernel<true, false, false, true, true>; }
+    if constexpr (!SPARSE) {
+      p.out = out; p.lse = lse; p.n_cap = c.batch;
+      auto fn = c.page_size > 0 ? dense_attn_kernel<true, false> : dense_attn_kernel<false, false>;
+      if (host) fn = dense_attn_kernel<false, true>;
+      const int n_ctas = fasa_dense_ctas(ctx);
+      FASA_CUDA_TRY(ctx, cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
+      FASA_CUDA_TRY(ctx, launch_after_predecessor(fn, dim3((unsigned)n_ctas), dim3(kMmaThreads), sizeof(MmaSmem<kMmaWarps>), s, 0, p));
+      FASA_LAUNCH_CHECK(ctx);
+      FASA_CUDA_TRY(ctx, launch_after_predecessor(dense_merge_kernel, dim3((unsigned)(c.batch * c.n_q_heads)), dim3(kMergeThreads),
+                                                  (size_t)0, s, 0, p, n_ctas));
+      FASA_LAUNCH_CHECK(ctx);
+      return FASA_OK;
+    } else {
+    auto fn = c.page_size > 0 ? decode_attn_mma_kernel<true, true, false> : decode_attn_mma_kernel<true, false, false>;
+    if (host) fn = decode_attn_mma_kernel<true, false, false, true>;
+    if (ksplit) fn = decode_attn_mma_kernel<true, false, false, true, true>;
     // (+ the slice of the index list: chunk <= 2048 rows)
-    const size_t smem = sizeof(MmaSmem<kMmaWarps>) + (SPARSE ? (size_t)plan.chunk * sizeof(int32_t) : 0);
+    const size_t smem = sizeof(MmaSmem<kMmaWarps>) + (size_t)plan.chunk * sizeof(int32_t);
     FASA_CUDA_TRY(ctx, cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
     FASA_CUDA_TRY(ctx, launch_after_predecessor(fn, grid, dim3(kMmaThreads), smem, s, 0, p));
+    }
   } else if (G == 1) decode_attn_kernel<1, 1, SPARSE><<<grid, kAttnThreads, 0, s>>>(p);
   else if (G == 2) decode_attn_kernel<2, 1, SPARSE><<<grid, kAttnThreads, 0, s>>>(p);
   else if (G == 3) decode_attn_kernel<3, 1, SPARSE><<<grid, kAttnThreads, 0, s>>>(p);
@@ -491,7 +637,7 @@ int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
   else decode_attn_kernel<4, 2, SPARSE><<<grid, kAttnThreads, 0, s>>>(p);
   FASA_LAUNCH_CHECK(ctx);
   FASA_CUDA_TRY(ctx, launch_after_predecessor(
-      decode_attn_merge_kernel<SPARSE>, dim3((unsigned)(n_seq * c.n_q_heads)), dim3(FASA_HEAD_DIM * kMergeWays),
+      decode_attn_merge_kernel<SPARSE>, dim3((unsigned)(n_seq * c.n_q_heads)), dim3(kMergeThreads),
       (size_t)0, s, 0, (const float*)workspace, n_rows, out, lse, ctx->d_status, (int)c.n_q_heads, (int)n_sets,
       (int)G, (int)c.max_len, (int)n_upper, (int)plan.chunk, (int)plan.n_splits));
   FASA_LAUNCH_CHECK(ctx);

@@ -73,6 +73,8 @@ struct fasa_split_plan {
   int chunk;      // rows per split (multiple of 32)
 };
 fasa_split_plan fasa_plan_splits(const fasa_ctx* ctx, int n_upper, int units);
+// CTAs of the dense pass over long contexts: what the device holds at once (six per SM, four on pages).
+static inline int fasa_dense_ctas(const fasa_ctx* ctx) { return (ctx->cfg.page_size > 0 ? 4 : 6) * (ctx->n_sm > 0 ? ctx->n_sm : 148); }
 
 // One-launch decode step (fasa_fused.cu): plan at context creation, launch per step.
 int fasa_fused_plan(fasa_ctx* ctx);

@@ -429,6 +429,38 @@ def test_large_selection_is_attended_by_the_split_k_kernel():
     assert r.fasa.device_status() == 0
 
 
+@pytest.mark.parametrize("heads,lens,page", [
+    ((8, 2), [20000, 0, 1, 16385, 17], 0),          # units shorter than a share, empty ones, shares that span several units
+    ((7, 1), [16900], 0),                           # one unit over all CTAs
+    ((16, 8), [0, 0, 0], 0),                        # nothing at all
+    ((5, 1), [63] * 40, 0),                         # more sequences than a warp has lanes; fewer tiles than CTAs
+    ((8, 2), [19999, 40, 8000], 32),
+])
+def test_dense_path_over_long_contexts_deals_rows_out_evenly(heads, lens, page):
+    w = C["c1"].replace(batch=len(lens), n_q_heads=heads[0], n_kv_heads=heads[1], max_len=20000, n_sink=0, n_recent=0, budget=16)
+    t = synth.make_inputs(w, "cpu", lens=torch.tensor(lens, dtype=torch.int32))
+    if page:
+        r, f, kp, vp, tab, table, need = _paged_twin(w, t, page)
+        f.full_decode_attn(r.q, kp, vp, r.seq_lens, r.dense, r.ws, r.dense_lse)
+    else:
+        r = Run(w, t)
+        f = r.fasa
+        r.dense_step()
+    torch.cuda.synchronize()
+    assert f.device_status() == 0
+    G = heads[0] // heads[1]
+    for b, L in enumerate(lens):
+        for g in range(heads[0]):
+            if L == 0:
+                assert float(r.dense[b, g].abs().max()) == 0.0 and float(r.dense_lse[b, g]) == float("-inf")
+                continue
+            k, v = (r.t[n][b, g // G, :L].double() for n in ("k", "v"))
+            lg = (k @ r.t["q"][b, g].double()) / math.sqrt(128.0)
+            # (the kernel's probabilities carry 17 bits and its sums 24: 1e-4 of the largest value covers both at 20000 rows)
+            err = (torch.softmax(lg, 0) @ v - r.dense[b, g].cpu().double()).abs().max()
+            assert float(err) <= 1e-4 * float(v.abs().max()) and abs(float(torch.logsumexp(lg, 0)) - float(r.dense_lse[b, g])) <= 1e-4
+
+
 # ---- index sets shared by fewer query heads than a KV head serves (Sec. 4.1: a set per head) ----
 
 @pytest.mark.parametrize("cfg,sel,kw", [
