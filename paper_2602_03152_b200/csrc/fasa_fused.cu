@@ -111,6 +111,10 @@ struct FusedParams {
   unsigned char* proxy_w;
   int32_t* seq_lens_w;
   int32_t* arrive;
+  // split key cache (append form; ndchan null otherwise): k_w holds the nd non-dominant channels of every key
+  const int16_t* ndchan;
+  int nd;
+  fasa_resident res;
   int early;               // at most one CTA per SM, all resident at once: launched early, and lets its successor be
   int shift_clusters, shift_ctas;   // phase shift of grids that run in rounds: clusters / CTAs resident at once (0: none)
   float* scores;           // nullable
@@ -345,7 +349,31 @@ fused_decode_kernel(const FusedParams p) {
       voff = page * p.vsb + h * p.vsh + (int64_t)prow * p.vst;
       poff = ((int64_t)page * p.n_kv_heads + h) * (1 << (p.pm.shift - 4)) * pg.tile_bytes;
     }
-    if (!row_ok) {
+    if (!PAGED && p.ndchan != nullptr) {
+      // Split (Algorithm 2), as in fasa_m_kv_append: the rows may lie in host memory, and cross the link while this kernel
+      // selects.  A sink position, and every new one while a recent window is kept, goes to its resident slot too.
+      const int slot = p.res.tags != nullptr && (len_old < p.res.n_sink || p.res.n_recent > 0) ? fasa_resident_slot(p.res, len_old) : -1;
+      uint16_t* res_row = slot >= 0 ? p.res.rows + ((int64_t)su.kv * p.res.slots + slot) * 2 * FASA_HEAD_DIM : nullptr;
+      uint16_t* k_row = p.k_w + ((int64_t)su.kv * p.max_len + len_old) * p.nd;
+      const int16_t* nch = p.ndchan + h * p.nd;
+      for (int i = tid; i < p.nd / 2; i += kFT) {
+        const uint32_t w = ksrc[nch[2 * i]] | ((uint32_t)ksrc[nch[2 * i + 1]] << 16);
+        *reinterpret_cast<uint32_t*>(k_row + 2 * i) = w;
+        if (res_row) *reinterpret_cast<uint32_t*>(res_row + 2 * i) = w;
+      }
+      for (int i = tid; i < 4 * p.chunks; i += kFT) {
+        const int16_t* ch = p.chan + h * p.chunks * 8 + 2 * i;
+        const uint32_t w = ksrc[ch[0]] | ((uint32_t)ksrc[ch[1]] << 16);
+        *reinterpret_cast<uint32_t*>(p.proxy_w + poff + proxy_word_offset(pg, prow, i)) = w;
+        if (res_row) *reinterpret_cast<uint32_t*>(res_row + p.nd + 2 * i) = w;
+      }
+      if (tid < 16) {
+        const uint4 x = *reinterpret_cast<const uint4*>(p.v_new + (int64_t)su.kv * FASA_HEAD_DIM + tid * 8);
+        *reinterpret_cast<uint4*>(p.v_w + voff + tid * 8) = x;
+        if (res_row) *reinterpret_cast<uint4*>(res_row + FASA_HEAD_DIM + tid * 8) = x;
+      }
+      if (tid == 0 && slot >= 0) p.res.tags[(int64_t)su.kv * p.res.slots_pad + slot] = len_old;
+    } else if (!row_ok) {
     } else if (tid < 16) {
       *reinterpret_cast<uint4*>(p.k_w + koff + tid * 8) = *reinterpret_cast<const uint4*>(ksrc + tid * 8);
     } else if (tid < 32) {
@@ -1106,7 +1134,7 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
                           const void* proxy_k, const int32_t* seq_lens, int32_t budget,
                           int32_t n_sel_max, float* scores, int32_t* idx, int32_t* n_sel,
                           float* out, float* lse, const void* k_new, const void* v_new,
-                          cudaStream_t stream, bool with_attention, float* out_mirror) {
+                          cudaStream_t stream, bool with_attention, float* out_mirror, bool split_keys) {
   const fasa_config_t& c = ctx->cfg;
   FusedParams p;
   p.out_mirror = out_mirror;
@@ -1116,6 +1144,9 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
   p.k_w = (uint16_t*)k_cache; p.v_w = (uint16_t*)v_cache; p.proxy_w = (unsigned char*)proxy_k;
   p.seq_lens_w = (int32_t*)seq_lens; p.arrive = ctx->d_arrive;
   p.shift_clusters = 0; p.shift_ctas = 0;
+  p.ndchan = split_keys ? ctx->d_ndchan : nullptr;
+  p.nd = FASA_HEAD_DIM - 2 * c.n_dom;
+  p.res = split_keys ? fasa_resident_of(ctx) : fasa_resident{};
   p.scores = scores; p.idx = idx; p.n_sel = n_sel; p.out = out; p.lse = lse; p.status = ctx->d_status;
   p.n_q_heads = c.n_q_heads; p.n_kv_heads = c.n_kv_heads; p.n_sets = ctx->n_sets; p.group = ctx->sel_heads; p.max_len = c.max_len;
   p.chunks = ctx->chunks; p.n_sink = c.n_sink; p.n_recent = c.n_recent; p.budget = budget;
