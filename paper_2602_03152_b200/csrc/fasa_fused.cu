@@ -1032,16 +1032,46 @@ int fasa_fused_plan(fasa_ctx* ctx) {
   const bool paged = c.page_size > 0;
   FusedFn fn = fused_fn(ctx->chunks, paged);
   auto cap_of = [&](int cs) { return (((c.max_len + cs - 1) / cs) + 31) & ~31; };
-  // Two CTAs per SM can be resident; a cluster is doubled while the whole grid still fits
-  // in one wave of them and every CTA keeps at least 512 tokens.
+  // Two CTAs per SM can be resident; a cluster is doubled while the whole grid still fits in one wave of them and the slices
+  // are worth it: at least 512 tokens, 2560 for clusters of 16, whose barriers cost more than their stream saves (8 units at
+  // 12 K: 18.6 us with 16, 16.1 with 8; at 25 K 20.5 / 18.9; at 60 K 24.0 / 25.5), and beyond one CTA per SM only from slices
+  // of 4608 on (20 units: at 6 K 23.1 us with 8 CTAs each or half as many wide ones, 20.2 with 4; at 12 K 24.5 / 22.4; at
+  // 25 K 27.5 / 27.2; at 50 K 33.0 / 34.7).
   const int slots = 2 * ctx->n_sm;
   int want = 1;
   while (want < 16 && cap_of(want) > kCapPair) want *= 2;
-  while (want < 16 && units * want * 2 <= slots && c.max_len / (2 * want) >= 512) want *= 2;
+  while (want < 16 && units * want * 2 <= slots && c.max_len / (2 * want) >= (want == 8 ? 2560 : 512) &&
+         (units * want * 2 <= ctx->n_sm || c.max_len / want >= 4608))
+    want *= 2;
   if (cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
     cudaGetLastError();
     if (want > 8) want = 8;
   }
+  // Clusters of the wide form with half of cs CTAs that the device holds at once; 0 where it is not available.
+  auto wide_clusters = [&](int cs) -> int {
+    if (cs < 4 || cap_of(cs / 2) > kCapWide) return 0;
+    const int limit_w = (int)fused_smem_layout(kCapWide, 32).total;
+    FusedFn fw = wide_fn(ctx->chunks, paged), fs = wide_select_fn(ctx->chunks, paged);
+    cudaLaunchConfig_t cw;
+    memset(&cw, 0, sizeof(cw));
+    cw.gridDim = dim3((unsigned)(cs / 2), (unsigned)units, 1);
+    cw.blockDim = dim3(1024, 1, 1);
+    cw.dynamicSmemBytes = (size_t)fused_smem_layout(cap_of(cs / 2), 32).total;
+    cudaLaunchAttribute aw[1];
+    aw[0].id = cudaLaunchAttributeClusterDimension;
+    aw[0].val.clusterDim.x = (unsigned)(cs / 2);
+    aw[0].val.clusterDim.y = 1;
+    aw[0].val.clusterDim.z = 1;
+    cw.attrs = aw;
+    cw.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute((const void*)fw, cudaFuncAttributeMaxDynamicSharedMemorySize, limit_w) == cudaSuccess &&
+        cudaFuncSetAttribute((const void*)fs, cudaFuncAttributeMaxDynamicSharedMemorySize, limit_w) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, (const void*)fw, &cw) == cudaSuccess)
+      return n;
+    cudaGetLastError();
+    return 0;
+  };
   for (int cs = want; cs >= 1; cs /= 2) {
     const int cap = cap_of(cs);
     if (cap > kCapMax) break;
@@ -1074,7 +1104,9 @@ int fasa_fused_plan(fasa_ctx* ctx) {
     // SMs over) would run a second round for the last few: half the cluster size instead.  Likewise the wide form below is
     // taken only if it holds every unit or the narrow one does not either.  16 units at 25 K (wide clusters of 8, 14 or 15
     // of them at once): 41.9 -> 22.8 us with 512-thread CTAs; at 60 K 50 -> 30 us; 36 units at 6 K 48 -> 26 us.
-    if (n_clusters < units && (long long)units * cs <= slots && cs > 1 && cap_of(cs / 2) <= kCapPair) continue;
+    if (n_clusters < units && (long long)units * cs <= slots && cs > 1 && cap_of(cs / 2) <= kCapPair &&
+        !((long long)units * cs > ctx->n_sm && wide_clusters(cs) >= units))
+      continue;
     // the form without attention runs with the same cluster shape
     if (cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit) != cudaSuccess ||
         (cs > 8 && cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
@@ -1093,37 +1125,13 @@ int fasa_fused_plan(fasa_ctx* ctx) {
     ctx->step_cs = cs;
     ctx->step_smem = smem;
     ctx->step_resident = n_clusters;
-    const long long ctas = (long long)units * cs;
     // (not down to clusters of one CTA: batch 32 x 4 heads of 7 query heads at 16 K lost 3-6 % that way)
-    if (cs >= 4 && ctas > ctx->n_sm && cap_of(cs / 2) <= kCapWide) {
-      const int cs_w = cs / 2;
-      const size_t smem_w = (size_t)fused_smem_layout(cap_of(cs_w), 32).total;
-      const int limit_w = (int)fused_smem_layout(kCapWide, 32).total;
-      FusedFn fw = wide_fn(ctx->chunks, paged), fs = wide_select_fn(ctx->chunks, paged);
-      cudaLaunchConfig_t cw;
-      memset(&cw, 0, sizeof(cw));
-      cw.gridDim = dim3((unsigned)cs_w, (unsigned)units, 1);
-      cw.blockDim = dim3(1024, 1, 1);
-      cw.dynamicSmemBytes = smem_w;
-      cudaLaunchAttribute aw[1];
-      aw[0].id = cudaLaunchAttributeClusterDimension;
-      aw[0].val.clusterDim.x = (unsigned)cs_w;
-      aw[0].val.clusterDim.y = 1;
-      aw[0].val.clusterDim.z = 1;
-      cw.attrs = aw;
-      cw.numAttrs = 1;
-      int n_w = 0;
-      if (cudaFuncSetAttribute((const void*)fw, cudaFuncAttributeMaxDynamicSharedMemorySize, limit_w) == cudaSuccess &&
-          cudaFuncSetAttribute((const void*)fs, cudaFuncAttributeMaxDynamicSharedMemorySize, limit_w) == cudaSuccess &&
-          cudaOccupancyMaxActiveClusters(&n_w, (const void*)fw, &cw) == cudaSuccess && n_w >= 1 &&
-          (n_w >= units || n_clusters < units)) {
-        ctx->step_threads = 1024;
-        ctx->step_cs = cs_w;
-        ctx->step_smem = smem_w;
-        ctx->step_resident = n_w;
-      } else {
-        cudaGetLastError();
-      }
+    const int n_w = (long long)units * cs > ctx->n_sm ? wide_clusters(cs) : 0;
+    if (n_w >= 1 && (n_w >= units || n_clusters < units)) {
+      ctx->step_threads = 1024;
+      ctx->step_cs = cs / 2;
+      ctx->step_smem = (size_t)fused_smem_layout(cap_of(cs / 2), 32).total;
+      ctx->step_resident = n_w;
     }
     return cs;
   }
