@@ -273,7 +273,8 @@ int32_t fasa_sparse_decode_attn_static(fasa_ctx_t* ctx, const void* q, const voi
  * fasa_step_cluster_size tells.
  * When a workspace is given and the selection is large (n_sel_max * ceil(heads per set / 4)
  * >= 2048; >= 512 when all units together reach 24576 such rows; >= 256 when the cluster
- * kernel's grid exceeds two CTAs per SM), mode 1 ends the
+ * kernel's grid exceeds two CTAs per SM; >= 64 when it has more than one of 512 threads per SM with slices
+ * of at least 4096 tokens), mode 1 ends the
  * cluster kernel after the selection and attends with the split-K tensor-core kernel of
  * fasa_sparse_decode_attn (two launches instead of one; three beyond 16384 selected rows).  The
  * same hand-over happens, whatever the selection size, when the caches are page-locked host

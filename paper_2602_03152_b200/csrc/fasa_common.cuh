@@ -99,8 +99,13 @@ static inline bool fasa_attend_separately(const fasa_ctx* ctx, int n_sel_max, co
   // at 1024; B 32 x 4 heads with 7 query heads each, context 4096: 48.2 vs 63.5 us; a batch-1
   // step with 8 units stays in one launch: 28.7 vs 33.7 us at budget 512).
   const long long all_rows = rows * ctx->cfg.batch * ctx->n_sets;
+  // More than one 512-thread CTA per SM on long slices: the pairs' attention phases keep SMs that the launch of their own
+  // would share (96 units at 25 K: 57.3 -> 45.0 us at budget 256, 52.5 -> 42.0 at 64; 128 units 59.5 -> 51.8; at 8 K 30.1 ->
+  // 29.0; one CTA per unit, 128 units at 3 K: 28.3 against 29.7 us, stays in one launch).
+  const bool pairs = ctx->step_threads == 512 && ctx->step_cs >= 2 && (long long)ctx->cfg.batch * ctx->n_sets * ctx->step_cs > ctx->n_sm &&
+                     ctx->cfg.max_len / ctx->step_cs >= 4096;
   return workspace != nullptr &&
-         (rows >= 2048 || (several_waves && rows >= 256) || (rows >= 512 && all_rows >= 24576));
+         (rows >= 2048 || (pairs && rows >= 64) || (several_waves && rows >= 256) || (rows >= 512 && all_rows >= 24576));
 }
 
 cudaError_t fasa_stage_from_mapped(void* dq, const void* sq, size_t q_bytes, void* dk, const void* sk, void* dv,
