@@ -459,7 +459,7 @@ decode_attn_merge_kernel(const float* partial, const int32_t* n_rows,
 // batch 1 at 30 K 34.3 -> 32 us; equal lengths that filled the last wave before: the same.
 struct DenseDeal {
   long long total;         // tiles of all units
-  int n;                   // CTAs that take part: at least four tiles each
+  int n;                   // CTAs that take part
   int mine;                // tiles of a KV head of sequence `lane`
 };
 // (Products of tiles and CTAs are formed in 32 bits where they fit: a 64-bit division costs more than the rest of the set-up.)
@@ -473,7 +473,9 @@ __device__ __forceinline__ DenseDeal dense_deal(const int32_t* seq_lens, int bat
   d.total = __reduce_add_sync(0xffffffffu, d.mine);
   for (int b0 = 32; b0 < batch; b0 += 32) d.total += __reduce_add_sync(0xffffffffu, dense_tiles(seq_lens, b0 + lane, batch, max_len, status));
   d.total *= n_kv_heads;
-  d.n = (int)min((long long)n_ctas, max(1ll, d.total >> 2));
+  // a few tiles to each of a third of the CTAs, then 32 tiles to each before the others join: below that a CTA's start and
+  // its partial result cost more than its share (34 MB of 2 x 4 heads at 17 K: 24.6 us with all CTAs, 21.5 with a third)
+  d.n = (int)max(1ll, min((long long)n_ctas, max(d.total >> 5, min(d.total >> 2, (long long)(n_ctas / 3)))));
   return d;
 }
 
@@ -539,7 +541,6 @@ dense_attn_kernel(const AttnParams p) {
 __global__ void __launch_bounds__(kMergeThreads)
 dense_merge_kernel(const AttnParams p, int n_ctas) {
   pdl_wait_for_predecessor();
-  pdl_release_successor();
   const int bh = blockIdx.x, b = bh / p.n_q_heads, hq = bh % p.n_q_heads, h = hq / p.group;
   const int lane = threadIdx.x & 31, batch = p.n_cap;
   const DenseDeal d = dense_deal(p.n_rows, batch, p.n_kv_heads, p.max_len, n_ctas, lane, p.status);
