@@ -474,7 +474,7 @@ __device__ __forceinline__ DenseDeal dense_deal(const int32_t* seq_lens, int bat
   for (int b0 = 32; b0 < batch; b0 += 32) d.total += __reduce_add_sync(0xffffffffu, dense_tiles(seq_lens, b0 + lane, batch, max_len, status));
   d.total *= n_kv_heads;
   // a few tiles to each of a third of the CTAs, then 32 tiles to each before the others join: below that a CTA's start and
-  // its partial result cost more than its share (34 MB of 2 x 4 heads at 17 K: 24.6 us with all CTAs, 21.5 with a third)
+  // its partial result cost more than its share (70 MB of 2 x 4 heads at 17 K: 24.6 us with all CTAs, 22.2 with a third)
   d.n = (int)max(1ll, min((long long)n_ctas, max(d.total >> 5, min(d.total >> 2, (long long)(n_ctas / 3)))));
   return d;
 }

@@ -299,33 +299,50 @@ fused_decode_kernel(const FusedParams p) {
   const unsigned char* unit = p.proxy + (int64_t)su.kv * ((p.max_len + 15) >> 4) * pg.tile_bytes;
   float* srow = p.scores ? p.scores + (int64_t)u * p.max_len : nullptr;
   const int tiles_alloc = (p.max_len + 15) >> 4;
-  // Paged caches: the tiles of a batch are located through the block table.  The table is read
-  // one batch ahead (tp_next) so that its latency overlaps the proxy loads in flight.
-  const unsigned char* tp[PAGED ? TPI : 1];
-  const unsigned char* tp_next[PAGED ? TPI : 1];
-  auto locate = [&](const unsigned char* (&out)[PAGED ? TPI : 1], int T) {
+  // Paged caches: the block-table entries of the slice's pages go to shared memory first (over the selection's bit masks,
+  // which come later), as the index in the pool of the page's first tile; only the first batch, which leaves before they are
+  // there, reads the table itself.  (Looking each tile up in the table, a batch ahead of its loads, took 8 registers and the
+  // issue slots of two 64-bit products per tile: 12 sequences of 3-28 K tokens in pages of 64 58.8 -> 52.0 us, 16 of 64-126 K
+  // 218 -> 174 us; contiguous caches of those lengths 47.4 and 175 us.)
+  uint32_t* s_pages = s_mask;
+  const int page0 = PAGED ? (crank * per) >> p.pm.shift : 0;
+  auto tile_at = [&](int T) {
     if constexpr (PAGED) {
-#pragma unroll
-      for (int j = 0; j < TPI; ++j)
-        out[j] = p.proxy + proxy_tile_offset(p.pm, b, h, p.n_kv_heads, min(T + j, tiles_alloc - 1), tiles_alloc,
-                                             pg.tile_bytes, (T + j) * 16 < c1 ? p.status : nullptr);
+      const int s = p.pm.shift - 4;
+      const uint32_t first = s_pages[(min(T, (c1 - 1) >> 4) >> s) - page0];
+      return p.proxy + (int64_t)(first + (uint32_t)(T & ((1 << s) - 1))) * pg.tile_bytes;
+    } else {
+      return unit + (int64_t)T * pg.tile_bytes;
     }
   };
-  auto fetch = [&](uint4 (&a)[TPI][KB], int T, int grp) {      // (paged: tp holds the tiles of batch T)
+  auto fetch = [&](uint4 (&a)[TPI][KB], int T, int grp) {
 #pragma unroll
-    for (int j = 0; j < TPI; ++j) {
-      const unsigned char* tile;
-      if constexpr (PAGED) tile = tp[j];
-      else tile = unit + (int64_t)(T + j) * pg.tile_bytes;
-      load_tile<KB>(a[j], tile, pg, lane, (T + j) * 16 < c1, grp * KB);
-    }
+    for (int j = 0; j < TPI; ++j) load_tile<KB>(a[j], tile_at(T + j), pg, lane, (T + j) * 16 < c1, grp * KB);
   };
   const int step = kFW * TPI;
   int T = ((crank * per) >> 4) + warp * TPI;                  // slices start on a tile boundary
   const bool own_new = grows && c0 <= len_old && len_old < c1;
   uint4 a[TPI][KB];
-  locate(tp, T);
-  if (!own_new) fetch(a, T, 0);
+  if (!own_new) {
+    if constexpr (PAGED) {
+#pragma unroll
+      for (int j = 0; j < TPI; ++j)
+        load_tile<KB>(a[j], p.proxy + proxy_tile_offset(p.pm, b, h, p.n_kv_heads, min(T + j, tiles_alloc - 1), tiles_alloc, pg.tile_bytes, nullptr),
+                      pg, lane, (T + j) * 16 < c1);
+    } else {
+      fetch(a, T, 0);
+    }
+  }
+  if constexpr (PAGED) {
+    for (int i = tid; i < (nloc > 0 ? ((c1 - 1) >> p.pm.shift) - page0 + 1 : 0); i += kFT) {
+      int page = page_of(p.pm, b, (page0 + i) << p.pm.shift);
+      if (!page_ok(p.pm, page)) {
+        atomicOr(p.status, FASA_DEV_PAGE_CLAMPED);
+        page = 0;
+      }
+      s_pages[i] = (uint32_t)(page * p.n_kv_heads + h) << (p.pm.shift - 4);
+    }
+  }
 
   if (own_new) {
     // this CTA's slice holds the new row: K and V copies (16 lanes each) and the packed
@@ -413,7 +430,6 @@ fused_decode_kernel(const FusedParams p) {
   // ---- 1. scoring stream -> keys + first histogram ------------------------------------------
   {
     if (own_new) fetch(a, T, 0);                              // (the new row is in place now)
-    locate(tp_next, T + step);
     // The loop exists twice.  When the head's dominant channels fill whole 16-channel blocks and
     // exactly the KB x NG blocks this kernel is compiled for (4 n_dom = 32 KB NG: 8, 16, 32 or 64
     // FCs), a tile's loads and products need no run-time test of the geometry: the loads of a batch
@@ -425,7 +441,7 @@ fused_decode_kernel(const FusedParams p) {
 #pragma unroll
           for (int j = 0; j < TPI; ++j) {
             const unsigned char* tile;
-            if constexpr (PAGED) tile = tp[j];
+            if constexpr (PAGED) tile = tile_at(TT + j);
             else tile = unit + (int64_t)(TT + j) * (KB * NG * 512);
             const bool ok = (TT + j) * 16 < c1;
 #pragma unroll
@@ -452,16 +468,8 @@ fused_decode_kernel(const FusedParams p) {
             }
           }
           // the registers are free again: the next group, or the next batch of tiles, at once
-          if (grp + 1 < NG) {
-            fetch_x(a, T, grp + 1);
-          } else if ((T + step) * 16 < c1) {
-            if constexpr (PAGED) {
-#pragma unroll
-              for (int j = 0; j < TPI; ++j) tp[j] = tp_next[j];
-            }
-            fetch_x(a, T + step, 0);
-            locate(tp_next, T + 2 * step);
-          }
+          if (grp + 1 < NG) fetch_x(a, T, grp + 1);
+          else if ((T + step) * 16 < c1) fetch_x(a, T + step, 0);
         }
 #pragma unroll
         for (int pr = 0; pr < TPI / 2; ++pr) {

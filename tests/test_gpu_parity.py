@@ -1048,6 +1048,29 @@ def _logical(pool, table, need, P, Lm):
     return out[:, :, :Lm]
 
 
+@pytest.mark.parametrize("n_dom", [5, 8, 16, 32, 64])
+@pytest.mark.parametrize("P,lo,hi", [(16, 1, 31), (16, 4000, 9001), (64, 33, 5121), (1024, 1000, 8193), (8192, 8191, 9001)])
+def test_paged_step_where_slices_and_pages_do_not_align(P, lo, hi, n_dom):
+    # a slice of the cluster kernel that starts inside a page, ends in one's first tile, lies within one, is empty, or
+    # takes many batches of tiles per warp: every output is the contiguous one, bit for bit
+    w = C["c1"].replace(index=77, batch=2, max_len=9001, len_lo=lo, len_hi=hi, n_dom=n_dom)
+    t = synth.make_inputs(w, "cpu")
+    t["seq_lens"][0], t["seq_lens"][1] = lo, hi
+    r, f, kp, vp, tab, table, need = _paged_twin(w, t, P)
+    proxy_p = f.alloc_proxy()
+    r.build_proxy()
+    f.proxy_build(kp, proxy_p, r.seq_lens)
+    out_p, scores_p, idx_p, n_sel_p = (torch.zeros_like(x) for x in (r.out, r.scores, r.idx, r.n_sel))
+    for x in (r.out, r.scores, r.idx, r.n_sel):
+        x.zero_()
+    f.decode_step(r.q, kp, vp, proxy_p, r.seq_lens, w.budget, scores_p, idx_p, n_sel_p, out_p, None)
+    r.fasa.decode_step(r.q, r.k, r.v, r.proxy, r.seq_lens, w.budget, r.scores, r.idx, r.n_sel, r.out, None)
+    torch.cuda.synchronize()
+    assert f.device_status() == r.fasa.device_status() == 0
+    for x, y in ((scores_p, r.scores), (idx_p, r.idx), (n_sel_p, r.n_sel), (out_p, r.out)):
+        assert torch.equal(x, y)
+
+
 @pytest.mark.parametrize("P,cfg,kw", [
     (16, "c1", dict(batch=2, max_len=1000, len_lo=300, len_hi=990)),
     (64, "c3", dict(batch=3, max_len=2100, len_lo=500, len_hi=2000)),
