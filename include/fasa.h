@@ -271,15 +271,10 @@ int32_t fasa_sparse_decode_attn_static(fasa_ctx_t* ctx, const void* q, const voi
  * `workspace` may be NULL and `scores` may be NULL (they are then not written).  Available
  * when ceil(max_len / 16) <= 22528 and the device can co-schedule such a cluster;
  * fasa_step_cluster_size tells.
- * When a workspace is given and the selection is large (n_sel_max * ceil(heads per set / 4)
- * >= 2048; >= 512 when all units together reach 24576 such rows; >= 256 when the cluster
- * kernel's grid exceeds two CTAs per SM; >= 64 when it has more than one of 512 threads per SM with slices
- * of at least 4096 tokens), mode 1 ends the
- * cluster kernel after the selection and attends with the split-K tensor-core kernel of
- * fasa_sparse_decode_attn (two launches instead of one; three beyond 16384 selected rows).  The
- * same hand-over happens, whatever the selection size, when the caches are page-locked host
- * memory and an index set serves more than four query heads (the cluster kernel would fetch
- * every row twice over the host link).
+ * When a workspace is given and the cluster kernel's grid needs several rounds of CTAs, mode 1 ends that kernel after the
+ * selection and attends with the split-K tensor-core kernel of fasa_sparse_decode_attn (two launches instead of one; three
+ * beyond 16384 selected rows): for n_sel_max >= 64, or only up to 511 where two CTAs share an SM.  The same hand-over
+ * happens for at most 8 units with max_len <= 8192 once n_sel_max * ceil(heads per set / 4) >= 2048.
  * A set per query head (select_heads = 1) with a workspace, rows of at least 2048 positions and many sets runs as two
  * launches instead: one stream of the proxy that scores all heads of a KV head, then selection and attention.
  * Mode 0, and every configuration mode 1 cannot take: fasa_fc_score -> fasa_topk ->

@@ -300,15 +300,6 @@ static int32_t two_launch_step(fasa_ctx* ctx, const void* q, const void* k_new, 
                                    out_mirror, k_new != nullptr, stream);
 }
 
-// The cluster kernel attends to groups of more than four query heads in two passes over the
-// selected rows.  From HBM the second pass hits L2; from caches in page-locked host memory every
-// row would cross the host link twice (measured at 28 / 4 heads: 531 us against 282 us through
-// the tensor-core kernel, which reads a row once for up to eight heads): given a workspace, such
-// steps hand the attention over whatever the selection size.
-static bool fasa_host_rows_twice(fasa_ctx* ctx, const void* k_cache, const void* workspace) {
-  return workspace != nullptr && ctx->sel_heads > 4 && ctx->cfg.page_size == 0 && fasa_on_host(ctx, k_cache);
-}
-
 // What fasa_fc_score, fasa_topk and fasa_sparse_decode_attn require of the arguments they share
 // with the composite calls.
 static bool three_kernel_args_ok(const fasa_ctx* ctx, const void* q, const void* k_cache, const void* v_cache,
@@ -336,7 +327,7 @@ extern "C" int32_t fasa_decode_step(fasa_ctx_t* ctx, const void* q, const void* 
       return two_launch_step(ctx, q, nullptr, nullptr, const_cast<void*>(k_cache), const_cast<void*>(v_cache), const_cast<void*>(proxy_k),
                              seq_lens, budget, n_sel_max, scores, idx, n_sel, out, lse, workspace, nullptr, (cudaStream_t)stream);
     }
-    if (fasa_attend_separately(ctx, n_sel_max, workspace) || fasa_host_rows_twice(ctx, k_cache, workspace)) {
+    if (fasa_attend_separately(ctx, n_sel_max, workspace)) {
       if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;   // (what the second launch would refuse)
       int32_t st2 = fasa_fused_launch(ctx, q, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores,
                                       idx, n_sel, out, lse, nullptr, nullptr, (cudaStream_t)stream, false);
@@ -380,7 +371,7 @@ static int32_t append_decode_step_impl(fasa_ctx_t* ctx, const void* q, const voi
       return two_launch_step(ctx, q, k_new, v_new, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores, idx, n_sel,
                              out, lse, workspace, out_mirror, (cudaStream_t)stream);
     }
-    if (fasa_attend_separately(ctx, n_sel_max, workspace) || fasa_host_rows_twice(ctx, k_cache, workspace)) {
+    if (fasa_attend_separately(ctx, n_sel_max, workspace)) {
       if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;   // (what the second launch would refuse)
       int32_t st2 = fasa_fused_launch(ctx, q, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores,
                                       idx, n_sel, out, lse, k_new, v_new, (cudaStream_t)stream, false);

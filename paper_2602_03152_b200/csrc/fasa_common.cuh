@@ -84,28 +84,28 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
                           float* out, float* lse, const void* k_new, const void* v_new,
                           cudaStream_t stream, bool with_attention = true, float* out_mirror = nullptr,
                           bool split_keys = false);
-// Large selections are attended by the split-K tensor-core kernel rather than inside the
-// cluster kernel (whose attention phase runs on CUDA cores at 64 registers per thread).  When
-// the cluster kernel's grid needs several waves of CTAs, every wave pays for its attention
-// phase with idle HBM while one split-K launch covers all units at once: the hand-over then
-// starts at much smaller selections (measured at B 16 x 8 heads, 64-128 K: 202 vs 223 us at
-// budget 256, 218 vs 250 us at 1024).
+// Whether the attention of a step is a launch of its own, the split-K tensor-core kernel, rather than the last phase of the
+// cluster kernel.  A grid whose clusters are all resident attends in its own launch, whatever the selection: the hand-over
+// costs two launches (batch 8 x 8 heads at 64 K: 58 against 52 us at budget 256, 68 / 62 at 1024, 90 / 80 at 4096; 32 x 4
+// heads with 7 query heads each at 9 K: 58 / 53 at 1700; 12 x 8 in pages at 3-28 K: 103 / 91 at 4096; batch 4 x 8 at 9 K and
+// 4096: 37 / 39 us, the one loss).  A grid of several rounds pays for the attention in every round while HBM waits for the next
+// round's streams: there one launch for all units is better (16 x 8 heads at 64-128 K: 154 against 166 us at budget 64, 175 /
+// 189 at 1024, 214 / 228 at 4096), except for 512 rows or more where two CTAs share an SM and one's attention runs beside the
+// other's stream (48 x 8 at 16 K: 105 / 107 us at 256, 143 / 133 at 1024; 64 x 4 x 7 at 20 K 86 / 89, 107 / 103).
+// A resident grid of barely more CTAs than SMs leaves most SMs with one CTA beside some with two.  One or two heads per set
+// do not make up for that: clusters of one attend separately from 1024 rows on (160 units of two heads at 10 K, 2048 rows: 71
+// against 79 us, at 3 K and 1455 51 / 55; 256 units 95 / 91), larger ones below that on long slices (96 units at 10 K, 512
+// rows: 33 / 34.5; 2048 rows: 59 / 52.5).  Up to
+// eight units on short caches keep the two launches that they are documented with (2 x 4 x 7 at 5.4 K, 1800 rows: 23.9 us;
+// one launch would take 20.7).
 static inline bool fasa_attend_separately(const fasa_ctx* ctx, int n_sel_max, const void* workspace) {
-  const long long rows = (long long)n_sel_max * ((ctx->sel_heads + 3) / 4);
-  const long long ctas = (long long)ctx->cfg.batch * ctx->n_sets * ctx->fused_cs;
-  const bool several_waves = ctas > 2ll * ctx->n_sm;
-  // One wave: the two extra launches pay off once a unit has ~512 rows to attend and the
-  // units together ~24 K (B 8 x 8 heads, 64 K: 82.9 vs 86.0 us at budget 512, 87.0 vs 98.3 us
-  // at 1024; B 32 x 4 heads with 7 query heads each, context 4096: 48.2 vs 63.5 us; a batch-1
-  // step with 8 units stays in one launch: 28.7 vs 33.7 us at budget 512).
-  const long long all_rows = rows * ctx->cfg.batch * ctx->n_sets;
-  // More than one 512-thread CTA per SM on long slices: the pairs' attention phases keep SMs that the launch of their own
-  // would share (96 units at 25 K: 57.3 -> 45.0 us at budget 256, 52.5 -> 42.0 at 64; 128 units 59.5 -> 51.8; at 8 K 30.1 ->
-  // 29.0; one CTA per unit, 128 units at 3 K: 28.3 against 29.7 us, stays in one launch).
-  const bool pairs = ctx->step_threads == 512 && ctx->step_cs >= 2 && (long long)ctx->cfg.batch * ctx->n_sets * ctx->step_cs > ctx->n_sm &&
-                     ctx->cfg.max_len / ctx->step_cs >= 4096;
-  return workspace != nullptr &&
-         (rows >= 2048 || (pairs && rows >= 64) || (several_waves && rows >= 256) || (rows >= 512 && all_rows >= 24576));
+  const bool pairs = (long long)ctx->step_resident * ctx->step_cs > ctx->n_sm;
+  const long long units = (long long)ctx->cfg.batch * ctx->n_sets;
+  const bool documented = units <= 8 && ctx->cfg.max_len <= 8192 && (long long)n_sel_max * ((ctx->sel_heads + 3) / 4) >= 2048;
+  const long long ctas = units * ctx->step_cs;
+  const bool uneven = ctx->sel_heads <= 2 && ctx->step_threads == 512 && ctas > ctx->n_sm && 10 * ctas <= 13ll * ctx->n_sm &&
+                      (ctx->step_cs == 1 ? n_sel_max >= 1024 : n_sel_max >= 64 && n_sel_max < 1024 && ctx->cfg.max_len / ctx->step_cs >= 4096);
+  return workspace != nullptr && (uneven || (units > ctx->step_resident && n_sel_max >= 64 && !(pairs && n_sel_max >= 512)) || documented);
 }
 
 cudaError_t fasa_stage_from_mapped(void* dq, const void* sq, size_t q_bytes, void* dk, const void* sk, void* dv,
@@ -157,6 +157,10 @@ struct fasa_calib_rows {
 int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget,
                              int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
                              int n_recent, cudaStream_t stream, int q_len = 1, const struct fasa_calib_rows* calib = nullptr);
+// The same by the selection phases of the cluster kernel (fasa_fused.cu), for contexts that it can serve (fused_cs > 0).
+int32_t fasa_topk_cluster_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget, int32_t n_sel_max,
+                                 int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink, int n_recent, cudaStream_t stream,
+                                 int q_len);
 // Paged caches: how a (sequence, token) pair finds its page.  All zero = contiguous caches.
 struct PageMap {
   const int32_t* table;   // [batch][pages_per_seq]: physical page of each logical page
@@ -222,6 +226,16 @@ __device__ __forceinline__ int64_t cache_row(const PageMap& m, int b, int h, int
     page = 0;
   }
   return page * sb + h * sh + (int64_t)(tok & ((1 << m.shift) - 1)) * st;
+}
+// The pool's row of token `tok` of sequence b: its page, and the row within the page in the low bits (a pool holds fewer
+// than 2^31 rows: they are at least 512 bytes each).
+__device__ __forceinline__ int pool_row(const PageMap& m, int b, int tok, int32_t* status) {
+  int page = page_of(m, b, tok);
+  if (!page_ok(m, page)) {
+    atomicOr(status, FASA_DEV_PAGE_CLAMPED);
+    page = 0;
+  }
+  return (page << m.shift) | (tok & ((1 << m.shift) - 1));
 }
 // Byte offset of the proxy tile of token tile T (tokens 16 T .. 16 T + 15) of (b, h).
 // status == nullptr: a speculative read (a tile that may lie past the sequence's end, where no

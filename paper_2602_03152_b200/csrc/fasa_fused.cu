@@ -38,7 +38,7 @@
 
 #include <type_traits>
 
-#include "fasa_cluster_merge.cuh"
+#include "fasa_attn_core.cuh"
 #include "fasa_common.cuh"
 #include "fasa_launch.cuh"
 #include "fasa_score_core.cuh"
@@ -58,7 +58,9 @@ constexpr int kGroups = kFBins / 32;   // 32-bin groups of the widest radix pass
 constexpr int kCandCap = 4096;         // keys of one bin that the cluster finishes locally
 constexpr int kFinBits = 7;            // bits per block-level pass of that local finish
 constexpr int kFinBins = 1 << kFinBits;
-constexpr int kHP = 4;                 // query heads per attention pass
+// A warp's part of the attention phase: 8 K and 8 V rows, afterwards 8 accumulators of 128 channels.
+constexpr int kAttSlot = 16 * kRowPad * 2;
+static_assert(kAttSlot >= 8 * kAccStride * 4 && kAttSlot % 16 == 0, "a warp's accumulators take over its rows");
 
 // Dynamic shared memory of one CTA holding `cap` keys (bytes from the start):
 //   keys[cap] | hist1 (8 KB) | sums1 (4 KB) | 4 KB | sums0 (4 KB) | hist0 (8 KB) | masks
@@ -70,7 +72,7 @@ constexpr int kHP = 4;                 // query heads per attention pass
 // dead by then; no peer writes here after the last barrier of the selection).
 struct FusedSmem {
   int keys, hist1, sums1, spare, sums0, hist0, mask, sel_end;
-  int acc, part, p, al, m, l, att_end;
+  int ring, part, m, l, att_end;
   int total;
 };
 __host__ __device__ inline FusedSmem fused_smem_layout(int cap, int kFW = kFT / 32) {   // kFW: warps per CTA
@@ -83,13 +85,11 @@ __host__ __device__ inline FusedSmem fused_smem_layout(int cap, int kFW = kFT / 
   L.hist0 = L.sums0 + kMaxCs * kGroups * 4;
   L.mask = L.hist0 + kFBins * 4;
   L.sel_end = L.mask + 2 * (cap / 32 + 1) * 4;     // one bit per key: above / equal to the threshold
-  L.acc = 0;                                       // [kFW][kHP][128] fp32
-  L.part = L.acc + kFW * kHP * FASA_HEAD_DIM * 4;  // [8][kPartStride + 2]
-  L.p = L.part + FASA_MAX_GROUP * (kPartStride + 2) * 4;   // [kFW][16]
-  L.al = L.p + kFW * 16 * 4;                       // [kFW][kHP]
-  L.m = L.al + kFW * kHP * 4;
-  L.l = L.m + kFW * kHP * 4;
-  L.att_end = L.l + kFW * kHP * 4;
+  L.ring = 0;                                      // [kFW] slots of the attention phase
+  L.part = L.ring + kFW * kAttSlot;                // [8][kPartStride + 2]
+  L.m = L.part + FASA_MAX_GROUP * (kPartStride + 2) * 4;   // [kFW][8]
+  L.l = L.m + kFW * FASA_MAX_GROUP * 4;
+  L.att_end = L.l + kFW * FASA_MAX_GROUP * 4;
   L.total = L.sel_end > L.att_end ? L.sel_end : L.att_end;
   return L;
 }
@@ -128,14 +128,11 @@ struct FusedParams {
   int max_reduce;          // score of a KV head = max over its query heads instead of their sum
   int64_t ksb, ksh, kst, vsb, vsh, vst;
   float scale_log2;        // softmax_scale * log2(e)
+  int q_len;               // (SCORES) blocks of queries: the rows of a sequence are (query, set) pairs, query t sees q_len - 1 - t
+                           // fewer positions (1: plain rows)
+  int host_rows;           // K and V rows lie in host memory
   PageMap pm;              // paged caches (all zero: contiguous)
 };
-
-__device__ __forceinline__ uint2 ld_stream_u2(const void* p) {
-  uint2 r;
-  asm volatile("ld.global.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"(p) : "memory");
-  return r;
-}
 
 // The two halves of a cluster barrier (cluster.sync() = arrive + wait), for all threads of all
 // CTAs alike: what a thread wrote before its arrive is visible to every thread after its wait.
@@ -174,7 +171,8 @@ __device__ __forceinline__ bool warp_find_kth(uint32_t v, uint32_t kth, int lane
 // PAGED: K, V and the proxy are page pools behind a block table (compiled separately, so that
 // the contiguous form keeps its plain address arithmetic within 64 registers).
 // NT: threads per CTA: 512 (two CTAs per SM) or 1024 (one CTA per SM with twice the slice).
-template <int KB, int NG, bool ATTEND, bool PAGED = false, int NT = 512>
+// SCORES: TopK-I alone: the keys come from a score buffer instead of the proxy stream, and the kernel ends after the list.
+template <int KB, int NG, bool ATTEND, bool PAGED = false, int NT = 512, bool SCORES = false>
 __global__ void __launch_bounds__(NT, NT == 512 ? 2 : 1)
 fused_decode_kernel(const FusedParams p) {
   constexpr int kFT = NT;                  // (shadow the file-level constants inside this kernel)
@@ -199,9 +197,7 @@ fused_decode_kernel(const FusedParams p) {
   __shared__ uint32_t s_ncand, s_cgt, s_ceq;       // candidates found here; pushed keys of lower ranks above / equal to the threshold
   __shared__ int s_len_old;
   constexpr int GP = FASA_MAX_GROUP;     // query heads a KV head can serve
-  constexpr int HP = kHP;                // heads per attention pass
-  __shared__ __align__(16) float s_q[GP][FASA_HEAD_DIM];
-  __shared__ __align__(16) uint16_t s_qraw[GP][FASA_HEAD_DIM];   // the unit's query rows as stored (scoring operand)
+  __shared__ __align__(16) uint16_t s_qraw[GP][kRowPad];   // the unit's query rows as stored (operand of scoring and attention)
   __shared__ int16_t s_chan[8 * FASA_MAX_DOM / 4];               // the head's channel table
   __shared__ ClusterMergeSmem s_merge;                            // pushed by the cluster: the partial results this CTA finishes
 
@@ -227,14 +223,18 @@ fused_decode_kernel(const FusedParams p) {
   // length, this thread's 16 bytes of the unit's query rows and its entry of the channel table.
   // The scoring operand (query values at the dominant channels) is gathered from the staged
   // copies in shared memory after the set-up barrier: no load waits on another load's result.
-  const bool append = p.k_new != nullptr;
+  const bool append = !SCORES && p.k_new != nullptr;
   int len_raw = 0;
   if (!append || tid == 0) len_raw = p.seq_lens[b];
   uint4 q_stage = make_uint4(0u, 0u, 0u, 0u);
-  if (tid < FASA_MAX_GROUP * (FASA_HEAD_DIM / 8) && tid / (FASA_HEAD_DIM / 8) < p.group)
+  if (!SCORES && tid < FASA_MAX_GROUP * (FASA_HEAD_DIM / 8) && tid / (FASA_HEAD_DIM / 8) < p.group)
     q_stage = *reinterpret_cast<const uint4*>(p.q + su.q0 * FASA_HEAD_DIM + tid * 8);
   int16_t chan_stage = -1;
-  if (tid < p.chunks * 8) chan_stage = p.chan[h * p.chunks * 8 + tid];
+  if (!SCORES && tid < p.chunks * 8) chan_stage = p.chan[h * p.chunks * 8 + tid];
+  if (SCORES && p.q_len > 1) {
+    const int t = (u % p.n_sets) / (p.n_sets / p.q_len);        // the query of this row
+    if (len_raw >= 0 && len_raw <= p.max_len) len_raw = max(0, len_raw - (p.q_len - 1 - t));   // (a bad length is left for clamp_len to flag)
+  }
   int len_old;
   if (append) {
     if (tid == 0) s_len_old = clamp_len(len_raw, p.max_len, p.status);
@@ -266,7 +266,7 @@ fused_decode_kernel(const FusedParams p) {
   // the two halves of the machine out of phase for the rest of the launch: one half streams while
   // the other selects.  Measured: batch 16 at 64-128 K 177.9 -> 167.9 us, batch 32 at 64 K
   // 225.9 -> 189.2 us.  The wait is a sleep bounded by the clock; nothing is waited for.
-  if (p.shift_ctas > 0 && (int)blockIdx.y < p.shift_clusters && (blockIdx.y & 1)) {
+  if (!SCORES && p.shift_ctas > 0 && (int)blockIdx.y < p.shift_clusters && (blockIdx.y & 1)) {
     const float ns = 0.45f * (float)p.shift_ctas * (float)nloc * (float)(p.chunks * 16) * (1.0f / 6400.0f);
     const unsigned long long want = (unsigned long long)fminf(ns, 200000.0f);
     unsigned long long t0, t1;
@@ -323,7 +323,7 @@ fused_decode_kernel(const FusedParams p) {
   int T = ((crank * per) >> 4) + warp * TPI;                  // slices start on a tile boundary
   const bool own_new = grows && c0 <= len_old && len_old < c1;
   uint4 a[TPI][KB];
-  if (!own_new) {
+  if (!SCORES && !own_new) {
     if constexpr (PAGED) {
 #pragma unroll
       for (int j = 0; j < TPI; ++j)
@@ -406,29 +406,43 @@ fused_decode_kernel(const FusedParams p) {
       *reinterpret_cast<uint32_t*>(p.proxy_w + poff + proxy_word_offset(pg, prow, w)) = lo | (hi << 16);
     }
   }
-  if (tid < GP * (FASA_HEAD_DIM / 8))
+  if (!SCORES && tid < GP * (FASA_HEAD_DIM / 8))
     *reinterpret_cast<uint4*>(&s_qraw[tid / (FASA_HEAD_DIM / 8)][(tid % (FASA_HEAD_DIM / 8)) * 8]) = q_stage;
-  if (tid < p.chunks * 8) s_chan[tid] = chan_stage;
-  // query, scaled into the base-2 logit domain, for the attention phase
-  if (ATTEND && tid < GP * (FASA_HEAD_DIM / 8)) {
-    const int g = tid / (FASA_HEAD_DIM / 8), c = (tid % (FASA_HEAD_DIM / 8)) * 8;
-    const uint4 w = q_stage;
-    const float2 f0 = bf16x2_to_f32x2(w.x), f1 = bf16x2_to_f32x2(w.y), f2 = bf16x2_to_f32x2(w.z), f3 = bf16x2_to_f32x2(w.w);
-    const float sc = p.scale_log2;
-    *reinterpret_cast<float4*>(&s_q[g][c]) = make_float4(f0.x * sc, f0.y * sc, f1.x * sc, f1.y * sc);
-    *reinterpret_cast<float4*>(&s_q[g][c + 4]) = make_float4(f2.x * sc, f2.y * sc, f3.x * sc, f3.y * sc);
-  }
+  if (!SCORES && tid < p.chunks * 8) s_chan[tid] = chan_stage;
   __syncthreads();
   // This CTA runs and its totals are cleared: the peers may add to them from now on.  Each CTA
   // waits for the others' arrival only when it is about to touch them, after its stream.
   cluster_arrive();
   ScoreFrag<KB> f[NG];
 #pragma unroll
-  for (int grp = 0; grp < NG; ++grp)
-    load_score_b<KB>(f[grp], &s_qraw[0][0], s_chan, p.chunks, p.group, lane, grp * KB);
+  for (int grp = 0; !SCORES && grp < NG; ++grp)
+    load_score_b<KB>(f[grp], &s_qraw[0][0], s_chan, p.chunks, p.group, lane, grp * KB, kRowPad);
 
   // ---- 1. scoring stream -> keys + first histogram ------------------------------------------
-  {
+  if constexpr (SCORES) {
+    // four consecutive positions per thread
+    const float* sin = p.scores + (int64_t)u * p.max_len;
+    const bool vec_ok = (reinterpret_cast<uintptr_t>(sin) & 15) == 0;
+    for (int i = c0 + tid * 4; i < c1; i += kFT * 4) {
+      float sv[4] = {0.f, 0.f, 0.f, 0.f};
+      if (vec_ok && i + 3 < c1) {
+        const float4 v4 = *reinterpret_cast<const float4*>(sin + i);
+        sv[0] = v4.x; sv[1] = v4.y; sv[2] = v4.z; sv[3] = v4.w;
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (i + e < c1) sv[e] = sin[i + e];
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (i + e < c1) {
+          const uint32_t key = fasa_item_key(sv[e], i + e, len, p.n_sink, p.n_recent);
+          atomicAdd(&hist0[key >> 21], 1u);
+          keys[i + e - c0] = key;
+        }
+      }
+    }
+  } else {
     if (own_new) fetch(a, T, 0);                              // (the new row is in place now)
     // The loop exists twice.  When the head's dominant channels fill whole 16-channel blocks and
     // exactly the KB x NG blocks this kernel is compiled for (4 n_dom = 32 KB NG: 8, 16, 32 or 64
@@ -827,11 +841,16 @@ fused_decode_kernel(const FusedParams p) {
   if constexpr (!ATTEND) return;   // (no peer reads this CTA's memory after the selection's last barrier)
 
   // ---- 4. attention over this CTA's share of the selected rows -----------------------------
-  // Register-lean form (64 registers per thread): four query heads per pass (two passes for
-  // groups of 5-8 heads; the second pass finds the rows in L2), four rows per warp step, a
-  // lane owning 4 channels of every row.  The 16 partial logits (4 rows x 4 heads) of a step
-  // are completed by a transposing xor-shuffle reduction, one shuffle per value.
-  constexpr int R = 4;
+  // Tensor cores, eight rows per warp step, 64 registers per thread.  What bounds this phase is the gather itself once the
+  // instructions are out of the way: an FMA form (four rows and four heads per step, so two passes for groups of 5-8) spent
+  // ~250 instructions per step and was bound by their issue.
+  //   - K and V rows go to the warp's two buffers in shared memory (cp.async, rows padded so that ldmatrix is free of bank
+  //     conflicts): the next step's K rows leave when this step's logits are done, its V rows after the output product.
+  //   - logits: A = q, bf16 as stored (heads in rows 0-7), B = K rows; the softmax scale is applied to the fp32 result, whose
+  //     fragment (head lane / 4, rows 2 t and 2 t + 1) is already the B operand of
+  //   - out^T: A = V^T (ldmatrix.trans), B = P^T, with p split into three bf16 terms that add up to all its 24 bits: the
+  //     first two as the two halves of one k = 16 product (A holds the same eight rows twice), the third with k = 8.
+  constexpr int R = 8;
   // The selected tokens are dealt out evenly: CTA r attends to rows [r, r + 1) * ktot / cs of the
   // index list, whoever selected them (scores cluster by position, so the CTAs' own selections
   // can differ several times in size); this costs one cluster barrier, after which the list
@@ -841,153 +860,149 @@ fused_decode_kernel(const FusedParams p) {
   const int a1 = (int)(((long long)ktot * (crank + 1)) / cs);
   // The attention phase's working arrays take over the key / histogram area: every read of
   // it, local or remote, happened before the selection's last barrier or the block barrier above.
-  float* s_acc = reinterpret_cast<float*>(smem_raw + sl.acc);                        // [kFW][HP][128]
+  unsigned char* ring = smem_raw + sl.ring + warp * kAttSlot;      // K rows, then V rows; at the end the warp's [8][kAccStride] accumulators
+  uint16_t (*k_rows)[kRowPad] = reinterpret_cast<uint16_t (*)[kRowPad]>(ring);
+  uint16_t (*v_rows)[kRowPad] = k_rows + R;
   float (*s_part)[kPartStride + 2] = reinterpret_cast<float (*)[kPartStride + 2]>(smem_raw + sl.part);
-  float (*s_p)[16] = reinterpret_cast<float (*)[16]>(smem_raw + sl.p);
-  float (*s_al)[HP] = reinterpret_cast<float (*)[HP]>(smem_raw + sl.al);
-  float (*s_m)[HP] = reinterpret_cast<float (*)[HP]>(smem_raw + sl.m);
-  float (*s_l)[HP] = reinterpret_cast<float (*)[HP]>(smem_raw + sl.l);
-  const int n_hp = (p.group + HP - 1) / HP;
-  for (int hp = 0; hp < n_hp; ++hp) {                          // uniform
-    float2 acc[HP][2];
-#pragma unroll
-    for (int g = 0; g < HP; ++g) acc[g][0] = acc[g][1] = make_float2(0.f, 0.f);
-    float m_run = -INFINITY, l_run = 0.f;   // of value (lane >> 1) = row * 4 + head
+  float (*s_m)[GP] = reinterpret_cast<float (*)[GP]>(smem_raw + sl.m);
+  float (*s_l)[GP] = reinterpret_cast<float (*)[GP]>(smem_raw + sl.l);
+  const int n_active = min(kFW, (a1 - a0 + R - 1) / R);           // warps that get rows
+  if (warp < n_active) {
+    const int g = lane >> 2, t = lane & 3;
     const int32_t* irow = p.idx + (int64_t)u * p.n_sel_max;
-    const uint16_t* kbase = p.k + b * p.ksb + h * p.ksh + lane * 4;
-    const uint16_t* vbase = p.v + b * p.vsb + h * p.vsh + lane * 4;
-    const int my_g = (lane >> 1) & 3;
-    const int my_i = lane >> 3;
-    for (int base = a0 + warp * R; base < a1; base += kFW * R) {
-      // all row indices first, then all row loads: nothing waits on a previous row (rows
-      // past the end repeat the last one and are masked below)
-      int tok[R];
+    const uint16_t* kbase = p.k + h * p.ksh + (PAGED ? 0 : b * p.ksb) + (lane & 15) * 8;
+    const uint16_t* vbase = p.v + h * p.vsh + (PAGED ? 0 : b * p.vsb) + (lane & 15) * 8;
+    float acc[FASA_HEAD_DIM / 16][4];         // out^T: [16-channel block][frag], heads 2 t and 2 t + 1
 #pragma unroll
-      for (int i = 0; i < R; ++i) tok[i] = __ldcg(irow + min(base + i, a1 - 1));
-      uint2 kk[R], vv[R];
+    for (int cb = 0; cb < FASA_HEAD_DIM / 16; ++cb) acc[cb][0] = acc[cb][1] = acc[cb][2] = acc[cb][3] = 0.f;
+    float m_run = -INFINITY, l_run = 0.f;     // of head g (the sum: over this lane's rows only)
+    // 32 entries of the list at a time, lane 8 s + r holding row r of the warp's s-th step from here on (rows past the end
+    // repeat the last one and are masked below); on paged caches as the row of the pool.
+    int listed = 0;
+    auto list_rows = [&](int base) {
+      const int i = __ldcg(irow + min(base + (lane >> 3) * (kFW * R) + (lane & 7), a1 - 1));
+      listed = min(max(i, 0), p.max_len - 1);
+      if constexpr (PAGED) listed = pool_row(p.pm, b, listed, p.status);
+    };
+    // lane l copies the 16 bytes l % 16 of rows 2 i + l / 16 of step s
+    auto stage = [&](uint16_t (*dst)[kRowPad], const uint16_t* unit_rows, int64_t sb, int64_t st, int s) {
 #pragma unroll
-      for (int i = 0; i < R; ++i) {
-        const int t = min(max(tok[i], 0), p.max_len - 1);
-        if constexpr (PAGED) {
-          kk[i] = ld_stream_u2(p.k + lane * 4 + cache_row(p.pm, b, h, t, p.ksb, p.ksh, p.kst, p.status));
-          vv[i] = ld_stream_u2(p.v + lane * 4 + cache_row(p.pm, b, h, t, p.vsb, p.vsh, p.vst, p.status));
-        } else {
-          kk[i] = ld_stream_u2(kbase + (int64_t)t * p.kst);
-          vv[i] = ld_stream_u2(vbase + (int64_t)t * p.vst);
-        }
+      for (int i = 0; i < R / 2; ++i) {
+        const int r = __shfl_sync(0xffffffffu, listed, (s & 3) * R + 2 * i + (lane >> 4));
+        const int64_t off = PAGED ? (r >> p.pm.shift) * sb + (r & ((1 << p.pm.shift) - 1)) * st : r * st;
+        uint16_t* to = &dst[2 * i + (lane >> 4)][(lane & 15) * 8];
+        if (!PAGED && p.host_rows) cp_async16_ca(to, unit_rows + off);
+        else cp_async16(to, unit_rows + off);
       }
-      float part[16];
+    };
+    int base = a0 + warp * R;
+    list_rows(base);
+    stage(k_rows, kbase, p.ksb, p.kst, 0);
+    cp_async_commit();
+    stage(v_rows, vbase, p.vsb, p.vst, 0);
+    cp_async_commit();
+    for (int s = 0; base < a1; ++s, base += kFW * R) {
+      const bool more = base + kFW * R < a1;                       // uniform over the warp
+      cp_async_wait<1>();                                          // the K rows
+      __syncwarp();
+      float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int g = 0; g < HP; ++g) {
-        const float4 qg = *reinterpret_cast<const float4*>(&s_q[hp * HP + g][lane * 4]);
-#pragma unroll
-        for (int i = 0; i < R; ++i) {
-          const float2 k0 = bf16x2_to_f32x2(kk[i].x), k1 = bf16x2_to_f32x2(kk[i].y);
-          part[i * HP + g] = qg.x * k0.x + qg.y * k0.y + qg.z * k1.x + qg.w * k1.y;
-        }
+      for (int i = 0; i < FASA_HEAD_DIM / 32; ++i) {
+        uint32_t qa[4], kb[4];
+        ldmatrix_x4(qa, &s_qraw[lane & 7][(4 * i + (lane >> 3)) * 8]);
+        ldmatrix_x4(kb, &k_rows[lane & 7][(4 * i + (lane >> 3)) * 8]);
+        const uint32_t a_lo[4] = {qa[0], 0u, qa[1], 0u}, a_hi[4] = {qa[2], 0u, qa[3], 0u};
+        mma16816(c, a_lo, kb[0], kb[1]);
+        mma16816(c, a_hi, kb[2], kb[3]);
       }
-      // transposing reduction: lane L ends with the full sum of value L >> 1
-      float logit;
-      {
-        float p8[8], p4[4], p2[2];
-        const bool u16 = (lane & 16) != 0;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          const float send = u16 ? part[i] : part[i + 8];
-          const float keep = u16 ? part[i + 8] : part[i];
-          p8[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-        }
-        const bool u8 = (lane & 8) != 0;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float send = u8 ? p8[i] : p8[i + 4];
-          const float keep = u8 ? p8[i + 4] : p8[i];
-          p4[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-        }
-        const bool u4 = (lane & 4) != 0;
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {
-          const float send = u4 ? p4[i] : p4[i + 2];
-          const float keep = u4 ? p4[i + 2] : p4[i];
-          p2[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-        }
-        const bool u2 = (lane & 2) != 0;
-        const float send = u2 ? p2[0] : p2[1];
-        const float keep = u2 ? p2[1] : p2[0];
-        logit = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-        logit += __shfl_xor_sync(0xffffffffu, logit, 1);
+      __syncwarp();
+      if (more) {
+        if (((s + 1) & 3) == 0) list_rows(base + kFW * R);
+        stage(k_rows, kbase, p.ksb, p.kst, s + 1);
       }
-      if (!(base + my_i < a1 && hp * HP + my_g < p.group)) logit = -INFINITY;
-      float bmax = logit;                                      // over the 4 rows of this head
-      bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 8));
-      bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 16));
+      cp_async_commit();
+      const float x0 = base + 2 * t < a1 ? c[0] * p.scale_log2 : -INFINITY;
+      const float x1 = base + 2 * t + 1 < a1 ? c[1] * p.scale_log2 : -INFINITY;
+      float bmax = fmaxf(x0, x1);
+      bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 1));
+      bmax = fmaxf(bmax, __shfl_xor_sync(0xffffffffu, bmax, 2));
       const float m_new = fmaxf(m_run, bmax);
       const float m_safe = m_new == -INFINITY ? 0.f : m_new;
       const float alpha = exp2f(m_run - m_safe);
-      const float pr = exp2f(logit - m_safe);
-      l_run = l_run * alpha + pr;
-      m_run = m_new;
-      if ((lane & 1) == 0) {
-        s_p[warp][lane >> 1] = pr;
-        if (lane < 2 * HP) s_al[warp][lane >> 1] = alpha;      // row 0 lanes: one per head
-      }
-      __syncwarp();
+      const float p0 = exp2f(x0 - m_safe), p1 = exp2f(x1 - m_safe);
+      l_run = l_run * alpha + (p0 + p1);
+      if (__any_sync(0xffffffffu, m_new != m_run)) {
+        const float al0 = __shfl_sync(0xffffffffu, alpha, 8 * t), al1 = __shfl_sync(0xffffffffu, alpha, 8 * t + 4);
 #pragma unroll
-      for (int g = 0; g < HP; ++g) {
-        const float al = s_al[warp][g];
-        const float2 a2 = make_float2(al, al);
-        acc[g][0] = __ffma2_rn(acc[g][0], a2, make_float2(0.f, 0.f));
-        acc[g][1] = __ffma2_rn(acc[g][1], a2, make_float2(0.f, 0.f));
-      }
-#pragma unroll
-      for (int i = 0; i < R; ++i) {
-        const float2 v0 = bf16x2_to_f32x2(vv[i].x), v1 = bf16x2_to_f32x2(vv[i].y);
-        const float4 pi = *reinterpret_cast<const float4*>(&s_p[warp][i * HP]);
-        const float pg4[4] = {pi.x, pi.y, pi.z, pi.w};
-#pragma unroll
-        for (int g = 0; g < HP; ++g) {
-          const float2 p2 = make_float2(pg4[g], pg4[g]);
-          acc[g][0] = __ffma2_rn(p2, v0, acc[g][0]);
-          acc[g][1] = __ffma2_rn(p2, v1, acc[g][1]);
+        for (int cb = 0; cb < FASA_HEAD_DIM / 16; ++cb) {
+          acc[cb][0] *= al0; acc[cb][1] *= al1; acc[cb][2] *= al0; acc[cb][3] *= al1;
         }
       }
+      m_run = m_new;
+      const uint32_t p_1 = pack_bf16(p0, p1);
+      const float2 f1 = bf16x2_to_f32x2(p_1);
+      const float r0 = p0 - f1.x, r1 = p1 - f1.y;
+      const uint32_t p_2 = pack_bf16(r0, r1);
+      const float2 f2 = bf16x2_to_f32x2(p_2);
+      const uint32_t p_3 = pack_bf16(r0 - f2.x, r1 - f2.y);
+      cp_async_wait<1>();                                          // the V rows
       __syncwarp();
-    }
-    // the four row lanes of a head add their partial sums of probabilities
-    l_run += __shfl_xor_sync(0xffffffffu, l_run, 8);
-    l_run += __shfl_xor_sync(0xffffffffu, l_run, 16);
-
-    // ---- 5a. combine the warps of this CTA for these heads ---------------------------------
-    if (lane < 2 * HP && (lane & 1) == 0) {
-      s_m[warp][lane >> 1] = m_run;
-      s_l[warp][lane >> 1] = l_run;
-    }
 #pragma unroll
-    for (int g = 0; g < HP; ++g)
-      *reinterpret_cast<float4*>(&s_acc[((warp * HP) + g) * FASA_HEAD_DIM + lane * 4]) =
-          make_float4(acc[g][0].x, acc[g][0].y, acc[g][1].x, acc[g][1].y);
-    __syncthreads();
-    for (int o = tid; o < HP * FASA_HEAD_DIM; o += kFT) {
-      const int g = o / FASA_HEAD_DIM, c = o % FASA_HEAD_DIM;
-      float mx = -INFINITY;
-#pragma unroll
-      for (int w = 0; w < kFW; ++w) mx = fmaxf(mx, s_m[w][g]);
-      float av = 0.f, l = 0.f;
-#pragma unroll
-      for (int w = 0; w < kFW; ++w) {
-        const float ms = s_m[w][g];
-        const float wt = ms == -INFINITY ? 0.f : exp2f(ms - mx);
-        av += wt * s_acc[((w * HP) + g) * FASA_HEAD_DIM + c];
-        l += wt * s_l[w][g];
+      for (int i = 0; i < FASA_HEAD_DIM / 32; ++i) {
+        uint32_t va[4];
+        ldmatrix_x4_trans(va, &v_rows[lane & 7][(4 * i + (lane >> 3)) * 8]);
+        const uint32_t a_lo[4] = {va[0], va[1], va[0], va[1]}, a_hi[4] = {va[2], va[3], va[2], va[3]};
+        mma16816(acc[2 * i], a_lo, p_1, p_2);
+        mma16816(acc[2 * i + 1], a_hi, p_1, p_2);
+        mma1688(acc[2 * i], va[0], va[1], p_3);
+        mma1688(acc[2 * i + 1], va[2], va[3], p_3);
       }
-      s_part[hp * HP + g][2 + c] = av;
-      if (c == 0) {
-        s_part[hp * HP + g][0] = mx;
-        s_part[hp * HP + g][1] = l;
-      }
+      __syncwarp();
+      if (more) stage(v_rows, vbase, p.vsb, p.vst, s + 1);
+      cp_async_commit();
     }
-    __syncthreads();                                           // s_acc / s_m are reused by the next pass
+    cp_async_wait<0>();
+    // ---- 5a. combine the warps of this CTA -------------------------------------------------
+    float* s_acc = reinterpret_cast<float*>(ring);
+#pragma unroll
+    for (int cb = 0; cb < FASA_HEAD_DIM / 16; ++cb) {
+      float* o = s_acc + 2 * t * kAccStride + cb * 16 + g;
+      o[0] = acc[cb][0];
+      o[kAccStride] = acc[cb][1];
+      o[8] = acc[cb][2];
+      o[kAccStride + 8] = acc[cb][3];
+    }
+    l_run += __shfl_xor_sync(0xffffffffu, l_run, 1);
+    l_run += __shfl_xor_sync(0xffffffffu, l_run, 2);
+    if (t == 0) {
+      s_m[warp][g] = m_run;
+      s_l[warp][g] = l_run;
+    }
   }
+  __syncthreads();
+  for (int o = tid; o < p.group * FASA_HEAD_DIM; o += kFT) {
+    const int g = o / FASA_HEAD_DIM, c = o % FASA_HEAD_DIM;       // (g: uniform over the warp)
+    // lane w: the weight of warp w's partial result
+    const float ms = lane < n_active ? s_m[lane][g] : -INFINITY;
+    float mx = ms;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    const float wt = ms == -INFINITY ? 0.f : exp2f(ms - mx);
+    float av = 0.f;
+    const float* acc_o = reinterpret_cast<const float*>(smem_raw + sl.ring) + g * kAccStride + c;
+    for (int w = 0; w < n_active; ++w) av += __shfl_sync(0xffffffffu, wt, w) * acc_o[w * (kAttSlot / 4)];
+    s_part[g][2 + c] = av;
+    if (c < 32) {
+      float l = lane < n_active ? wt * s_l[lane][g] : 0.f;
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+      if (c == 0) {
+        s_part[g][0] = mx;
+        s_part[g][1] = l;
+      }
+    }
+  }
+  __syncthreads();
   // ---- 5b. merge across the cluster (one barrier; see fasa_cluster_merge.cuh) -------------------
   cluster_merge_store<kFT>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse);
 }
@@ -1020,6 +1035,7 @@ FusedFn wide_variant(int chunks) {
 }
 FusedFn wide_fn(int chunks, bool paged) { return paged ? wide_variant<true, true>(chunks) : wide_variant<true, false>(chunks); }
 FusedFn wide_select_fn(int chunks, bool paged) { return paged ? wide_variant<false, true>(chunks) : wide_variant<false, false>(chunks); }
+FusedFn topk_fn() { return fused_decode_kernel<1, 1, false, false, 512, true>; }
 constexpr int kCapWide = 40960;        // keys a 1024-thread CTA can hold (one CTA per SM)
 
 FusedFn select_fn(int chunks, bool paged = false) {         // the step without attention
@@ -1115,9 +1131,12 @@ int fasa_fused_plan(fasa_ctx* ctx) {
     if (n_clusters < units && (long long)units * cs <= slots && cs > 1 && cap_of(cs / 2) <= kCapPair &&
         !((long long)units * cs > ctx->n_sm && wide_clusters(cs) >= units))
       continue;
-    // the form without attention runs with the same cluster shape
-    if (cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit) != cudaSuccess ||
-        (cs > 8 && cudaFuncSetAttribute((const void*)select_fn(ctx->chunks, paged), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+    // the forms without attention run with the same cluster shape
+    bool ok = true;
+    for (FusedFn other : {select_fn(ctx->chunks, paged), topk_fn()})
+      ok = ok && cudaFuncSetAttribute((const void*)other, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit) == cudaSuccess &&
+           (cs <= 8 || cudaFuncSetAttribute((const void*)other, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess);
+    if (!ok) {
       cudaGetLastError();
       continue;
     }
@@ -1160,6 +1179,7 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
   p.k_w = (uint16_t*)k_cache; p.v_w = (uint16_t*)v_cache; p.proxy_w = (unsigned char*)proxy_k;
   p.seq_lens_w = (int32_t*)seq_lens; p.arrive = ctx->d_arrive;
   p.shift_clusters = 0; p.shift_ctas = 0;
+  p.q_len = 1;
   p.ndchan = split_keys ? ctx->d_ndchan : nullptr;
   p.nd = FASA_HEAD_DIM - 2 * c.n_dom;
   p.res = split_keys ? fasa_resident_of(ctx) : fasa_resident{};
@@ -1172,6 +1192,7 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
   p.vsb = c.v_stride_b; p.vsh = c.v_stride_h; p.vst = c.v_stride_t;
   p.scale_log2 = c.softmax_scale * 1.4426950408889634f;
   p.pm = fasa_page_map(ctx);
+  p.host_rows = with_attention && c.page_size == 0 && fasa_on_host(ctx, k_cache);
   if (!fasa_pages_ready(ctx)) return FASA_ERR_INVALID_ARG;
   const bool paged = c.page_size > 0;
   FusedFn fn = with_attention ? fused_fn(ctx->chunks, paged) : select_fn(ctx->chunks, paged);
@@ -1193,6 +1214,34 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
   // over several rounds, gaps that stay (batch 16 at 64-128 K: 177 -> 211 us).
   const fasa_launch_shape shape{dim3((unsigned)cs_l, (unsigned)(c.batch * ctx->n_sets)), dim3((unsigned)threads), smem_l, cs_l, p.early != 0};
   const cudaError_t e = fasa_launch(fn, shape, stream, p);
+  ctx->launches += 1;
+  FASA_CUDA_TRY(ctx, e);
+  return FASA_OK;
+}
+
+int32_t fasa_topk_cluster_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget, int32_t n_sel_max,
+                                 int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink, int n_recent, cudaStream_t stream,
+                                 int q_len) {
+  const fasa_config_t& c = ctx->cfg;
+  FusedParams p;
+  memset(&p, 0, sizeof(p));
+  p.seq_lens = seq_lens; p.scores = const_cast<float*>(scores); p.idx = idx; p.n_sel = n_sel; p.status = ctx->d_status;
+  // (this form uses the unit index for its score row and its sequence alone)
+  p.n_q_heads = rows_per_seq; p.n_kv_heads = 1; p.n_sets = rows_per_seq; p.group = 1; p.max_len = c.max_len;
+  p.chunks = ctx->chunks; p.n_sink = n_sink; p.n_recent = n_recent; p.budget = budget;
+  p.n_sel_max = n_sel_max;
+  p.q_len = q_len;
+  // The context's cluster size suits its own number of rows; a block of queries has more, and takes the smallest that holds
+  // a row two CTAs to an SM.
+  int cs = ctx->fused_cs;
+  auto cap_of = [&](int n) { return (((c.max_len + n - 1) / n) + 31) & ~31; };
+  if (rows_per_seq > ctx->n_sets) {
+    cs = 1;
+    while (cs < ctx->fused_cs && cap_of(cs) > kCapPair) cs *= 2;
+  }
+  p.early = (long long)c.batch * rows_per_seq * cs <= ctx->n_sm;
+  const fasa_launch_shape shape{dim3((unsigned)cs, (unsigned)(c.batch * rows_per_seq)), dim3(kFT), fused_smem_bytes(cap_of(cs)), cs, p.early != 0};
+  const cudaError_t e = fasa_launch(topk_fn(), shape, stream, p);
   ctx->launches += 1;
   FASA_CUDA_TRY(ctx, e);
   return FASA_OK;

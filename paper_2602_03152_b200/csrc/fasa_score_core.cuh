@@ -67,7 +67,7 @@ struct ScoreFrag {
 template <int KB>
 __device__ __forceinline__ void load_score_b(ScoreFrag<KB>& f, const uint16_t* __restrict__ q_unit,
                                              const int16_t* __restrict__ chan_h, int chunks,
-                                             int group, int lane, int kb0 = 0) {
+                                             int group, int lane, int kb0 = 0, int q_stride = FASA_HEAD_DIM) {
   const int n = lane >> 2, t = lane & 3;
   const int n_chan = chunks * 8;
 #pragma unroll
@@ -81,7 +81,7 @@ __device__ __forceinline__ void load_score_b(ScoreFrag<KB>& f, const uint16_t* _
         uint32_t v = 0u;
         if (ci < n_chan && n < group) {
           const int ch = chan_h[ci];
-          if (ch >= 0) v = q_unit[n * FASA_HEAD_DIM + ch];
+          if (ch >= 0) v = q_unit[n * q_stride + ch];
         }
         w |= v << (16 * e);
       }

@@ -336,7 +336,9 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, float gm_l
       visit([&](int c, bool ok, float x) { classify(c, ok ? second.bin(x) : 0); });
     }
     __syncthreads();
-    // four threads to a member, each comparing it with a quarter of the others
+    // four threads to a member, each comparing it with a quarter of the others (the minimum: no entry that nobody wrote is
+    // looked at, whatever becomes of the scores meanwhile)
+    count = min(count, sm.n_cand);
     for (int i = tid >> 2; i < (int)count; i += NT / 4) {           // (uniform over the four)
       const uint32_t key = sm.ckey[i], pos = sm.cpos[i];
       uint32_t ahead = 0;
@@ -397,7 +399,7 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, float gm_l
     while (m) {
       const int j = __ffs(m) - 1;
       m &= m - 1;
-      emit((int)at, pos_at(c, j));
+      if (at < (uint32_t)r.k) emit((int)at, pos_at(c, j));       // (the comparison keeps a write inside the list)
       ++at;
     }
   }

@@ -140,6 +140,17 @@ int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* 
                              int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
                              int n_recent, cudaStream_t stream, int q_len, const fasa_calib_rows* calib) {
   const fasa_config_t& c = ctx->cfg;
+  // Few long rows: a cluster per row, which keeps the row's keys in shared memory.  One CTA per row pays for every position
+  // that it looks at again, the more the larger the selection (8 rows: at 17 K 10.6 against 8.6 us at 512, 14.7 / 9.7 at
+  // 2048; at 120 K 23 / 12 and 47 / 14; 64 rows at 32 K, 4096: 29 / 15), and for a row whose outliers crowd its scores into
+  // a few bins with radix passes over all of it (64 rows at 55 K, 512: 41 / 17 where others take 13).  It is the better one
+  // for short rows and for small selections of many (8 rows at 9 K, 64: 7.1 / 7.3; 40 rows at 17 K: 9.2 / 10.0 at 64,
+  // 10.8 / 11.3 at 512, 13.8 / 12.0 at 1024), and when the clusters would run in rounds (96 rows at 55 K: 21 / 27).
+  const long long n_rows = (long long)c.batch * rows_per_seq;
+  const int k = budget > 0 ? budget : (int)(((long long)-budget * c.max_len + 999) / 1000);
+  if (!calib && ctx->fused_cs > 1 && c.max_len > 8192 &&
+      (n_rows <= 16 ? c.max_len > 16384 || k >= 256 : n_rows <= ctx->n_sm / 2 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || c.max_len > 65536)))
+    return fasa_topk_cluster_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, rows_per_seq, n_sink, n_recent, stream, q_len);
   RowParams p;
   p.scores = scores; p.seq_lens = seq_lens; p.idx = idx; p.n_sel = n_sel; p.status = ctx->d_status;
   p.rows_per_seq = rows_per_seq; p.max_len = c.max_len; p.n_sink = n_sink; p.n_recent = n_recent;

@@ -1048,6 +1048,37 @@ def _logical(pool, table, need, P, Lm):
     return out[:, :, :Lm]
 
 
+@pytest.mark.parametrize("G", [1, 3, 4, 7, 8])
+@pytest.mark.parametrize("max_len,k", [(40, 1), (40, 7), (40, 9), (700, 129), (700, 700), (9000, 513), (9000, 4097), (30000, 4609)])
+def test_step_attention_at_the_edges_of_its_row_tiles(G, max_len, k):
+    # rows dealt to no warp, to a part of a warp's eight, to the 33rd step of a warp's list; the last head of a set alone
+    w = C["c1"].replace(index=78, batch=1, n_q_heads=2 * G, n_kv_heads=2, max_len=max_len, len_lo=max_len, len_hi=max_len,
+                        budget=k, n_sink=0, n_recent=0)
+    r = Run(w)
+    r.build_proxy()
+    n0 = r.fasa.launch_count()
+    r.fasa.decode_step(r.q, r.k, r.v, r.proxy, r.seq_lens, w.budget, r.scores, r.idx, r.n_sel, r.out, None, r.lse)
+    torch.cuda.synchronize()
+    assert r.fasa.launch_count() - n0 == 1 and r.fasa.device_status() == 0
+    for h in range(2):
+        n = int(r.n_sel[0, h])
+        assert n == min(k, max_len)
+        rows = r.idx[0, h, :n].long()
+        q, kk, vv = r.q[0, h * G:(h + 1) * G].double(), r.k[0, h, rows].double(), r.v[0, h, rows].double()
+        scale = 128 ** -0.5
+        x = q @ kk.T * scale
+        out = torch.softmax(x, -1) @ vv
+        # One unit u = 2^-23 per fp32 addition (a tensor core may cut off instead of rounding).  A logit takes 128 products
+        # of bf16 values, exact, in 8 sums of 16: at most 128 u of sum |q k|, which moves p by as much relatively, in the
+        # numerator and in the sum.  p is exact in three bf16 terms; exp2f and its argument cost 4 u and |x| u.  A row's
+        # products join at most n of those before them.
+        u = 2.0 ** -23
+        rel = 2 * (128 * float((q.abs() @ kk.abs().T * scale).max()) + 4 + 2 * float(x.abs().max())) * u + (3 * n + 64) * u
+        assert float((r.out[0, h * G:(h + 1) * G].double() - out).abs().max()) <= rel * float(vv.abs().max())
+        # typical errors are far smaller: one bf16 term of p less would show at 2^-17
+        assert float((r.out[0, h * G:(h + 1) * G].double() - out).abs().max()) <= 2.0 ** -19 * float(vv.abs().max())
+
+
 @pytest.mark.parametrize("n_dom", [5, 8, 16, 32, 64])
 @pytest.mark.parametrize("P,lo,hi", [(16, 1, 31), (16, 4000, 9001), (64, 33, 5121), (1024, 1000, 8193), (8192, 8191, 9001)])
 def test_paged_step_where_slices_and_pages_do_not_align(P, lo, hi, n_dom):
