@@ -302,6 +302,7 @@ template <bool SPARSE, bool PAGED, bool CLUSTER, bool HOSTMEM = false, bool KSPL
 __global__ void __launch_bounds__(kMmaThreads, KSPLIT || PAGED ? 4 : 5)
 decode_attn_mma_kernel(const AttnParams p) {
   __shared__ ClusterMergeSmem s_merge;              // (CLUSTER only: written by the peers)
+  if constexpr (CLUSTER) cluster_arrive();          // this CTA runs; each waits for that much before it writes to a peer
   pdl_wait_for_predecessor();
   pdl_release_successor();
   const int u = blockIdx.y;
@@ -362,6 +363,7 @@ decode_attn_mma_kernel(const AttnParams p) {
   });
   if constexpr (CLUSTER) {
     __syncthreads();
+    cluster_wait();
     cg::cluster_group cluster = cg::this_cluster();
     cluster_merge_store<kMmaThreads>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse);
   }

@@ -15,6 +15,11 @@
 constexpr int kMergePartStride = FASA_HEAD_DIM + 4;   // a head's partial in shared memory: m, l, acc[128], padding
 constexpr int kMergeMaxCs = 16;                        // CTAs per cluster at most
 
+// The two halves of a cluster barrier (cluster.sync() = arrive + wait), for all threads of all CTAs alike: what a thread
+// wrote before its arrive is visible to every thread after its wait.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 // What the peers write into: must not share memory with anything the owning CTA still uses
 // when the first peer finishes its part.
 struct ClusterMergeSmem {
@@ -25,7 +30,8 @@ struct ClusterMergeSmem {
 // part[g] = (m, l, acc[128]) of head g of this CTA, base-2 logit domain, complete and visible to
 // the whole block.  NT threads call this together, in every CTA of the cluster (the cluster
 // size must be a power of two <= 16).  out / lse rows start at query head q0; out_mirror and
-// lse may be null.
+// lse may be null.  The peers must be known to run before this is called (their shared memory is written): a cluster barrier
+// since the kernel's start, or cluster_arrive() at the start and cluster_wait() before the call.
 template <int NT>
 __device__ __forceinline__ void cluster_merge_store(cooperative_groups::cluster_group& cluster,
                                                     const float (*part)[kMergePartStride], ClusterMergeSmem& sm,

@@ -134,11 +134,6 @@ struct FusedParams {
   PageMap pm;              // paged caches (all zero: contiguous)
 };
 
-// The two halves of a cluster barrier (cluster.sync() = arrive + wait), for all threads of all
-// CTAs alike: what a thread wrote before its arrive is visible to every thread after its wait.
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t v, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {

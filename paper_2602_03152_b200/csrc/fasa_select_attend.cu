@@ -53,7 +53,7 @@ select_attend_kernel(const SelAttnParams p) {
   __shared__ int s_last;
   const int tid = threadIdx.x, lane = tid & 31;
   // (the merge writes into the peers' shared memory: each CTA says that it runs, and waits for that much at the end)
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  cluster_arrive();
   cg::cluster_group cluster = cg::this_cluster();
   const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
   const int u = blockIdx.y;
@@ -118,7 +118,7 @@ select_attend_kernel(const SelAttnParams p) {
   // new ones, below
   if (p.append && tid == 0) s_last = atomicAdd(p.arrive, 1) == (int)(gridDim.x * gridDim.y) - 1;
   __syncthreads();
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_wait();
   cluster_merge_store<NT>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse);
   if (p.append && tid < 32 && s_last) {
     if (tid == 0) *p.arrive = 0;

@@ -429,6 +429,42 @@ def test_large_selection_is_attended_by_the_split_k_kernel():
     assert r.fasa.device_status() == 0
 
 
+def _attention_error(q, k, v, rows, out, lse):
+    """Largest deviation of one head's output from float64 over the listed rows, relative to the largest value, and that
+    of the log-sum-exp."""
+    lg = (k[rows].double() @ q.double()) / math.sqrt(128.0)
+    err = (torch.softmax(lg, 0) @ v[rows].double() - out.double()).abs().max() / v[rows].double().abs().max()
+    return float(err), abs(float(torch.logsumexp(lg, 0)) - float(lse))
+
+
+@pytest.mark.parametrize("n_sel_max", [64, 300, 2048, 16384])       # clusters of 1, 4 and 8 splits
+def test_sparse_attention_over_lists_shorter_than_the_splits(n_sel_max):
+    # a split without rows reaches the merge, in which the splits of a unit write into each other's shared memory,
+    # before the others have started
+    w = C["c1"].replace(batch=40, n_q_heads=8, n_kv_heads=2, max_len=2048, len_lo=2048, len_hi=2048, n_sink=0, n_recent=0, budget=16)
+    r = Run(w, n_sel_max=n_sel_max)
+    most = min(n_sel_max, 2048)
+    counts = torch.tensor([[0, 1, 31, 32, 33, 257, most, 0, 16, most - 1][(3 * b + h) % 10] for b in range(40) for h in range(2)]).clamp(max=most)
+    r.n_sel.copy_(counts.view(40, 2))
+    g = torch.Generator().manual_seed(n_sel_max)
+    rows = [torch.randperm(2048, generator=g)[:int(n)].sort().values for n in counts]
+    for u, ids in enumerate(rows):
+        r.idx[u // 2, u % 2, :ids.numel()] = ids.int().cuda()
+    r.fasa.sparse_decode_attn(r.q, r.k, r.v, r.idx, r.n_sel, r.out, r.ws, r.lse)
+    torch.cuda.synchronize()
+    assert r.fasa.device_status() == 0
+    out, lse = r.out.cpu(), r.lse.cpu()
+    for u, ids in enumerate(rows):
+        b, h = u // 2, u % 2
+        for hq in range(4 * h, 4 * h + 4):
+            if ids.numel() == 0:
+                assert float(out[b, hq].abs().max()) == 0.0 and float(lse[b, hq]) == float("-inf")
+                continue
+            # (the kernel's probabilities carry 17 bits and its sums 24: 1e-4 of the largest value covers both)
+            e, el = _attention_error(r.t["q"][b, hq], r.t["k"][b, h], r.t["v"][b, h], ids, out[b, hq], lse[b, hq])
+            assert e <= 1e-4 and el <= 1e-4, (u, hq)
+
+
 @pytest.mark.parametrize("heads,lens,page", [
     ((8, 2), [20000, 0, 1, 16385, 17], 0),          # units shorter than a share, empty ones, shares that span several units
     ((7, 1), [16900], 0),                           # one unit over all CTAs
