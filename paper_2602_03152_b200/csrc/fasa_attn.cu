@@ -340,7 +340,7 @@ decode_attn_mma_kernel(const AttnParams p) {
   int32_t* s_idx = reinterpret_cast<int32_t*>(attn_smem_raw + sizeof(MmaSmem<kMmaWarps>));
   if (SPARSE) {
     for (int i = threadIdx.x; i < r1 - r0; i += kMmaThreads) {
-      int tok = __ldg(irow + r0 + i);
+      int tok = irow[r0 + i];                        // (not through the read-only path: the kernel ahead may have written it)
       if (tok < 0 || tok >= p.max_len) {
         atomicOr(p.status, FASA_DEV_IDX_CLAMPED);
         tok = 0;

@@ -103,8 +103,7 @@ calib_score_kernel(const uint16_t* __restrict__ q, const uint16_t* __restrict__ 
 // marked positions of an FC list at a time.
 constexpr int kParts = 8;
 __global__ void __launch_bounds__(256)
-calib_intersect_kernel(const int32_t* __restrict__ idx, const int32_t* __restrict__ seq_lens,
-                       unsigned long long* __restrict__ counts, unsigned long long* __restrict__ n_used,
+calib_intersect_kernel(const int32_t* idx, const int32_t* seq_lens, unsigned long long* counts, unsigned long long* n_used,
                        int n_q_heads, int max_len, int top_k) {
   extern __shared__ uint32_t marked[];
   const int u = blockIdx.x;

@@ -213,7 +213,8 @@ __device__ __forceinline__ float dot8(const float2 (&q)[4], const uint4& k) {
 
 __device__ __forceinline__ bool page_ok(const PageMap& m, int page) { return page >= 0 && page < m.n_pages; }
 __device__ __forceinline__ int page_of(const PageMap& m, int b, int tok) {
-  return __ldg(m.table + (int64_t)b * m.pages_per_seq + (tok >> m.shift));
+  // (not through the read-only path: the table may change in stream order, and kernels wait for their predecessor inside)
+  return m.table[(int64_t)b * m.pages_per_seq + (tok >> m.shift)];
 }
 // Element offset of row `tok` of (sequence b, KV head h) in a K or V cache, for reading: an
 // entry outside the pool reads page 0 and raises the status bit.

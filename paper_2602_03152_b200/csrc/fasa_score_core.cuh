@@ -65,8 +65,7 @@ struct ScoreFrag {
 // q_unit: first query head of the KV head; chan_h: the head's 8 * chunks channel ids (-1 =
 // padding).  Column n = lane / 4 of the B matrix is query head n (zero for n >= group).
 template <int KB>
-__device__ __forceinline__ void load_score_b(ScoreFrag<KB>& f, const uint16_t* __restrict__ q_unit,
-                                             const int16_t* __restrict__ chan_h, int chunks,
+__device__ __forceinline__ void load_score_b(ScoreFrag<KB>& f, const uint16_t* q_unit, const int16_t* chan_h, int chunks,
                                              int group, int lane, int kb0 = 0, int q_stride = FASA_HEAD_DIM) {
   const int n = lane >> 2, t = lane & 3;
   const int n_chan = chunks * 8;

@@ -102,3 +102,22 @@ def test_calib_select_is_host_only_and_agrees_with_the_oracle(lib):
         binding.calib_select(torch.from_numpy(counts), torch.from_numpy(used), Hkv, top_k, 65)
     with pytest.raises(binding.FasaError):
         binding.calib_select(torch.from_numpy(counts), torch.from_numpy(used), 5, top_k, 4)
+
+
+def test_kernels_that_wait_inside_read_nothing_through_the_read_only_path():
+    # A kernel launched early starts before the one ahead of it has written: what it reads must not be declared constant
+    # for its lifetime (const __restrict__ parameters, __ldg).  The channel tables are written when the context is created.
+    kernels = 0
+    for name in sorted(os.listdir(build.CSRC)):
+        text = open(os.path.join(build.CSRC, name)).read()
+        if name.endswith(".cuh"):
+            assert "__ldg(" not in text and not re.search(r"const \w+\* __restrict__", text), name
+        for part in text.split("__global__")[1:]:
+            part = part.split("\nextern \"C\"")[0]
+            if "pdl_wait_for_predecessor()" not in part:
+                continue
+            kernels += 1
+            constant = re.findall(r"const \w+\* __restrict__ (\w+)", part[:part.index("{")])
+            assert set(constant) <= {"chan", "ndchan"}, (name, constant)
+            assert "__ldg(" not in part, name
+    assert kernels >= 10
