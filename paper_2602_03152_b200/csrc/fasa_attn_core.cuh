@@ -98,8 +98,9 @@ __device__ __forceinline__ float (*mma_part(unsigned char* smem))[kMergePartStri
 }
 
 // B operand of the logits: q[head g][channels], bf16 as stored, for the 8 blocks of 16 channels.
-// P: launch parameters with the fields of the attention kernels (q, k, v and their strides, group, ks ...).
-template <bool KSPLIT, typename P>
+// P: launch parameters with the fields of the attention kernels (q, k, v and their strides, group, ks ...).  FROM_L2: the
+// loads bypass L1 (a kernel that has not waited for its predecessor yet).
+template <bool KSPLIT, bool FROM_L2 = false, typename P>
 __device__ __forceinline__ void attn_load_query(uint32_t (&qb)[8][2], const P& p, const SelUnit& su, int lane) {
   const int g = lane >> 2, t = lane & 3, h = su.h;
   const uint16_t* qh = p.q + (su.q0 + (g < p.group ? g : 0)) * FASA_HEAD_DIM;
@@ -115,8 +116,9 @@ __device__ __forceinline__ void attn_load_query(uint32_t (&qb)[8][2], const P& p
       w0 = q_at(kb * 16 + 2 * t) | (q_at(kb * 16 + 2 * t + 1) << 16);
       w1 = q_at(kb * 16 + 2 * t + 8) | (q_at(kb * 16 + 2 * t + 9) << 16);
     } else {
-      w0 = *reinterpret_cast<const uint32_t*>(qh + kb * 16 + 2 * t);
-      w1 = *reinterpret_cast<const uint32_t*>(qh + kb * 16 + 2 * t + 8);
+      const uint32_t* qw = reinterpret_cast<const uint32_t*>(qh + kb * 16 + 2 * t);
+      w0 = FROM_L2 ? __ldcg(qw) : qw[0];
+      w1 = FROM_L2 ? __ldcg(qw + 4) : qw[4];
     }
     qb[kb][0] = g < p.group ? w0 : 0u;
     qb[kb][1] = g < p.group ? w1 : 0u;

@@ -58,18 +58,16 @@ select_attend_kernel(const SelAttnParams p) {
   const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
   const int u = blockIdx.y;
   const SelUnit su = sel_unit(u, p.n_sets, p.group, p.n_q_heads, p.n_kv_heads);
-  // Before the first half has ended: only what it does not write.  (It lets this kernel start after its own wait, so
-  // everything older is complete; an appended token's length is stored below.)
-  const int old_len = clamp_len(p.seq_lens[su.b], p.max_len, p.status);
+  // Before the first half has ended: its inputs alone, the lengths and the query, are read, and no result is written.  The
+  // first half lets this kernel start after its own wait, so what is older than it is complete, and these loads take it
+  // from L2: nothing says that an L1 line of that age is current before this kernel's own wait.  (The appended token's
+  // length is stored below.)
+  const int old_len = clamp_len(__ldcg(p.seq_lens + su.b), p.max_len, p.status);
   const int len = p.append && old_len < p.max_len ? old_len + 1 : old_len;
   uint32_t qb[8][2];
-  attn_load_query<false>(qb, p, su, lane);
+  attn_load_query<false, true>(qb, p, su, lane);
   sel_begin<NT>(sm);
   const SelPlan plan = sel_plan(len, p.budget, p.n_sink, p.n_recent, p.n_sel_max);
-  if (crank == 0 && tid == 0) {
-    if (plan.clamped) atomicOr(p.status, FASA_DEV_NSEL_CLAMPED);
-    p.n_sel[u] = plan.ktot;
-  }
   // this CTA's share of the list
   const int a0 = (int)(((long long)plan.ktot * crank) / cs), a1 = (int)(((long long)plan.ktot * (crank + 1)) / cs);
   int32_t* s_idx = reinterpret_cast<int32_t*>(dsm + p.idx_off);
@@ -80,11 +78,6 @@ select_attend_kernel(const SelAttnParams p) {
       out_idx[rank] = pos;
     }
   };
-  for (int i = tid; i < plan.n_forced; i += NT) {
-    int rank, pos;
-    sel_forced(plan, i, &rank, &pos);
-    take(rank, pos);
-  }
   SelRow<SelScores> row;
   row.src = SelScores{p.scores + (int64_t)u * p.max_len};
   row.lo = plan.lo;
@@ -96,6 +89,15 @@ select_attend_kernel(const SelAttnParams p) {
   if (gs > 0 && !(row.k > 0 && row.k < n_free && (long long)row.k * (gs == 3 ? 12 : 43) <= n_free)) gs = 0;
   pdl_wait_for_predecessor();
   pdl_release_successor();
+  if (crank == 0 && tid == 0) {
+    if (plan.clamped) atomicOr(p.status, FASA_DEV_NSEL_CLAMPED);
+    p.n_sel[u] = plan.ktot;
+  }
+  for (int i = tid; i < plan.n_forced; i += NT) {
+    int rank, pos;
+    sel_forced(plan, i, &rank, &pos);
+    take(rank, pos);
+  }
   float gm_lo = INFINITY, gm_hi = -INFINITY;
   if (gs > 0) {
     float* gm = reinterpret_cast<float*>(dsm);

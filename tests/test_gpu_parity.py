@@ -613,6 +613,35 @@ def test_index_sets_per_query_head_in_two_launches(kw, page):
         assert torch.equal(px[0][b, :, :L // 16], px[1][b, :, :L // 16])
 
 
+def test_two_launch_steps_back_to_back_see_their_own_query_and_lengths():
+    # the second launch starts before the first has ended and reads the lengths and the query then: in a loop that rewrites
+    # the query's buffer on the stream and lets the lengths grow, every step must equal the one that had the GPU to itself
+    w = C["c1"].replace(batch=4, max_len=2200, len_lo=300, len_hi=2100, budget=48, n_sink=4, n_recent=32, sel_heads=1)
+    steps = [synth.make_step_inputs(w, s, "cuda") for s in range(12)]
+    got = []
+    for alone in (True, False):
+        r = Run(w)
+        r.build_proxy()
+        q = torch.empty_like(steps[0]["q"])
+        outs = []
+        torch.cuda.synchronize()
+        for s in steps:
+            q.copy_(s["q"])
+            o = (torch.empty_like(r.idx).fill_(-7), torch.empty_like(r.n_sel), torch.empty_like(r.out))
+            if alone:
+                torch.cuda.synchronize()
+            r.fasa.append_decode_step(q, s["k_new"], s["v_new"], r.k, r.v, r.proxy, r.seq_lens, w.budget, None, *o, r.ws)
+            if alone:
+                torch.cuda.synchronize()
+            outs.append(o)
+        torch.cuda.synchronize()
+        assert r.fasa.device_status() == 0
+        got.append((outs, r.seq_lens.clone()))
+    assert torch.equal(got[0][1], got[1][1])
+    for a, b in zip(got[0][0], got[1][0]):
+        assert all(torch.equal(x, y) for x, y in zip(a, b))
+
+
 def test_index_sets_per_query_head_large_selection_and_static_scratch():
     # one head per set: the split route starts at n_sel_max >= 2048; the no-workspace variant agrees
     w = C["c1"].replace(batch=1, n_q_heads=8, n_kv_heads=2, max_len=6000, len_lo=5000, len_hi=6000, budget=2500,
