@@ -365,7 +365,22 @@ decode_attn_mma_kernel(const AttnParams p) {
     __syncthreads();
     cluster_wait();
     cg::cluster_group cluster = cg::this_cluster();
-    cluster_merge_store<kMmaThreads>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse);
+    if constexpr (SPARSE && !KSPLIT)
+      cluster_merge_store<kMmaThreads>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse, [&](int g) {
+        const int u = unit_again();
+        const SelUnit s = sel_unit(u, p.n_sets, p.group, p.n_q_heads, p.n_kv_heads);
+        ExactOutput<PAGED> e;
+        e.q = p.q + (s.q0 + g) * FASA_HEAD_DIM;
+        e.k = p.k + s.h * p.ksh + (PAGED ? 0 : (s.b / p.q_len) * p.ksb);
+        e.v = p.v + s.h * p.vsh + (PAGED ? 0 : (s.b / p.q_len) * p.vsb);
+        e.list = p.idx + (int64_t)u * p.n_sel_max;
+        e.n = min(max(p.n_rows[u], 0), p.n_cap);
+        e.status = p.status; e.pm = p.pm; e.ksb = p.ksb; e.kst = p.kst; e.vsb = p.vsb; e.vst = p.vst;
+        e.b = (s.b / p.q_len); e.max_len = p.max_len; e.scale_log2 = p.scale_log2;
+        return e;
+      });
+    else   // (the dense pass and split key caches go without)
+      cluster_merge_store<kMmaThreads>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse);
   }
 }
 

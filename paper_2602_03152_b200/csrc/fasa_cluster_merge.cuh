@@ -10,6 +10,8 @@
 
 #include <cooperative_groups.h>
 
+#include <type_traits>
+
 #include "fasa_common.cuh"
 
 constexpr int kMergePartStride = FASA_HEAD_DIM + 4;   // a head's partial in shared memory: m, l, acc[128], padding
@@ -27,15 +29,84 @@ struct ClusterMergeSmem {
   alignas(8) float rml[kMergeMaxCs][FASA_MAX_GROUP][2];                 // every CTA's (m, l) per head
 };
 
+// Infinite values.  A probability enters the output products of the tensor-core forms as a sum of bf16 terms, of which the
+// later ones may be zero or negative, and rows past the end of a tile repeat the last one with probability zero: an infinite
+// entry of V then gives NaN where its sum with the other rows is an infinity.  An output that is not finite is therefore
+// computed once more by a warp, row by row with multiply-adds.  (Here, because the attention loops have no register to
+// spare: a test at their end, a branch in them or a second copy of them cost 2 to 10 % of a step; this costs 0.2 us of the
+// smallest ones, 13.4 -> 13.6 us, and nothing that shows of most others.)
+template <bool PAGED>
+struct ExactOutput {
+  const uint16_t* q;              // the query head
+  const uint16_t* k;              // (of the KV head; contiguous caches: of the sequence)
+  const uint16_t* v;
+  const int32_t* list;            // n rows
+  int32_t* status;
+  PageMap pm;
+  int64_t ksb, kst, vsb, vst;
+  int n, b, max_len;
+  float scale_log2;
+};
+// One warp: channel c of the output.
+template <bool PAGED>
+__device__ __forceinline__ float exact_output(const ExactOutput<PAGED>& r, int c) {
+  const int lane = threadIdx.x & 31;
+  const uint2 qw = *reinterpret_cast<const uint2*>(r.q + lane * 4);
+  const float2 q0 = bf16x2_to_f32x2(qw.x), q1 = bf16x2_to_f32x2(qw.y);
+  float m = -INFINITY, l = 0.f, a = 0.f;
+#pragma unroll 1
+  for (int i = 0; i < r.n; ++i) {
+    const int tok = min(max(r.list[i], 0), r.max_len - 1);
+    const int row = PAGED ? pool_row(r.pm, r.b, tok, r.status) : tok;
+    const int page = PAGED ? row >> r.pm.shift : 0, in = PAGED ? row & ((1 << r.pm.shift) - 1) : row;
+    const uint16_t* kr = r.k + page * r.ksb + in * r.kst;
+    const uint16_t* vr = r.v + page * r.vsb + in * r.vst;
+    const uint2 kw = *reinterpret_cast<const uint2*>(kr + lane * 4);
+    const float2 k0 = bf16x2_to_f32x2(kw.x), k1 = bf16x2_to_f32x2(kw.y);
+    float x = q0.x * k0.x + q0.y * k0.y + q1.x * k1.x + q1.y * k1.y;
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    x *= r.scale_log2;
+    const float m_new = fmaxf(m, x), m_safe = m_new == -INFINITY ? 0.f : m_new;
+    const float alpha = exp2f(m - m_safe), pr = exp2f(x - m_safe);
+    l = l * alpha + pr;
+    a = fmaf(pr, bf16_bits_to_f32(vr[c]), a * alpha);
+    m = m_new;
+  }
+  return l > 0.f ? a / l : 0.f;
+}
+struct NoExactOutput {};
+// The CTA's unit, read anew: what is derived from it where exact_output is called shall not be kept since the kernel's start.
+__device__ __forceinline__ int unit_again() {
+  int u;
+  asm volatile("mov.u32 %0, %%ctaid.y;" : "=r"(u));
+  return u;
+}
+
 // part[g] = (m, l, acc[128]) of head g of this CTA, base-2 logit domain, complete and visible to
 // the whole block.  NT threads call this together, in every CTA of the cluster (the cluster
 // size must be a power of two <= 16).  out / lse rows start at query head q0; out_mirror and
 // lse may be null.  The peers must be known to run before this is called (their shared memory is written): a cluster barrier
-// since the kernel's start, or cluster_arrive() at the start and cluster_wait() before the call.
-template <int NT>
+// since the kernel's start, or cluster_arrive() at the start and cluster_wait() before the call.  exact(g): what is needed to
+// compute the outputs of head g of this unit row by row (ExactOutput), for those that are not finite.
+template <int NT, typename Exact = NoExactOutput>
 __device__ __forceinline__ void cluster_merge_store(cooperative_groups::cluster_group& cluster,
                                                     const float (*part)[kMergePartStride], ClusterMergeSmem& sm,
-                                                    int group, int64_t q0, float* out, float* out_mirror, float* lse) {
+                                                    int group, int64_t q0, float* out, float* out_mirror, float* lse,
+                                                    Exact exact = Exact()) {
+  // a warp: the value of a lane that has one at (g, c), computed anew where it is not finite
+  auto settled = [&](float ov, bool has, int g, int c) -> float {
+    if constexpr (!std::is_same<Exact, NoExactOutput>::value) {
+#pragma unroll 1
+      for (uint32_t odd = __ballot_sync(0xffffffffu, has && !(fabsf(ov) < INFINITY)); odd != 0u; odd &= odd - 1u) {
+        const int l = __ffs(odd) - 1;
+        const auto e = exact(__shfl_sync(0xffffffffu, g, l));
+        const float x = exact_output(e, __shfl_sync(0xffffffffu, c, l));
+        if ((int)(threadIdx.x & 31) == l) ov = x;
+      }
+    }
+    return ov;
+  };
   const int cs = (int)cluster.num_blocks();
   const int crank = (int)cluster.block_rank();
   const int tid = threadIdx.x;
@@ -44,7 +115,7 @@ __device__ __forceinline__ void cluster_merge_store(cooperative_groups::cluster_
   if (cs == 1) {                              // nothing to merge
     for (int o = tid; o < n_out; o += NT) {
       const int g = o / FASA_HEAD_DIM, c = o % FASA_HEAD_DIM;
-      const float l = part[g][1], ov = l > 0.f ? part[g][2 + c] / l : 0.f;
+      const float l = part[g][1], ov = settled(l > 0.f ? part[g][2 + c] / l : 0.f, true, g, c);
       out[q0 * FASA_HEAD_DIM + o] = ov;
       if (out_mirror) out_mirror[q0 * FASA_HEAD_DIM + o] = ov;
       if (lse && c == 0) lse[q0 + g] = l > 0.f ? (part[g][0] + log2f(l)) * 0.6931471805599453f : -INFINITY;
@@ -79,10 +150,10 @@ __device__ __forceinline__ void cluster_merge_store(cooperative_groups::cluster_
       av += __shfl_xor_sync(0xffffffffu, av, off);
       l += __shfl_xor_sync(0xffffffffu, l, off);
     }
+    const int c = (crank << lw) + (t & (cw - 1));
+    const float ov = settled(l > 0.f ? av / l : 0.f, ok && r == 0, g, c);
     if (ok && r == 0) {
-      const int c = (crank << lw) + (t & (cw - 1));
       const int64_t hq = q0 + g;
-      const float ov = l > 0.f ? av / l : 0.f;
       out[hq * FASA_HEAD_DIM + c] = ov;
       if (out_mirror) out_mirror[hq * FASA_HEAD_DIM + c] = ov;
       if (lse && c == 0) lse[hq] = l > 0.f ? (mx + log2f(l)) * 0.6931471805599453f : -INFINITY;

@@ -999,7 +999,19 @@ fused_decode_kernel(const FusedParams p) {
   }
   __syncthreads();
   // ---- 5b. merge across the cluster (one barrier; see fasa_cluster_merge.cuh) -------------------
-  cluster_merge_store<kFT>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse);
+  cluster_merge_store<kFT>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse, [&](int g) {
+    const int u = unit_again();
+    const SelUnit s = sel_unit(u, p.n_sets, p.group, p.n_q_heads, p.n_kv_heads);
+    ExactOutput<PAGED> e;
+    e.q = p.q + (s.q0 + g) * FASA_HEAD_DIM;
+    e.k = p.k + s.h * p.ksh + (PAGED ? 0 : s.b * p.ksb);
+    e.v = p.v + s.h * p.vsh + (PAGED ? 0 : s.b * p.vsb);
+    e.list = p.idx + (int64_t)u * p.n_sel_max;
+    e.n = p.n_sel[u];
+    e.status = p.status; e.pm = p.pm; e.ksb = p.ksb; e.kst = p.kst; e.vsb = p.vsb; e.vst = p.vst;
+    e.b = s.b; e.max_len = p.max_len; e.scale_log2 = p.scale_log2;
+    return e;
+  });
 }
 
 size_t fused_smem_bytes(int cap) { return (size_t)fused_smem_layout(cap).total; }

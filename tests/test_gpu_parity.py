@@ -465,6 +465,53 @@ def test_sparse_attention_over_lists_shorter_than_the_splits(n_sel_max):
             assert e <= 1e-4 and el <= 1e-4, (u, hq)
 
 
+@pytest.mark.parametrize("launches,kw", [
+    (1, dict(batch=2, n_q_heads=14, n_kv_heads=2, max_len=900, budget=77)),                            # the cluster kernel
+    (2, dict(batch=48, n_q_heads=32, n_kv_heads=8, max_len=256, len_lo=256, len_hi=256, budget=77)),   # several rounds: a launch of its own
+    (2, dict(batch=2, n_q_heads=32, n_kv_heads=8, max_len=2100, budget=77, sel_heads=1)),              # select-and-attend
+])
+def test_infinite_values_among_the_selected_rows(launches, kw):
+    # an infinite entry of V in a selected row gives an infinity, as the sum over the rows does (NaN only where both signs
+    # meet), wherever in a tile of rows it lies, and leaves the other channels and the other heads alone
+    w = C["c1"].replace(**dict(dict(len_lo=kw["max_len"] - 100, len_hi=kw["max_len"], n_sink=0, n_recent=0), **kw))
+    r = Run(w)
+    r.build_proxy()
+    r.q.mul_(0.05)                                                       # (no probability underflows)
+    f = r.fasa
+
+    def step():
+        n0 = f.launch_count()
+        f.decode_step(r.q, r.k, r.v, r.proxy, r.seq_lens, w.budget, None, r.idx, r.n_sel, r.out, r.ws, r.lse)
+        torch.cuda.synchronize()
+        assert f.launch_count() - n0 == launches and f.device_status() == 0
+
+    step()
+    idx = r.idx.clone()
+    per = w.n_q_heads // w.n_sets
+    sets_per_head = w.n_sets // w.n_kv_heads
+    for b in range(w.batch):
+        for s in range(w.n_sets):
+            rows = idx[b, s, :77].long()
+            v = r.v[b, s // sets_per_head]
+            v[rows[76], 5] = float("inf")                                # the last row of the list
+            v[rows[40], 9] = float("-inf")
+            v[rows[0], 77], v[rows[75], 77] = float("inf"), float("-inf")
+    step()
+    assert torch.equal(r.idx, idx)
+    for b in range(0, w.batch, max(1, w.batch // 3)):
+        for hq in range(w.n_q_heads):
+            k, v = (x[b, hq * w.n_kv_heads // w.n_q_heads][idx[b, hq // per, :77].long()].double() for x in (r.k, r.v))
+            p = torch.softmax((k @ r.q[b, hq].double()) / math.sqrt(128.0), 0)
+            ref = (p[:, None] * v).sum(0)
+            got = r.out[b, hq].double()
+            assert torch.equal(torch.isnan(got), torch.isnan(ref)) and (sets_per_head > 1 or bool(torch.isnan(ref[77])))
+            inf = torch.isinf(ref)
+            assert bool(inf[5]) and bool(inf[9]) and torch.equal(got[inf], ref[inf]) and not bool(torch.isinf(got[~inf]).any())
+            fin = torch.isfinite(ref)
+            # (the kernel's probabilities carry 17 bits and its sums 24: 1e-4 of the largest value covers both)
+            assert float((got - ref)[fin].abs().max()) <= 1e-4 * float(v[:, fin].abs().max())
+
+
 @pytest.mark.parametrize("heads,lens,page", [
     ((8, 2), [20000, 0, 1, 16385, 17], 0),          # units shorter than a share, empty ones, shares that span several units
     ((7, 1), [16900], 0),                           # one unit over all CTAs
