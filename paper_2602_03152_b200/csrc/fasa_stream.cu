@@ -20,7 +20,9 @@
 //
 // With at most four query heads to a KV head the eight columns of an instruction hold the four heads twice, once
 // zeroed for each tile of a pair: both tiles accumulate into one fragment, lanes t < 2 of a quad holding the first
-// tile's heads and t >= 2 the second's, which halves the work after the products.
+// tile's heads and t >= 2 the second's, which halves the work after the products.  A key that is not finite gives NaN in
+// the zeroed columns too, that is in the score of a token of the other tile: a slot with such a score is scored again with
+// a fragment for each tile.
 //
 // The new token's row is scored from k_new itself: the warp that owns its tile writes the K, V and proxy rows
 // and replaces the row in its fragments, so nothing waits for those writes.  The lengths themselves grow in the
@@ -255,7 +257,8 @@ score_stream_kernel(const StreamParams p) {
     };
     constexpr int NC = G4 ? 1 : 2;                    // fragments of a pair
     // Maxima of the groups of a head's scores in the fragments of one column: v[o] = octet 2 (t >> 1) + o (G4), or octet o
-    auto store_max_head = [&](const float (&v)[2 * NC], float* hgm, bool mine, int pair) {
+    // (returned: a maximum over some of them, over all of them within the warp)
+    auto store_max_head = [&](const float (&v)[2 * NC], float* hgm, bool mine, int pair) -> float {
       const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0;
       float m;
       int octet;
@@ -277,7 +280,9 @@ score_stream_kernel(const StreamParams p) {
         m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, G4 ? 2 : 8));
         if (mine && g == 0 && (!G4 || t < 2)) hgm[pair] = m;
       }
+      return m;
     };
+    float seen = 0.f;                                // G4: NaN once a score of the slot is not finite
     // where this lane's values go: rows g, g + 8, ... of its two heads' score rows
     const int head0 = G4 ? 2 * (t & 1) : 2 * t;
     float* const lane_row = srow0 + (int64_t)head0 * p.max_len + (G4 ? 16 * (t >> 1) : 0) + g;
@@ -316,7 +321,13 @@ score_stream_kernel(const StreamParams p) {
             v[o] = c[i][o >> 1][(o & 1) * 2 + e] + 0.0f;               // (-0 becomes +0)
             if (mine) hrow[8 * o] = v[o];
           }
-          if (p.gs > 0) store_max_head(v, lane_gm + (int64_t)e * p.gm_stride, mine, pair);
+          if (p.gs > 0) {
+            const float m = store_max_head(v, lane_gm + (int64_t)e * p.gm_stride, mine, pair);
+            if (G4) seen = fmaf(m, 0.f, seen);
+          } else if (G4) {
+#pragma unroll
+            for (int o = 0; o < 2 * NC; ++o) seen = fmaf(v[o], 0.f, seen);
+          }
         }
       }
     };
@@ -337,14 +348,6 @@ score_stream_kernel(const StreamParams p) {
             a[e][kb] = make_uint4(x.x, x.y, 0u, 0u);
           }
         }
-        if (pair * 32 + 32 > w.len) {                // (uniform) rows past the end, whatever they hold, must not meet another tile's
-          const int row = pair * 32 + e * 16 + g;
-#pragma unroll
-          for (int kb = 0; kb < KB; ++kb) {
-            if (row >= w.len) a[e][kb].x = a[e][kb].z = 0u;
-            if (row + 8 >= w.len) a[e][kb].y = a[e][kb].w = 0u;
-          }
-        }
         if constexpr (PATCH) {
           const int r = new_row & 15;
           if ((new_row >> 4) == 2 * pair + e && g == (r & 7)) {
@@ -359,15 +362,19 @@ score_stream_kernel(const StreamParams p) {
           }
         }
       }
-      float c[NC][4];
+      float c[2][4];                                 // a fragment for each tile: what one holds never meets the other
 #pragma unroll
-      for (int e = 0; e < NC; ++e) c[e][0] = c[e][1] = c[e][2] = c[e][3] = 0.f;
+      for (int e = 0; e < 2; ++e) c[e][0] = c[e][1] = c[e][2] = c[e][3] = 0.f;
 #pragma unroll
       for (int kb = 0; kb < KB; ++kb) {
         if (kb < pg.n16 + pg.n8) {
 #pragma unroll
-          for (int e = 0; e < 2; ++e) mma_bf16_16816(c[G4 ? 0 : e], a[e][kb], f[G4 ? e : 0].b[kb]);
+          for (int e = 0; e < 2; ++e) mma_bf16_16816(c[e], a[e][kb], f[G4 ? e : 0].b[kb]);
         }
+      }
+      if constexpr (G4) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) c[0][i] = t < 2 ? c[0][i] : c[1][i];
       }
 #pragma unroll
       for (int e = 0; e < 2; ++e) {
@@ -411,6 +418,13 @@ score_stream_kernel(const StreamParams p) {
           general(std::false_type{}, src + j * pair_bytes, pair);
         }
         ++j;
+      }
+      if constexpr (G4) {
+        if (__any_sync(0xffffffffu, seen != 0.f)) {  // (NaN != 0)
+          for (j = 0; j < n; ++j)
+            if (first + j >= plain0 && first + j < plain1) general(std::false_type{}, src + j * pair_bytes, first + j);
+          seen = 0.f;
+        }
       }
       __syncwarp();                                  // every lane is done with the slot
       issue(slot);

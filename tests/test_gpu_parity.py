@@ -660,6 +660,40 @@ def test_index_sets_per_query_head_in_two_launches(kw, page):
         assert torch.equal(px[0][b, :, :L // 16], px[1][b, :, :L // 16])
 
 
+@pytest.mark.parametrize("kw", [
+    dict(budget=40),                                # groups of 8; whole 16-channel blocks
+    dict(budget=2),                                 # groups of 32
+    dict(budget=900, n_dom=12),                     # no group maxima; a block of 8 channels
+    dict(budget=40, n_q_heads=28, n_kv_heads=4),    # more than four heads: a fragment for each tile throughout
+])
+def test_score_stream_keeps_a_key_that_is_not_finite_to_itself(kw):
+    w = C["c1"].replace(**dict(dict(batch=3, max_len=3000, len_lo=2900, len_hi=2990, n_sink=0, n_recent=0, sel_heads=1), **kw))
+    r = Run(w)
+
+    def scores():
+        r.build_proxy()
+        r.scores.fill_(SENTINEL)
+        n0 = r.fasa.launch_count()
+        r.fasa.decode_step(r.q, r.k, r.v, r.proxy, r.seq_lens, w.budget, r.scores, r.idx, r.n_sel, r.out, r.ws)
+        torch.cuda.synchronize()
+        assert r.fasa.launch_count() - n0 == 2 and r.fasa.device_status() == 0
+        return r.scores.clone()
+
+    clean = scores()
+    odd = torch.zeros_like(clean, dtype=torch.bool)
+    per = w.n_q_heads // w.n_kv_heads
+    for n, (b, h, j) in enumerate([(0, 0, 0), (0, 1, 100), (0, 2, 117), (1, 3, 2047), (2, 0, 1031), (2, 1, int(r.seq_lens[2]) - 1)]):
+        r.k[b, h, j, int(r.dom[h, n % 4])] = float("inf") if n % 2 else float("-inf")
+        odd[b, h * per:(h + 1) * per, j] = True
+    got = scores()
+    assert torch.equal(got[~odd], clean[~odd]) and not bool(torch.isfinite(got[odd]).any())
+    for b in range(w.batch):
+        L = int(r.seq_lens[b])
+        for s in range(w.n_sets):
+            ref, _ = O.select(got[b, s, :L].double().cpu().numpy(), w.budget, 0, 0)
+            assert np.array_equal(r.idx[b, s, :ref.size].cpu().numpy(), ref), (b, s)
+
+
 def test_two_launch_steps_back_to_back_see_their_own_query_and_lengths():
     # the second launch starts before the first has ended and reads the lengths and the query then: in a loop that rewrites
     # the query's buffer on the stream and lets the lengths grow, every step must equal the one that had the GPU to itself
