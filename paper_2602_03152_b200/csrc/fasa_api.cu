@@ -332,7 +332,9 @@ extern "C" int32_t fasa_decode_step(fasa_ctx_t* ctx, const void* q, const void* 
       int32_t st2 = fasa_fused_launch(ctx, q, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores,
                                       idx, n_sel, out, lse, nullptr, nullptr, (cudaStream_t)stream, false);
       if (st2 != FASA_OK) return st2;
-      return fasa_sparse_decode_attn(ctx, q, k_cache, v_cache, idx, n_sel, n_sel_max, out, lse, workspace, stream);
+      bool mirrored;
+      return fasa_sparse_attn_mirrored(ctx, q, k_cache, v_cache, idx, n_sel, n_sel_max, out, lse, workspace, (cudaStream_t)stream,
+                                       nullptr, &mirrored, fasa_full_probabilities(ctx, n_sel_max));
     }
     return fasa_fused_launch(ctx, q, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores,
                              idx, n_sel, out, lse, nullptr, nullptr, (cudaStream_t)stream);
@@ -377,7 +379,7 @@ static int32_t append_decode_step_impl(fasa_ctx_t* ctx, const void* q, const voi
                                       idx, n_sel, out, lse, k_new, v_new, (cudaStream_t)stream, false);
       if (st2 != FASA_OK) return st2;
       return fasa_sparse_attn_mirrored(ctx, q, k_cache, v_cache, idx, n_sel, n_sel_max, out, lse, workspace,
-                                       (cudaStream_t)stream, out_mirror, mirrored);
+                                       (cudaStream_t)stream, out_mirror, mirrored, fasa_full_probabilities(ctx, n_sel_max));
     }
     *mirrored = out_mirror != nullptr;
     return fasa_fused_launch(ctx, q, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores,

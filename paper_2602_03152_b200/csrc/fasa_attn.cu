@@ -298,7 +298,8 @@ constexpr int kMmaWarps = kMmaThreads / 32;
 // query operand is loaded in the same channel order, so the logits are the same dot products
 // summed in another order.
 // (CTAs per SM: as many as the registers allow)
-template <bool SPARSE, bool PAGED, bool CLUSTER, bool HOSTMEM = false, bool KSPLIT = false>
+// TERMS: of a probability (see fasa_attn_core.cuh).
+template <bool SPARSE, bool PAGED, bool CLUSTER, bool HOSTMEM = false, bool KSPLIT = false, int TERMS = 2>
 __global__ void __launch_bounds__(kMmaThreads, KSPLIT || PAGED ? 4 : 5)
 decode_attn_mma_kernel(const AttnParams p) {
   __shared__ ClusterMergeSmem s_merge;              // (CLUSTER only: written by the peers)
@@ -337,7 +338,7 @@ decode_attn_mma_kernel(const AttnParams p) {
 
   // The CTA's slice of the index list goes to shared memory in one coalesced read (checked
   // once): a tile then costs one memory round trip (its rows), not two (its indices first).
-  int32_t* s_idx = reinterpret_cast<int32_t*>(attn_smem_raw + sizeof(MmaSmem<kMmaWarps>));
+  int32_t* s_idx = reinterpret_cast<int32_t*>(attn_smem_raw + sizeof(MmaSmem<kMmaWarps, TERMS>));
   if (SPARSE) {
     for (int i = threadIdx.x; i < r1 - r0; i += kMmaThreads) {
       int tok = irow[r0 + i];                        // (not through the read-only path: the kernel ahead may have written it)
@@ -358,7 +359,7 @@ decode_attn_mma_kernel(const AttnParams p) {
   }
 
   float (*s_part)[kMergePartStride] = mma_part<kMmaWarps>(attn_smem_raw);
-  attn_rows<kMmaWarps, SPARSE, PAGED, HOSTMEM, KSPLIT>(p, su, b / p.q_len, qb, r0, r1, s_idx, attn_smem_raw, [&](int gl) {
+  attn_rows<kMmaWarps, SPARSE, PAGED, HOSTMEM, KSPLIT, TERMS>(p, su, b / p.q_len, qb, r0, r1, s_idx, attn_smem_raw, [&](int gl) {
     return CLUSTER ? &s_part[gl][0] : p.partial + ((su.q0 + gl) * p.n_splits + split) * kPartialStride;
   });
   if constexpr (CLUSTER) {
@@ -539,7 +540,7 @@ dense_attn_kernel(const AttnParams p) {
     uint32_t qb[8][2];
     attn_load_query<false>(qb, p, su, lane);
     float* const dst = p.partial + (int64_t)(i + b * p.n_kv_heads + h) * p.group * kPartialStride;
-    attn_rows<kMmaWarps, false, PAGED, HOSTMEM, false>(p, su, b, qb, t0 * 16, min(len, (t0 + n) * 16), nullptr, attn_smem_raw,
+    attn_rows<kMmaWarps, false, PAGED, HOSTMEM, false, 2>(p, su, b, qb, t0 * 16, min(len, (t0 + n) * 16), nullptr, attn_smem_raw,
                                                        [&](int gl) { return dst + gl * kPartialStride; });
     x += n;
     if (x < end) {
@@ -577,12 +578,12 @@ dense_merge_kernel(const AttnParams p, int n_ctas) {
 }
 
 // out_mirror (nullable): a second destination of out; *mirrored tells whether it was written
-// (only the form that merges inside the attention launch can do that).
+// (only the form that merges inside the attention launch can do that).  full_p: three terms of a probability (that form too).
 template <bool SPARSE>
 int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
                     const int32_t* idx, const int32_t* n_rows, int n_upper, int n_sel_max,
                     float* out, float* lse, void* workspace, cudaStream_t s, float* out_mirror = nullptr,
-                    bool* mirrored = nullptr, int q_len = 1, const fasa_ksplit* ksplit = nullptr) {
+                    bool* mirrored = nullptr, int q_len = 1, const fasa_ksplit* ksplit = nullptr, bool full_p = false) {
   if (mirrored) *mirrored = false;
   const fasa_config_t& c = ctx->cfg;
   if (!fasa_pages_ready(ctx)) return FASA_ERR_INVALID_ARG;
@@ -607,7 +608,7 @@ int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
   p.scale_log2 = c.softmax_scale * 1.4426950408889634f;
   dim3 grid((unsigned)plan.n_splits, (unsigned)(n_seq * n_sets));
   if (ctx->use_fused) {   // default: the tensor-core kernel (mode 0 keeps the scalar one)
-    const int max_smem = (int)(sizeof(MmaSmem<kMmaWarps>) + 2080 * sizeof(int32_t));
+    const int max_smem = (int)(sizeof(MmaSmem<kMmaWarps, 3>) + 2080 * sizeof(int32_t));
     // One launch where the splits of a unit fit a portable cluster: the split count becomes a
     // power of two <= 8 (the nearest to the planned one) and the cluster merges by itself.
     int cs = 1;
@@ -619,8 +620,14 @@ int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
       if (mirrored) *mirrored = out_mirror != nullptr;
       auto fn = c.page_size > 0 ? decode_attn_mma_kernel<SPARSE, true, true> : decode_attn_mma_kernel<SPARSE, false, true>;
       if (host) fn = decode_attn_mma_kernel<SPARSE, false, true, true>;
-      if constexpr (SPARSE) { if (ksplit) fn = decode_attn_mma_kernel<true, false, true, true, true>; }
-      const size_t smem = sizeof(MmaSmem<kMmaWarps>) + (SPARSE ? (size_t)cchunk * sizeof(int32_t) : 0);
+      if constexpr (SPARSE) {
+        if (full_p) {
+          fn = c.page_size > 0 ? decode_attn_mma_kernel<true, true, true, false, false, 3> : decode_attn_mma_kernel<true, false, true, false, false, 3>;
+          if (host) fn = decode_attn_mma_kernel<true, false, true, true, false, 3>;
+        }
+        if (ksplit) fn = decode_attn_mma_kernel<true, false, true, true, true>;
+      }
+      const size_t smem = (full_p ? sizeof(MmaSmem<kMmaWarps, 3>) : sizeof(MmaSmem<kMmaWarps>)) + (SPARSE ? (size_t)cchunk * sizeof(int32_t) : 0);
       FASA_CUDA_TRY(ctx, cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
       FASA_CUDA_TRY(ctx, launch_after_predecessor(fn, dim3((unsigned)cs, grid.y), dim3(kMmaThreads), smem, s, cs, p));
       FASA_LAUNCH_CHECK(ctx);
@@ -682,10 +689,10 @@ extern "C" int32_t fasa_sparse_decode_attn(fasa_ctx_t* ctx, const void* q, const
 // fasa_sparse_decode_attn with a second destination for the output (the host-buffer step).
 int32_t fasa_sparse_attn_mirrored(fasa_ctx* ctx, const void* q, const void* k_cache, const void* v_cache,
                                   const int32_t* idx, const int32_t* n_sel, int32_t n_sel_max, float* out,
-                                  float* lse, void* workspace, cudaStream_t stream, float* out_mirror, bool* mirrored) {
+                                  float* lse, void* workspace, cudaStream_t stream, float* out_mirror, bool* mirrored, bool full_p) {
   const int n_upper = n_sel_max < ctx->cfg.max_len ? n_sel_max : ctx->cfg.max_len;
   return launch_attn<true>(ctx, q, k_cache, v_cache, idx, n_sel, n_upper, n_sel_max, out, lse, workspace, stream,
-                           out_mirror, mirrored);
+                           out_mirror, mirrored, 1, nullptr, full_p);
 }
 
 // FAC over a split key cache (Algorithm 2: Combine, then Eq. 6-7): k_nondom holds the non-dominant

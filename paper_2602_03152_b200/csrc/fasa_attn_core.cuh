@@ -20,9 +20,9 @@
 //     is applied to the fp32 result;
 //   - online softmax per head on the accumulator fragment (a thread owns heads 2t, 2t+1 of
 //     rows g, g+8; row maxima and sums by xor-shuffles over g);
-//   - output: A = V^T via ldmatrix.x4.trans, B = P^T.  P is split into two bf16 terms
-//     (p = hi + lo, error 2^-17 p) because one bf16 term would cost up to 2^-9 |v| of the
-//     2e-3 tolerance; two MMAs per block.
+//   - output: A = V^T via ldmatrix.x4.trans, B = P^T, split into bf16 terms; a MMA per block and term.
+//     Two terms hold 17 bits of a probability, three all 24 (outputs of 64 to 256 rows: 1.6e-6 and
+//     2.5e-7 of their norm); fasa_full_probabilities says where the third is taken.
 constexpr int kRowPad = FASA_HEAD_DIM + 8;          // bf16 elements per staged row (272 bytes)
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -77,12 +77,11 @@ __device__ __forceinline__ uint32_t f32_to_bf16_bits(float f) {
   return (u + 0x7fffu + ((u >> 16) & 1u)) >> 16;
 }
 
-template <int WARPS>
+template <int WARPS, int TERMS = 2>
 struct MmaSmem {
   uint16_t k[WARPS][16][kRowPad];
   uint16_t v[WARPS][16][kRowPad];
-  uint16_t p_hi[WARPS][8][16];                      // P^T: [head][row]
-  uint16_t p_lo[WARPS][8][16];
+  uint16_t p[TERMS][WARPS][8][16];                  // terms of P^T: [head][row]
 };
 // After the last row the staging memory becomes the combine area: [WARPS][8] accumulators of 128 channels, then
 // [WARPS][8][2] running maxima and sums, then one partial result per head.  (The stride of an accumulator keeps a
@@ -128,15 +127,15 @@ __device__ __forceinline__ void attn_load_query(uint32_t (&qb)[8][2], const P& p
 // Attention of the unit's query heads over rows [r0, r1): a warp takes 16 rows at a time.  SPARSE: row r is token
 // s_idx[r - r0] (shared memory), else token r.  bc: the sequence whose cache is read.  part(head) receives the
 // block's partial result (m, l, acc[128]); the threads must be synchronised before another reads it.  smem: at least
-// MmaSmem<WARPS>; it must not be in use by anything else when the first warp arrives.  HOSTMEM: K and V rows are
+// MmaSmem<WARPS, TERMS>; it must not be in use by anything else when the first warp arrives.  HOSTMEM: K and V rows are
 // copied through L1 (caches in page-locked host memory).  KSPLIT: Algorithm 2's Combine, see fasa_attn.cu.
-template <int WARPS, bool SPARSE, bool PAGED, bool HOSTMEM, bool KSPLIT, typename P, typename Part>
+template <int WARPS, bool SPARSE, bool PAGED, bool HOSTMEM, bool KSPLIT, int TERMS, typename P, typename Part>
 __device__ __forceinline__ void attn_rows(const P& p, const SelUnit& su, int bc, const uint32_t (&qb)[8][2], int r0, int r1,
                                           const int32_t* s_idx, unsigned char* smem, Part part) {
-  static_assert(sizeof(MmaSmem<WARPS>) >= mma_combine_bytes<WARPS>(), "combine area");
+  static_assert(sizeof(MmaSmem<WARPS, TERMS>) >= mma_combine_bytes<WARPS>(), "combine area");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3, h = su.h;
-  MmaSmem<WARPS>& sm = *reinterpret_cast<MmaSmem<WARPS>*>(smem);
+  MmaSmem<WARPS, TERMS>& sm = *reinterpret_cast<MmaSmem<WARPS, TERMS>*>(smem);
   float acc[8][4];                                  // out^T: [16-channel block][frag], heads 2t, 2t+1
 #pragma unroll
   for (int cb = 0; cb < 8; ++cb) acc[cb][0] = acc[cb][1] = acc[cb][2] = acc[cb][3] = 0.f;
@@ -247,14 +246,17 @@ __device__ __forceinline__ void attn_rows(const P& p, const SelUnit& su, int bc,
       l_run[e] = l_run[e] * alpha[e] + lg[e] + lg[2 + e];   // this thread's rows; the g lanes are added at the end
       m_run[e] = m_new;
     }
-    // P^T[head][row] as two bf16 terms
+    // P^T[head][row] as bf16 terms
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int head = 2 * t + (e & 1), row = g + 8 * (e >> 1);
-      const uint32_t hi = f32_to_bf16_bits(lg[e]);
-      const float rest = lg[e] - __uint_as_float(hi << 16);
-      sm.p_hi[warp][head][row] = (uint16_t)hi;
-      sm.p_lo[warp][head][row] = (uint16_t)f32_to_bf16_bits(rest);
+      float rest = lg[e];
+#pragma unroll
+      for (int i = 0; i < TERMS; ++i) {
+        const uint32_t term = f32_to_bf16_bits(rest);
+        sm.p[i][warp][head][row] = (uint16_t)term;
+        rest -= __uint_as_float(term << 16);
+      }
     }
     __syncwarp();                                   // P is visible; every lane is done with the K buffer
     if (more) stage_k(base + kTileStep);
@@ -262,10 +264,12 @@ __device__ __forceinline__ void attn_rows(const P& p, const SelUnit& su, int bc,
     cp_async_wait<1>();                             // this tile's V rows have landed
     __syncwarp();
     // B operand of the output product: B[k = row][n = head g]: rows 2t, 2t+1 and 2t+8, 2t+9
-    const uint32_t ph0 = *reinterpret_cast<const uint32_t*>(&sm.p_hi[warp][g][2 * t]);
-    const uint32_t ph1 = *reinterpret_cast<const uint32_t*>(&sm.p_hi[warp][g][2 * t + 8]);
-    const uint32_t pl0 = *reinterpret_cast<const uint32_t*>(&sm.p_lo[warp][g][2 * t]);
-    const uint32_t pl1 = *reinterpret_cast<const uint32_t*>(&sm.p_lo[warp][g][2 * t + 8]);
+    uint32_t pt[TERMS][2];
+#pragma unroll
+    for (int i = 0; i < TERMS; ++i) {
+      pt[i][0] = *reinterpret_cast<const uint32_t*>(&sm.p[i][warp][g][2 * t]);
+      pt[i][1] = *reinterpret_cast<const uint32_t*>(&sm.p[i][warp][g][2 * t + 8]);
+    }
 
     // ---- output: out^T[16 ch x 8 heads] += V^T[16 ch x 16 rows] . P^T[16 rows x 8 heads] ------
 #pragma unroll
@@ -275,8 +279,8 @@ __device__ __forceinline__ void attn_rows(const P& p, const SelUnit& su, int bc,
       // source blocks (token rows x channels), transposed on load:
       // (rows 0-7, ch 0-7), (rows 0-7, ch 8-15), (rows 8-15, ch 0-7), (rows 8-15, ch 8-15)
       ldmatrix_x4_trans(a, &sm.v[warp][(lane & 7) + 8 * (lane >> 4)][cb * 16 + 8 * ((lane >> 3) & 1)]);
-      mma16816(acc[cb], a, ph0, ph1);
-      mma16816(acc[cb], a, pl0, pl1);
+#pragma unroll
+      for (int i = 0; i < TERMS; ++i) mma16816(acc[cb], a, pt[i][0], pt[i][1]);
     }
     __syncwarp();                                   // every lane is done with the V buffer
     if (more) stage_v(base + kTileStep);

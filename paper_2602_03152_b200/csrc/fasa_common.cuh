@@ -108,12 +108,20 @@ static inline bool fasa_attend_separately(const fasa_ctx* ctx, int n_sel_max, co
   return workspace != nullptr && (uneven || (units > ctx->step_resident && n_sel_max >= 64 && !(pairs && n_sel_max >= 512)) || documented);
 }
 
+// Whether the attention of a step that runs on 16-row tiles (a launch of its own, or select-and-attend) keeps all 24 bits of a
+// probability.  The cluster kernel does; the split-K kernel's 17 bits are for lists that are long, or of which there are so many
+// that the gather decides (the third term costs 1 to 4 % there: 16 x 32 sets of 4096 rows 325 -> 332 us).
+static inline bool fasa_full_probabilities(const fasa_ctx* ctx, int n_sel_max) {
+  const long long rows = (long long)n_sel_max * ((ctx->sel_heads + 3) / 4), units = (long long)ctx->cfg.batch * ctx->n_sets;
+  return !(rows >= 2048 || (rows >= 256 && units * ctx->fused_cs > 2ll * ctx->n_sm) || (rows >= 512 && rows * units >= 24576));
+}
+
 cudaError_t fasa_stage_from_mapped(void* dq, const void* sq, size_t q_bytes, void* dk, const void* sk, void* dv,
                                    const void* sv, size_t kv_bytes, cudaStream_t stream);
 
 int32_t fasa_sparse_attn_mirrored(fasa_ctx* ctx, const void* q, const void* k_cache, const void* v_cache,
                                   const int32_t* idx, const int32_t* n_sel, int32_t n_sel_max, float* out,
-                                  float* lse, void* workspace, cudaStream_t stream, float* out_mirror, bool* mirrored);
+                                  float* lse, void* workspace, cudaStream_t stream, float* out_mirror, bool* mirrored, bool full_p);
 
 // Split key cache (memory-optimised variant): what the attention kernels need besides k_nondom.
 // The rows every step attends to (the sink positions and the recent window) can stay on the GPU:

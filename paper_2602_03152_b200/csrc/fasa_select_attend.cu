@@ -43,7 +43,7 @@ struct SelAttnParams {
   fasa_ksplit ks;                         // (unused: attn_load_query's general form)
 };
 
-template <int NT, bool PAGED>
+template <int NT, bool PAGED, int TERMS>
 __global__ void __launch_bounds__(NT, NT == 256 ? 2 : 1)
 select_attend_kernel(const SelAttnParams p) {
   constexpr int WARPS = NT / 32;
@@ -115,7 +115,7 @@ select_attend_kernel(const SelAttnParams p) {
   sel_row<NT>(row, gs, gm_lo, gm_hi, sm, dsm, p.lay, [&](int r, int pos) { take(plan.sink + r, pos); });
   __syncthreads();                                   // the list is complete, the selection's memory free
   float (*s_part)[kMergePartStride] = mma_part<WARPS>(dsm);
-  attn_rows<WARPS, true, PAGED, false, false>(p, su, su.b, qb, a0, a1, s_idx, dsm, [&](int gl) { return &s_part[gl][0]; });
+  attn_rows<WARPS, true, PAGED, false, false, TERMS>(p, su, su.b, qb, a0, a1, s_idx, dsm, [&](int gl) { return &s_part[gl][0]; });
   // append: every CTA of the launch has read the old length by the time that it arrives here; the last one stores the
   // new ones, below
   if (p.append && tid == 0) s_last = atomicAdd(p.arrive, 1) == (int)(gridDim.x * gridDim.y) - 1;
@@ -190,7 +190,7 @@ int32_t fasa_select_attend_launch(fasa_ctx* ctx, const void* q, const void* k_ca
   const int need = (c.max_len + 63) & ~31, room = 2 * p.lay.gm_cap > (wide ? 24576 : 12288) ? 2 * p.lay.gm_cap : (wide ? 24576 : 12288);
   p.lay.uni_cap = need < room ? need : room;
   p.lay.word_cap = (c.max_len >> 5) + 2;
-  const size_t stage = wide ? sizeof(MmaSmem<16>) : sizeof(MmaSmem<8>);
+  const size_t stage = wide ? sizeof(MmaSmem<16, 3>) : sizeof(MmaSmem<8, 3>);
   p.idx_off = (int)fasa_align_up(stage > (size_t)p.lay.bytes() ? stage : (size_t)p.lay.bytes(), 16);
   const size_t smem = (size_t)p.idx_off + (size_t)share_cap * 4;
   auto go = [&](auto kernel, int threads) -> cudaError_t {
@@ -200,7 +200,11 @@ int32_t fasa_select_attend_launch(fasa_ctx* ctx, const void* q, const void* k_ca
   };
   const bool paged = c.page_size > 0;
   ctx->launches += 1;
-  if (wide) FASA_CUDA_TRY(ctx, paged ? go(select_attend_kernel<512, true>, 512) : go(select_attend_kernel<512, false>, 512));
-  else FASA_CUDA_TRY(ctx, paged ? go(select_attend_kernel<256, true>, 256) : go(select_attend_kernel<256, false>, 256));
+  auto form = [&](auto terms_tag) -> cudaError_t {
+    constexpr int T = decltype(terms_tag)::value;
+    if (wide) return paged ? go(select_attend_kernel<512, true, T>, 512) : go(select_attend_kernel<512, false, T>, 512);
+    return paged ? go(select_attend_kernel<256, true, T>, 256) : go(select_attend_kernel<256, false, T>, 256);
+  };
+  FASA_CUDA_TRY(ctx, fasa_full_probabilities(ctx, n_sel_max) ? form(std::integral_constant<int, 3>{}) : form(std::integral_constant<int, 2>{}));
   return FASA_OK;
 }

@@ -512,6 +512,37 @@ def test_infinite_values_among_the_selected_rows(launches, kw):
             assert float((got - ref)[fin].abs().max()) <= 1e-4 * float(v[:, fin].abs().max())
 
 
+@pytest.mark.parametrize("launches,kw", [
+    (1, dict(batch=2, n_q_heads=28, n_kv_heads=4, max_len=900, budget=200)),
+    (2, dict(batch=48, n_q_heads=32, n_kv_heads=8, max_len=256, len_lo=256, len_hi=256, budget=200)),
+    (2, dict(batch=2, n_q_heads=32, n_kv_heads=8, max_len=2100, budget=200, sel_heads=1)),
+    (2, dict(batch=2, n_q_heads=28, n_kv_heads=4, max_len=2400, len_lo=2200, budget=200, sel_heads=1)),
+])
+def test_attention_keeps_32_bits_on_every_route(launches, kw):
+    # a flat distribution, whose probabilities use all their bits: products and sums of 24 bits leave some 3e-7 of the norm
+    # (the roundings of 200 terms, and of logits of up to 3 in magnitude, add up as their root: a few units of 2^-24); 17 bits
+    # in a probability would show as 1.6e-6
+    w = C["c1"].replace(**dict(dict(len_lo=kw["max_len"] - 100, len_hi=kw["max_len"], n_sink=0, n_recent=0), **kw))
+    r = Run(w)
+    r.build_proxy()
+    g = torch.Generator(device="cuda").manual_seed(3)
+    r.v.normal_(generator=g)
+    r.q.mul_(0.05)
+    n0 = r.fasa.launch_count()
+    r.fasa.decode_step(r.q, r.k, r.v, r.proxy, r.seq_lens, w.budget, None, r.idx, r.n_sel, r.out, r.ws, r.lse)
+    torch.cuda.synchronize()
+    assert r.fasa.launch_count() - n0 == launches and r.fasa.device_status() == 0
+    per = w.n_q_heads // w.n_sets
+    num = den = 0.0
+    for b in range(0, w.batch, max(1, w.batch // 3)):
+        for hq in range(w.n_q_heads):
+            k, v = (x[b, hq * w.n_kv_heads // w.n_q_heads][r.idx[b, hq // per, :200].long()].double() for x in (r.k, r.v))
+            ref = torch.softmax((k @ r.q[b, hq].double()) / math.sqrt(128.0), 0) @ v
+            num += float((r.out[b, hq].double() - ref).pow(2).sum())
+            den += float(ref.pow(2).sum())
+    assert math.sqrt(num / den) <= 6e-7
+
+
 @pytest.mark.parametrize("heads,lens,page", [
     ((8, 2), [20000, 0, 1, 16385, 17], 0),          # units shorter than a share, empty ones, shares that span several units
     ((7, 1), [16900], 0),                           # one unit over all CTAs
