@@ -285,9 +285,10 @@ int32_t fasa_sparse_decode_attn_static(fasa_ctx_t* ctx, const void* q, const voi
  * ceil(0.189 * L) + n_sink + n_recent for a permille budget) rather than the bound at
  * max_len; idx is addressed with whatever n_sel_max is passed as its row stride. */
 int32_t fasa_set_step_mode(fasa_ctx_t* ctx, int32_t mode);
-/* (The mode also selects the kernel behind fasa_topk: one CTA per score row for rows of up to 524288
- * tokens, a register-resident cluster kernel beyond that and in mode 0; the results are identical.
- * Mode 2 is mode 1.) */
+/* (The mode also selects the kernel behind fasa_topk and fasa_topk_batched, with identical results.  Mode 1: one CTA per
+ * score row, or the cluster kernel's selection phases for few long rows; beyond 524288 tokens a register-resident
+ * cluster kernel, which is also that of mode 0.  Mode 2 is mode 1 with one CTA per row up to 524288 tokens whatever the
+ * number of rows.) */
 /* Cluster size mode 1 runs with for this context; 0 = fasa_decode_step uses mode 0. */
 int32_t fasa_step_cluster_size(const fasa_ctx_t* ctx);
 int32_t fasa_decode_step(fasa_ctx_t* ctx, const void* q, const void* k_cache,

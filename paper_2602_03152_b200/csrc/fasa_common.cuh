@@ -39,6 +39,7 @@ struct fasa_ctx {
   size_t step_smem;
   int step_resident;      // clusters of the step's shape that the device holds at once
   int use_fused;          // fasa_decode_step takes the one-launch kernel when it is available
+  int topk_rows;          // fasa_topk and fasa_topk_batched by the one-CTA-per-row kernel whatever the rows (fasa_set_step_mode 2)
   // host-buffer step: the last host pointers seen and what the device can use in their place
   // (null: not page-locked + mapped), so that a decode loop with fixed buffers asks the driver once
   const void* host_seen[4];

@@ -148,7 +148,7 @@ int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* 
   // 10.8 / 11.3 at 512, 13.8 / 12.0 at 1024), and when the clusters would run in rounds (96 rows at 55 K: 21 / 27).
   const long long n_rows = (long long)c.batch * rows_per_seq;
   const int k = budget > 0 ? budget : (int)(((long long)-budget * c.max_len + 999) / 1000);
-  if (!calib && ctx->fused_cs > 1 && c.max_len > 8192 &&
+  if (!calib && !ctx->topk_rows && ctx->fused_cs > 1 && c.max_len > 8192 &&
       (n_rows <= 16 ? c.max_len > 16384 || k >= 256 : n_rows <= ctx->n_sm / 2 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || c.max_len > 65536)))
     return fasa_topk_cluster_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, rows_per_seq, n_sink, n_recent, stream, q_len);
   RowParams p;

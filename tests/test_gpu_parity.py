@@ -1614,7 +1614,8 @@ def test_device_status_bits_instead_of_faults():
 # ------------------------------------------------------------------ top-k alone ----
 
 def _topk_only(scores_cpu, lens, budget, n_sink, n_recent, n_sel_max, mode=1):
-    """mode 1: the cluster kernel's selection phases; mode 0: the register-resident kernel; mode 2: one CTA per row."""
+    """mode 1: the cluster kernel's selection phases or one CTA per row, by the rows; mode 0: the register-resident kernel; mode 2: one
+    CTA per row."""
     B, H, Lm = scores_cpu.shape
     dom = torch.arange(4, dtype=torch.int32).repeat(H, 1)
     f = binding.Fasa(B, H, H, Lm, dom, n_sink=n_sink, n_recent=n_recent)
@@ -1672,8 +1673,7 @@ def test_topk_exact_on_crowded_bins():
             _assert_topk_exact(sc, lens, budget)
         _assert_topk_exact(sc, lens, 500, n_sink=3, n_recent=100)
         _assert_topk_exact(sc, lens, -189)
-    # exactly 4096 / 4097 keys in the bin (the capacity of the cluster kernel's candidate area), and
-    # 8192 / 8193 (that of the one-CTA-per-row kernel's list), the rest far below
+    # exactly 4096 / 4097 keys in the bin (the capacity of the cluster kernel's candidate area), and twice that, the rest far below
     for n_in in (4096, 4097, 8192, 8193):
         sc = torch.full((1, 1, 30000), -5.0)
         sc[0, 0, torch.randperm(30000, generator=g)[:n_in]] = 1.0 + 0.2 * torch.rand(n_in, generator=g)
@@ -1709,6 +1709,31 @@ def test_topk_exact_at_the_edges_of_its_groups(L, budget, n_sink, n_recent):
     sc[0, 3, L // 3:L // 3 + max(1, budget)] = 2.5
     sc[0, 4] = sc[0, 4].abs() ** 9
     _assert_topk_exact(sc, [L], budget, n_sink=n_sink, n_recent=n_recent)
+
+
+@pytest.mark.parametrize("rows,L,budget", [
+    (100, 20001, 40), (100, 20001, 1700),                       # a thread block of 1024
+    (160, 9001, 64), (160, 9001, 900), (160, 65553, 300),       # 512
+    (320, 5003, 30), (320, 70001, 100), (320, 70001, 2000),     # 256; groups of 32 and whole rows beyond 65536 positions
+])
+def test_topk_exact_for_each_size_of_thread_block(rows, L, budget):
+    # many rows, each kind of row among them, by the kernel of one CTA per row; all of them against the register-resident
+    # kernel, one of each kind against the oracle
+    g = torch.Generator().manual_seed(rows + L + budget)
+    sc = torch.randn(rows // 4, 4, L, generator=g)
+    sc[:, 0] = torch.where(torch.rand(rows // 4, L, generator=g) < 2e-3, sc[:, 0] + 3e3, sc[:, 0])      # crowded but for a few outliers
+    sc[:, 1] = torch.randint(-3, 4, (rows // 4, L), generator=g).float()                                # runs of equal scores
+    sc[1::2, 1] = sc[1::2, 1] * 1e-3 + 1.0
+    sc[1, 2, 5::97] = float("inf")
+    sc[2, 2, 7::3] = float("-inf")
+    sc[3, 2, L - 3] = float("nan")
+    lens = [L - 13 * b for b in range(rows // 4)]
+    for n_sink, n_recent in ((0, 0), (4, 64)):
+        got = [_topk_only(sc, lens, budget, n_sink, n_recent, budget + n_sink + n_recent, mode) for mode in (0, 2)]
+        assert all(np.array_equal(x, y) for x, y in zip(*got))
+        for b, h in [(0, 0), (0, 1), (1, 1), (1, 2), (2, 2), (rows // 4 - 1, 3)]:
+            ref, _ = O.select(sc[b, h, :lens[b]].double().numpy(), budget, n_sink, n_recent)
+            assert int(got[1][1][b, h]) == ref.size and np.array_equal(got[1][0][b, h, :ref.size], ref), (b, h)
 
 
 @pytest.mark.parametrize("L,B,H", [(32768, 1, 8), (131072, 2, 2), (140001, 1, 2), (20000, 3, 5)])
