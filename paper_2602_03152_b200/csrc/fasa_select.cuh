@@ -16,9 +16,11 @@
 //   4. the bit masks of the selected positions become ranks (a block-wide prefix sum).
 // What bounds this is instructions and block barriers (seven), not bytes: a pass touches a score with
 // a dozen instructions per 32 of them, so the fewer positions a pass visits the better.  Bins are
-// monotone in the score, whatever the rounding, so the result is exact; scores that even bins cannot
-// spread (infinities and NaNs, hundreds of equal scores at the threshold) are settled by an
-// 11 / 11 / 10-bit radix select on order-preserving keys instead.
+// monotone in the score, whatever the rounding, so the result is exact.  A few scores far above the others (outlier keys,
+// sinks) would leave the rest in one or two bins: where some warp's largest value is far below the largest of all, the bins
+// end a little above it, and what lies beyond falls into the last one.  A histogram whose bin of interest is crowded all the
+// same is taken again over that bin's range, what lies above or below falling into the outermost bins.  Scores that this cannot spread either (infinities and
+// NaNs, hundreds of equal scores at the threshold) are settled by an 11 / 11 / 10-bit radix select on order-preserving keys.
 #pragma once
 
 #include "fasa_common.cuh"
@@ -80,6 +82,20 @@ __device__ __forceinline__ SelBinning sel_binning(float lo, float hi) {
   return b;
 }
 
+// Bins over the range of one bin alone (and a little to either side; the last one reaches up to `hi`, the largest value);
+// scale 0 where that is too narrow.
+constexpr int kSelTries = 3;             // histograms taken at most
+__device__ __forceinline__ SelBinning sel_narrower(const SelBinning& b, int bin, float hi) {
+  const float lo = b.lo + ((float)bin - 1.0625f) / b.scale;
+  return sel_binning(lo, bin == kSelBins - 1 ? hi : lo + 1.125f / b.scale);
+}
+// Where the bins of values in [lo, hi] end if they are to spread the kth largest: mid = the least of the warps' largest values.
+template <int NT>
+__device__ __forceinline__ float sel_reach(float lo, float hi, float mid, int k) {
+  const float r = 1.25f * (mid - lo);
+  return k >= NT / 16 && r > 0.f && hi - lo > 4.f * r ? lo + r : hi;
+}
+
 __device__ __forceinline__ uint32_t sel_scan(uint32_t v, int lane) {
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -123,14 +139,17 @@ __device__ __forceinline__ void sel_find(const uint32_t* hist, uint32_t kth, int
   }
 }
 
-// Block-wide min and max of the threads' values (one barrier); false when one of them is not finite.
+// Block-wide min and max of the threads' values, and the least of the warps' maxima (of those that have values: the others
+// come with -inf); one barrier.  false when a value is not finite.
 template <int NT>
-__device__ __forceinline__ bool sel_minmax(SelShared& sm, float& lo, float& hi, int warp, int lane) {
+__device__ __forceinline__ bool sel_minmax(SelShared& sm, float& lo, float& hi, float& mid, int warp, int lane) {
   const uint32_t kl = __reduce_min_sync(0xffffffffu, fasa_order_key(lo)), kh = __reduce_max_sync(0xffffffffu, fasa_order_key(hi));
   if (lane == 0) { sm.wlo[warp] = kl; sm.whi[warp] = kh; }
   __syncthreads();
   lo = sel_key_value(__reduce_min_sync(0xffffffffu, lane < NT / 32 ? sm.wlo[lane] : 0xffffffffu));
-  hi = sel_key_value(__reduce_max_sync(0xffffffffu, lane < NT / 32 ? sm.whi[lane] : 0u));
+  const uint32_t w = lane < NT / 32 ? sm.whi[lane] : 0u;
+  hi = sel_key_value(__reduce_max_sync(0xffffffffu, w));
+  mid = sel_key_value(__reduce_min_sync(0xffffffffu, w > fasa_order_key(-INFINITY) ? w : 0xffffffffu));
   return hi - lo < 3.0e38f;                                         // (false for NaN)
 }
 
@@ -176,7 +195,7 @@ struct SelRow {
   int k;                                 // 0 <= k <= hi - lo
 };
 
-// Before a row: clears what the row's histograms add to (a barrier must follow).
+// Before a row: clears what the row's histograms add to.
 template <int NT>
 __device__ __forceinline__ void sel_begin(SelShared& sm) {
   for (int i = threadIdx.x; i < kSelRadixBins / 4; i += NT) reinterpret_cast<uint4*>(&sm.hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
@@ -194,11 +213,12 @@ __host__ __device__ __forceinline__ int sel_group_shift(int n, int k, int gm_cap
 }
 
 // Calls emit(r, position) for the r-th selected position in ascending order, r = 0 .. k - 1.
-// gs > 0: dyn starts with the maxima (float) of the groups (r.lo >> gs) .. ((r.hi - 1) >> gs), positions
-// outside [lo, hi) left out, and gm_lo / gm_hi are the least and the largest of those that this thread
-// has written.  sel_begin comes before; all threads call.
-template <int NT, typename Src, typename Emit>
-__device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, float gm_lo, float gm_hi, SelShared& sm, unsigned char* dyn,
+// gs > 0: fill(gm, lo, hi), called by all threads, once or up to kSelTries times, writes the maxima (float) of the groups
+// (r.lo >> gs) .. ((r.hi - 1) >> gs), positions outside [lo, hi) left out, and the least and the largest of those that this
+// thread has written to lo and hi.  sel_begin comes before (the first barrier is behind the first reads of the row, so that
+// nothing delays them); all threads call.
+template <int NT, typename Src, typename Fill, typename Emit>
+__device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill, SelShared& sm, unsigned char* dyn,
                                         const SelLayout& lay, Emit emit) {
   constexpr int NW = NT / 32;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -215,26 +235,47 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, float gm_l
 
   bool radix = false;                    // the even bins do not apply
   int n_list = 0;
-  float bound = 0.f;
+  float bound = 0.f, top = 0.f, reach = 0.f;                       // the largest value; where the bins end
   int g0 = 0;
   if (gs > 0) {
     // ---- 1, 2: the groups that can hold one of the k best -------------------------------------
     g0 = r.lo >> gs;
     const int n_groups = ((r.hi - 1) >> gs) + 1 - g0;
-    if (!sel_minmax<NT>(sm, gm_lo, gm_hi, warp, lane)) {            // (the maxima are complete after its barrier)
-      radix = true;
-      gs = 0;
-    } else {
-      const SelBinning first = sel_binning(gm_lo, gm_hi);
+    SelBinning first{0.f, 0.f};
+    int b0 = 0;
+#pragma unroll 1
+    for (int t = 0; t < kSelTries; ++t) {
+      float lo = INFINITY, hi = -INFINITY, mid;
+      fill(gm, lo, hi);
+      if (t == 0) {
+        if (!sel_minmax<NT>(sm, lo, hi, mid, warp, lane)) {              // (the maxima are complete after its barrier)
+          radix = true;
+          gs = 0;
+          break;
+        }
+        top = hi;
+        reach = sel_reach<NT>(lo, hi, mid, r.k);
+        first = sel_binning(lo, reach);
+      } else {
+        __syncthreads();
+      }
       for (int i = tid; i < n_groups; i += NT) {
         const int bin = first.bin(gm[i]);
         atomicAdd(&sm.hist[0][bin], 1u);
         gm[i] = __int_as_float(bin);
       }
       __syncthreads();
-      int b0;
       uint32_t rank, count;
       sel_find<kSelBins>(sm.hist[0], (uint32_t)r.k, lane, &b0, &rank, &count);
+      // crowded: its groups would all be listed, and 8 or 32 positions of each visited
+      if (count <= 64u + (uint32_t)r.k / 2u || t + 1 == kSelTries || !(first.scale > 0.f)) break;
+      const SelBinning nb = sel_narrower(first, b0, top);
+      if (!(nb.scale > 0.f)) break;
+      first = nb;
+      __syncthreads();                   // (every warp has read the histogram)
+      for (int i = tid; i < kSelBins / 4; i += NT) reinterpret_cast<uint4*>(&sm.hist[0][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    if (!radix) {
       const int per = ((n_groups + NW - 1) / NW + 31) & ~31;        // a warp takes a run of groups
       const int s0 = min(n_groups, warp * per), s1 = min(n_groups, s0 + per);
       uint32_t mine = 0;
@@ -289,28 +330,38 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, float gm_l
   };
   SelBinning second{0.f, 0.f};
   if (listed) {
-    second = sel_binning(bound, gm_hi);
+    second = sel_binning(bound, reach > bound ? reach : top);
   } else if (!radix) {
-    float lo = INFINITY, hi = -INFINITY;
+    float lo = INFINITY, hi = -INFINITY, mid;
     visit([&](int, bool ok, float x) {
       if (ok) { lo = fminf(lo, x); hi = max_nan(hi, x); }           // (a NaN shows in hi)
     });
-    if (!sel_minmax<NT>(sm, lo, hi, warp, lane)) radix = true;
-    else second = sel_binning(lo, hi);
+    if (!sel_minmax<NT>(sm, lo, hi, mid, warp, lane)) radix = true;
+    else second = sel_binning(lo, sel_reach<NT>(lo, hi, mid, r.k));
+    top = hi;
   }
   uint32_t rank = 0, count = 0;
   int b1 = 0;
   if (!radix) {
-    visit([&](int c, bool ok, float x) {
-      const int bin = ok ? second.bin(x) : 0;
-      if (bin > 0) atomicAdd(&sm.hist[1][bin], 1u);
-      if (held) bins16[c * 32 + lane] = (uint16_t)bin;
-    });
-    __syncthreads();
-    sel_find<kSelBins>(sm.hist[1], (uint32_t)r.k, lane, &b1, &rank, &count);
-    if (count > (uint32_t)kSelRank || b1 == 0) {
-      radix = true;
+#pragma unroll 1
+    for (int t = 0; t < kSelTries; ++t) {
+      visit([&](int c, bool ok, float x) {
+        const int bin = ok ? second.bin(x) : 0;
+        if (bin > 0) atomicAdd(&sm.hist[1][bin], 1u);
+        if (held) bins16[c * 32 + lane] = (uint16_t)bin;
+      });
+      __syncthreads();
+      const uint32_t was = count;
+      sel_find<kSelBins>(sm.hist[1], (uint32_t)r.k, lane, &b1, &rank, &count);
+      if (count <= (uint32_t)kSelRank && b1 > 0) break;
+      const SelBinning nb = sel_narrower(second, b1, top);
+      // (as many as before: equal scores)
+      radix = b1 == 0 || t + 1 == kSelTries || count == was || !(second.scale > 0.f) || !(nb.scale > 0.f);
       __syncthreads();                   // (every warp has read the histogram)
+      if (radix) break;
+      second = nb;
+      for (int i = tid; i < kSelBins / 4; i += NT) reinterpret_cast<uint4*>(&sm.hist[1][0])[i] = make_uint4(0u, 0u, 0u, 0u);
+      __syncthreads();
     }
   }
 

@@ -89,18 +89,7 @@ select_attend_kernel(const SelAttnParams p) {
   if (gs > 0 && !(row.k > 0 && row.k < n_free && (long long)row.k * (gs == 3 ? 12 : 43) <= n_free)) gs = 0;
   pdl_wait_for_predecessor();
   pdl_release_successor();
-  if (crank == 0 && tid == 0) {
-    if (plan.clamped) atomicOr(p.status, FASA_DEV_NSEL_CLAMPED);
-    p.n_sel[u] = plan.ktot;
-  }
-  for (int i = tid; i < plan.n_forced; i += NT) {
-    int rank, pos;
-    sel_forced(plan, i, &rank, &pos);
-    take(rank, pos);
-  }
-  float gm_lo = INFINITY, gm_hi = -INFINITY;
-  if (gs > 0) {
-    float* gm = reinterpret_cast<float*>(dsm);
+  auto maxima = [&](float* gm, float& gm_lo, float& gm_hi) {
     const int g0 = row.lo >> gs, n_groups = ((row.hi - 1) >> gs) + 1 - g0;
     const float* src = p.gm + (int64_t)u * p.gm_stride + g0;
 #pragma unroll 8
@@ -110,9 +99,17 @@ select_attend_kernel(const SelAttnParams p) {
       gm_lo = fminf(gm_lo, m);
       gm_hi = max_nan(gm_hi, m);
     }
+  };
+  sel_row<NT>(row, gs, maxima, sm, dsm, p.lay, [&](int r, int pos) { take(plan.sink + r, pos); });
+  for (int i = tid; i < plan.n_forced; i += NT) {
+    int rank, pos;
+    sel_forced(plan, i, &rank, &pos);
+    take(rank, pos);
   }
-  __syncthreads();
-  sel_row<NT>(row, gs, gm_lo, gm_hi, sm, dsm, p.lay, [&](int r, int pos) { take(plan.sink + r, pos); });
+  if (crank == 0 && tid == 0) {
+    if (plan.clamped) atomicOr(p.status, FASA_DEV_NSEL_CLAMPED);
+    p.n_sel[u] = plan.ktot;
+  }
   __syncthreads();                                   // the list is complete, the selection's memory free
   float (*s_part)[kMergePartStride] = mma_part<WARPS>(dsm);
   attn_rows<WARPS, true, PAGED, false, false, TERMS>(p, su, su.b, qb, a0, a1, s_idx, dsm, [&](int gl) { return &s_part[gl][0]; });

@@ -44,10 +44,8 @@ __device__ __forceinline__ void topk_row(const RowParams& p, const Src& src, int
   row.hi = plan.hi;
   row.k = plan.k;
   const int gs = row.k > 0 && row.k < row.hi - row.lo ? sel_group_shift(row.hi - row.lo, row.k, p.lay.gm_cap) : 0;
-  float gm_lo = INFINITY, gm_hi = -INFINITY;
-  if (gs > 0) {
+  auto maxima = [&](float* gm, float& gm_lo, float& gm_hi) {
     // A thread takes eight consecutive positions: their maximum needs no other lane (groups of 32: two shuffles).
-    float* gm = reinterpret_cast<float*>(rsm);
     const int g0 = row.lo >> gs, first = g0 << gs;
     const bool vec_ok = src.aligned();
     constexpr int UNR = 2, STEP = NT * 8;
@@ -88,15 +86,14 @@ __device__ __forceinline__ void topk_row(const RowParams& p, const Src& src, int
         }
       }
     }
-  }
-  __syncthreads();
+  };
   int32_t* out = p.idx + (int64_t)u * p.n_sel_max;
+  sel_row<NT>(row, gs, maxima, sm, rsm, p.lay, [&](int r, int pos) { out[plan.sink + r] = pos; });
   for (int i = tid; i < plan.n_forced; i += NT) {
     int rank, pos;
     sel_forced(plan, i, &rank, &pos);
     if (rank < plan.ktot) out[rank] = pos;
   }
-  sel_row<NT>(row, gs, gm_lo, gm_hi, sm, rsm, p.lay, [&](int r, int pos) { out[plan.sink + r] = pos; });
 }
 
 // CALIB: row r < 64 of a sample (sequence, query head) is FC r alone, computed from the channel pairs as it is read, row

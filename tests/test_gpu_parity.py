@@ -1736,6 +1736,22 @@ def test_topk_exact_for_each_size_of_thread_block(rows, L, budget):
             assert int(got[1][1][b, h]) == ref.size and np.array_equal(got[1][0][b, h, :ref.size], ref), (b, h)
 
 
+@pytest.mark.parametrize("far", [1e2, 1e4, 1e6, 1e9, 1e30])
+@pytest.mark.parametrize("L,budget", [(3000, 20), (3000, 700), (40000, 30), (40000, 512), (40000, 9000)])
+def test_topk_exact_below_outliers(L, budget, far):
+    # a few scores far above (or below) the others, at one or several distances: the selection's even histograms crowd and
+    # are refined, up to where the radix select takes over
+    g = torch.Generator().manual_seed(L + budget)
+    sc = torch.randn(1, 4, L, generator=g)
+    pos = torch.randperm(L, generator=g)
+    sc[0, 0, pos[:budget // 4]] += far
+    sc[0, 1, pos[:3]] += torch.tensor([far, far ** 0.5, -far])
+    sc[0, 2] = sc[0, 2] * 1e-4 + 100.0
+    sc[0, 2, pos[:budget - 1]] = far
+    sc[0, 3] = sc[0, 3] ** 5
+    _assert_topk_exact(sc, [L], budget)
+
+
 @pytest.mark.parametrize("L,B,H", [(32768, 1, 8), (131072, 2, 2), (140001, 1, 2), (20000, 3, 5)])
 def test_topk_exact_at_scale(L, B, H):
     # 131072 fills the register-resident capacity of an 8-CTA cluster; 140001 takes the
