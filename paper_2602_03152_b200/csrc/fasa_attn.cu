@@ -469,12 +469,12 @@ decode_attn_merge_kernel(const float* partial, const int32_t* n_rows,
 }
 
 // ---- dense pass over long contexts -----------------------------------------------------------------
-// As many CTAs as the device holds at once; the rows of all (sequence, KV head) units, laid end to end in tiles of 16, are
-// dealt out to them evenly by the lengths on the device, so ragged batches end together and no last wave is left over.
+// The rows of all (sequence, KV head) units, laid end to end in tiles of 16, are dealt out to the CTAs evenly by the lengths on
+// the device, so ragged batches end together.
 // A CTA whose share spans several units writes a partial result for each; segment (CTA i, unit u) is number i + u of
 // the partial results (from one segment to the next exactly one of the two grows).  Bound by HBM.  Measured (back to back,
-// with the merge) against splits of a fixed size: batch 4 at 20-60 K 126 -> 119 us, batch 16 x 4 heads at 9-18 K 94 -> 88 us,
-// batch 1 at 30 K 34.3 -> 32 us; equal lengths that filled the last wave before: the same.
+// with the merge) against splits of a fixed size: batch 4 at 20-60 K 131 -> 116 us, batch 16 x 4 heads at 9-18 K 94 -> 88 us,
+// batch 1 at 30 K 32.2 -> 27.9 us, batch 8 at 64 K 336 -> 330 us; batch 4, 40 / 8 heads, 12-22 K 54.2 / 55.9 us.
 struct DenseDeal {
   long long total;         // tiles of all units
   int n;                   // CTAs that take part
@@ -484,16 +484,24 @@ struct DenseDeal {
 __device__ __forceinline__ int dense_tiles(const int32_t* seq_lens, int b, int batch, int max_len, int32_t* status) {
   return b < batch ? (clamp_len(seq_lens[b], max_len, status) + 15) >> 4 : 0;
 }
-// One warp.
-__device__ __forceinline__ DenseDeal dense_deal(const int32_t* seq_lens, int batch, int n_kv_heads, int max_len, int n_ctas, int lane, int32_t* status) {
+// One warp.  n_ctas: CTAs launched, of which the device holds `resident` at once; n_sm: 0 on pages.
+__device__ __forceinline__ DenseDeal dense_deal(const int32_t* seq_lens, int batch, int n_kv_heads, int max_len, int n_ctas, int resident, int n_sm,
+                                                int lane, int32_t* status) {
   DenseDeal d;
   d.mine = dense_tiles(seq_lens, lane, batch, max_len, status);
   d.total = __reduce_add_sync(0xffffffffu, d.mine);
   for (int b0 = 32; b0 < batch; b0 += 32) d.total += __reduce_add_sync(0xffffffffu, dense_tiles(seq_lens, b0 + lane, batch, max_len, status));
   d.total *= n_kv_heads;
-  // a few tiles to each of a third of the CTAs, then 32 tiles to each before the others join: below that a CTA's start and
-  // its partial result cost more than its share (70 MB of 2 x 4 heads at 17 K: 24.6 us with all CTAs, 22.2 with a third)
-  d.n = (int)max(1ll, min((long long)n_ctas, max(d.total >> 5, min(d.total >> 2, (long long)(n_ctas / 3)))));
+  // Long contexts: 1.8 times as many shares as CTAs are resident.  With one share to each, the slowest SM ends last by a
+  // twentieth of the launch (batch 8 x 8 heads at 64 K: 350 us, 330 with 1.8; batch 16 at 32 K 355 / 334; batch 4 at 64 K 184 /
+  // 176); a number of shares just above a whole multiple leaves most SMs idle at the end (1.4: 348 us, 1.9: 346, 2.3: 339).
+  // Less than 64 tiles to each: as many CTAs to each SM as get 64 (batch 1 at 73 K 60 -> 57 us, batch 4 at 17 K 55.7 -> 53.5).
+  // Pages keep one share to each resident CTA (batch 8 at 64 K: 374 us, 414 with 1.8), and short contexts a few tiles to
+  // each of a third of the CTAs, then 32 tiles to each before the others join: below that a CTA's start and its partial
+  // result cost more than its share (70 MB of 2 x 4 heads at 17 K: 24.6 us with all CTAs, 22.2 with a third).
+  if (n_sm > 0 && d.total >= (long long)kDenseTiles * resident) d.n = n_ctas;
+  else if (n_sm > 0 && d.total >= 2ll * kDenseTiles * n_sm) d.n = (int)(d.total / ((long long)kDenseTiles * n_sm)) * n_sm;
+  else d.n = (int)max(1ll, min((long long)resident, max(d.total >> 5, min(d.total >> 2, (long long)(resident / 3)))));
   return d;
 }
 
@@ -504,11 +512,11 @@ dense_attn_kernel(const AttnParams p) {
   pdl_release_successor();
   const int lane = threadIdx.x & 31;
   const int batch = p.n_cap;                        // (the launch's number of sequences)
-  const DenseDeal d = dense_deal(p.n_rows, batch, p.n_kv_heads, p.max_len, (int)gridDim.x, lane, p.status);
+  const DenseDeal d = dense_deal(p.n_rows, batch, p.n_kv_heads, p.max_len, (int)gridDim.x, p.n_splits, p.chunk, lane, p.status);
   const int i = blockIdx.x;
   if (i >= d.n) return;
-  long long x = d.total < (1 << 22) ? (uint32_t)d.total * (uint32_t)i / (uint32_t)d.n : d.total * i / d.n;
-  const long long end = d.total < (1 << 22) ? (uint32_t)d.total * (uint32_t)(i + 1) / (uint32_t)d.n : d.total * (i + 1) / d.n;
+  long long x = d.total < (1 << 21) ? (uint32_t)d.total * (uint32_t)i / (uint32_t)d.n : d.total * i / d.n;
+  const long long end = d.total < (1 << 21) ? (uint32_t)d.total * (uint32_t)(i + 1) / (uint32_t)d.n : d.total * (i + 1) / d.n;
   if (x >= end) return;
   // the sequence that tile x lies in
   int b = 0, tiles = 0;
@@ -561,7 +569,7 @@ dense_merge_kernel(const AttnParams p, int n_ctas) {
   pdl_wait_for_predecessor();
   const int bh = blockIdx.x, b = bh / p.n_q_heads, hq = bh % p.n_q_heads, h = hq / p.group;
   const int lane = threadIdx.x & 31, batch = p.n_cap;
-  const DenseDeal d = dense_deal(p.n_rows, batch, p.n_kv_heads, p.max_len, n_ctas, lane, p.status);
+  const DenseDeal d = dense_deal(p.n_rows, batch, p.n_kv_heads, p.max_len, n_ctas, p.n_splits, p.chunk, lane, p.status);
   long long first = 0;                              // this unit's first tile
   for (int b0 = 0; b0 < b; b0 += 32)
     first += __reduce_add_sync(0xffffffffu, b0 + lane < b ? (b0 == 0 ? d.mine : dense_tiles(p.n_rows, b0 + lane, batch, p.max_len, p.status)) : 0);
@@ -569,7 +577,7 @@ dense_merge_kernel(const AttnParams p, int n_ctas) {
   first = first * p.n_kv_heads + (long long)h * tiles;
   // tile x belongs to CTA ((x + 1) n - 1) / total
   auto cta_of = [&](long long y) {                  // y = x + 1
-    return d.total < (1 << 22) ? (int)(((uint32_t)y * (uint32_t)d.n - 1u) / (uint32_t)d.total) : (int)((y * d.n - 1) / d.total);
+    return d.total < (1 << 21) ? (int)(((uint32_t)y * (uint32_t)d.n - 1u) / (uint32_t)d.total) : (int)((y * d.n - 1) / d.total);
   };
   const int i0 = tiles > 0 ? cta_of(first + 1) : 0;
   const int ns = tiles > 0 ? cta_of(first + tiles) - i0 + 1 : 0;
@@ -635,6 +643,7 @@ int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
     }
     if constexpr (!SPARSE) {
       p.out = out; p.lse = lse; p.n_cap = c.batch;
+      p.n_splits = fasa_dense_resident(ctx); p.chunk = c.page_size > 0 ? 0 : ctx->n_sm;   // (what dense_deal asks for)
       auto fn = c.page_size > 0 ? dense_attn_kernel<true, false> : dense_attn_kernel<false, false>;
       if (host) fn = dense_attn_kernel<false, true>;
       const int n_ctas = fasa_dense_ctas(ctx);

@@ -74,8 +74,15 @@ struct fasa_split_plan {
   int chunk;      // rows per split (multiple of 32)
 };
 fasa_split_plan fasa_plan_splits(const fasa_ctx* ctx, int n_upper, int units);
-// CTAs of the dense pass over long contexts: what the device holds at once (six per SM, four on pages).
-static inline int fasa_dense_ctas(const fasa_ctx* ctx) { return (ctx->cfg.page_size > 0 ? 4 : 6) * (ctx->n_sm > 0 ? ctx->n_sm : 148); }
+// CTAs of the dense pass over long contexts: what the device holds at once (six per SM, four on pages), and how many are
+// launched: 1.8 times that where contiguous caches can hold 64 tiles of 16 rows for each (see dense_deal).
+constexpr int kDenseTiles = 64;
+static inline int fasa_dense_resident(const fasa_ctx* ctx) { return (ctx->cfg.page_size > 0 ? 4 : 6) * (ctx->n_sm > 0 ? ctx->n_sm : 148); }
+static inline int fasa_dense_ctas(const fasa_ctx* ctx) {
+  const int res = fasa_dense_resident(ctx);
+  const long long tiles = (long long)ctx->cfg.batch * ctx->cfg.n_kv_heads * ((ctx->cfg.max_len + 15) / 16);
+  return ctx->cfg.page_size == 0 && tiles >= (long long)kDenseTiles * res ? res * 9 / 5 : res;
+}
 
 // One-launch decode step (fasa_fused.cu): plan at context creation, launch per step.
 int fasa_fused_plan(fasa_ctx* ctx);

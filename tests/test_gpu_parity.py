@@ -575,6 +575,32 @@ def test_dense_path_over_long_contexts_deals_rows_out_evenly(heads, lens, page):
             assert float(err) <= 1e-4 * float(v.abs().max()) and abs(float(torch.logsumexp(lg, 0)) - float(r.dense_lse[b, g])) <= 1e-4
 
 
+@pytest.mark.parametrize("lens", [
+    [14208] * 8, [14208] * 7 + [14192],                                  # 64 tiles to each resident CTA of a B200, and one tile less
+    [16400, 16385, 16000, 15000, 14999, 13001, 12000, 11000],
+    [4736] * 8, [4736] * 7 + [4720], [6001, 0, 9000, 1, 16400, 33, 17, 5000],
+])
+def test_dense_path_where_the_number_of_shares_changes(lens):
+    w = C["c1"].replace(batch=8, n_q_heads=16, n_kv_heads=8, max_len=16400, n_sink=0, n_recent=0, budget=16)
+    f = binding.Fasa(8, 16, 8, w.max_len, torch.arange(4, dtype=torch.int32).repeat(8, 1))
+    g = torch.Generator(device="cuda").manual_seed(sum(lens))
+    q = torch.randn(8, 16, 128, device="cuda", generator=g).bfloat16()
+    k, v = (torch.empty(8, 8, w.max_len, 128, dtype=torch.bfloat16, device="cuda").normal_(generator=g) for _ in range(2))
+    out, lse = torch.full((8, 16, 128), SENTINEL, device="cuda"), torch.full((8, 16), SENTINEL, device="cuda")
+    ws = f.alloc_workspace(16)
+    guard = torch.full((ws.numel() + 4096,), 77, dtype=torch.uint8, device="cuda")          # (nothing is written past the workspace)
+    f.full_decode_attn(q, k, v, torch.tensor(lens, dtype=torch.int32, device="cuda"), out, guard[:ws.numel()], lse)
+    torch.cuda.synchronize()
+    assert f.device_status() == 0 and bool((guard[ws.numel():] == 77).all())
+    for b, L in enumerate(lens):
+        for hq in range(16):
+            if L == 0:
+                assert float(out[b, hq].abs().max()) == 0.0 and float(lse[b, hq]) == float("-inf")
+                continue
+            e, el = _attention_error(q[b, hq], k[b, hq // 2], v[b, hq // 2], slice(0, L), out[b, hq], lse[b, hq])
+            assert e <= 1e-4 and el <= 1e-4, (b, hq)     # (17 bits in a probability, 24 in the sums)
+
+
 # ---- index sets shared by fewer query heads than a KV head serves (Sec. 4.1: a set per head) ----
 
 @pytest.mark.parametrize("cfg,sel,kw", [
