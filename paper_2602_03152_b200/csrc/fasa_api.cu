@@ -472,7 +472,9 @@ extern "C" int32_t fasa_decode_step_host(fasa_ctx_t* ctx, const void* q_host,
   const void* mk = mapped(1, k_new_host);
   const void* mv = mapped(2, v_new_host);
   const bool all_mapped = mq && mk && mv && !((uintptr_t)mq & 15) && !((uintptr_t)mk & 15) && !((uintptr_t)mv & 15);
-  const bool one_wave_one_launch = ctx->use_fused && ctx->fused_cs > 0 && !fasa_attend_separately(ctx, n_sel_max, workspace) &&
+  // (a set per query head at 16 K, batch 1: every warp of the score stream would fetch its query over the link, 105 us against 45)
+  const bool one_wave_one_launch = ctx->use_fused && ctx->fused_cs > 0 && !two_launches(ctx, k_cache, n_sel_max, workspace) &&
+                                   !fasa_attend_separately(ctx, n_sel_max, workspace) &&
                                    (long long)c.batch * ctx->n_sets * ctx->fused_cs <= 2ll * ctx->n_sm;
   if (all_mapped && one_wave_one_launch) {
     dq = (char*)mq; dk = (char*)mk; dv = (char*)mv;

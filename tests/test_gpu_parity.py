@@ -751,6 +751,30 @@ def test_score_stream_keeps_a_key_that_is_not_finite_to_itself(kw):
             assert np.array_equal(r.idx[b, s, :ref.size].cpu().numpy(), ref), (b, s)
 
 
+def test_host_step_of_two_launches_stages_its_inputs():
+    # pinned buffers are read in place by a step of one launch and one wave only: both kernels of a two-launch step would
+    # fetch them over the link CTA by CTA, so a kernel brings them to the staging area first
+    w = C["c1"].replace(batch=1, max_len=2100, len_lo=2000, len_hi=2000, budget=64, sel_heads=1)
+    a, b = Run(w), Run(w)
+    s = synth.make_step_inputs(w, 1, "cpu")
+    for r in (a, b):
+        r.build_proxy()
+    n0 = a.fasa.launch_count()
+    a.fasa.append_decode_step(*(s[n].cuda() for n in ("q", "k_new", "v_new")), a.k, a.v, a.proxy, a.seq_lens, w.budget, None, a.idx,
+                              a.n_sel, a.out, a.ws)
+    assert a.fasa.launch_count() - n0 == 2
+    stage = torch.zeros(b.fasa.stage_bytes(), dtype=torch.uint8, device="cuda")
+    host = torch.zeros(b.out.shape).pin_memory()
+    n0 = b.fasa.launch_count()
+    b.fasa.decode_step_host(*(s[n].pin_memory() for n in ("q", "k_new", "v_new")), stage, b.k, b.v, b.proxy, b.seq_lens, w.budget, None,
+                            b.idx, b.n_sel, b.out, host, b.ws)
+    assert b.fasa.launch_count() - n0 == 3
+    torch.cuda.synchronize()
+    assert a.fasa.device_status() == 0 and b.fasa.device_status() == 0
+    for x, y in ((a.idx, b.idx), (a.n_sel, b.n_sel), (a.out, b.out), (a.out.cpu(), host), (a.seq_lens, b.seq_lens), (a.k, b.k)):
+        assert torch.equal(x, y)
+
+
 def test_two_launch_steps_back_to_back_see_their_own_query_and_lengths():
     # the second launch starts before the first has ended and reads the lengths and the query then: in a loop that rewrites
     # the query's buffer on the stream and lets the lengths grow, every step must equal the one that had the GPU to itself
