@@ -137,16 +137,19 @@ int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* 
                              int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
                              int n_recent, cudaStream_t stream, int q_len, const fasa_calib_rows* calib) {
   const fasa_config_t& c = ctx->cfg;
-  // Few long rows: a cluster per row, which keeps the row's keys in shared memory.  One CTA per row pays for every position
-  // that it looks at again, the more the larger the selection (8 rows: at 17 K 10.6 against 8.6 us at 512, 14.7 / 9.7 at
-  // 2048; at 120 K 23 / 12 and 47 / 14; 64 rows at 32 K, 4096: 29 / 15), and for a row whose outliers crowd its scores into
-  // a few bins with radix passes over all of it (64 rows at 55 K, 512: 41 / 17 where others take 13).  It is the better one
-  // for short rows and for small selections of many (8 rows at 9 K, 64: 7.1 / 7.3; 40 rows at 17 K: 9.2 / 10.0 at 64,
-  // 10.8 / 11.3 at 512, 13.8 / 12.0 at 1024), and when the clusters would run in rounds (96 rows at 55 K: 21 / 27).
+  // A cluster per row keeps the row's keys in shared memory and selects by their bits, whatever their distribution.  One CTA per
+  // row pays for every position that it looks at again: the more, the larger the selection (8 rows: at 17 K 10.6 against 8.6
+  // us at 512, 14.7 / 9.7 at 2048; at 120 K 23 / 12 and 47 / 14; 64 rows at 32 K, 4096: 29 / 15) and the more scores are
+  // outliers (64 rows at 16 K, 256, one score in 500 an outlier: 18 / 14).  It is the better one for short rows and for small
+  // selections of many (40 rows at 17 K: 9.2 / 10.0 at 64, 10.8 / 11.3 at 512, 13.8 / 12.0 at 1024), and when the clusters would
+  // run in rounds (96 rows at 55 K: 21 / 27), unless nothing narrows a row down (96 rows at 65 K, 12387 of each: 48 / 35; 320 rows:
+  // 172 / 102; 320 rows at 16 K, 2048 of each: 42 / 29): then a row held in shared memory is read once, here three times.
   const long long n_rows = (long long)c.batch * rows_per_seq;
   const int k = budget > 0 ? budget : (int)(((long long)-budget * c.max_len + 999) / 1000);
-  if (!calib && !ctx->topk_rows && ctx->fused_cs > 1 && c.max_len > 8192 &&
-      (n_rows <= 16 ? c.max_len > 16384 || k >= 256 : n_rows <= ctx->n_sm / 2 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || c.max_len > 65536)))
+  const bool narrowed = sel_group_shift(c.max_len, k < c.max_len ? k : c.max_len, 16386) > 0, whole = !narrowed && c.max_len > 8192;
+  const bool few = n_rows <= 16 && c.max_len >= 2048 && (c.max_len > 16384 || (k >= 128 && (narrowed || whole)));
+  const bool large = n_rows <= ctx->n_sm / 2 && c.max_len > 8192 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || c.max_len > 65536);
+  if (!calib && !ctx->topk_rows && ((whole && ctx->fused_cs > 0) || ((few || large) && ctx->fused_cs > 1)))
     return fasa_topk_cluster_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, rows_per_seq, n_sink, n_recent, stream, q_len);
   RowParams p;
   p.scores = scores; p.seq_lens = seq_lens; p.idx = idx; p.n_sel = n_sel; p.status = ctx->d_status;

@@ -1762,13 +1762,14 @@ def test_topk_exact_at_the_edges_of_its_groups(L, budget, n_sink, n_recent):
 
 
 @pytest.mark.parametrize("rows,L,budget", [
+    (16, 4096, 256), (16, 2048, 128),                           # few rows
     (100, 20001, 40), (100, 20001, 1700),                       # a thread block of 1024
     (160, 9001, 64), (160, 9001, 900), (160, 65553, 300),       # 512
     (320, 5003, 30), (320, 70001, 100), (320, 70001, 2000),     # 256; groups of 32 and whole rows beyond 65536 positions
 ])
 def test_topk_exact_for_each_size_of_thread_block(rows, L, budget):
-    # many rows, each kind of row among them, by the kernel of one CTA per row; all of them against the register-resident
-    # kernel, one of each kind against the oracle
+    # many rows, each kind of row among them, by the kernel of one CTA per row, and by the one that the rows ask for; all of them
+    # against the register-resident kernel, one of each kind against the oracle
     g = torch.Generator().manual_seed(rows + L + budget)
     sc = torch.randn(rows // 4, 4, L, generator=g)
     sc[:, 0] = torch.where(torch.rand(rows // 4, L, generator=g) < 2e-3, sc[:, 0] + 3e3, sc[:, 0])      # crowded but for a few outliers
@@ -1779,8 +1780,8 @@ def test_topk_exact_for_each_size_of_thread_block(rows, L, budget):
     sc[3, 2, L - 3] = float("nan")
     lens = [L - 13 * b for b in range(rows // 4)]
     for n_sink, n_recent in ((0, 0), (4, 64)):
-        got = [_topk_only(sc, lens, budget, n_sink, n_recent, budget + n_sink + n_recent, mode) for mode in (0, 2)]
-        assert all(np.array_equal(x, y) for x, y in zip(*got))
+        got = [_topk_only(sc, lens, budget, n_sink, n_recent, budget + n_sink + n_recent, mode) for mode in (0, 2, 1)]
+        assert all(np.array_equal(x, y) and np.array_equal(x, z) for x, y, z in zip(*got))
         for b, h in [(0, 0), (0, 1), (1, 1), (1, 2), (2, 2), (rows // 4 - 1, 3)]:
             ref, _ = O.select(sc[b, h, :lens[b]].double().numpy(), budget, n_sink, n_recent)
             assert int(got[1][1][b, h]) == ref.size and np.array_equal(got[1][0][b, h, :ref.size], ref), (b, h)
