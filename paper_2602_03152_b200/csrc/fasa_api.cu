@@ -269,12 +269,18 @@ extern "C" int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max
 // 4 K 24 -> 19 us; 28 / 4 heads, batch 4 at 50 K 89 -> 33 us.  Few sets with long lists stay with the cluster kernel, whose
 // CTAs share one selection (batch 1 at 16 K, 1024 rows a set: 24 against 28 us), as do groups of two or three, where the
 // stream saves less (16 / 8 heads, batch 4 at 50 K: 40 against 42 us; batch 16 at 16 K: 71 -> 50 us), and rows shorter
-// than 2048, which are one launch whatever the batch.
+// than 2048, which are one launch whatever the batch.  Every CTA of the second launch selects for itself, which large selections do
+// not repay: beyond a sixteenth of the context nothing narrows a row down (batch 16 at 16 K, 1536 rows a set: 180 against
+// 166 us by cluster kernel and split-K attention, 4096: 324 / 238; rows of up to 4096 are cheap to take whole, and of up to
+// 8192 in larger groups: batch 16 at 4 K, 2048 rows 103 / 116; batch 8, 28 / 4 heads, at 8 K, 1024 rows 43 / 47), and beyond 2048
+// rows a set has several such CTAs (batch 4 at 64 K: 2048 89 / 129, 3072 130 / 140, 8192 376 / 189).
 static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, const void* workspace) {
   const fasa_config_t& c = ctx->cfg;
   if (workspace == nullptr || !set_per_head(ctx) || c.max_len < 2048 || !fasa_select_attend_ok(ctx, n_sel_max)) return false;
   const long long sets = (long long)c.batch * ctx->n_sets;
-  if (ctx->group < 4 ? sets < 192 : sets < 96 && n_sel_max > 512) return false;
+  if (ctx->group < 4 ? sets < 192 || n_sel_max > 1024 : sets < 96 && n_sel_max > 512) return false;
+  if (n_sel_max > (sets <= ctx->n_sm ? 3072 : 2048)) return false;
+  if (16ll * n_sel_max > c.max_len && c.max_len > (ctx->group > 4 ? 8192 : 4096)) return false;
   return !(c.page_size == 0 && fasa_on_host(ctx, k_cache));
 }
 

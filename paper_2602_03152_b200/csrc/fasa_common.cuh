@@ -103,9 +103,15 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
 // A resident grid of barely more CTAs than SMs leaves most SMs with one CTA beside some with two.  One or two heads per set
 // do not make up for that: clusters of one attend separately from 1024 rows on (160 units of two heads at 10 K, 2048 rows: 71
 // against 79 us, at 3 K and 1455 51 / 55; 256 units 95 / 91), larger ones below that on long slices (96 units at 10 K, 512
-// rows: 33 / 34.5; 2048 rows: 59 / 52.5).  Up to
-// eight units on short caches keep the two launches that they are documented with (2 x 4 x 7 at 5.4 K, 1800 rows: 23.9 us;
-// one launch would take 20.7).
+// rows: 33 / 34.5; 2048 rows: 59 / 52.5).
+// From some thousand rows on the attention itself decides.  Clusters of four 512-thread CTAs, each alone on its SM, have 16
+// warps an SM to gather with, the split-K kernel 20 and more (4 x 8 at 16 K: 25.5 / 26.4 us at 1024, 35.7 / 40.7 at 4096, 50.2 /
+// 59.1 at 8192).  And where several sets read the rows of one KV head they come from L2, and what counts is the instructions
+// per row, of which 16-row tiles need fewer: four sets or more to a KV head from 1024 rows on (a set per head, 16 x 32 at 16 K:
+// 209 / 226 us at 3072, 352 / 444 at 8192; 4 x 28 at 32 K 97 / 116 at 6144), two sets of several heads once they hold a fifth
+// of the context (16 x 16 sets of two heads at 16 K: 201 / 233 at 8192, 32 x 16 at 8 K 208 / 236 at 4096).
+// Up to eight units on short caches keep the two launches that they are documented with (2 x 4 x 7 at 5.4 K, 1800 rows: 23.9
+// us; one launch would take 20.7).
 static inline bool fasa_attend_separately(const fasa_ctx* ctx, int n_sel_max, const void* workspace) {
   const bool pairs = (long long)ctx->step_resident * ctx->step_cs > ctx->n_sm;
   const long long units = (long long)ctx->cfg.batch * ctx->n_sets;
@@ -113,7 +119,11 @@ static inline bool fasa_attend_separately(const fasa_ctx* ctx, int n_sel_max, co
   const long long ctas = units * ctx->step_cs;
   const bool uneven = ctx->sel_heads <= 2 && ctx->step_threads == 512 && ctas > ctx->n_sm && 10 * ctas <= 13ll * ctx->n_sm &&
                       (ctx->step_cs == 1 ? n_sel_max >= 1024 : n_sel_max >= 64 && n_sel_max < 1024 && ctx->cfg.max_len / ctx->step_cs >= 4096);
-  return workspace != nullptr && (uneven || (units > ctx->step_resident && n_sel_max >= 64 && !(pairs && n_sel_max >= 512)) || documented);
+  const bool lone = ctx->step_threads == 512 && ctx->step_cs == 4 && ctas <= ctx->n_sm && 8 * units >= ctx->n_sm && n_sel_max >= 1024;
+  const int sharing = ctx->group / ctx->sel_heads;
+  const bool from_l2 = (sharing >= 4 && units >= 96 && n_sel_max >= 1024) ||
+                       (sharing >= 2 && ctx->sel_heads >= 2 && n_sel_max >= 2048 && 5ll * n_sel_max >= ctx->cfg.max_len);
+  return workspace != nullptr && (uneven || lone || from_l2 || (units > ctx->step_resident && n_sel_max >= 64 && !(pairs && n_sel_max >= 512)) || documented);
 }
 
 // Whether the attention of a step that runs on 16-row tiles (a launch of its own, or select-and-attend) keeps all 24 bits of a

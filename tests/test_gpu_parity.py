@@ -751,6 +751,32 @@ def test_score_stream_keeps_a_key_that_is_not_finite_to_itself(kw):
             assert np.array_equal(r.idx[b, s, :ref.size].cpu().numpy(), ref), (b, s)
 
 
+@pytest.mark.parametrize("kw,budget,launches", [
+    (dict(batch=3, max_len=5000, sel_heads=1), 312, 2),             # score stream, select-and-attend: up to a sixteenth of the context
+    (dict(batch=3, max_len=5000, sel_heads=1), 313, 1),             # the cluster kernel, one proxy stream per set
+    (dict(batch=3, max_len=5000, sel_heads=1), 1024, 2),            # its selection, then split-K attention of rows from L2
+    (dict(batch=3, max_len=4000, sel_heads=1), 1536, 2),            # short rows are taken whole
+    (dict(batch=5, max_len=4000, sel_heads=1), 2048, 2), (dict(batch=5, max_len=4000, sel_heads=1), 2049, 2),
+    (dict(batch=4, n_q_heads=28, n_kv_heads=4, max_len=6000, sel_heads=1), 900, 2),
+    (dict(batch=8, max_len=10240, sel_heads=2), 2047, 1), (dict(batch=8, max_len=10240, sel_heads=2), 2048, 2),
+    (dict(batch=4, max_len=8192), 1023, 1), (dict(batch=4, max_len=8192), 1024, 2),      # clusters of four, one CTA to an SM
+])
+def test_large_selections_where_the_route_changes(kw, budget, launches):
+    w = C["c1"].replace(**dict(dict(len_lo=kw["max_len"] - 700, len_hi=kw["max_len"], n_sink=0, n_recent=0, budget=budget), **kw))
+    r = Run(w)
+    r.build_proxy()
+    r.step(fused=True)                                                # no workspace: one launch
+    one = [x.clone() for x in (r.idx, r.n_sel, r.out, r.lse)]
+    r.reset_outputs()
+    n0 = r.fasa.launch_count()
+    r.fasa.decode_step(r.q, r.k, r.v, r.proxy, r.seq_lens, w.budget, r.scores, r.idx, r.n_sel, r.out, r.ws, r.lse)
+    torch.cuda.synchronize()
+    assert r.fasa.launch_count() - n0 == launches and r.fasa.device_status() == 0
+    assert torch.equal(one[0], r.idx) and torch.equal(one[1], r.n_sel)
+    # (17 bits in a probability, 24 in the sums)
+    assert float((one[2] - r.out).abs().max()) <= 1e-4 and float((one[3] - r.lse).abs().max()) <= 1e-4
+
+
 def test_host_step_of_two_launches_stages_its_inputs():
     # pinned buffers are read in place by a step of one launch and one wave only: both kernels of a two-launch step would
     # fetch them over the link CTA by CTA, so a kernel brings them to the staging area first
