@@ -238,18 +238,23 @@ fasa_split_plan fasa_plan_splits(const fasa_ctx* ctx, int n_upper, int units) {
   return p;
 }
 
-// Workspace: split-K partial results, then (sets per query head) what the two-launch step passes from its first half to
-// its second, a score row and a row of group maxima per index set.  The partial-result area is sized for the largest
+// Workspace: split-K partial results, then (contexts whose steps can run as two launches) what the first half passes to the
+// second, a score row and a row of group maxima per index set.  The partial-result area is sized for the largest
 // split count any call can use (the bound at max_len for the fewest units a launch can have, one per KV head), so
 // nothing here depends on the selection size.
 static bool set_per_head(const fasa_ctx* ctx) { return ctx->sel_heads == 1 && ctx->group > 1; }
+// Whether any step of this context can run as two launches (see two_launches).
+static bool two_launches_possible(const fasa_ctx* ctx) {
+  return set_per_head(ctx) && ctx->cfg.max_len >= 2048 && fasa_select_attend_ok(ctx, 1) &&
+         (ctx->group >= 4 || (long long)ctx->cfg.batch * ctx->n_sets >= 192);
+}
 struct fasa_ws {
   size_t scores, gm, total;
 };
 static fasa_ws ws_layout(const fasa_ctx* ctx) {
   const fasa_config_t& c = ctx->cfg;
   const int n = split_count_bound(ctx, c.max_len, c.batch * c.n_kv_heads);
-  const size_t per_split = (size_t)c.batch * c.n_q_heads * (FASA_HEAD_DIM + 2) * sizeof(float), rows = set_per_head(ctx) ? (size_t)c.batch * ctx->n_sets : 0;
+  const size_t per_split = (size_t)c.batch * c.n_q_heads * (FASA_HEAD_DIM + 2) * sizeof(float), rows = two_launches_possible(ctx) ? (size_t)c.batch * ctx->n_sets : 0;
   fasa_ws w;
   const size_t dense = ((size_t)fasa_dense_ctas(ctx) + (size_t)c.batch * c.n_kv_heads) * ctx->group * (FASA_HEAD_DIM + 2) * sizeof(float);
   w.scores = fasa_align_up(std::max(per_split * (size_t)n, dense), 256) + 256;
@@ -276,10 +281,9 @@ extern "C" int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max
 // rows a set has several such CTAs (batch 4 at 64 K: 2048 89 / 129, 3072 130 / 140, 8192 376 / 189).
 static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, const void* workspace) {
   const fasa_config_t& c = ctx->cfg;
-  if (workspace == nullptr || !set_per_head(ctx) || c.max_len < 2048 || !fasa_select_attend_ok(ctx, n_sel_max)) return false;
   const long long sets = (long long)c.batch * ctx->n_sets;
-  if (ctx->group < 4 ? sets < 192 || n_sel_max > 1024 : sets < 96 && n_sel_max > 512) return false;
-  if (n_sel_max > (sets <= ctx->n_sm ? 3072 : 2048)) return false;
+  if (workspace == nullptr || !two_launches_possible(ctx) || n_sel_max > (sets <= ctx->n_sm ? 3072 : 2048)) return false;
+  if (ctx->group < 4 ? n_sel_max > 1024 : sets < 96 && n_sel_max > 512) return false;
   if (16ll * n_sel_max > c.max_len && c.max_len > (ctx->group > 4 ? 8192 : 4096)) return false;
   return !(c.page_size == 0 && fasa_on_host(ctx, k_cache));
 }

@@ -751,6 +751,19 @@ def test_score_stream_keeps_a_key_that_is_not_finite_to_itself(kw):
             assert np.array_equal(r.idx[b, s, :ref.size].cpu().numpy(), ref), (b, s)
 
 
+def test_workspace_holds_score_rows_only_where_a_step_can_use_them():
+    def need(heads, max_len, sel, batch=4):
+        f = binding.Fasa(batch, heads[0], heads[1], max_len, torch.arange(4, dtype=torch.int32).repeat(heads[1], 1), select_heads=sel)
+        return f.workspace_bytes(64)
+
+    score_rows = 4 * 32 * 2048 * 4
+    assert need((32, 8), 2048, 1) >= need((32, 8), 2048, 0) + score_rows
+    assert need((32, 8), 2047, 1) == need((32, 8), 2047, 0)                     # too short for two launches
+    assert need((32, 8), 262145, 1) == need((32, 8), 262145, 0)                 # too long
+    assert need((16, 8), 4096, 1) == need((16, 8), 4096, 0)                     # groups of two, few sets
+    assert need((16, 8), 4096, 1, 12) > need((16, 8), 4096, 0, 12)
+
+
 @pytest.mark.parametrize("kw,budget,launches", [
     (dict(batch=3, max_len=5000, sel_heads=1), 312, 2),             # score stream, select-and-attend: up to a sixteenth of the context
     (dict(batch=3, max_len=5000, sel_heads=1), 313, 1),             # the cluster kernel, one proxy stream per set
