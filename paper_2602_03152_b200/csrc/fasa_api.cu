@@ -288,6 +288,14 @@ static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, cons
   return !(c.page_size == 0 && fasa_on_host(ctx, k_cache));
 }
 
+// A workspace that is not 256-byte aligned is refused where the list is one for the split-K kernel, and goes unused by steps
+// that can do without: one launch.
+static bool usable_workspace(const fasa_ctx* ctx, int n_sel_max, void** workspace) {
+  if (((uintptr_t)*workspace & 255) == 0) return true;
+  *workspace = nullptr;
+  return fasa_full_probabilities(ctx, n_sel_max);
+}
+
 // The groups whose maxima the first half takes: those that suit a row of max_len.
 static int stream_group_shift(const fasa_ctx* ctx, int budget) {
   const long long n = ctx->cfg.max_len, k = budget > 0 ? budget : ((long long)-budget * n + 999) / 1000;
@@ -333,13 +341,11 @@ extern "C" int32_t fasa_decode_step(fasa_ctx_t* ctx, const void* q, const void* 
         ((uintptr_t)v_cache & 15) || (scores && ((uintptr_t)scores & 3)))
       return FASA_ERR_INVALID_ARG;
     if (!fasa_pages_ready(ctx)) return FASA_ERR_INVALID_ARG;
-    if (two_launches(ctx, k_cache, n_sel_max, workspace)) {
-      if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;
+    if (!usable_workspace(ctx, n_sel_max, &workspace)) return FASA_ERR_INVALID_ARG;
+    if (two_launches(ctx, k_cache, n_sel_max, workspace))
       return two_launch_step(ctx, q, nullptr, nullptr, const_cast<void*>(k_cache), const_cast<void*>(v_cache), const_cast<void*>(proxy_k),
                              seq_lens, budget, n_sel_max, scores, idx, n_sel, out, lse, workspace, nullptr, (cudaStream_t)stream);
-    }
     if (fasa_attend_separately(ctx, n_sel_max, workspace)) {
-      if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;   // (what the second launch would refuse)
       int32_t st2 = fasa_fused_launch(ctx, q, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores,
                                       idx, n_sel, out, lse, nullptr, nullptr, (cudaStream_t)stream, false);
       if (st2 != FASA_OK) return st2;
@@ -378,14 +384,13 @@ static int32_t append_decode_step_impl(fasa_ctx_t* ctx, const void* q, const voi
         (scores && ((uintptr_t)scores & 3)))
       return FASA_ERR_INVALID_ARG;
     if (!fasa_pages_ready(ctx)) return FASA_ERR_INVALID_ARG;
+    if (!usable_workspace(ctx, n_sel_max, &workspace)) return FASA_ERR_INVALID_ARG;
     if (two_launches(ctx, k_cache, n_sel_max, workspace)) {
-      if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;
       *mirrored = out_mirror != nullptr;
       return two_launch_step(ctx, q, k_new, v_new, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores, idx, n_sel,
                              out, lse, workspace, out_mirror, (cudaStream_t)stream);
     }
     if (fasa_attend_separately(ctx, n_sel_max, workspace)) {
-      if ((uintptr_t)workspace & 255) return FASA_ERR_INVALID_ARG;   // (what the second launch would refuse)
       int32_t st2 = fasa_fused_launch(ctx, q, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max, scores,
                                       idx, n_sel, out, lse, k_new, v_new, (cudaStream_t)stream, false);
       if (st2 != FASA_OK) return st2;

@@ -751,6 +751,26 @@ def test_score_stream_keeps_a_key_that_is_not_finite_to_itself(kw):
             assert np.array_equal(r.idx[b, s, :ref.size].cpu().numpy(), ref), (b, s)
 
 
+@pytest.mark.parametrize("kw", [dict(batch=2, n_q_heads=32, n_kv_heads=8, max_len=2100, sel_heads=1), dict(batch=48, n_q_heads=32, n_kv_heads=8, max_len=256)])
+def test_misaligned_workspace_is_refused_for_long_lists_only(kw):
+    w = C["c1"].replace(**dict(dict(len_lo=kw["max_len"], len_hi=kw["max_len"], n_sink=0, n_recent=0, budget=100), **kw))
+    r = Run(w)
+    r.build_proxy()
+    ws = torch.empty(r.ws.numel() + 16, dtype=torch.uint8, device="cuda")[16:]
+    n0 = r.fasa.launch_count()
+    r.fasa.decode_step(r.q, r.k, r.v, r.proxy, r.seq_lens, w.budget, r.scores, r.idx, r.n_sel, r.out, ws)
+    torch.cuda.synchronize()
+    assert r.fasa.launch_count() - n0 == 1 and r.fasa.device_status() == 0
+    got = (r.idx.clone(), r.out.clone())
+    r.step(fused=True)
+    assert torch.equal(got[0], r.idx) and torch.equal(got[1], r.out)
+    long = torch.empty((w.batch, w.n_sets, 2048), dtype=torch.int32, device="cuda")
+    with pytest.raises(binding.FasaError) as e:
+        r.fasa.decode_step(r.q, r.k, r.v, r.proxy, r.seq_lens, w.budget, r.scores, long, r.n_sel, r.out, ws)
+    assert e.value.status == binding.ERR_INVALID_ARG
+    torch.cuda.synchronize()
+
+
 def test_workspace_holds_score_rows_only_where_a_step_can_use_them():
     def need(heads, max_len, sel, batch=4):
         f = binding.Fasa(batch, heads[0], heads[1], max_len, torch.arange(4, dtype=torch.int32).repeat(heads[1], 1), select_heads=sel)
