@@ -31,8 +31,10 @@ split_rows_kernel(const uint16_t* k_src, const uint16_t* v_src, uint16_t* k_nond
                   int max_len, int chunks, int nd, int64_t ksb, int64_t ksh, int64_t kst, int64_t vsb, int64_t vsh,
                   int64_t vst, const fasa_resident res) {
   __shared__ __align__(16) uint16_t s_k[kSplitRows][FASA_HEAD_DIM];
-  pdl_wait_for_predecessor();
-  pdl_release_successor();
+  if constexpr (APPEND) {                           // (the other form is launched the ordinary way: see bulk_rows_kernel)
+    pdl_wait_for_predecessor();
+    pdl_release_successor();
+  }
   const int u = blockIdx.y, h = u % n_kv_heads, b = u / n_kv_heads, tid = threadIdx.x;
   const int len = clamp_len(seq_lens[b], max_len, status);
   const int n0 = blockIdx.x * kSplitRows;
@@ -158,8 +160,8 @@ extern "C" int32_t fasa_m_split(fasa_ctx_t* ctx, const void* k_cache, void* k_no
   if (!split_ok(ctx)) return FASA_ERR_UNSUPPORTED;
   const fasa_config_t& c = ctx->cfg;
   dim3 grid((unsigned)((c.max_len + kSplitRows - 1) / kSplitRows), (unsigned)(c.batch * c.n_kv_heads));
-  FASA_CUDA_TRY(ctx, launch_after_predecessor(
-      split_rows_kernel<false>, grid, dim3(256), (size_t)0, (cudaStream_t)stream, 0, (const uint16_t*)k_cache, (const uint16_t*)nullptr,
+  FASA_CUDA_TRY(ctx, fasa_launch(
+      split_rows_kernel<false>, fasa_launch_shape{grid, dim3(256), 0, 0, false}, (cudaStream_t)stream, (const uint16_t*)k_cache, (const uint16_t*)nullptr,
       (uint16_t*)k_nondom, (uint16_t*)nullptr, (unsigned char*)nullptr, seq_lens, (int32_t*)nullptr, (int32_t*)nullptr,
       (const int16_t*)ctx->d_chan, (const int16_t*)ctx->d_ndchan, ctx->d_status, 0, (int)c.n_kv_heads, (int)c.max_len, ctx->chunks,
       (int)(FASA_HEAD_DIM - 2 * c.n_dom), c.k_stride_b, c.k_stride_h, c.k_stride_t, c.v_stride_b, c.v_stride_h, c.v_stride_t, fasa_resident{}));
