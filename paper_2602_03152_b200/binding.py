@@ -16,6 +16,8 @@ from typing import Optional
 
 import torch
 
+from . import build
+
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libfasa.so")
 MARSHAL_PATH = os.path.join(_PKG, "_marshal.so")
@@ -127,6 +129,8 @@ def _load_marshal():
     if _invoke is None:
         if not os.path.exists(MARSHAL_PATH):
             raise FileNotFoundError(f"{MARSHAL_PATH} is missing: build it with `python -m paper_2602_03152_b200.build`")
+        if not build.marshal_fits(MARSHAL_PATH):
+            raise ImportError(f"{MARSHAL_PATH} was not built as {build.marshal_tag()!r}: run `python -m paper_2602_03152_b200.build`")
         spec = importlib.util.spec_from_file_location("_marshal", MARSHAL_PATH)
         module = importlib.util.module_from_spec(spec)
         spec.loader.exec_module(module)

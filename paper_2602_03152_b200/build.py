@@ -6,6 +6,7 @@ argument marshalling of the Python binding) with the host compiler.
 from __future__ import annotations
 
 import glob
+import importlib.metadata
 import os
 import subprocess
 import sys
@@ -36,16 +37,32 @@ def _stale() -> bool:
     return any(os.path.getmtime(d) > os.path.getmtime(LIB) for d in deps)
 
 
+def marshal_tag() -> str:
+    """The interpreter and torch that an extension module built now is for; a string that the file holds."""
+    return "_marshal for %s, torch %s" % (sysconfig.get_config_var("SOABI"), importlib.metadata.version("torch"))
+
+
+def marshal_fits(path: str) -> bool:
+    """Whether the extension module at `path` was built for this interpreter and this torch."""
+    with open(path, "rb") as f:
+        return marshal_tag().encode() in f.read()
+
+
+def _marshal_stale() -> bool:
+    return not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL_SRC) > os.path.getmtime(MARSHAL) or not marshal_fits(MARSHAL)
+
+
 def build_marshal(force: bool = False) -> str:
     """The binding's extension module, against the headers and libraries of the installed torch."""
-    if not force and os.path.exists(MARSHAL) and os.path.getmtime(MARSHAL_SRC) <= os.path.getmtime(MARSHAL):
+    if not force and not _marshal_stale():
         return MARSHAL
     import torch
 
     root = os.path.dirname(torch.__file__)
     libs = os.path.join(root, "lib")
     tmp = MARSHAL + ".tmp.%d" % os.getpid()
-    cmd = ["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI]
+    cmd = ["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-D_GLIBCXX_USE_CXX11_ABI=%d" % torch._C._GLIBCXX_USE_CXX11_ABI,
+           '-DFASA_BUILT_FOR="%s"' % marshal_tag()]
     for path in (sysconfig.get_paths()["include"], "/usr/local/cuda/include"):
         cmd += ["-I", path]
     for path in ("include", os.path.join("include", "torch", "csrc", "api", "include")):
@@ -60,7 +77,7 @@ def build_marshal(force: bool = False) -> str:
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every kernel into one shared object, and the binding's extension; returns the former's path."""
     marshal = subprocess.Popen([sys.executable, os.path.abspath(__file__), "--marshal"] + (["--force"] if force else [])) \
-        if force or not os.path.exists(MARSHAL) or os.path.getmtime(MARSHAL_SRC) > os.path.getmtime(MARSHAL) else None
+        if force or _marshal_stale() else None
     if force or _stale():
         nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
         tmp = LIB + ".tmp.%d" % os.getpid()

@@ -121,3 +121,15 @@ def test_kernels_that_wait_inside_read_nothing_through_the_read_only_path():
             assert set(constant) <= {"chan", "ndchan"}, (name, constant)
             assert "__ldg(" not in part, name
     assert kernels >= 10
+
+
+def test_extension_built_for_another_interpreter_or_torch_is_stale_and_not_loaded(monkeypatch):
+    build.build()
+    assert build.marshal_fits(build.MARSHAL)
+    monkeypatch.setattr(build, "marshal_tag", lambda: "_marshal for another interpreter")
+    assert not build.marshal_fits(build.MARSHAL) and build._marshal_stale()
+    monkeypatch.setattr(binding, "_invoke", None)
+    with pytest.raises(ImportError):
+        binding._load_marshal()
+    monkeypatch.undo()
+    assert callable(binding._load_marshal())
