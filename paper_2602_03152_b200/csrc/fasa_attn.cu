@@ -366,7 +366,7 @@ decode_attn_mma_kernel(const AttnParams p) {
     __syncthreads();
     cluster_wait();
     cg::cluster_group cluster = cg::this_cluster();
-    if constexpr (SPARSE && !KSPLIT)
+    if constexpr (TERMS == 3)
       cluster_merge_store<kMmaThreads>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse, [&](int g) {
         const int u = unit_again();
         const SelUnit s = sel_unit(u, p.n_sets, p.group, p.n_q_heads, p.n_kv_heads);
@@ -380,7 +380,7 @@ decode_attn_mma_kernel(const AttnParams p) {
         e.b = (s.b / p.q_len); e.max_len = p.max_len; e.scale_log2 = p.scale_log2;
         return e;
       });
-    else   // (the dense pass and split key caches go without)
+    else   // (long lists, the dense pass and split key caches go without, as ever)
       cluster_merge_store<kMmaThreads>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse);
   }
 }

@@ -34,7 +34,7 @@ struct ClusterMergeSmem {
 // entry of V then gives NaN where its sum with the other rows is an infinity.  An output that is not finite is therefore
 // computed once more by a warp, row by row with multiply-adds.  (Here, because the attention loops have no register to
 // spare: a test at their end, a branch in them or a second copy of them cost 2 to 10 % of a step; this costs 0.2 us of the
-// smallest ones, 13.4 -> 13.6 us, and nothing that shows of most others.)
+// smallest ones, 13.4 -> 13.6 us, nothing that shows of most others, and 3 % of the cluster kernel's lists of 4096 rows.)
 template <bool PAGED>
 struct ExactOutput {
   const uint16_t* q;              // the query head

@@ -118,19 +118,22 @@ select_attend_kernel(const SelAttnParams p) {
   if (p.append && tid == 0) s_last = atomicAdd(p.arrive, 1) == (int)(gridDim.x * gridDim.y) - 1;
   __syncthreads();
   cluster_wait();
-  cluster_merge_store<NT>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse, [&](int g) {
-    const int u = unit_again();
-    const SelUnit s = sel_unit(u, p.n_sets, p.group, p.n_q_heads, p.n_kv_heads);
-    ExactOutput<PAGED> e;
-    e.q = p.q + (s.q0 + g) * FASA_HEAD_DIM;
-    e.k = p.k + s.h * p.ksh + (PAGED ? 0 : s.b * p.ksb);
-    e.v = p.v + s.h * p.vsh + (PAGED ? 0 : s.b * p.vsb);
-    e.list = p.idx + (int64_t)u * p.n_sel_max;
-    e.n = p.n_sel[u];
-    e.status = p.status; e.pm = p.pm; e.ksb = p.ksb; e.kst = p.kst; e.vsb = p.vsb; e.vst = p.vst;
-    e.b = s.b; e.max_len = p.max_len; e.scale_log2 = p.scale_log2;
-    return e;
-  });
+  if constexpr (TERMS == 3)
+    cluster_merge_store<NT>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse, [&](int g) {
+      const int u = unit_again();
+      const SelUnit s = sel_unit(u, p.n_sets, p.group, p.n_q_heads, p.n_kv_heads);
+      ExactOutput<PAGED> e;
+      e.q = p.q + (s.q0 + g) * FASA_HEAD_DIM;
+      e.k = p.k + s.h * p.ksh + (PAGED ? 0 : s.b * p.ksb);
+      e.v = p.v + s.h * p.vsh + (PAGED ? 0 : s.b * p.vsb);
+      e.list = p.idx + (int64_t)u * p.n_sel_max;
+      e.n = p.n_sel[u];
+      e.status = p.status; e.pm = p.pm; e.ksb = p.ksb; e.kst = p.kst; e.vsb = p.vsb; e.vst = p.vst;
+      e.b = s.b; e.max_len = p.max_len; e.scale_log2 = p.scale_log2;
+      return e;
+    });
+  else   // (long lists go without: see fasa_attn.cu)
+    cluster_merge_store<NT>(cluster, s_part, s_merge, p.group, su.q0, p.out, p.out_mirror, p.lse);
   if (p.append && tid < 32 && s_last) {
     if (tid == 0) *p.arrive = 0;
     for (int b = tid; b < p.batch; b += 32) {
