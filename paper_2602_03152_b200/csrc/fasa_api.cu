@@ -153,17 +153,13 @@ extern "C" int32_t fasa_create(const fasa_config_t* cfg, const int32_t* dom_fc_h
   return FASA_OK;
 }
 
-// Whether a K/V cache pointer is host memory (the memory-optimised variant keeps the caches in
-// page-locked host memory): asked of the driver once per pointer, a decode loop passes the same one.
-bool fasa_on_host(fasa_ctx* ctx, const void* p) {
-  if (ctx->cache_seen == p && p) return ctx->cache_on_host != 0;
+// Whether a K/V cache pointer is host memory (the memory-optimised variant keeps the caches in page-locked host memory).  The
+// driver is asked each time, 60 ns: an answer kept by address would be wrong for what is allocated there next.
+bool fasa_on_host(const void* p) {
   cudaPointerAttributes at;
-  bool host = false;
-  if (cudaPointerGetAttributes(&at, p) == cudaSuccess) host = at.type == cudaMemoryTypeHost;
-  else cudaGetLastError();
-  ctx->cache_seen = p;
-  ctx->cache_on_host = host ? 1 : 0;
-  return host;
+  if (cudaPointerGetAttributes(&at, p) == cudaSuccess) return at.type == cudaMemoryTypeHost;
+  cudaGetLastError();
+  return false;
 }
 
 extern "C" int32_t fasa_set_block_table(fasa_ctx_t* ctx, const int32_t* block_table) {
@@ -285,7 +281,7 @@ static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, cons
   if (workspace == nullptr || !two_launches_possible(ctx) || n_sel_max > (sets <= ctx->n_sm ? 3072 : 2048)) return false;
   if (ctx->group < 4 ? n_sel_max > 1024 : sets < 96 && n_sel_max > 512) return false;
   if (16ll * n_sel_max > c.max_len && c.max_len > (ctx->group > 4 ? 8192 : 4096)) return false;
-  return !(c.page_size == 0 && fasa_on_host(ctx, k_cache));
+  return !(c.page_size == 0 && fasa_on_host(k_cache));
 }
 
 // A workspace that is not 256-byte aligned is refused where the list is one for the split-K kernel, and goes unused by steps
@@ -468,24 +464,17 @@ extern "C" int32_t fasa_decode_step_host(fasa_ctx_t* ctx, const void* q_host,
   // of one launch its kernel reads them in place (the few KB cross the host link inside the
   // launch); where it is several launches or several waves of CTAs, one small kernel first
   // brings all three to the staging area, so that no CTA's start waits on the link.  Anything
-  // else is copied to the staging area with cudaMemcpyAsync.  The driver is asked about a
-  // pointer once: a decode loop passes the same buffers every step.
-  auto mapped = [&](int slot, const void* hp) -> void* {
-    if (ctx->host_seen[slot] == hp) return ctx->host_mapped[slot];
+  // else is copied to the staging area with cudaMemcpyAsync.  The driver is asked about each
+  // pointer in every call (see fasa_on_host; a buffer that is no longer pinned must not be touched by a kernel).
+  auto mapped = [](const void* hp) -> void* {
     cudaPointerAttributes at;
-    void* dp = nullptr;
-    if (cudaPointerGetAttributes(&at, hp) == cudaSuccess) {
-      if (at.type == cudaMemoryTypeHost) dp = at.devicePointer;
-    } else {
-      cudaGetLastError();
-    }
-    ctx->host_seen[slot] = hp;
-    ctx->host_mapped[slot] = dp;
-    return dp;
+    if (cudaPointerGetAttributes(&at, hp) == cudaSuccess) return at.type == cudaMemoryTypeHost ? at.devicePointer : nullptr;
+    cudaGetLastError();
+    return nullptr;
   };
-  const void* mq = mapped(0, q_host);
-  const void* mk = mapped(1, k_new_host);
-  const void* mv = mapped(2, v_new_host);
+  const void* mq = mapped(q_host);
+  const void* mk = mapped(k_new_host);
+  const void* mv = mapped(v_new_host);
   const bool all_mapped = mq && mk && mv && !((uintptr_t)mq & 15) && !((uintptr_t)mk & 15) && !((uintptr_t)mv & 15);
   // (a set per query head at 16 K, batch 1: every warp of the score stream would fetch its query over the link, 105 us against 45)
   const bool one_wave_one_launch = ctx->use_fused && ctx->fused_cs > 0 && !two_launches(ctx, k_cache, n_sel_max, workspace) &&
@@ -503,7 +492,7 @@ extern "C" int32_t fasa_decode_step_host(fasa_ctx_t* ctx, const void* q_host,
   }
   // A pinned out_host is written by the step's kernel itself (next to `out`), where the path
   // taken has a single kernel to do it; otherwise `out` is copied back.
-  float* mo = (float*)mapped(3, out_host);
+  float* mo = (float*)mapped(out_host);
   if ((uintptr_t)mo & 3) mo = nullptr;
   bool mirrored = false;
   int32_t st = append_decode_step_impl(ctx, dq, dk, dv, k_cache, v_cache, proxy_k, seq_lens, budget, n_sel_max,

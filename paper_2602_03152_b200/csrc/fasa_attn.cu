@@ -605,7 +605,7 @@ int32_t launch_attn(fasa_ctx* ctx, const void* q, const void* k, const void* v,
   memset(&p.ks, 0, sizeof(p.ks));
   if (ksplit) p.ks = *ksplit;
   // caches in page-locked host memory are copied through L1 (contiguous caches, tensor-core kernel)
-  const bool host = c.page_size == 0 && ctx->use_fused && (ksplit != nullptr || fasa_on_host(ctx, k));
+  const bool host = c.page_size == 0 && ctx->use_fused && (ksplit != nullptr || fasa_on_host(k));
   p.q = (const uint16_t*)q; p.k = (const uint16_t*)k; p.v = (const uint16_t*)v;
   p.idx = idx; p.n_rows = n_rows; p.partial = (float*)workspace; p.out = nullptr; p.out_mirror = nullptr; p.lse = nullptr; p.status = ctx->d_status;
   p.n_q_heads = c.n_q_heads; p.n_kv_heads = c.n_kv_heads; p.n_sets = n_sets; p.group = G;

@@ -40,12 +40,6 @@ struct fasa_ctx {
   int step_resident;      // clusters of the step's shape that the device holds at once
   int use_fused;          // fasa_decode_step takes the one-launch kernel when it is available
   int topk_rows;          // fasa_topk and fasa_topk_batched by the one-CTA-per-row kernel whatever the rows (fasa_set_step_mode 2)
-  // host-buffer step: the last host pointers seen and what the device can use in their place
-  // (null: not page-locked + mapped), so that a decode loop with fixed buffers asks the driver once
-  const void* host_seen[4];
-  void* host_mapped[4];
-  const void* cache_seen;   // the last K/V cache pointer asked about, and whether it is host memory
-  int cache_on_host;
   long long launches;     // kernels launched through this context
   char cuda_err[256];
 };
@@ -166,7 +160,7 @@ fasa_resident fasa_resident_of(const fasa_ctx* ctx);
 int32_t fasa_attn_split_keys(fasa_ctx* ctx, const void* q, const void* k_nondom, const void* v_cache, const void* proxy_k,
                              const int32_t* idx, const int32_t* n_sel, int32_t n_sel_max, float* out, float* lse,
                              void* workspace, cudaStream_t stream);
-bool fasa_on_host(fasa_ctx* ctx, const void* p);
+bool fasa_on_host(const void* p);
 
 bool fasa_topk_row_ok(const fasa_ctx* ctx);
 // Calibration: the single-FC rows of a (sequence, query head) are not stored, they are computed from the KV head's

@@ -1199,7 +1199,7 @@ int32_t fasa_fused_launch(fasa_ctx* ctx, const void* q, const void* k_cache, con
   p.vsb = c.v_stride_b; p.vsh = c.v_stride_h; p.vst = c.v_stride_t;
   p.scale_log2 = c.softmax_scale * 1.4426950408889634f;
   p.pm = fasa_page_map(ctx);
-  p.host_rows = with_attention && c.page_size == 0 && fasa_on_host(ctx, k_cache);
+  p.host_rows = with_attention && c.page_size == 0 && fasa_on_host(k_cache);
   if (!fasa_pages_ready(ctx)) return FASA_ERR_INVALID_ARG;
   const bool paged = c.page_size > 0;
   FusedFn fn = with_attention ? fused_fn(ctx->chunks, paged) : select_fn(ctx->chunks, paged);

@@ -834,6 +834,38 @@ def test_host_step_of_two_launches_stages_its_inputs():
         assert torch.equal(x, y)
 
 
+def test_host_step_with_buffers_that_are_pinned_for_a_while():
+    # the same addresses, page-locked, then not, then again: what the device may read in place is decided in every call
+    w = C["c1"].replace(batch=1, max_len=3000, len_lo=2000, len_hi=2000, budget=64)
+    rt = torch.cuda.cudart()
+    outs = []
+    for pin in ([False] * 3, [True, False, True]):
+        r = Run(w)
+        r.build_proxy()
+        stage = torch.zeros(r.fasa.stage_bytes(), dtype=torch.uint8, device="cuda")
+        host = torch.zeros(4, 1 << 16, dtype=torch.uint8)                       # (a buffer each)
+        q, kn, vn, out = (host[i][4096:] for i in range(4))
+        q, kn, vn = (x[:n * 256].view(torch.bfloat16).view(s) for x, n, s in ((q, w.n_q_heads, (1, w.n_q_heads, 128)),
+                     (kn, w.n_kv_heads, (1, w.n_kv_heads, 1, 128)), (vn, w.n_kv_heads, (1, w.n_kv_heads, 1, 128))))
+        out = out[:w.n_q_heads * 512].view(torch.float32).view(1, w.n_q_heads, 128)
+        got = []
+        for step, on in enumerate(pin):
+            s = synth.make_step_inputs(w, step, "cpu")
+            for dst, n in ((q, "q"), (kn, "k_new"), (vn, "v_new")):
+                dst.copy_(s[n])
+            out.zero_()
+            if on:
+                assert int(rt.cudaHostRegister(host.data_ptr(), host.numel(), 0)) == 0
+            r.fasa.decode_step_host(q, kn, vn, stage, r.k, r.v, r.proxy, r.seq_lens, w.budget, None, r.idx, r.n_sel, r.out, out, r.ws)
+            if on:
+                assert int(rt.cudaHostUnregister(host.data_ptr())) == 0
+            got.append((r.idx.clone(), r.out.cpu(), out.clone()))
+        assert r.fasa.device_status() == 0
+        outs.append(got)
+    for a, b in zip(*outs):
+        assert all(torch.equal(x, y) for x, y in zip(a, b)) and torch.equal(a[1], a[2])
+
+
 def test_two_launch_steps_back_to_back_see_their_own_query_and_lengths():
     # the second launch starts before the first has ended and reads the lengths and the query then: in a loop that rewrites
     # the query's buffer on the stream and lets the lengths grow, every step must equal the one that had the GPU to itself
