@@ -18,11 +18,8 @@
 // Measured (ncu, batch 4, 32 / 8 heads, 30-56 K): 31 us for 88 MB of proxy and 22 MB of scores, and 23 us for the second
 // half, against 79 + 10 us for a cluster per set.
 //
-// With at most four query heads to a KV head the eight columns of an instruction hold the four heads twice, once
-// zeroed for each tile of a pair: both tiles accumulate into one fragment, lanes t < 2 of a quad holding the first
-// tile's heads and t >= 2 the second's, which halves the work after the products.  A key that is not finite gives NaN in
-// the zeroed columns too, that is in the score of a token of the other tile: a slot with such a score is scored again with
-// a fragment for each tile.
+// With at most four query heads to a KV head the eight columns of an instruction hold the four heads twice: of a pair of tiles
+// the lanes t < 2 of a quad keep the first one's scores and t >= 2 the second's, which halves the work after the products.
 //
 // The new token's row is scored from k_new itself: the warp that owns its tile writes the K, V and proxy rows
 // and replaces the row in its fragments, so nothing waits for those writes.  The lengths themselves grow in the
@@ -208,13 +205,10 @@ score_stream_kernel(const StreamParams p) {
   bool ok = true;
   while (w.left > 0 && ok) {
     const int run = min(w.left, w.pairs - w.pair);   // pairs of this (sequence, KV head)
-    // Operands: column n of the product is query head n; G4: head n - 4 e for tile e of a pair, zero elsewhere.
-    constexpr int OPS = G4 ? 2 : 1;
-    ScoreFrag<KB> f[OPS];
-#pragma unroll
-    for (int e = 0; e < OPS; ++e)
-      load_score_b<KB>(f[e], p.q + ((int64_t)w.b * p.n_q_heads + (int64_t)w.h * p.group) * FASA_HEAD_DIM, p.chan + w.h * p.chunks * 8, p.chunks,
-                       G4 && (lane >> 4) != e ? 0 : p.group, G4 ? (lane & 15) : lane);
+    // Operand: column n of the product is query head n; G4: head n mod 4.
+    ScoreFrag<KB> f;
+    load_score_b<KB>(f, p.q + ((int64_t)w.b * p.n_q_heads + (int64_t)w.h * p.group) * FASA_HEAD_DIM, p.chan + w.h * p.chunks * 8, p.chunks, p.group,
+                     G4 ? (lane & 15) : lane);
     const int64_t row0 = (int64_t)w.b * p.n_q_heads + w.h * p.group;                    // its first score row
     float* const srow0 = p.scores + row0 * p.max_len;
     float* const gm0 = p.gm + row0 * p.gm_stride;
@@ -257,8 +251,7 @@ score_stream_kernel(const StreamParams p) {
     };
     constexpr int NC = G4 ? 1 : 2;                    // fragments of a pair
     // Maxima of the groups of a head's scores in the fragments of one column: v[o] = octet 2 (t >> 1) + o (G4), or octet o
-    // (returned: a maximum over some of them, over all of them within the warp)
-    auto store_max_head = [&](const float (&v)[2 * NC], float* hgm, bool mine, int pair) -> float {
+    auto store_max_head = [&](const float (&v)[2 * NC], float* hgm, bool mine, int pair) {
       const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0;
       float m;
       int octet;
@@ -280,9 +273,8 @@ score_stream_kernel(const StreamParams p) {
         m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, G4 ? 2 : 8));
         if (mine && g == 0 && (!G4 || t < 2)) hgm[pair] = m;
       }
-      return m;
     };
-    float seen = 0.f;                                // G4: NaN once a score of the slot is not finite
+
     // where this lane's values go: rows g, g + 8, ... of its two heads' score rows
     const int head0 = G4 ? 2 * (t & 1) : 2 * t;
     float* const lane_row = srow0 + (int64_t)head0 * p.max_len + (G4 ? 16 * (t >> 1) : 0) + g;
@@ -297,17 +289,24 @@ score_stream_kernel(const StreamParams p) {
         for (int e = 0; e < 2; ++e)
 #pragma unroll
           for (int kb = 0; kb < KB; ++kb) a[i][e][kb] = *reinterpret_cast<const uint4*>(src + ((i * 2 + e) * KB + kb) * 512 + lane * 16);
-      float c[NP][NC][4];
+      float c[NP][2][4];                             // (a fragment for each tile: in a common one, each tile meeting zeros in the other's
+                                                     // columns, a key that is not finite made scores of the other tile NaN)
 #pragma unroll
       for (int i = 0; i < NP; ++i)
 #pragma unroll
-        for (int e = 0; e < NC; ++e) c[i][e][0] = c[i][e][1] = c[i][e][2] = c[i][e][3] = 0.f;
+        for (int e = 0; e < 2; ++e) c[i][e][0] = c[i][e][1] = c[i][e][2] = c[i][e][3] = 0.f;
 #pragma unroll
       for (int kb = 0; kb < KB; ++kb)
 #pragma unroll
         for (int e = 0; e < 2; ++e)
 #pragma unroll
-          for (int i = 0; i < NP; ++i) mma_bf16_16816(c[i][G4 ? 0 : e], a[i][e][kb], f[G4 ? e : 0].b[kb]);
+          for (int i = 0; i < NP; ++i) mma_bf16_16816(c[i][e], a[i][e][kb], f.b[kb]);
+      if constexpr (G4) {
+#pragma unroll
+        for (int i = 0; i < NP; ++i)
+#pragma unroll
+          for (int k = 0; k < 4; ++k) c[i][0][k] = t < 2 ? c[i][0][k] : c[i][1][k];
+      }
 #pragma unroll
       for (int i = 0; i < NP; ++i) {
         const int pair = pair0 + i;
@@ -321,13 +320,7 @@ score_stream_kernel(const StreamParams p) {
             v[o] = c[i][o >> 1][(o & 1) * 2 + e] + 0.0f;               // (-0 becomes +0)
             if (mine) hrow[8 * o] = v[o];
           }
-          if (p.gs > 0) {
-            const float m = store_max_head(v, lane_gm + (int64_t)e * p.gm_stride, mine, pair);
-            if (G4) seen = fmaf(m, 0.f, seen);
-          } else if (G4) {
-#pragma unroll
-            for (int o = 0; o < 2 * NC; ++o) seen = fmaf(v[o], 0.f, seen);
-          }
+          if (p.gs > 0) store_max_head(v, lane_gm + (int64_t)e * p.gm_stride, mine, pair);
         }
       }
     };
@@ -362,14 +355,14 @@ score_stream_kernel(const StreamParams p) {
           }
         }
       }
-      float c[2][4];                                 // a fragment for each tile: what one holds never meets the other
+      float c[2][4];
 #pragma unroll
       for (int e = 0; e < 2; ++e) c[e][0] = c[e][1] = c[e][2] = c[e][3] = 0.f;
 #pragma unroll
       for (int kb = 0; kb < KB; ++kb) {
         if (kb < pg.n16 + pg.n8) {
 #pragma unroll
-          for (int e = 0; e < 2; ++e) mma_bf16_16816(c[e], a[e][kb], f[G4 ? e : 0].b[kb]);
+          for (int e = 0; e < 2; ++e) mma_bf16_16816(c[e], a[e][kb], f.b[kb]);
         }
       }
       if constexpr (G4) {
@@ -418,13 +411,6 @@ score_stream_kernel(const StreamParams p) {
           general(std::false_type{}, src + j * pair_bytes, pair);
         }
         ++j;
-      }
-      if constexpr (G4) {
-        if (__any_sync(0xffffffffu, seen != 0.f)) {  // (NaN != 0)
-          for (j = 0; j < n; ++j)
-            if (first + j >= plain0 && first + j < plain1) general(std::false_type{}, src + j * pair_bytes, first + j);
-          seen = 0.f;
-        }
       }
       __syncwarp();                                  // every lane is done with the slot
       issue(slot);
