@@ -270,15 +270,21 @@ int32_t fasa_sparse_decode_attn_static(fasa_ctx_t* ctx, const void* q, const voi
  * `workspace` may be NULL and `scores` may be NULL (they are then not written).  Available
  * when ceil(max_len / 16) <= 22528 and the device can co-schedule such a cluster;
  * fasa_step_cluster_size tells.
- * When a workspace is given and the cluster kernel's grid needs several rounds of CTAs, mode 1 ends that kernel after the
- * selection and attends with the split-K tensor-core kernel of fasa_sparse_decode_attn (two launches instead of one; three
- * beyond 16384 selected rows): for n_sel_max >= 64, or only up to 511 where two CTAs share an SM.  The same hand-over
- * happens for at most 8 units with max_len <= 8192 once n_sel_max * ceil(heads per set / 4) >= 2048.
- * A set per query head (select_heads = 1) with a workspace, rows of at least 2048 positions and many sets runs as two
- * launches instead: one stream of the proxy that scores all heads of a KV head, then selection and attention.
+ * When a workspace is given, mode 1 may end that kernel after the selection and attend with the split-K tensor-core
+ * kernel of fasa_sparse_decode_attn (two launches instead of one; three beyond 16384 selected rows):
+ *   - where the cluster kernel's grid needs several rounds of CTAs, for n_sel_max >= 64, or only up to 511 where two
+ *     CTAs share an SM;
+ *   - where its CTAs are all resident but one or two heads to a set leave barely more of them than SMs, or clusters of
+ *     four stand alone on their SMs, for 1024 rows or more (64 to 1023 on long slices in the former case);
+ *   - for large selections (from 1024 or 2048 rows) of sets that share a KV head, whose rows come from L2;
+ *   - for at most 8 units with max_len <= 8192 once n_sel_max * ceil(heads per set / 4) >= 2048.
+ * A set per query head (select_heads = 1) with a workspace, rows of at least 2048 positions, many sets and selections of
+ * up to a sixteenth of the context (short rows: up to 2048) runs as two launches instead: one stream of the proxy that
+ * scores all heads of a KV head, then selection and attention.
  * Mode 0, and every configuration mode 1 cannot take: fasa_fc_score -> fasa_topk ->
  * fasa_sparse_decode_attn; scores and workspace are then required (INVALID_ARG if NULL).
- * Both modes select identical index sets; outputs agree to fp32 rounding.
+ * Both modes select identical index sets; outputs agree to fp32 rounding, or to 17 bits of each probability where a long
+ * list is attended by the split-K kernel (there, an infinite V entry of a selected row may give NaN; elsewhere an infinity).
  * n_sel_max is also the bound the launch shapes are planned with (route, split count): a
  * caller that knows the current lengths should pass the tightest bound it can (e.g.
  * ceil(0.189 * L) + n_sink + n_recent for a permille budget) rather than the bound at

@@ -215,8 +215,8 @@ extern "C" int32_t fasa_topk(fasa_ctx_t* ctx, const float* scores, const int32_t
   if (budget < -1000) return FASA_ERR_INVALID_ARG;
   const fasa_config_t& c = ctx->cfg;
   const int units = c.batch * ctx->n_sets;
-  // One CTA per row from the maxima of the row's groups; the register-resident cluster kernel below
-  // remains for longer rows and as mode 0.
+  // One CTA per row from the maxima of the row's groups, or the cluster kernel's selection phases (see fasa_topk_row_launch); the
+  // register-resident cluster kernel below remains for longer rows and as mode 0.
   if (ctx->use_fused && fasa_topk_row_ok(ctx))
     return fasa_topk_row_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, ctx->n_sets, c.n_sink, c.n_recent,
                                 (cudaStream_t)stream);
