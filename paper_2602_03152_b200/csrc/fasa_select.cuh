@@ -234,6 +234,7 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
   const uint32_t below = (1u << lane) - 1u;
 
   bool radix = false;                    // the even bins do not apply
+  bool equal_maxima = false;             // the threshold lies among many equal scores, it seems
   int n_list = 0;
   float bound = 0.f, top = 0.f, reach = 0.f;                       // the largest value; where the bins end
   int g0 = 0;
@@ -243,6 +244,7 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
     const int n_groups = ((r.hi - 1) >> gs) + 1 - g0;
     SelBinning first{0.f, 0.f};
     int b0 = 0;
+    uint32_t rank, count = 0;
 #pragma unroll 1
     for (int t = 0; t < kSelTries; ++t) {
       float lo = INFINITY, hi = -INFINITY, mid;
@@ -265,10 +267,13 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
         gm[i] = __int_as_float(bin);
       }
       __syncthreads();
-      uint32_t rank, count;
+      const uint32_t was = count;
       sel_find<kSelBins>(sm.hist[0], (uint32_t)r.k, lane, &b0, &rank, &count);
       // crowded: its groups would all be listed, and 8 or 32 positions of each visited
       if (count <= 64u + (uint32_t)r.k / 2u || t + 1 == kSelTries || !(first.scale > 0.f)) break;
+      // a thousandth of the range with half the maxima in it: no bins spread these (the same token again and again)
+      equal_maxima = 2u * count > was && t > 0;
+      if (equal_maxima) break;
       const SelBinning nb = sel_narrower(first, b0, top);
       if (!(nb.scale > 0.f)) break;
       first = nb;
@@ -355,8 +360,8 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
       sel_find<kSelBins>(sm.hist[1], (uint32_t)r.k, lane, &b1, &rank, &count);
       if (count <= (uint32_t)kSelRank && b1 > 0) break;
       const SelBinning nb = sel_narrower(second, b1, top);
-      // (as many as before: equal scores)
-      radix = b1 == 0 || t + 1 == kSelTries || count == was || !(second.scale > 0.f) || !(nb.scale > 0.f);
+      // (half as many as before: equal scores)
+      radix = b1 == 0 || t + 1 == kSelTries || (t > 0 && 2u * count > was) || equal_maxima || !(second.scale > 0.f) || !(nb.scale > 0.f);
       __syncthreads();                   // (every warp has read the histogram)
       if (radix) break;
       second = nb;

@@ -1894,6 +1894,19 @@ def test_topk_exact_below_outliers(L, budget, far):
     _assert_topk_exact(sc, [L], budget)
 
 
+@pytest.mark.parametrize("repeats", [200, 300, 1500, 2900])
+@pytest.mark.parametrize("L,budget", [(3328, 256), (7001, 256), (7001, 20), (20000, 1024)])
+def test_topk_exact_where_one_token_repeats(L, budget, repeats):
+    # the same score at the threshold again and again, among others: the histograms are refined once, then give way
+    g = torch.Generator().manual_seed(L + budget + repeats)
+    sc = torch.randn(1, 4, L, generator=g)
+    for h, above in enumerate((0, budget // 2, budget - 1, budget + 5)):
+        value = 9.0 if above == 0 else sc[0, h].sort(descending=True).values[above].item()
+        at = L - repeats if h % 2 else L // 9
+        sc[0, h, at:at + repeats] = value
+    _assert_topk_exact(sc, [L], budget)
+
+
 @pytest.mark.parametrize("L,B,H", [(32768, 1, 8), (131072, 2, 2), (140001, 1, 2), (20000, 3, 5)])
 def test_topk_exact_at_scale(L, B, H):
     # 131072 fills the register-resident capacity of an 8-CTA cluster; 140001 takes the
