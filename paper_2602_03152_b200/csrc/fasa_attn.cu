@@ -303,7 +303,7 @@ template <bool SPARSE, bool PAGED, bool CLUSTER, bool HOSTMEM = false, bool KSPL
 __global__ void __launch_bounds__(kMmaThreads, KSPLIT || PAGED ? 4 : 5)
 decode_attn_mma_kernel(const AttnParams p) {
   __shared__ ClusterMergeSmem s_merge;              // (CLUSTER only: written by the peers)
-  if constexpr (CLUSTER) cluster_arrive();          // this CTA runs; each waits for that much before it writes to a peer
+  if constexpr (CLUSTER) cluster_arrive_running();  // each waits for that much before it writes to a peer
   pdl_wait_for_predecessor();
   pdl_release_successor();
   const int u = blockIdx.y;
@@ -340,20 +340,31 @@ decode_attn_mma_kernel(const AttnParams p) {
   // once): a tile then costs one memory round trip (its rows), not two (its indices first).
   int32_t* s_idx = reinterpret_cast<int32_t*>(attn_smem_raw + sizeof(MmaSmem<kMmaWarps, TERMS>));
   if (SPARSE) {
-    for (int i = threadIdx.x; i < r1 - r0; i += kMmaThreads) {
-      int tok = irow[r0 + i];                        // (not through the read-only path: the kernel ahead may have written it)
-      if (tok < 0 || tok >= p.max_len) {
-        atomicOr(p.status, FASA_DEV_IDX_CLAMPED);
-        tok = 0;
-      }
-      if constexpr (KSPLIT) {
-        // a row that is resident on the GPU is entered as -1 - slot: it is then copied from there
-        if (p.ks.res.tags != nullptr) {
-          const int slot = fasa_resident_slot(p.ks.res, tok);
-          if (slot >= 0 && p.ks.res.tags[(int64_t)su.kv * p.ks.res.slots_pad + slot] == tok) tok = -1 - slot;
+    // Four entries in flight per thread: they are plain loads, as the kernel ahead may have written the list, which the compiler
+    // does not move over the check's atomic (13 x 8 lists of 12 K rows: one at a time 226.8 us a step, four 224).
+    constexpr int kAhead = 4;
+    for (int i0 = threadIdx.x; i0 < r1 - r0; i0 += kAhead * kMmaThreads) {
+      int ahead[kAhead];
+#pragma unroll
+      for (int j = 0; j < kAhead; ++j) ahead[j] = i0 + j * kMmaThreads < r1 - r0 ? irow[r0 + i0 + j * kMmaThreads] : 0;
+#pragma unroll
+      for (int j = 0; j < kAhead; ++j) {
+        const int i = i0 + j * kMmaThreads;
+        if (i >= r1 - r0) break;
+        int tok = ahead[j];
+        if (tok < 0 || tok >= p.max_len) {
+          atomicOr(p.status, FASA_DEV_IDX_CLAMPED);
+          tok = 0;
         }
+        if constexpr (KSPLIT) {
+          // a row that is resident on the GPU is entered as -1 - slot: it is then copied from there
+          if (p.ks.res.tags != nullptr) {
+            const int slot = fasa_resident_slot(p.ks.res, tok);
+            if (slot >= 0 && p.ks.res.tags[(int64_t)su.kv * p.ks.res.slots_pad + slot] == tok) tok = -1 - slot;
+          }
+        }
+        s_idx[i] = tok;
       }
-      s_idx[i] = tok;
     }
     __syncthreads();
   }

@@ -20,6 +20,8 @@ constexpr int kMergeMaxCs = 16;                        // CTAs per cluster at mo
 // The two halves of a cluster barrier (cluster.sync() = arrive + wait), for all threads of all CTAs alike: what a thread
 // wrote before its arrive is visible to every thread after its wait.
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+// (the first half where nothing was written that a peer may touch: the CTA only says that it runs, without a fence)
+__device__ __forceinline__ void cluster_arrive_running() { asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 
 // What the peers write into: must not share memory with anything the owning CTA still uses
@@ -87,7 +89,7 @@ __device__ __forceinline__ int unit_again() {
 // the whole block.  NT threads call this together, in every CTA of the cluster (the cluster
 // size must be a power of two <= 16).  out / lse rows start at query head q0; out_mirror and
 // lse may be null.  The peers must be known to run before this is called (their shared memory is written): a cluster barrier
-// since the kernel's start, or cluster_arrive() at the start and cluster_wait() before the call.  exact(g): what is needed to
+// since the kernel's start, or cluster_arrive_running() at the start and cluster_wait() before the call.  exact(g): what is needed to
 // compute the outputs of head g of this unit row by row (ExactOutput), for those that are not finite.
 template <int NT, typename Exact = NoExactOutput>
 __device__ __forceinline__ void cluster_merge_store(cooperative_groups::cluster_group& cluster,

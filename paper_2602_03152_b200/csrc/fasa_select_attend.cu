@@ -53,7 +53,7 @@ select_attend_kernel(const SelAttnParams p) {
   __shared__ int s_last;
   const int tid = threadIdx.x, lane = tid & 31;
   // (the merge writes into the peers' shared memory: each CTA says that it runs, and waits for that much at the end)
-  cluster_arrive();
+  cluster_arrive_running();
   cg::cluster_group cluster = cg::this_cluster();
   const int cs = (int)cluster.num_blocks(), crank = (int)cluster.block_rank();
   const int u = blockIdx.y;
