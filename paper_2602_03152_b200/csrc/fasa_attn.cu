@@ -341,7 +341,8 @@ decode_attn_mma_kernel(const AttnParams p) {
   int32_t* s_idx = reinterpret_cast<int32_t*>(attn_smem_raw + sizeof(MmaSmem<kMmaWarps, TERMS>));
   if (SPARSE) {
     // Four entries in flight per thread: they are plain loads, as the kernel ahead may have written the list, which the compiler
-    // does not move over the check's atomic (13 x 8 lists of 12 K rows: one at a time 226.8 us a step, four 224).
+    // does not move over the check's atomic (13 x 8 lists of 9-12 K rows: one at a time, and a fence at the start, 207.4 us a
+    // step, now 203.6).
     constexpr int kAhead = 4;
     for (int i0 = threadIdx.x; i0 < r1 - r0; i0 += kAhead * kMmaThreads) {
       int ahead[kAhead];
