@@ -929,7 +929,7 @@ def run_paged(args):
 
 def run_batched(args):
     """Blocks of query tokens (q_len > 1) on --config's shape: the three batched calls (scoring of all
-    queries of a block in one pass over the proxy on the tcgen05 tensor cores, selection and attention
+    queries of a block in one pass over the proxy on the tensor cores, selection and attention
     per query) next to q_len repetitions of the single-query calls.  One JSON object."""
     import numpy as np
     import torch

@@ -342,7 +342,7 @@ int32_t fasa_select_step(fasa_ctx_t* ctx, const void* q, const void* k_new, cons
  * [batch][q_len][n_sets]; out fp32 [batch][q_len][n_q_heads][128]; lse [batch][q_len][n_q_heads].
  * What the q_len steps share is the proxy stream: fasa_fc_score_batched reads it ONCE and
  * scores all queries as one matrix product P[L x 2F] . Q[2F x (heads per set * q_len)] on the
- * tcgen05 tensor cores (fp32 accumulation in tensor memory), then reduces each query's heads
+ * tensor cores (fp32 accumulation), then reduces each query's heads
  * (sum, or max with group_reduce = 1).  q_len = 1 gives the results of the single-query calls
  * up to the rounding order of the fp32 accumulation.  fasa_topk_batched and
  * fasa_sparse_decode_attn_batched are fasa_topk and fasa_sparse_decode_attn over the

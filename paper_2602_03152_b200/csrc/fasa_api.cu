@@ -256,6 +256,8 @@ static fasa_ws ws_layout(const fasa_ctx* ctx) {
   w.scores = fasa_align_up(std::max(per_split * (size_t)n, dense), 256) + 256;
   w.gm = w.scores + fasa_align_up(rows * (size_t)c.max_len * sizeof(float), 256);
   w.total = w.gm + fasa_align_up(rows * (size_t)fasa_stream_gm_stride(ctx) * sizeof(float), 256);
+  // (a block of queries keeps its group maxima here between scoring and selection, before any partial result)
+  w.total = std::max(w.total, fasa_block_maxima_bytes(ctx));
   return w;
 }
 extern "C" int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max, size_t* out_bytes) {

@@ -176,7 +176,18 @@ struct fasa_calib_rows {
 // pairs, query-major, and query t of the block sees seq_lens[b] - (q_len - 1 - t) positions.
 int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget,
                              int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
-                             int n_recent, cudaStream_t stream, int q_len = 1, const struct fasa_calib_rows* calib = nullptr);
+                             int n_recent, cudaStream_t stream, int q_len = 1, const struct fasa_calib_rows* calib = nullptr,
+                             const struct fasa_row_maxima* given = nullptr);
+// Where the scoring pass leaves the maxima of groups of 1 << gs scores, a row of `stride` of them for each score row; the size
+// of the groups that a selection of n_rows rows would use (0: it would not).
+struct fasa_row_maxima {
+  float* gm;
+  int gs, stride;
+};
+size_t fasa_block_maxima_bytes(const fasa_ctx* ctx);   // of the largest block of queries, a set to a KV head
+int fasa_row_maxima_shift(const fasa_ctx* ctx, int budget, long long n_rows);
+// Floats per row of such a buffer with groups of 8.
+int fasa_stream_gm_stride(const fasa_ctx* ctx);
 // The same by the selection phases of the cluster kernel (fasa_fused.cu), for contexts that it can serve (fused_cs > 0).
 int32_t fasa_topk_cluster_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget, int32_t n_sel_max,
                                  int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink, int n_recent, cudaStream_t stream,

@@ -461,6 +461,18 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
   }
 }
 
+// fill for sel_row where the maxima of groups [g0, g1) of a row were left in memory by the scoring pass.
+template <int NT>
+__device__ __forceinline__ void sel_copy_maxima(float* gm, const float* src, int g0, int g1, float& lo, float& hi) {
+#pragma unroll 8
+  for (int i = threadIdx.x; i < g1 - g0; i += NT) {
+    const float m = src[g0 + i];
+    gm[i] = m;
+    lo = fminf(lo, m);
+    hi = max_nan(hi, m);
+  }
+}
+
 // The selection of a row of `len` positions with forced ones: how the budget, the forced positions and
 // the size of the list combine (the forced ones are taken first, in ascending order).
 struct SelPlan {

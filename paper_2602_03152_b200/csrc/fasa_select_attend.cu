@@ -90,15 +90,7 @@ select_attend_kernel(const SelAttnParams p) {
   pdl_wait_for_predecessor();
   pdl_release_successor();
   auto maxima = [&](float* gm, float& gm_lo, float& gm_hi) {
-    const int g0 = row.lo >> gs, n_groups = ((row.hi - 1) >> gs) + 1 - g0;
-    const float* src = p.gm + (int64_t)u * p.gm_stride + g0;
-#pragma unroll 8
-    for (int i = tid; i < n_groups; i += NT) {
-      const float m = src[i];
-      gm[i] = m;
-      gm_lo = fminf(gm_lo, m);
-      gm_hi = max_nan(gm_hi, m);
-    }
+    sel_copy_maxima<NT>(gm, p.gm + (int64_t)u * p.gm_stride, row.lo >> gs, ((row.hi - 1) >> gs) + 1, gm_lo, gm_hi);
   };
   sel_row<NT>(row, gs, maxima, sm, dsm, p.lay, [&](int r, int pos) { take(plan.sink + r, pos); });
   for (int i = tid; i < plan.n_forced; i += NT) {

@@ -5,9 +5,6 @@
 
 #include "fasa_common.cuh"
 
-// Floats per score row of the group-maxima buffer (groups of 8).
-int fasa_stream_gm_stride(const fasa_ctx* ctx);
-
 // First half: scores [batch][n_q_heads][max_len] (and maxima of groups of 1 << gs positions, gs > 0) of every cached
 // token; k_new != null: the appended token first.
 struct fasa_stream_args {

@@ -21,10 +21,11 @@ struct RowParams {
   int32_t* status;
   int rows_per_seq, max_len, n_sink, n_recent, budget, n_sel_max, q_len;
   SelLayout lay;
+  fasa_row_maxima given;                // (MAXIMA) what the scoring pass has left
 };
 
 // One row: unit u = blockIdx.x of sequence b.
-template <int NT, typename Src>
+template <int NT, bool MAXIMA, typename Src>
 __device__ __forceinline__ void topk_row(const RowParams& p, const Src& src, int b, SelShared& sm, unsigned char* rsm) {
   const int tid = threadIdx.x, lane = tid & 31, u = blockIdx.x;
   int len_raw = p.seq_lens[b];
@@ -43,8 +44,15 @@ __device__ __forceinline__ void topk_row(const RowParams& p, const Src& src, int
   row.lo = plan.lo;
   row.hi = plan.hi;
   row.k = plan.k;
-  const int gs = row.k > 0 && row.k < row.hi - row.lo ? sel_group_shift(row.hi - row.lo, row.k, p.lay.gm_cap) : 0;
+  int gs = row.k > 0 && row.k < row.hi - row.lo ? sel_group_shift(row.hi - row.lo, row.k, p.lay.gm_cap) : 0;
+  // (given maxima are of the groups that suit max_len, which a short row may do without)
+  const bool given = MAXIMA && gs > 0 && (long long)row.k * (p.given.gs == 3 ? 12 : 43) <= row.hi - row.lo;
+  if (given) gs = p.given.gs;
   auto maxima = [&](float* gm, float& gm_lo, float& gm_hi) {
+    if (given) {
+      sel_copy_maxima<NT>(gm, p.given.gm + (int64_t)u * p.given.stride, row.lo >> gs, ((row.hi - 1) >> gs) + 1, gm_lo, gm_hi);
+      return;
+    }
     // A thread takes eight consecutive positions: their maximum needs no other lane (groups of 32: two shuffles).
     const int g0 = row.lo >> gs, first = g0 << gs;
     const bool vec_ok = src.aligned();
@@ -99,7 +107,7 @@ __device__ __forceinline__ void topk_row(const RowParams& p, const Src& src, int
 // CALIB: row r < 64 of a sample (sequence, query head) is FC r alone, computed from the channel pairs as it is read, row
 // 64 the full head: the 64 rows of the four to eight query heads of a KV head share 4 bytes per position and FC
 // instead of having 4 bytes each.
-template <int NT, bool CALIB>
+template <int NT, bool CALIB, bool MAXIMA = false>
 __global__ void __launch_bounds__(NT, 1024 / NT)
 topk_row_kernel(const RowParams p) {
   extern __shared__ __align__(16) unsigned char rsm[];
@@ -117,12 +125,12 @@ topk_row_kernel(const RowParams p) {
       src.p = p.calib.pairs + ((int64_t)kv * 64 + fc) * p.calib.stride;
       src.q0 = bf16_bits_to_f32(q[p.calib.pairing == 0 ? fc : 2 * fc]);
       src.q1 = bf16_bits_to_f32(q[p.calib.pairing == 0 ? fc + 64 : 2 * fc + 1]);
-      topk_row<NT>(p, src, b, sm, rsm);
+      topk_row<NT, false>(p, src, b, sm, rsm);
     } else {
-      topk_row<NT>(p, SelScores{p.scores + (int64_t)sample * p.calib.stride}, b, sm, rsm);
+      topk_row<NT, false>(p, SelScores{p.scores + (int64_t)sample * p.calib.stride}, b, sm, rsm);
     }
   } else {
-    topk_row<NT>(p, SelScores{p.scores + (int64_t)blockIdx.x * p.max_len}, b, sm, rsm);
+    topk_row<NT, MAXIMA>(p, SelScores{p.scores + (int64_t)blockIdx.x * p.max_len}, b, sm, rsm);
   }
 }
 
@@ -133,34 +141,49 @@ static constexpr int kTopkRowMaxLen = 524288;
 
 bool fasa_topk_row_ok(const fasa_ctx* ctx) { return ctx->cfg.max_len <= kTopkRowMaxLen; }
 
-int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget,
-                             int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
-                             int n_recent, cudaStream_t stream, int q_len, const fasa_calib_rows* calib) {
+// A cluster per row keeps the row's keys in shared memory and selects by their bits, whatever their distribution.  One CTA per
+// row pays for every position that it looks at again: the more, the larger the selection (8 rows: at 17 K 10.6 against 8.6
+// us at 512, 14.7 / 9.7 at 2048; at 120 K 23 / 12 and 47 / 14; 64 rows at 32 K, 4096: 29 / 15) and the more scores are
+// outliers (64 rows at 16 K, 256, one score in 500 an outlier: 18 / 14).  It is the better one for short rows and for small
+// selections of many (40 rows at 17 K: 9.2 / 10.0 at 64, 10.8 / 11.3 at 512, 13.8 / 12.0 at 1024), and when the clusters would
+// run in rounds (96 rows at 55 K: 21 / 27), unless nothing narrows a row down (96 rows at 65 K, 12387 of each: 48 / 35; 320 rows:
+// 172 / 102; 320 rows at 16 K, 2048 of each: 42 / 29): then a row held in shared memory is read once, here three times.
+static bool topk_by_clusters(const fasa_ctx* ctx, long long n_rows, int budget) {
   const fasa_config_t& c = ctx->cfg;
-  // A cluster per row keeps the row's keys in shared memory and selects by their bits, whatever their distribution.  One CTA per
-  // row pays for every position that it looks at again: the more, the larger the selection (8 rows: at 17 K 10.6 against 8.6
-  // us at 512, 14.7 / 9.7 at 2048; at 120 K 23 / 12 and 47 / 14; 64 rows at 32 K, 4096: 29 / 15) and the more scores are
-  // outliers (64 rows at 16 K, 256, one score in 500 an outlier: 18 / 14).  It is the better one for short rows and for small
-  // selections of many (40 rows at 17 K: 9.2 / 10.0 at 64, 10.8 / 11.3 at 512, 13.8 / 12.0 at 1024), and when the clusters would
-  // run in rounds (96 rows at 55 K: 21 / 27), unless nothing narrows a row down (96 rows at 65 K, 12387 of each: 48 / 35; 320 rows:
-  // 172 / 102; 320 rows at 16 K, 2048 of each: 42 / 29): then a row held in shared memory is read once, here three times.
-  const long long n_rows = (long long)c.batch * rows_per_seq;
   const int k = budget > 0 ? budget : (int)(((long long)-budget * c.max_len + 999) / 1000);
   const bool narrowed = sel_group_shift(c.max_len, k < c.max_len ? k : c.max_len, 16386) > 0, whole = !narrowed && c.max_len > 8192;
   const bool few = n_rows <= 16 && c.max_len >= 2048 && (c.max_len > 16384 || (k >= 128 && (narrowed || whole)));
   const bool large = n_rows <= ctx->n_sm / 2 && c.max_len > 8192 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || c.max_len > 65536);
-  if (!calib && !ctx->topk_rows && ((whole && ctx->fused_cs > 0) || ((few || large) && ctx->fused_cs > 1)))
+  return !ctx->topk_rows && ((whole && ctx->fused_cs > 0) || ((few || large) && ctx->fused_cs > 1));
+}
+
+// Group maxima that fit: groups of 8 up to 65536 positions, groups of 32 beyond (16 KB + 8 KB to 64 KB + 32 KB of shared memory).
+static int row_maxima_cap(const fasa_ctx* ctx) {
+  const int by32 = (ctx->cfg.max_len >> 5) + 2, by8 = (ctx->cfg.max_len >> 3) + 2;
+  return by32 > 8194 ? by32 : (by8 < 8194 ? by8 : 8194);
+}
+
+int fasa_row_maxima_shift(const fasa_ctx* ctx, int budget, long long n_rows) {
+  const long long n = ctx->cfg.max_len, k = budget > 0 ? budget : ((long long)-budget * n + 999) / 1000;
+  if (!fasa_topk_row_ok(ctx) || topk_by_clusters(ctx, n_rows, budget)) return 0;
+  return sel_group_shift((int)n, (int)(k < n ? k : n), row_maxima_cap(ctx));
+}
+
+int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* seq_lens, int32_t budget,
+                             int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
+                             int n_recent, cudaStream_t stream, int q_len, const fasa_calib_rows* calib, const fasa_row_maxima* given) {
+  const fasa_config_t& c = ctx->cfg;
+  if (!calib && !given && topk_by_clusters(ctx, (long long)c.batch * rows_per_seq, budget))
     return fasa_topk_cluster_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, rows_per_seq, n_sink, n_recent, stream, q_len);
   RowParams p;
   p.scores = scores; p.seq_lens = seq_lens; p.idx = idx; p.n_sel = n_sel; p.status = ctx->d_status;
   p.rows_per_seq = rows_per_seq; p.max_len = c.max_len; p.n_sink = n_sink; p.n_recent = n_recent;
   p.budget = budget; p.n_sel_max = n_sel_max; p.q_len = q_len;
   p.calib = calib ? *calib : fasa_calib_rows{};
-  // Groups of 8 up to 65536 positions, groups of 32 beyond (16 KB + 8 KB to 64 KB + 32 KB of shared memory).
-  const int by32 = (c.max_len >> 5) + 2, by8 = (c.max_len >> 3) + 2;
-  p.lay.gm_cap = by32 > 8194 ? by32 : (by8 < 8194 ? by8 : 8194);
+  p.given = given ? *given : fasa_row_maxima{};
+  p.lay.gm_cap = row_maxima_cap(ctx);
   const int rows = c.batch * rows_per_seq;
-  p.lay.word_cap = by32;
+  p.lay.word_cap = (c.max_len >> 5) + 2;
   const int room = 2 * p.lay.gm_cap > 8192 ? 2 * p.lay.gm_cap : 8192, need = (c.max_len + 63) & ~31;
   p.lay.uni_cap = need < room ? need : room;
   auto go = [&](auto kernel, int threads) -> int32_t {
@@ -173,6 +196,11 @@ int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* 
   // warp scans the histograms) and needs all of them resident: 320 rows of 64 K took two rounds of 512 threads,
   // 38 us, and fit in one round of 256.
   if (calib) return go(topk_row_kernel<256, true>, 256);
+  if (given) {
+    if (rows <= ctx->n_sm && c.max_len > 16384) return go(topk_row_kernel<1024, false, true>, 1024);
+    if (rows <= 2 * ctx->n_sm) return go(topk_row_kernel<512, false, true>, 512);
+    return go(topk_row_kernel<256, false, true>, 256);
+  }
   if (rows <= ctx->n_sm && c.max_len > 16384) return go(topk_row_kernel<1024, false>, 1024);
   if (rows <= 2 * ctx->n_sm) return go(topk_row_kernel<512, false>, 512);
   return go(topk_row_kernel<256, false>, 256);

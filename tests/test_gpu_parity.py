@@ -354,6 +354,18 @@ def test_batched_queries_shapes(cfg, kw, T):
     _batched_run(C[cfg].replace(**kw), T)
 
 
+@pytest.mark.parametrize("kw,T", [
+    # odd max_len: no two scores are stored at once; maxima in groups of 8; sinks and a window that end inside a group
+    (dict(batch=3, max_len=2047, len_lo=1025, len_hi=2047, budget=40, n_sink=3, n_recent=13), 7),
+    (dict(batch=3, max_len=4096, len_lo=4063, len_hi=4096, budget=2, n_recent=33), 3),                      # groups of 32, tiles end with the row
+    (dict(batch=2, n_q_heads=10, n_kv_heads=2, max_len=2080, len_lo=2049, len_hi=2080, n_dom=32, budget=50, group_reduce=1), 6),   # odd group, max
+    (dict(batch=2, n_q_heads=14, n_kv_heads=2, max_len=2100, len_lo=2063, len_hi=2100, n_dom=64, budget=60), 5),   # one tile in registers, 4 pairs of heads
+    (dict(batch=2, n_q_heads=6, n_kv_heads=1, max_len=1200, len_lo=5, len_hi=1200, n_dom=28, budget=30, n_sink=40), 8),   # seven chunks; a row shorter than the block
+])
+def test_batched_queries_at_the_edges_of_tiles_and_groups(kw, T):
+    _batched_run(C["c1"].replace(**kw), T)
+
+
 def test_batched_queries_on_paged_caches_equal_the_contiguous_results():
     # a block of 4 queries after a 4-token append, page pools in random order: the batched calls read
     # the proxy and the K/V rows through the block table and must give the contiguous bits
