@@ -103,8 +103,7 @@ extern "C" {
 #define FASA_DEV_IDX_CLAMPED    4   /* sparse attention met an index outside [0, max_len)  */
 #define FASA_DEV_NSEL_CLAMPED   8   /* n_sel exceeded n_sel_max                            */
 #define FASA_DEV_PAGE_CLAMPED  16   /* a block-table entry was < 0 or >= n_pages           */
-#define FASA_DEV_TIMEOUT       32   /* a bounded wait inside a kernel ran out; results of  */
-                                    /* that launch are undefined, the context stays usable */
+#define FASA_DEV_TIMEOUT       32   /* reserved: no kernel spins on anything                */
 
 typedef struct fasa_ctx fasa_ctx_t;
 

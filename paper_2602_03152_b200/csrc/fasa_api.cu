@@ -305,15 +305,16 @@ static int32_t two_launch_step(fasa_ctx* ctx, const void* q, const void* k_new, 
                                int32_t* idx, int32_t* n_sel, float* out, float* lse, void* workspace, float* out_mirror,
                                cudaStream_t stream) {
   const fasa_ws w = ws_layout(ctx);
-  fasa_stream_args a;
+  fasa_stream_args a{};
   a.q = q; a.proxy_k = proxy_k; a.seq_lens = seq_lens;
   a.scores = scores ? scores : (float*)((char*)workspace + w.scores);
-  a.gm = (float*)((char*)workspace + w.gm);
-  a.gs = stream_group_shift(ctx, budget);
+  a.maxima.gm = (float*)((char*)workspace + w.gm);
+  a.maxima.gs = stream_group_shift(ctx, budget);
+  a.maxima.stride = fasa_stream_gm_stride(ctx);
   a.k_new = k_new; a.v_new = v_new; a.k_cache = k_cache; a.v_cache = v_cache;
   int32_t st = fasa_stream_launch(ctx, a, stream);
   if (st != FASA_OK) return st;
-  return fasa_select_attend_launch(ctx, q, k_cache, v_cache, a.scores, a.gm, a.gs, seq_lens, budget, n_sel_max, idx, n_sel, out, lse,
+  return fasa_select_attend_launch(ctx, q, k_cache, v_cache, a.scores, a.maxima.gm, a.maxima.gs, seq_lens, budget, n_sel_max, idx, n_sel, out, lse,
                                    out_mirror, k_new != nullptr, stream);
 }
 

@@ -1,19 +1,20 @@
-// The two halves of the two-launch decode step, for index sets per query head.
+// The two halves of the two-launch decode step; the first one also scores blocks of queries.
 #pragma once
 
 #include <type_traits>
 
 #include "fasa_common.cuh"
 
-// First half: scores [batch][n_q_heads][max_len] (and maxima of groups of 1 << gs positions, gs > 0) of every cached
-// token; k_new != null: the appended token first.
+// First half: scores [batch][n_sets][max_len] (and group maxima, gs > 0) of every cached token; k_new != null: the appended
+// token first.  q_len > 0: of a block of queries, [batch][q_len][n_sets][max_len].  Index sets of one head or of as many as a
+// block takes.
 struct fasa_stream_args {
   const void* q;
   const void* proxy_k;
   const int32_t* seq_lens;
   float* scores;
-  float* gm;
-  int gs;
+  fasa_row_maxima maxima;
+  int q_len;
   const void* k_new;
   const void* v_new;
   void* k_cache;
