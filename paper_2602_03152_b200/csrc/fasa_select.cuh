@@ -14,8 +14,11 @@
 //      k-th largest score; its few members are ranked against each other by (score, index), which
 //      settles which of them are taken;
 //   4. the bit masks of the selected positions become ranks (a block-wide prefix sum).
-// What bounds this is instructions and block barriers (seven), not bytes: a pass touches a score with
-// a dozen instructions per 32 of them, so the fewer positions a pass visits the better.  Bins are
+// What bounds this is latency, instructions and block barriers (ten), not bytes: a pass touches a score with a dozen
+// instructions per 32 of them, so the fewer positions a pass visits the better.  A row of 53 K with its maxima given, 256 of it,
+// 512 threads, in thousands of cycles: the maxima 2.6, their histogram 3.4 with the search, the list 2.7, the scores of its
+// groups 3.5, their threshold 1.1, classes 1.3, ties 1.2, ranks 1.7; before loads went in batches without a serial rest, shares of
+// the bins were summed by warps, and ranks went by bytes: 4.0, 3.6, 2.8, 5.1 for scores and threshold, 3.5, 2.2.  Bins are
 // monotone in the score, whatever the rounding, so the result is exact.  A few scores far above the others (outlier keys,
 // sinks) would leave the rest in one or two bins: where some warp's largest value is far below the largest of all, the bins
 // end a little above it, and what lies beyond falls into the last one.  A histogram whose bin of interest is crowded all the
@@ -35,7 +38,7 @@ constexpr int kSelRadixBins = 2048;
 struct SelShared {
   alignas(16) uint32_t hist[2][kSelBins];   // (read 16 bytes at a time) group maxima; scores.  Together: the bins of a radix pass
   uint32_t ckey[kSelRank], cpos[kSelRank];
-  uint32_t wlo[32], whi[32], wcnt[32];
+  uint32_t wlo[32], whi[32], wcnt[32], share[32];
   uint32_t n_cand;
 };
 static_assert(2 * kSelBins == kSelRadixBins, "the radix passes use both histograms");
@@ -137,6 +140,56 @@ __device__ __forceinline__ void sel_find(const uint32_t* hist, uint32_t kth, int
     left -= __shfl_sync(0xffffffffu, ci, 31);
     top -= 32;
   }
+}
+
+// The same for the histograms of kSelBins bins, by the whole block: every warp sums its share of the bins, then looks at the
+// sums and at one share alone.  (Every warp scanning all bins moves 4 KB of shared memory for each: 1200 cycles with 16 warps,
+// 450 this way.)  One barrier, behind the one that completes the histogram.
+template <int NT>
+__device__ __forceinline__ void sel_find_block(SelShared& sm, const uint32_t* hist, uint32_t kth, int warp, int lane, int* bin, uint32_t* rank,
+                                               uint32_t* count) {
+  constexpr int NW = NT / 32, PER = kSelBins / NW, EACH = PER / 32;  // bins of a share / of a lane: 1, 2 or 4
+  static_assert(EACH == 1 || EACH == 2 || EACH == 4, "a lane reads its bins at once");
+  auto share = [&](int w, uint32_t (&c)[EACH]) {                    // the lane's bins of share w, highest first (share 0 is the highest)
+    const uint32_t* p = hist + kSelBins - PER * w - EACH * (lane + 1);
+    if constexpr (EACH == 4) {
+      const uint4 q = *reinterpret_cast<const uint4*>(p);
+      c[0] = q.w; c[1] = q.z; c[2] = q.y; c[3] = q.x;
+    } else if constexpr (EACH == 2) {
+      const uint2 q = *reinterpret_cast<const uint2*>(p);
+      c[0] = q.y; c[1] = q.x;
+    } else {
+      c[0] = *p;
+    }
+  };
+  uint32_t c[EACH], sum = 0;
+  share(warp, c);
+#pragma unroll
+  for (int j = 0; j < EACH; ++j) sum += c[j];
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  if (lane == 0) sm.share[warp] = sum;
+  __syncthreads();
+  const uint32_t v = lane < NW ? sm.share[lane] : 0u, incl = sel_scan(v, lane);
+  const uint32_t hits = __ballot_sync(0xffffffffu, incl >= kth);
+  const int w = hits ? __ffs(hits) - 1 : NW - 1;
+  const uint32_t left = kth - __shfl_sync(0xffffffffu, incl - v, w);
+  share(w, c);
+  sum = 0;
+#pragma unroll
+  for (int j = 0; j < EACH; ++j) sum += c[j];
+  const uint32_t ci = sel_scan(sum, lane);
+  const uint32_t h2 = __ballot_sync(0xffffffffu, ci >= left);
+  const int at = h2 ? __ffs(h2) - 1 : 31;
+  uint32_t r = left - (ci - sum);                                   // (of the lane `at`)
+  int j = 0;
+  uint32_t n = c[0];
+#pragma unroll
+  for (int i = 1; i < EACH; ++i) {
+    if (j == i - 1 && r > n) { r -= n; n = c[i]; j = i; }
+  }
+  *bin = __shfl_sync(0xffffffffu, kSelBins - PER * w - EACH * lane - 1 - j, at);
+  *rank = __shfl_sync(0xffffffffu, r, at);
+  *count = __shfl_sync(0xffffffffu, n, at);
 }
 
 // Block-wide min and max of the threads' values, and the least of the warps' maxima (of those that have values: the others
@@ -261,14 +314,22 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
       } else {
         __syncthreads();
       }
-      for (int i = tid; i < n_groups; i += NT) {
-        const int bin = first.bin(gm[i]);
-        atomicAdd(&sm.hist[0][bin], 1u);
-        gm[i] = __int_as_float(bin);
+      for (int i0 = tid; i0 < n_groups; i0 += NT * 4) {
+        float m[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) m[j] = gm[min(i0 + j * NT, n_groups - 1)];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (i0 + j * NT < n_groups) {
+            const int bin = first.bin(m[j]);
+            atomicAdd(&sm.hist[0][bin], 1u);
+            gm[i0 + j * NT] = __int_as_float(bin);
+          }
+        }
       }
       __syncthreads();
       const uint32_t was = count;
-      sel_find<kSelBins>(sm.hist[0], (uint32_t)r.k, lane, &b0, &rank, &count);
+      sel_find_block<NT>(sm, sm.hist[0], (uint32_t)r.k, warp, lane, &b0, &rank, &count);
       // crowded: its groups would all be listed, and 8 or 32 positions of each visited
       if (count <= 64u + (uint32_t)r.k / 2u || t + 1 == kSelTries || !(first.scale > 0.f)) break;
       // a thousandth of the range with half the maxima in it: no bins spread these (the same token again and again)
@@ -284,6 +345,7 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
       const int per = ((n_groups + NW - 1) / NW + 31) & ~31;        // a warp takes a run of groups
       const int s0 = min(n_groups, warp * per), s1 = min(n_groups, s0 + per);
       uint32_t mine = 0;
+#pragma unroll 4
       for (int i = s0 + lane; i < s1; i += 32) mine += __float_as_int(gm[i]) >= b0 ? 1u : 0u;
       mine = __reduce_add_sync(0xffffffffu, mine);
       if (lane == 0) sm.wcnt[warp] = mine;
@@ -291,11 +353,16 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
       const uint32_t w = lane < NW ? sm.wcnt[lane] : 0u, incl = sel_scan(w, lane);
       n_list = (int)__shfl_sync(0xffffffffu, incl, 31);
       uint32_t at = __shfl_sync(0xffffffffu, incl - w, warp);
-      for (int i = s0; i < s1; i += 32) {                           // uniform over the warp
-        const bool in = i + lane < s1 && __float_as_int(gm[i + lane]) >= b0;
-        const uint32_t m = __ballot_sync(0xffffffffu, in);
-        if (in) list[at + __popc(m & below)] = (uint16_t)(i + lane);
-        at += __popc(m);
+      for (int i = s0; i < s1; i += 128) {                          // uniform over the warp
+        bool in[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) in[j] = __float_as_int(gm[min(i + 32 * j + lane, n_groups - 1)]) >= b0 && i + 32 * j + lane < s1;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint32_t m = __ballot_sync(0xffffffffu, in[j]);
+          if (in[j]) list[at + __popc(m & below)] = (uint16_t)(i + 32 * j + lane);
+          at += __popc(m);
+        }
       }
       // (a little below the bin's edge, so that rounding leaves none of the listed maxima under it)
       bound = first.scale > 0.f ? first.lo + ((float)b0 - 1.0625f) / first.scale : first.lo;
@@ -357,7 +424,7 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
       });
       __syncthreads();
       const uint32_t was = count;
-      sel_find<kSelBins>(sm.hist[1], (uint32_t)r.k, lane, &b1, &rank, &count);
+      sel_find_block<NT>(sm, sm.hist[1], (uint32_t)r.k, warp, lane, &b1, &rank, &count);
       if (count <= (uint32_t)kSelRank && b1 > 0) break;
       const SelBinning nb = sel_narrower(second, b1, top);
       // (half as many as before: equal scores)
@@ -445,31 +512,48 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
   __syncthreads();
 
   // ---- 4: ranks in ascending order ---------------------------------------------------------------
-  const int wpt = (n_chunks + NT - 1) / NT;
-  const int w0 = min(n_chunks, tid * wpt), w1 = min(n_chunks, w0 + wpt);
+  // A thread takes a run of bytes of the masks (a byte is a group of 8), or of words where there are enough of them: as few bits
+  // after one another as there are threads for.
+  const bool bytes = 2 * n_chunks <= NT;
+  const uint8_t* mask8 = reinterpret_cast<const uint8_t*>(words);
+  const int n_parts = bytes ? 4 * n_chunks : n_chunks, each = (n_parts + NT - 1) / NT;
+  const int w0 = min(n_parts, tid * each), w1 = min(n_parts, w0 + each);
   uint32_t mine = 0;
-  for (int c = w0; c < w1; ++c) mine += __popc(words[c]);
+  for (int c = w0; c < w1; ++c) mine += __popc(bytes ? (uint32_t)mask8[c] : words[c]);
   uint32_t total, at = sel_block_prefix<NT>(sm, mine, warp, lane, &total);
   for (int c = w0; c < w1; ++c) {
-    uint32_t m = words[c];
+    uint32_t m = bytes ? (uint32_t)mask8[c] : words[c];
+    if (m == 0u) continue;
+    const int first = bytes ? pos_at(c >> 2, (c & 3) * 8) : 0;
     while (m) {
       const int j = __ffs(m) - 1;
       m &= m - 1;
-      if (at < (uint32_t)r.k) emit((int)at, pos_at(c, j));       // (the comparison keeps a write inside the list)
+      if (at < (uint32_t)r.k) emit((int)at, bytes ? first + j : pos_at(c, j));     // (the comparison keeps a write inside the list)
       ++at;
     }
   }
 }
 
-// fill for sel_row where the maxima of groups [g0, g1) of a row were left in memory by the scoring pass.
+// fill for sel_row where the maxima of groups [g0, g1) of a row were left in memory by the scoring pass.  Eight or sixteen loads in flight
+// per thread, the last ones predicated: a loop that takes what is left over one by one waits for memory each time.
 template <int NT>
 __device__ __forceinline__ void sel_copy_maxima(float* gm, const float* src, int g0, int g1, float& lo, float& hi) {
-#pragma unroll 8
-  for (int i = threadIdx.x; i < g1 - g0; i += NT) {
-    const float m = src[g0 + i];
-    gm[i] = m;
-    lo = fminf(lo, m);
-    hi = max_nan(hi, m);
+  constexpr int UNR = NT == 256 ? 8 : 16;         // (64 registers)
+  const int n = g1 - g0;
+  src += g0;
+  for (int i0 = threadIdx.x; i0 < n; i0 += NT * UNR) {
+    float m[UNR];
+#pragma unroll
+    for (int j = 0; j < UNR; ++j)
+      if (i0 + j * NT < n) m[j] = src[i0 + j * NT];
+#pragma unroll
+    for (int j = 0; j < UNR; ++j) {
+      if (i0 + j * NT < n) {
+        gm[i0 + j * NT] = m[j];
+        lo = fminf(lo, m[j]);
+        hi = max_nan(hi, m[j]);
+      }
+    }
   }
 }
 
