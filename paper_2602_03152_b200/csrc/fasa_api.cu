@@ -239,10 +239,16 @@ fasa_split_plan fasa_plan_splits(const fasa_ctx* ctx, int n_upper, int units) {
 // split count any call can use (the bound at max_len for the fewest units a launch can have, one per KV head), so
 // nothing here depends on the selection size.
 static bool set_per_head(const fasa_ctx* ctx) { return ctx->sel_heads == 1 && ctx->group > 1; }
+// Whether the clusters of the one-launch step run in rounds, or some SMs hold two CTAs of it and others one.
+static bool clusters_crowd(const fasa_ctx* ctx) {
+  const long long units = (long long)ctx->cfg.batch * ctx->n_sets;
+  return ctx->fused_cs > 0 && (units * ctx->step_cs > ctx->n_sm || units > ctx->step_resident);
+}
 // Whether any step of this context can run as two launches (see two_launches).
 static bool two_launches_possible(const fasa_ctx* ctx) {
-  return set_per_head(ctx) && ctx->cfg.max_len >= 2048 && fasa_select_attend_ok(ctx, 1) &&
-         (ctx->group >= 4 || (long long)ctx->cfg.batch * ctx->n_sets >= 192);
+  if (ctx->cfg.max_len < 2048 || !fasa_select_attend_ok(ctx, 1)) return false;
+  if (set_per_head(ctx)) return ctx->group >= 4 || (long long)ctx->cfg.batch * ctx->n_sets >= 192;
+  return ctx->sel_heads == ctx->group && clusters_crowd(ctx);
 }
 struct fasa_ws {
   size_t scores, gm, total;
@@ -277,10 +283,24 @@ extern "C" int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max
 // 166 us by cluster kernel and split-K attention, 4096: 324 / 238; rows of up to 4096 are cheap to take whole, and of up to
 // 8192 in larger groups: batch 16 at 4 K, 2048 rows 103 / 116; batch 8, 28 / 4 heads, at 8 K, 1024 rows 43 / 47), and beyond 2048
 // rows a set has several such CTAs (batch 4 at 64 K: 2048 89 / 129, 3072 130 / 140, 8192 376 / 189).
+//
+// A set for all heads of a KV head takes two launches where the one-launch step's clusters run in rounds or lie unevenly on the
+// SMs: the score stream deals tokens out whatever the lengths, and all sets are selected at once.  Batch 12, 32 / 8 heads, 24-28 K,
+// 512 rows 60 -> 49 us, on pages 61 -> 54, 3-28 K 47 -> 42 and 47.5 -> 45.4; batch 32 at 16-28 K, 256 rows 104 -> 88; batch 8 at 50-120 K,
+// 512 rows 98 -> 88; batch 16 at 4-7 K, 256 rows 33 -> 26.  Resident clusters with an SM to each CTA are faster (batch 8 at 57 K 52 / 57,
+// batch 4 at 60-120 K 47 / 53), and lists are attended by one CTA each here, which long ones do not repay: batch 32 at 28 K, 2048 rows
+// 160 / 172; on pages batch 16 at 20-56 K, 1024 rows 96 / 100; 128 sets of 96 K, 1024 rows 168 / 170.  Beyond a set to an SM a CTA has
+// half the threads: 160 sets of 44 K, 256 rows 107 / 105, 1024 118 / 127; 256 sets of 4-7 K, 64 rows 33 / 32, 256 38 / 39.
 static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, const void* workspace) {
   const fasa_config_t& c = ctx->cfg;
   const long long sets = (long long)c.batch * ctx->n_sets;
   if (workspace == nullptr || !two_launches_possible(ctx) || n_sel_max > (sets <= ctx->n_sm ? 3072 : 2048)) return false;
+  if (!set_per_head(ctx)) {
+    int most = c.page_size > 0 || c.max_len > 65536 ? 512 : 1024;
+    if (sets > ctx->n_sm && 5 * sets < 6ll * ctx->n_sm) most = 256;
+    if (sets > ctx->n_sm && c.max_len <= 8192) most = 64;
+    return n_sel_max <= most && 8ll * n_sel_max <= c.max_len && !(c.page_size == 0 && fasa_on_host(k_cache));
+  }
   if (ctx->group < 4 ? n_sel_max > 1024 : sets < 96 && n_sel_max > 512) return false;
   if (16ll * n_sel_max > c.max_len && c.max_len > (ctx->group > 4 ? 8192 : 4096)) return false;
   return !(c.page_size == 0 && fasa_on_host(k_cache));
@@ -314,8 +334,10 @@ static int32_t two_launch_step(fasa_ctx* ctx, const void* q, const void* k_new, 
   a.k_new = k_new; a.v_new = v_new; a.k_cache = k_cache; a.v_cache = v_cache;
   int32_t st = fasa_stream_launch(ctx, a, stream);
   if (st != FASA_OK) return st;
+  // (a probability keeps as many bits as on the route that this one replaces)
+  const bool full_p = fasa_full_probabilities(ctx, n_sel_max) || (!set_per_head(ctx) && !fasa_attend_separately(ctx, n_sel_max, workspace));
   return fasa_select_attend_launch(ctx, q, k_cache, v_cache, a.scores, a.maxima.gm, a.maxima.gs, seq_lens, budget, n_sel_max, idx, n_sel, out, lse,
-                                   out_mirror, k_new != nullptr, stream);
+                                   out_mirror, k_new != nullptr, full_p, stream);
 }
 
 // What fasa_fc_score, fasa_topk and fasa_sparse_decode_attn require of the arguments they share

@@ -156,7 +156,7 @@ bool fasa_select_attend_ok(const fasa_ctx* ctx, int n_sel_max) {
 
 int32_t fasa_select_attend_launch(fasa_ctx* ctx, const void* q, const void* k_cache, const void* v_cache, const float* scores,
                                   const float* gm, int gs, const int32_t* seq_lens, int32_t budget, int32_t n_sel_max,
-                                  int32_t* idx, int32_t* n_sel, float* out, float* lse, float* out_mirror, bool append,
+                                  int32_t* idx, int32_t* n_sel, float* out, float* lse, float* out_mirror, bool append, bool full_p,
                                   cudaStream_t stream) {
   const fasa_config_t& c = ctx->cfg;
   SelAttnParams p;
@@ -197,6 +197,6 @@ int32_t fasa_select_attend_launch(fasa_ctx* ctx, const void* q, const void* k_ca
     if (wide) return paged ? go(select_attend_kernel<512, true, T>, 512) : go(select_attend_kernel<512, false, T>, 512);
     return paged ? go(select_attend_kernel<256, true, T>, 256) : go(select_attend_kernel<256, false, T>, 256);
   };
-  FASA_CUDA_TRY(ctx, fasa_full_probabilities(ctx, n_sel_max) ? form(std::integral_constant<int, 3>{}) : form(std::integral_constant<int, 2>{}));
+  FASA_CUDA_TRY(ctx, full_p ? form(std::integral_constant<int, 3>{}) : form(std::integral_constant<int, 2>{}));
   return FASA_OK;
 }

@@ -40,11 +40,13 @@ constexpr int kStreamMaxTiles = 1024;          // proxy tiles of a CTA at most (
 // Tiles that a warp holds in registers (positions are finished 32 at a time), and CTAs on an SM.  About 32 KB of loads in flight
 // on an SM are enough; more CTAs with fewer tiles each beat fewer with more (batch 8, 40-65 K, 16 FCs, 5 queries: 47 us with 4
 // CTAs of two tiles a warp, 51 with 2 or 3 of four).
+// HP 0: a single row, whose heads are the rows of the product.
 template <int KB, int HP>
 struct StreamShape {
   static constexpr int tiles = KB == 1 ? 4 : (KB == 8 ? 1 : 2);
   static constexpr int step = tiles < 2 ? 2 : tiles;        // tiles per warp and iteration
   static constexpr int ctas = KB <= 2 && HP <= 2 ? 4 : 3;
+  static constexpr int pairs = HP > 0 ? HP : 1;
 };
 
 // A unit is what one pass over a KV head's proxy serves: `rows` score rows (up to 8), each the sum (or the maximum) over `heads`
@@ -94,18 +96,21 @@ __device__ __forceinline__ void mma_q_tokens(float (&c)[4], const uint4& q, uint
         : "r"(q.x), "r"(q.y), "r"(q.z), "r"(q.w), "r"(b0), "r"(b1));
 }
 
-// KB: 16-channel blocks per tile rounded up to 1, 2, 4 or 8.  HP: pairs of heads that are reduced.
+// KB: 16-channel blocks per tile rounded up to 1, 2, 4 or 8.  HP: pairs of heads that are reduced; 0: one row, whose up to eight
+// heads are rows 0-7 of the product (an eighth of the products that HP > 0 takes for a single row).  Their sum is a tree over
+// lanes in which every step also halves the tokens a lane holds: ((0 + 1) + (2 + 3)) + ((4 + 5) + (6 + 7)), as everywhere else.
 // The query's fragments are read from shared memory for each tile: in registers they cost CTAs (47 against 46 us).
 // APPEND: the sequence grows by a token first.
 template <int KB, int HP, bool PAGED, bool APPEND>
 __global__ void __launch_bounds__(kStreamThreads, StreamShape<KB, HP>::ctas)
 score_stream_kernel(const StreamParams p) {
-  constexpr int NT = StreamShape<KB, HP>::tiles, STEP = StreamShape<KB, HP>::step;
+  constexpr int NT = StreamShape<KB, HP>::tiles, STEP = StreamShape<KB, HP>::step, HQ = StreamShape<KB, HP>::pairs;
+  constexpr bool TREE = HP == 0;
   const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (known to be uniform)
   const int g = lane >> 2, t = lane & 3;
   const int u = blockIdx.y;
   const int b = u / p.n_units, hs = u - b * p.n_units, h = hs / (p.n_units / p.n_kv_heads), kv = b * p.n_kv_heads + h;
-  __shared__ __align__(16) uint32_t s_q[HP * KB][32][4];
+  __shared__ __align__(16) uint32_t s_q[HQ * KB][32][4];
   extern __shared__ uint32_t s_first[];                       // (PAGED) the pool's index of the first tile of each page
   pdl_wait_for_predecessor();
   pdl_release_successor();
@@ -148,16 +153,17 @@ score_stream_kernel(const StreamParams p) {
   }
   // The query as operand A: rows 0-7 are the rows of head 2 hp, rows 8-15 those of head 2 hp + 1.
 #pragma unroll
-  for (int n = 0; n < (KB < 2 ? (HP + 1) / 2 : HP * NW); ++n) {
+  for (int n = 0; n < (KB < 2 ? (HQ + 1) / 2 : HQ * NW); ++n) {
     const int hp = KB < 2 ? 2 * n + (tid >> 7) : n / NW, i = n % NW, kb = KB < 2 ? 0 : qkb + 2 * i;
-    const int head = 2 * hp + (qe & 1), query = ql >> 2;
+    // (TREE: up to four heads are there twice, so that a lane's first halving of its tokens needs no other lane)
+    const int head = TREE ? ((qe & 1) ? p.heads : (p.heads <= 4 ? (ql >> 2) & 3 : ql >> 2)) : 2 * hp + (qe & 1), query = TREE ? 0 : ql >> 2;
     uint32_t x = 0u;
     if (head < p.heads && query < p.rows) {
       const uint16_t* qrow = p.q + (int64_t)b * p.q_seq + hs * p.q_unit + query * p.q_row + head * FASA_HEAD_DIM;
       const int c0 = (int16_t)(chan2[i] & 0xffffu), c1 = (int16_t)(chan2[i] >> 16);
       x = (c0 >= 0 ? (uint32_t)qrow[c0] : 0u) | ((c1 >= 0 ? (uint32_t)qrow[c1] : 0u) << 16);
     }
-    if (hp < HP) s_q[hp * KB + kb][ql][qe] = x;
+    if (hp < HQ) s_q[hp * KB + kb][ql][qe] = x;
   }
   __syncthreads();
   auto tile_at = [&](int TT) -> const unsigned char* {
@@ -173,13 +179,17 @@ score_stream_kernel(const StreamParams p) {
     for (int j = 0; j < NT; ++j) load_tile<KB>(a[j], tile_at(T + j), pg, lane, (T + j) * 16 < row1);
   }
   // this lane's row, and the positions that compete there
-  const bool mine = g < p.rows;
-  const int64_t row = (int64_t)b * p.row_seq + hs * p.row_unit + (mine ? g : 0) * p.row_step;
-  float* const srow = p.scores + row * p.max_len + 2 * t;
+  const bool mine = TREE || g < p.rows;
+  const int64_t row = (int64_t)b * p.row_seq + hs * p.row_unit + (mine && !TREE ? g : 0) * p.row_step;
+  float* const srow = p.scores + row * p.max_len + (TREE ? 0 : 2 * t);
   float* const gmrow = p.gm + row * p.gm_stride;
-  const int len_q = max(0, len - (p.causal ? p.rows - 1 - g : 0)), lo = min(len_q, p.n_sink), hi = len_q - min(p.n_recent, len_q - lo);
+  const int len_q = TREE ? len : max(0, len - (p.causal ? p.rows - 1 - g : 0)), lo = min(len_q, p.n_sink), hi = len_q - min(p.n_recent, len_q - lo);
   const int all = max(0, len - (p.causal ? p.rows - 1 : 0));  // positions that every row sees
   const bool even_heads = (p.heads & 1) == 0;
+  // TREE: the octet of a pair of tiles and the position that this lane ends with
+  const bool four = p.heads <= 4, b0 = (lane & 4) != 0, b1 = (lane & 8) != 0, b2 = (lane & 16) != 0;
+  const int octet = four ? 2 * (int)b2 + (int)b0 : 2 * (int)b0 + (int)b1, mine_at = 8 * octet + 2 * t + (int)(four ? b1 : b2);
+  const bool no_head = TREE && p.max_reduce && (four ? g & 3 : g) >= p.heads;
   const bool pairs_ok = ((p.max_len & 1) == 0) && (reinterpret_cast<uintptr_t>(p.scores) & 7) == 0;
 
   // Channel pair i of the appended row, from its source: the row is scored from there (its tile's fragments take it as they are
@@ -241,9 +251,9 @@ score_stream_kernel(const StreamParams p) {
             take_new(a[j]);
             store_new();
           }
-          float c[HP][2][4];
+          float c[HQ][2][4];
 #pragma unroll
-          for (int hp = 0; hp < HP; ++hp) {
+          for (int hp = 0; hp < HQ; ++hp) {
             const uint4 qa = lds_u4(s_q[hp * KB][lane]);
             mma_q_tokens<true>(c[hp][0], qa, a[j][0].x, a[j][0].z);
             mma_q_tokens<true>(c[hp][1], qa, a[j][0].y, a[j][0].w);
@@ -252,7 +262,7 @@ score_stream_kernel(const StreamParams p) {
           for (int kb = 1; kb < KB; ++kb) {
             if (EXACT || kb < n_blocks) {
 #pragma unroll
-              for (int hp = 0; hp < HP; ++hp) {
+              for (int hp = 0; hp < HQ; ++hp) {
                 const uint4 qa = lds_u4(s_q[hp * KB + kb][lane]);
                 mma_q_tokens<false>(c[hp][0], qa, a[j][kb].x, a[j][kb].z);
                 mma_q_tokens<false>(c[hp][1], qa, a[j][kb].y, a[j][kb].w);
@@ -276,7 +286,9 @@ score_stream_kernel(const StreamParams p) {
 #pragma unroll
           for (int o = 0; o < 2; ++o) {
             float2 s;                                         // (-0 becomes +0)
-            if (p.max_reduce) {                               // uniform
+            if constexpr (TREE) {
+              s = no_head ? make_float2(-INFINITY, -INFINITY) : make_float2(c[0][o][0], c[0][o][1]);
+            } else if (p.max_reduce) {                               // uniform
               s = make_float2(c[0][o][0], c[0][o][1]);
 #pragma unroll
               for (int hp = 0; hp < HP; ++hp) {
@@ -299,6 +311,43 @@ score_stream_kernel(const StreamParams p) {
           }
         }
         const int pos = (T + 2 * jp) * 16;                    // of the pair of tiles
+        if constexpr (TREE) {
+          float s;
+          auto tree = [&](auto op) {
+            float x[2][2];                                    // [octet of the kept tile][position]
+#pragma unroll
+            for (int o = 0; o < 2; ++o)
+#pragma unroll
+              for (int i = 0; i < 2; ++i) {
+                if (four) x[o][i] = b2 ? v[2 + o][i] : v[o][i];
+                else x[o][i] = op(b0 ? v[2 + o][i] : v[o][i], __shfl_xor_sync(0xffffffffu, b0 ? v[o][i] : v[2 + o][i], 4));
+              }
+            const bool bo = four ? b0 : b1, bi = four ? b1 : b2;
+            const int lo_ = four ? 4 : 8, li = four ? 8 : 16;
+            const float y0 = op(bo ? x[1][0] : x[0][0], __shfl_xor_sync(0xffffffffu, bo ? x[0][0] : x[1][0], lo_));
+            const float y1 = op(bo ? x[1][1] : x[0][1], __shfl_xor_sync(0xffffffffu, bo ? x[0][1] : x[1][1], lo_));
+            s = op(bi ? y1 : y0, __shfl_xor_sync(0xffffffffu, bi ? y0 : y1, li));
+          };
+          if (p.max_reduce) tree([](float u, float w) { return fmaxf(u, w); });     // uniform
+          else tree([](float u, float w) { return u + w; });
+          s += 0.0f;                                          // (-0 becomes +0)
+          const int i = pos + mine_at;
+          if (i < len) srow[i] = s;
+          if (p.gs > 0) {                                     // uniform
+            float m = i >= lo && i < hi ? s : -INFINITY;
+            m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 1));
+            m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 2));
+            m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, four ? 8 : 16));
+            if (p.gs == 3) {
+              if (t == 0 && !(four ? b1 : b2)) gmrow[(pos >> 3) + octet] = m;
+            } else {
+              m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, 4));
+              m = max_nan(m, __shfl_xor_sync(0xffffffffu, m, four ? 16 : 8));
+              if (lane == 0) gmrow[pos >> 5] = m;
+            }
+          }
+          continue;
+        }
         if (mine) {
           if (pos + 32 <= all && pairs_ok) {
 #pragma unroll
@@ -400,6 +449,7 @@ int32_t fasa_stream_launch(fasa_ctx* ctx, const fasa_stream_args& a, cudaStream_
   const int nb = (ctx->chunks + 1) / 2;                // 16-channel blocks per tile, the 8-channel one included
   auto pick = [&](auto kb_tag) -> cudaError_t {
     constexpr int K = decltype(kb_tag)::value;
+    if (p.rows == 1 && a.q_len == 0 && p.heads > 1) return launch_stream<K, 0>(ctx, p, stream);
     switch ((p.heads + 1) / 2) {
       case 1: return launch_stream<K, 1>(ctx, p, stream);
       case 2: return launch_stream<K, 2>(ctx, p, stream);

@@ -27,5 +27,5 @@ int32_t fasa_stream_launch(fasa_ctx* ctx, const fasa_stream_args& a, cudaStream_
 bool fasa_select_attend_ok(const fasa_ctx* ctx, int n_sel_max);
 int32_t fasa_select_attend_launch(fasa_ctx* ctx, const void* q, const void* k_cache, const void* v_cache, const float* scores,
                                   const float* gm, int gs, const int32_t* seq_lens, int32_t budget, int32_t n_sel_max,
-                                  int32_t* idx, int32_t* n_sel, float* out, float* lse, float* out_mirror, bool append,
+                                  int32_t* idx, int32_t* n_sel, float* out, float* lse, float* out_mirror, bool append, bool full_p,
                                   cudaStream_t stream);

@@ -822,6 +822,48 @@ def test_large_selections_where_the_route_changes(kw, budget, launches):
     assert float((one[2] - r.out).abs().max()) <= 1e-4 and float((one[3] - r.lse).abs().max()) <= 1e-4
 
 
+@pytest.mark.parametrize("kw,page", [
+    (dict(batch=20, max_len=2500, len_lo=1900, len_hi=2500, budget=50, n_sink=3, n_recent=9), 0),       # more sets than SMs, four heads: half the tree
+    (dict(batch=40, n_q_heads=28, n_kv_heads=4, max_len=2051, len_lo=1, len_hi=2051, budget=60, n_dom=5, group_reduce=1), 0),  # seven heads, max, odd chunks
+    (dict(batch=52, n_q_heads=9, n_kv_heads=3, max_len=2100, len_lo=2017, len_hi=2100, budget=33, n_dom=64), 16),               # three heads, one tile in registers
+    (dict(batch=40, n_q_heads=20, n_kv_heads=4, max_len=2304, len_lo=2200, len_hi=2303, budget=64, n_dom=28), 0),               # five heads, seven chunks
+    (dict(batch=12, max_len=9472, len_lo=700, len_hi=9471, budget=300), 64),                            # a set to an SM, short rows taken whole
+])
+def test_two_launches_for_a_set_to_a_kv_head_equal_one(kw, page):
+    # steps that append: first rows of a page, a sequence that fills up; against one launch (no workspace) on a copy
+    w = C["c1"].replace(**dict(dict(n_sink=0, n_recent=0), **kw))
+    t = synth.make_inputs(w, "cpu")
+    t["seq_lens"][0] = w.max_len - 1
+    t["seq_lens"][1] = 16 * (w.len_hi // 16 - 1)
+    if page:
+        r, f, k, v, tab, table, need = _paged_twin(w, t, page, extra_tokens=2)
+    else:
+        r, f2 = Run(w, t), Run(w, {n: (x.clone() if torch.is_tensor(x) else x) for n, x in t.items()})
+        f, k, v = f2.fasa, f2.k, f2.v
+    r.build_proxy()
+    proxy, lens = f.alloc_proxy(), r.seq_lens.clone()
+    f.proxy_build(k, proxy, lens)
+    ws = f.alloc_workspace(r.n_sel_max)
+    o = [torch.full_like(x, -7) for x in (r.scores, r.idx, r.n_sel, r.out, r.lse)]
+    for step in range(2):
+        s = synth.make_step_inputs(w, step, "cuda")
+        r.scores.fill_(-7)
+        r.idx.fill_(-7)
+        r.fasa.append_decode_step(s["q"], s["k_new"], s["v_new"], r.k, r.v, r.proxy, r.seq_lens, w.budget, r.scores, r.idx, r.n_sel,
+                                  r.out, None, r.lse)
+        n0 = f.launch_count()
+        f.append_decode_step(s["q"], s["k_new"], s["v_new"], k, v, proxy, lens, w.budget, o[0], o[1], o[2], o[3], ws, o[4])
+        torch.cuda.synchronize()
+        assert f.launch_count() - n0 == 2
+        for x, y in zip((r.scores, r.idx, r.n_sel, r.seq_lens), (*o[:3], lens)):
+            assert torch.equal(x, y)
+        # (24 bits in a probability on both routes)
+        assert float((r.out - o[3]).abs().max()) <= 1e-5 and float((r.lse - o[4]).abs().max()) <= 1e-5
+        assert r.fasa.device_status() == f.device_status() == (binding.DEV_APPEND_FULL if step == 1 else 0)
+    if not page:
+        assert torch.equal(r.k, k) and torch.equal(r.v, v) and torch.equal(r.proxy, proxy)
+
+
 def test_host_step_of_two_launches_stages_its_inputs():
     # pinned buffers are read in place by a step of one launch and one wave only: both kernels of a two-launch step would
     # fetch them over the link CTA by CTA, so a kernel brings them to the staging area first
