@@ -290,7 +290,8 @@ extern "C" int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max
 // 512 rows 98 -> 88; batch 16 at 4-7 K, 256 rows 33 -> 26.  Resident clusters with an SM to each CTA are faster (batch 8 at 57 K 52 / 57,
 // batch 4 at 60-120 K 47 / 53), and lists are attended by one CTA each here, which long ones do not repay: batch 32 at 28 K, 2048 rows
 // 160 / 172; on pages batch 16 at 20-56 K, 1024 rows 96 / 100; 128 sets of 96 K, 1024 rows 168 / 170.  Beyond a set to an SM a CTA has
-// half the threads: 160 sets of 44 K, 256 rows 107 / 105, 1024 118 / 127; 256 sets of 4-7 K, 64 rows 33 / 32, 256 38 / 39.
+// half the threads: 160 sets of 44 K, 256 rows 107 / 105, 1024 118 / 127; 256 sets of 4-7 K, 64 rows 33 / 32, 256 38 / 39, on
+// pages of 16, 4-10 K, 64 rows 40 / 42.
 static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, const void* workspace) {
   const fasa_config_t& c = ctx->cfg;
   const long long sets = (long long)c.batch * ctx->n_sets;
@@ -299,6 +300,7 @@ static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, cons
     int most = c.page_size > 0 || c.max_len > 65536 ? 512 : 1024;
     if (sets > ctx->n_sm && 5 * sets < 6ll * ctx->n_sm) most = 256;
     if (sets > ctx->n_sm && c.max_len <= 8192) most = 64;
+    if (sets > ctx->n_sm && c.page_size > 0 && c.max_len < 16384) most = 0;
     return n_sel_max <= most && 8ll * n_sel_max <= c.max_len && !(c.page_size == 0 && fasa_on_host(k_cache));
   }
   if (ctx->group < 4 ? n_sel_max > 1024 : sets < 96 && n_sel_max > 512) return false;

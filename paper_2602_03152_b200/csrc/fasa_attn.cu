@@ -348,6 +348,11 @@ decode_attn_mma_kernel(const AttnParams p) {
       int ahead[kAhead];
 #pragma unroll
       for (int j = 0; j < kAhead; ++j) ahead[j] = i0 + j * kMmaThreads < r1 - r0 ? irow[r0 + i0 + j * kMmaThreads] : 0;
+      int pages[kAhead];                            // (looked up here once, not for each copy of a row's K and V)
+      if constexpr (PAGED) {
+#pragma unroll
+        for (int j = 0; j < kAhead; ++j) pages[j] = page_of(p.pm, b / p.q_len, ahead[j] < 0 || ahead[j] >= p.max_len ? 0 : ahead[j]);
+      }
 #pragma unroll
       for (int j = 0; j < kAhead; ++j) {
         const int i = i0 + j * kMmaThreads;
@@ -356,6 +361,14 @@ decode_attn_mma_kernel(const AttnParams p) {
         if (tok < 0 || tok >= p.max_len) {
           atomicOr(p.status, FASA_DEV_IDX_CLAMPED);
           tok = 0;
+        }
+        if constexpr (PAGED) {
+          int page = pages[j];
+          if (!page_ok(p.pm, page)) {
+            atomicOr(p.status, FASA_DEV_PAGE_CLAMPED);
+            page = 0;
+          }
+          tok = (page << p.pm.shift) | (tok & ((1 << p.pm.shift) - 1));
         }
         if constexpr (KSPLIT) {
           // a row that is resident on the GPU is entered as -1 - slot: it is then copied from there

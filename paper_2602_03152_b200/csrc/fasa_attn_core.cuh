@@ -125,7 +125,7 @@ __device__ __forceinline__ void attn_load_query(uint32_t (&qb)[8][2], const P& p
 }
 
 // Attention of the unit's query heads over rows [r0, r1): a warp takes 16 rows at a time.  SPARSE: row r is token
-// s_idx[r - r0] (shared memory), else token r.  bc: the sequence whose cache is read.  part(head) receives the
+// s_idx[r - r0] (shared memory; on pages that token's row of the pool), else token r.  bc: the sequence whose cache is read.  part(head) receives the
 // block's partial result (m, l, acc[128]); the threads must be synchronised before another reads it.  smem: at least
 // MmaSmem<WARPS, TERMS>; it must not be in use by anything else when the first warp arrives.  HOSTMEM: K and V rows are
 // copied through L1 (caches in page-locked host memory).  KSPLIT: Algorithm 2's Combine, see fasa_attn.cu.
@@ -158,7 +158,9 @@ __device__ __forceinline__ void attn_rows(const P& p, const SelUnit& su, int bc,
       const int tok = SPARSE ? s_idx[r - r0] : r;
       const int c8 = (lane & 15) * 8;
       // (contiguous caches keep the plain address arithmetic: the page map costs registers)
-      if constexpr (PAGED) cp_async16(&dst[row][c8], unit + cache_row(p.pm, bc, h, tok, sb, sh, st, p.status) + c8);
+      if constexpr (PAGED && SPARSE)
+        cp_async16(&dst[row][c8], unit + (tok >> p.pm.shift) * sb + h * sh + (tok & ((1 << p.pm.shift) - 1)) * st + c8);
+      else if constexpr (PAGED) cp_async16(&dst[row][c8], unit + cache_row(p.pm, bc, h, tok, sb, sh, st, p.status) + c8);
       else if constexpr (HOSTMEM) cp_async16_ca(&dst[row][c8], unit + (int64_t)tok * st + c8);
       else cp_async16(&dst[row][c8], unit + (int64_t)tok * st + c8);
     }

@@ -825,8 +825,9 @@ def test_large_selections_where_the_route_changes(kw, budget, launches):
 @pytest.mark.parametrize("kw,page", [
     (dict(batch=20, max_len=2500, len_lo=1900, len_hi=2500, budget=50, n_sink=3, n_recent=9), 0),       # more sets than SMs, four heads: half the tree
     (dict(batch=40, n_q_heads=28, n_kv_heads=4, max_len=2051, len_lo=1, len_hi=2051, budget=60, n_dom=5, group_reduce=1), 0),  # seven heads, max, odd chunks
-    (dict(batch=52, n_q_heads=9, n_kv_heads=3, max_len=2100, len_lo=2017, len_hi=2100, budget=33, n_dom=64), 16),               # three heads, one tile in registers
+    (dict(batch=52, n_q_heads=9, n_kv_heads=3, max_len=2100, len_lo=2017, len_hi=2100, budget=33, n_dom=64), 0),                # three heads, one tile in registers
     (dict(batch=40, n_q_heads=20, n_kv_heads=4, max_len=2304, len_lo=2200, len_hi=2303, budget=64, n_dom=28), 0),               # five heads, seven chunks
+    (dict(batch=24, n_q_heads=12, n_kv_heads=4, max_len=9344, len_lo=300, len_hi=9343, budget=100), 16),  # pages of one tile
     (dict(batch=12, max_len=9472, len_lo=700, len_hi=9471, budget=300), 64),                            # a set to an SM, short rows taken whole
 ])
 def test_two_launches_for_a_set_to_a_kv_head_equal_one(kw, page):
