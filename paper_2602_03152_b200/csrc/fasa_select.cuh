@@ -400,6 +400,11 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
         if (c + j < c1) f(c + j, ok[j], x[j]);
     }
   };
+  // Listed groups of 8 are visited by a thread each where they occupy 128 of 256 threads, or all of more: two 16-byte loads, eight
+  // bins kept as 16 bytes, a byte of the masks.  Against positions in chunks of 32 to a warp, 1024 rows a set: batch 4 at 30-56 K, a
+  // set per query head 51.8 -> 49.3 us a step, batch 32 at 16-31 K 122 -> 117; calibration, 512 of 8-16 K 80 -> 67.5, 128 of 12-24 K 44.5
+  // -> 42.6.  With fewer groups than threads the chunks are more parallel: 512 threads, 256 of 3-7 K 26.3 / 27.2.
+  const bool octets = gs == 3 && held && (NT == 256 ? 2 : 1) * n_list >= NT;
   SelBinning second{0.f, 0.f};
   if (listed) {
     second = sel_binning(bound, reach > bound ? reach : top);
@@ -417,11 +422,36 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
   if (!radix) {
 #pragma unroll 1
     for (int t = 0; t < kSelTries; ++t) {
-      visit([&](int c, bool ok, float x) {
-        const int bin = ok ? second.bin(x) : 0;
-        if (bin > 0) atomicAdd(&sm.hist[1][bin], 1u);
-        if (held) bins16[c * 32 + lane] = (uint16_t)bin;
-      });
+      if (octets) {
+        const bool whole = r.src.aligned();
+#pragma unroll 2
+        for (int e = tid; e < n_list; e += NT) {
+          const int p = base + ((int)list[e] << 3);
+          float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
+          const bool plain = whole && p >= r.lo && p + 8 <= r.hi;
+          if (plain) {
+            x = r.src.four(p);
+            y = r.src.four(p + 4);
+          }
+          const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+          uint32_t bin[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            bin[i] = 0u;
+            if (plain) bin[i] = (uint32_t)second.bin(v[i]);
+            else if (p + i >= r.lo && p + i < r.hi) bin[i] = (uint32_t)second.bin(r.src(p + i));
+            if (bin[i] > 0u) atomicAdd(&sm.hist[1][bin[i]], 1u);
+          }
+          *reinterpret_cast<uint4*>(bins16 + e * 8) =
+              make_uint4(bin[0] | bin[1] << 16, bin[2] | bin[3] << 16, bin[4] | bin[5] << 16, bin[6] | bin[7] << 16);
+        }
+      } else {
+        visit([&](int c, bool ok, float x) {
+          const int bin = ok ? second.bin(x) : 0;
+          if (bin > 0) atomicAdd(&sm.hist[1][bin], 1u);
+          if (held) bins16[c * 32 + lane] = (uint16_t)bin;
+        });
+      }
       __syncthreads();
       const uint32_t was = count;
       sel_find_block<NT>(sm, sm.hist[1], (uint32_t)r.k, warp, lane, &b1, &rank, &count);
@@ -452,7 +482,31 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
         }
       }
     };
-    if (held) {
+    if (octets) {
+      for (int e = tid; e < 4 * n_chunks; e += NT) {
+        uint32_t mask = 0u, equal = 0u;
+        if (e < n_list) {
+          const uint4 q = *reinterpret_cast<const uint4*>(bins16 + e * 8);
+          const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int lo = (int)(w[i] & 0xffffu), hi = (int)(w[i] >> 16);
+            mask |= (lo > b1 ? 1u : 0u) << (2 * i) | (hi > b1 ? 2u : 0u) << (2 * i);
+            equal |= (lo == b1 ? 1u : 0u) << (2 * i) | (hi == b1 ? 2u : 0u) << (2 * i);
+          }
+        }
+        reinterpret_cast<uint8_t*>(words)[e] = (uint8_t)mask;
+        while (equal) {
+          const int i = __ffs(equal) - 1;
+          equal &= equal - 1;
+          const uint32_t at = atomicAdd(&sm.n_cand, 1u);
+          if (at < (uint32_t)kSelRank) {
+            sm.cpos[at] = (uint32_t)(e * 8 + i);
+            sm.ckey[at] = fasa_order_key(r.src(base + ((int)list[e] << 3) + i));
+          }
+        }
+      }
+    } else if (held) {
 #pragma unroll 4
       for (int c = c0; c < c1; ++c) classify(c, bins16[c * 32 + lane]);
     } else {
