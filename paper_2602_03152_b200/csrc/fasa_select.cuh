@@ -223,6 +223,10 @@ struct SelScores {
   const float* p;
   __device__ __forceinline__ float operator()(int i) const { return p[i]; }
   __device__ __forceinline__ float4 four(int i) const { return *reinterpret_cast<const float4*>(p + i); }
+  __device__ __forceinline__ float max8(int i) const {              // of eight positions; i: as four wants it
+    const float4 a = four(i), b = four(i + 4);
+    return max_nan(max_nan(a.x, a.y, a.z), max_nan(a.w, b.x, b.y), max_nan(b.z, b.w));
+  }
   __device__ __forceinline__ bool aligned() const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 };
 struct SelPairs {
@@ -236,6 +240,17 @@ struct SelPairs {
   __device__ __forceinline__ float4 four(int i) const {
     const uint4 w = *reinterpret_cast<const uint4*>(p + i);
     return make_float4(score(w.x), score(w.y), score(w.z), score(w.w));
+  }
+  // Two positions to an instruction (the values are the same; a maximum needs no +0).
+  __device__ __forceinline__ float2 two(uint32_t a, uint32_t b) const {
+    const float2 x = make_float2(__uint_as_float(a << 16), __uint_as_float(b << 16));
+    const float2 y = make_float2(__uint_as_float(a & 0xffff0000u), __uint_as_float(b & 0xffff0000u));
+    return __ffma2_rn(make_float2(q0, q0), x, __fmul2_rn(make_float2(q1, q1), y));
+  }
+  __device__ __forceinline__ float max8(int i) const {
+    const uint4 a = *reinterpret_cast<const uint4*>(p + i), b = *reinterpret_cast<const uint4*>(p + i + 4);
+    const float2 s = two(a.x, a.y), t = two(a.z, a.w), u = two(b.x, b.y), v = two(b.z, b.w);
+    return max_nan(max_nan(s.x, s.y, t.x), max_nan(t.y, u.x, u.y), max_nan(v.x, v.y));
   }
   __device__ __forceinline__ bool aligned() const { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 };

@@ -61,15 +61,8 @@ __device__ __forceinline__ void topk_row(const RowParams& p, const Src& src, int
       const int i0 = w0 + lane * 8;
       float m[UNR];
       if (vec_ok && w0 >= row.lo && w0 + STEP * (UNR - 1) + 256 <= row.hi) {        // plain positions only
-        float4 v[UNR][2];
 #pragma unroll
-        for (int j = 0; j < UNR; ++j) {
-          v[j][0] = src.four(i0 + j * STEP);
-          v[j][1] = src.four(i0 + j * STEP + 4);
-        }
-#pragma unroll
-        for (int j = 0; j < UNR; ++j)
-          m[j] = max_nan(max_nan(v[j][0].x, v[j][0].y, v[j][0].z), max_nan(v[j][0].w, v[j][1].x, v[j][1].y), max_nan(v[j][1].z, v[j][1].w));
+        for (int j = 0; j < UNR; ++j) m[j] = src.max8(i0 + j * STEP);
       } else {
 #pragma unroll
         for (int j = 0; j < UNR; ++j) {
