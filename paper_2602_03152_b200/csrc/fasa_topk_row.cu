@@ -135,19 +135,31 @@ static constexpr int kTopkRowMaxLen = 524288;
 bool fasa_topk_row_ok(const fasa_ctx* ctx) { return ctx->cfg.max_len <= kTopkRowMaxLen; }
 
 // A cluster per row keeps the row's keys in shared memory and selects by their bits, whatever their distribution.  One CTA per
-// row pays for every position that it looks at again: the more, the larger the selection (8 rows: at 17 K 10.6 against 8.6
-// us at 512, 14.7 / 9.7 at 2048; at 120 K 23 / 12 and 47 / 14; 64 rows at 32 K, 4096: 29 / 15) and the more scores are
-// outliers (64 rows at 16 K, 256, one score in 500 an outlier: 18 / 14).  It is the better one for short rows and for small
-// selections of many (40 rows at 17 K: 9.2 / 10.0 at 64, 10.8 / 11.3 at 512, 13.8 / 12.0 at 1024), and when the clusters would
-// run in rounds (96 rows at 55 K: 21 / 27), unless nothing narrows a row down (96 rows at 65 K, 12387 of each: 48 / 35; 320 rows:
-// 172 / 102; 320 rows at 16 K, 2048 of each: 42 / 29): then a row held in shared memory is read once, here three times.
-static bool topk_by_clusters(const fasa_ctx* ctx, long long n_rows, int budget) {
+// row pays for every position that it looks at again: the more, the larger the selection (8 rows: at 16 K 7.6 against 8.2 us at 256,
+// 8.9 / 17.0 at 2048; at 128 K 12 / 16 and 13 / 47) and the more scores are outliers (64 rows at 16 K, 256, one score in 500 an
+// outlier: 18 / 14).  It is the better one for short rows, for small selections of many, and when the clusters have large slices
+// or run in rounds, which is what more than 32 rows beyond 32 K come to (40 rows of 64 K: 15.2 / 12.0 at 256, 15.5 / 14.9 at 1024, 15.6 /
+// 21.2 at 2048; of 128 K 27.6 / 16.4, 29.7 / 30.8, 29.6 / 47.6; 32 rows of 64 K 12.0 / 11.9, 13.8 / 14.8, 13.1 / 21.2; 64 and 72 rows of 32 K, 1024:
+// 12.9 / 14.3 and 19.8 / 14.5), unless nothing narrows a row down (96 rows at 65 K, 12387 of each: 48 / 35; 320 rows: 172 / 102; 320 rows
+// at 16 K, 2048 of each: 42 / 29): then a row held in shared memory is read once, here three times.
+// block: of a block of queries; given: the scoring pass has left the rows' maxima, which spares the pass over the row (blocks of queries, 64 rows of 120 K,
+// 128: 64 us a block by clusters, 48; 16 rows of 64 K 34.7 / 31.5; 16 K, 1024: 31.4 / 35.5; 32 rows of 120 K, 512: 43.0 / 45.8).
+static bool topk_by_clusters(const fasa_ctx* ctx, long long n_rows, int budget, bool block, bool given) {
   const fasa_config_t& c = ctx->cfg;
   const int k = budget > 0 ? budget : (int)(((long long)-budget * c.max_len + 999) / 1000);
   const bool narrowed = sel_group_shift(c.max_len, k < c.max_len ? k : c.max_len, 16386) > 0, whole = !narrowed && c.max_len > 8192;
-  const bool few = n_rows <= 16 && c.max_len >= 2048 && (c.max_len > 16384 || (k >= 128 && (narrowed || whole)));
-  const bool large = n_rows <= ctx->n_sm / 2 && c.max_len > 8192 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || c.max_len > 65536);
-  return !ctx->topk_rows && ((whole && ctx->fused_cs > 0) || ((few || large) && ctx->fused_cs > 1));
+  if (ctx->topk_rows) return false;
+  if (whole && ctx->fused_cs > 0) return true;
+  if (ctx->fused_cs <= 1) return false;
+  // up to 16, 32, 64 and 74 of 148 SMs' rows
+  const bool r16 = n_rows <= 16, r32 = 9 * n_rows <= 2ll * ctx->n_sm, r64 = 9 * n_rows <= 4ll * ctx->n_sm, r74 = 2 * n_rows <= ctx->n_sm;
+  const bool few = r16 && c.max_len >= 2048 && (c.max_len > 16384 || (k >= 128 && (narrowed || whole) && (n_rows <= 12 || c.max_len > 8192)));
+  const bool large = r32   ? c.max_len > 8192 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || (c.max_len > 65536 && k >= 128))
+                     : r64 ? c.max_len > 8192 && (k >= 2048 || (k >= 1024 && (c.max_len <= 32768 || c.max_len > 65536)))
+                           : r74 && c.max_len > 65536 && k >= 2048;
+  if (given && !(k >= 1024 && (r32 || (r74 && c.max_len <= 32768))) && !(r32 && k >= 512 && c.max_len > 65536)) return false;
+  // (a block's rows have smaller clusters of their own)
+  return few || large || (block && r74 && k >= 1024 && c.max_len > 8192 && c.max_len <= 32768);
 }
 
 // Group maxima that fit: groups of 8 up to 65536 positions, groups of 32 beyond (16 KB + 8 KB to 64 KB + 32 KB of shared memory).
@@ -158,7 +170,7 @@ static int row_maxima_cap(const fasa_ctx* ctx) {
 
 int fasa_row_maxima_shift(const fasa_ctx* ctx, int budget, long long n_rows) {
   const long long n = ctx->cfg.max_len, k = budget > 0 ? budget : ((long long)-budget * n + 999) / 1000;
-  if (!fasa_topk_row_ok(ctx) || topk_by_clusters(ctx, n_rows, budget)) return 0;
+  if (!fasa_topk_row_ok(ctx) || topk_by_clusters(ctx, n_rows, budget, true, true)) return 0;
   return sel_group_shift((int)n, (int)(k < n ? k : n), row_maxima_cap(ctx));
 }
 
@@ -166,7 +178,7 @@ int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* 
                              int32_t n_sel_max, int32_t* idx, int32_t* n_sel, int rows_per_seq, int n_sink,
                              int n_recent, cudaStream_t stream, int q_len, const fasa_calib_rows* calib, const fasa_row_maxima* given) {
   const fasa_config_t& c = ctx->cfg;
-  if (!calib && !given && topk_by_clusters(ctx, (long long)c.batch * rows_per_seq, budget))
+  if (!calib && !given && topk_by_clusters(ctx, (long long)c.batch * rows_per_seq, budget, rows_per_seq > ctx->n_sets, false))
     return fasa_topk_cluster_launch(ctx, scores, seq_lens, budget, n_sel_max, idx, n_sel, rows_per_seq, n_sink, n_recent, stream, q_len);
   RowParams p;
   p.scores = scores; p.seq_lens = seq_lens; p.idx = idx; p.n_sel = n_sel; p.status = ctx->d_status;
