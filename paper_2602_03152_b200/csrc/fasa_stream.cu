@@ -9,16 +9,21 @@
 // the next head of the sum, whose scores then meet in one thread.  The heads are reduced without a shuffle; a lane holds two
 // consecutive tokens of one row, and eight tokens' maximum is two shuffles away.  A warp goes from its loads to its stores alone.
 //
-// Measured (batch 8, 32 / 8 heads, 40-65 K, 16 FCs, T = 5): 46.4 us, 6.1 TB/s.  Before, tcgen05.mma with both operands in shared
-// memory took 71.8 us: the proxy had to be scattered into its operand layout, four warps met at a barrier for each 128 tokens,
+// The tokens of a unit are shared out to its CTAs by its length, read from the device: a batch of short sequences in long caches
+// takes as many CTAs as it has work for, and nothing is read past a length.  With shares cut from max_len, 4 K tokens of four
+// sequences in caches of 64 K lay on two or three CTAs of several iterations each, and the others read 21 MB of nothing: a step with a
+// set per head 24.4 us, now 19.2; 16 sequences of 2 K in 32 K 45.6 -> 37.8; blocks of five, 8 sequences of 4 K in 64 K 44.6 -> 34.5.
+//
+// Measured (batch 8, 32 / 8 heads, 40-65 K, 16 FCs, T = 5): 45.7 us, 5.9 TB/s.  Before, tcgen05.mma with both operands in shared
+// memory took 71.0 us: the proxy had to be scattered into its operand layout, four warps met at a barrier for each 128 tokens,
 // 250 instructions per 32 tokens and warp against 146 here.  The tensor pipe is no limit: 16 products of 8 cycles per 32 tokens
-// and scheduler, a quarter of the time that the tokens take to arrive.  At 8 FCs and five heads a set 59.8 -> 34.2 us, 32 FCs
-// 50.4 -> 40.8, 64 FCs 53.5 -> 44.6, 12 FCs (no whole blocks) 86 -> 46.7; the same bits throughout.
+// and scheduler, a quarter of the time that the tokens take to arrive.  At 8 FCs and five heads a set 59.6 -> 33.0 us, 32 FCs
+// 97.5 -> 77.4, 64 FCs 189 -> 139, 12 FCs (no whole blocks) 82.6 -> 42.1; the same bits throughout.
 //
 // A set per query head took another kernel, a persistent grid with rings of bulk copies whose every warp had an equal share, 171
 // instructions per 32 tokens and heads in columns that shuffles brought together; its SMs were busy for 31 to 50 thousand cycles.
-// The step (scoring, then selection and attention), 32 / 8 heads, batch 4, 30-56 K: 43.4 -> 40.7 us, on pages of 64 53.9 -> 41.4,
-// with 32 FCs 68.4 -> 51.5, 64 FCs and batch 2 75.4 -> 50.1; batch 16, 12-16 K 74.8 -> 68.4.
+// The step (scoring, then selection and attention), 32 / 8 heads, batch 4, 30-56 K: 42.7 -> 36.0 us, on pages of 64 53.4 -> 36.0,
+// with 32 FCs 65.2 -> 45.3, 64 FCs and batch 2 74.6 -> 44.3; batch 16, 12-16 K 74.3 -> 62.5.
 //
 // The new token's row is scored from k_new itself: the warp that owns its tile writes the K, V and proxy rows and replaces the
 // row in its fragments, so nothing waits for those writes.  The lengths themselves grow in the second half, which reads the old
@@ -59,7 +64,7 @@ struct StreamParams {
   float* scores;                // rows of max_len
   float* gm;                    // gs > 0: maxima of groups of 1 << gs positions, a row of gm_stride per score row
   int32_t* status;
-  int n_kv_heads, n_units, rows, heads, max_len, chunks, tiles_per_cta, max_reduce;      // n_units: to a sequence
+  int n_kv_heads, n_units, rows, heads, max_len, chunks, max_reduce;      // n_units: to a sequence
   int q_seq, q_unit, q_row;     // elements of q from one sequence / unit / row to the next (a head's 128 follow each other)
   int row_seq, row_unit, row_step;   // score rows likewise
   int causal;                   // row r sees rows - 1 - r fewer positions (a block of queries)
@@ -73,6 +78,13 @@ struct StreamParams {
   int64_t ksb, ksh, kst, vsb, vsh, vst;
   PageMap pm;
 };
+
+// Tiles of each of n shares of a unit with `tiles` of them: whole iterations of a CTA.
+template <int KB, int HP>
+__host__ __device__ __forceinline__ int stream_share(int tiles, int n) {
+  constexpr int kStep = kStreamWarps * StreamShape<KB, HP>::step;
+  return (((tiles + n - 1) / n) + kStep - 1) / kStep * kStep;
+}
 
 // (volatile: read where it is used, not kept in registers around the loop)
 __device__ __forceinline__ uint4 lds_u4(const void* p) {
@@ -117,17 +129,21 @@ score_stream_kernel(const StreamParams p) {
   const ProxyGeom pg = proxy_geom(p.chunks);
   const int n_blocks = pg.n16 + pg.n8;
   const int tiles_alloc = (p.max_len + 15) >> 4;
-  const int tile0 = blockIdx.x * p.tiles_per_cta, tile1 = min(tiles_alloc, tile0 + p.tiles_per_cta);
+  // The unit's tokens are shared out to the CTAs of its row of the grid as its length stands on the device: nothing is read past
+  // it, and a short sequence in a long cache takes as many CTAs as it has work for.
+  const int old_len = clamp_len(p.seq_lens[b], p.max_len, p.status);
+  const int new_row = APPEND && old_len < p.max_len ? old_len : -1, len = new_row >= 0 ? old_len + 1 : old_len;
+  const int share = stream_share<KB, HP>((len + 15) >> 4, (int)gridDim.x), tile0 = blockIdx.x * share;
+  if (tile0 * 16 >= len) return;
+  const int row1 = min(len, (tile0 + share) * 16);
   const unsigned char* unit = p.proxy + (int64_t)kv * tiles_alloc * pg.tile_bytes;
   int T = tile0 + warp * STEP;
   uint4 a[NT][KB];
-  // (every tile up to max_len is allocated: the first loads do not wait for the length)
   if constexpr (!PAGED) {
 #pragma unroll
-    for (int j = 0; j < NT; ++j) load_tile<KB>(a[j], unit + (int64_t)(T + j) * pg.tile_bytes, pg, lane, T + j < tile1);
+    for (int j = 0; j < NT; ++j) load_tile<KB>(a[j], unit + (int64_t)(T + j) * pg.tile_bytes, pg, lane, (T + j) * 16 < row1);
   }
-  // (nor do those of the channel pairs that this thread's words of the query operand take: a thread meets every second block,
-  // or the only one)
+  // the channel pairs that this thread's words of the query operand take: a thread meets every second block, or the only one
   constexpr int NW = KB < 2 ? 1 : KB / 2;
   const int qe = tid & 3, ql = (tid >> 2) & 31, qkb = KB < 2 ? 0 : tid >> 7;
   uint32_t chan2[NW];
@@ -136,10 +152,6 @@ score_stream_kernel(const StreamParams p) {
     const int w = (qkb + 2 * i) * 8 + (qe >> 1) * 4 + (ql & 3);
     chan2[i] = w < 4 * p.chunks ? *reinterpret_cast<const uint32_t*>(p.chan + (h * p.chunks * 8 + 2 * w)) : 0xffffffffu;
   }
-  const int old_len = clamp_len(p.seq_lens[b], p.max_len, p.status);
-  const int new_row = APPEND && old_len < p.max_len ? old_len : -1, len = new_row >= 0 ? old_len + 1 : old_len;
-  if (tile0 * 16 >= len) return;
-  const int row1 = min(len, tile1 * 16);
   const int sh = p.pm.shift - 4, page0 = PAGED ? tile0 >> sh : 0;
   if constexpr (PAGED) {
     for (int i = tid; i <= ((row1 - 1) >> p.pm.shift) - page0; i += kStreamThreads) {
@@ -401,16 +413,28 @@ cudaError_t launch_stream(fasa_ctx* ctx, StreamParams& p, cudaStream_t stream) {
   constexpr int kStep = kStreamWarps * StreamShape<KB, HP>::step;
   const fasa_config_t& c = ctx->cfg;
   const int units = c.batch * p.n_units, tiles = (c.max_len + 15) / 16;
-  // Ten CTAs to an SM, so that the SMs end together (they pull at different rates); but six iterations to a CTA, whose start
-  // costs one or two, as long as every SM still gets all it can hold.
-  const long long total = (long long)units * tiles, fine = total / (10ll * ctx->n_sm), one_wave = total / (StreamShape<KB, HP>::ctas * (long long)ctx->n_sm);
-  const long long want = std::max(fine, std::min(6ll * kStep, one_wave));
-  const int per = (int)std::min((long long)kStreamMaxTiles, std::max(1ll, (want + kStep - 1) / kStep) * kStep);
-  p.tiles_per_cta = per;
-  const dim3 grid((unsigned)((tiles + per - 1) / per), (unsigned)units);
+  // CTAs to a unit: as many as fit in one to eight waves, whichever a full cache is scored in soonest.  A CTA's start costs two
+  // iterations or so, and the last ones end up to a fifth of their time apart.  Measured, one wave against two, three and four: a
+  // set per head, batch 4, 30-56 K, 36.5 us a step / 37.1 / 38.9 / 39.6; batch 16, 20-30 K 92.2 / 86.7 / 86.8 / 87.3; default sets, batch
+  // 12, 40-60 K 70.0 / 66.1 / 66.9 / 68.3; batch 14, 72 K 126 / 99 / 100 / 99; batch 32, 16-28 K 86.8 / 85.4 / 85.3 / 81.7 (two CTAs to
+  // each of 256 units leave a seventh of a wave empty); blocks of three, batch 3, 84-108 K 49.1 / 52.0 / 52.8 / 55.1.
+  const int least = (tiles + kStreamMaxTiles - 1) / kStreamMaxTiles, most = (tiles + kStep - 1) / kStep;
+  const long long slots = (long long)StreamShape<KB, HP>::ctas * ctx->n_sm;
+  int n = least;
+  float best = INFINITY;
+  for (int w = 1; w <= 8; ++w) {
+    const int m = std::max(least, (int)std::min((long long)most, w * slots / units));
+    const float each = std::max(1.f, (float)tiles / (float)(m * kStep)), waves = (float)((m * (long long)units + slots - 1) / slots);
+    const float time = waves * (each + 2.f) + 0.2f * each;
+    if (time < best) {
+      best = time;
+      n = m;
+    }
+  }
+  const dim3 grid((unsigned)n, (unsigned)units);
   auto go = [&](auto kernel, size_t smem) { return launch_after_predecessor(kernel, grid, dim3(kStreamThreads), smem, stream, 0, p); };
   if (c.page_size > 0) {
-    const size_t smem = (size_t)((per >> (p.pm.shift - 4)) + 2) * 4;
+    const size_t smem = (size_t)((stream_share<KB, HP>(tiles, n) >> (p.pm.shift - 4)) + 2) * 4;
     return p.k_new ? go(score_stream_kernel<KB, HP, true, true>, smem) : go(score_stream_kernel<KB, HP, true, false>, smem);
   }
   return p.k_new ? go(score_stream_kernel<KB, HP, false, true>, 0) : go(score_stream_kernel<KB, HP, false, false>, 0);

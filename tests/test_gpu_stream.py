@@ -1,0 +1,42 @@
+"""The score stream and the selections that follow it, where the shapes of its launches change."""
+import pytest
+import torch
+
+from paper_2602_03152_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _device_us(call, n=20, reps=9):
+    """Median device time of a call among n of them, captured once."""
+    call()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(n):
+            call()
+    times = []
+    for _ in range(reps):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        graph.replay()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) / n * 1e3)
+    return sorted(times)[reps // 2]
+
+
+def test_short_sequences_in_a_long_cache_are_scored_as_in_a_short_one():
+    # What the stream takes goes by the lengths, not by max_len: 4000 tokens of 16 sequences in caches of 4096 and of
+    # 65536: 8.2 and 10.2 us.  (Shares of max_len put all of a sequence on two CTAs while the others read where nothing is: 21.3.)
+    us = {}
+    for max_len in (4096, 65536):
+        B, T, H = 16, 3, 8
+        f = binding.Fasa(B, 4 * H, H, max_len, torch.arange(16, dtype=torch.int32).repeat(H, 1))
+        proxy = f.alloc_proxy()
+        q = torch.ones((B, T, 4 * H, 128), dtype=torch.bfloat16, device="cuda")
+        lens = torch.full((B,), 4000, dtype=torch.int32, device="cuda")
+        scores = torch.empty((B, T, H, max_len), dtype=torch.float32, device="cuda")
+        us[max_len] = _device_us(lambda: f.fc_score_batched(q, proxy, lens, scores))
+        del proxy, scores
+    assert us[65536] <= 1.8 * us[4096], us
