@@ -40,3 +40,24 @@ def test_short_sequences_in_a_long_cache_are_scored_as_in_a_short_one():
         us[max_len] = _device_us(lambda: f.fc_score_batched(q, proxy, lens, scores))
         del proxy, scores
     assert us[65536] <= 1.8 * us[4096], us
+
+
+@pytest.mark.parametrize("B,H,max_len,n,launches", [
+    (34, 8, 8704, 256, 1),      # 272 clusters of one CTA, two to an SM: one round that leaves nothing to even out
+    (34, 8, 8704, 128, 2),
+    (18, 8, 17408, 512, 1),     # 144 clusters of two
+    (18, 8, 17408, 256, 2),
+    (20, 8, 8704, 512, 2),      # 160 clusters of one: some SMs with two CTAs, others with one
+    (20, 8, 8704, 1024, 1),
+    (48, 8, 4352, 512, 1),      # rounds of clusters of one
+    (48, 8, 4352, 256, 2),
+])
+def test_default_sets_take_two_launches_only_where_they_gain(B, H, max_len, n, launches):
+    f = binding.Fasa(B, 4 * H, H, max_len, torch.arange(16, dtype=torch.int32).repeat(H, 1))
+    k = torch.zeros((B, H, max_len, 128), dtype=torch.bfloat16, device="cuda")
+    q = torch.ones((B, 4 * H, 128), dtype=torch.bfloat16, device="cuda")
+    idx, n_sel = torch.empty((B, H, n), dtype=torch.int32, device="cuda"), torch.empty((B, H), dtype=torch.int32, device="cuda")
+    lens = torch.full((B,), max_len // 2, dtype=torch.int32, device="cuda")
+    n0 = f.launch_count()
+    f.decode_step(q, k, k, f.alloc_proxy(), lens, n, None, idx, n_sel, torch.empty((B, 4 * H, 128), device="cuda"), f.alloc_workspace(n))
+    assert f.launch_count() - n0 == launches
