@@ -12,22 +12,25 @@
 // The tokens of a unit are shared out to its CTAs by its length, read from the device: a batch of short sequences in long caches
 // takes as many CTAs as it has work for, and nothing is read past a length.  With shares cut from max_len, 4 K tokens of four
 // sequences in caches of 64 K lay on two or three CTAs of several iterations each, and the others read 21 MB of nothing: a step with a
-// set per head 24.4 us, now 19.2; 16 sequences of 2 K in 32 K 45.6 -> 37.8; blocks of five, 8 sequences of 4 K in 64 K 44.6 -> 34.5.
+// set per head 24.4 us, now 18.4; 16 sequences of 2 K in 32 K 45.6 -> 35.6; blocks of five, 8 sequences of 4 K in 64 K 44.6 -> 34.6.
 //
-// Measured (batch 8, 32 / 8 heads, 40-65 K, 16 FCs, T = 5): 45.7 us, 5.9 TB/s.  Before, tcgen05.mma with both operands in shared
+// Measured (batch 8, 32 / 8 heads, 40-65 K, 16 FCs, T = 5): 45.6 us, 6.0 TB/s.  Before, tcgen05.mma with both operands in shared
 // memory took 71.0 us: the proxy had to be scattered into its operand layout, four warps met at a barrier for each 128 tokens,
 // 250 instructions per 32 tokens and warp against 146 here.  The tensor pipe is no limit: 16 products of 8 cycles per 32 tokens
-// and scheduler, a quarter of the time that the tokens take to arrive.  At 8 FCs and five heads a set 59.6 -> 33.0 us, 32 FCs
-// 97.5 -> 77.4, 64 FCs 189 -> 139, 12 FCs (no whole blocks) 82.6 -> 42.1; the same bits throughout.
+// and scheduler, a quarter of the time that the tokens take to arrive.  At 8 FCs and five heads a set 59.6 -> 32.9 us, 32 FCs
+// 97.5 -> 77.4, 64 FCs 189 -> 139, 12 FCs (no whole blocks) 82.6 -> 42.2; the same bits throughout.
 //
 // A set per query head took another kernel, a persistent grid with rings of bulk copies whose every warp had an equal share, 171
 // instructions per 32 tokens and heads in columns that shuffles brought together; its SMs were busy for 31 to 50 thousand cycles.
-// The step (scoring, then selection and attention), 32 / 8 heads, batch 4, 30-56 K: 42.7 -> 36.0 us, on pages of 64 53.4 -> 36.0,
-// with 32 FCs 65.2 -> 45.3, 64 FCs and batch 2 74.6 -> 44.3; batch 16, 12-16 K 74.3 -> 62.5.
+// The step (scoring, then selection and attention), 32 / 8 heads, batch 4, 30-56 K: 42.7 -> 31.3 us, on pages of 64 53.4 -> 32.5,
+// with 32 FCs 65.2 -> 43.9, 64 FCs and batch 2 74.6 -> 41.8; batch 16, 12-16 K 74.3 -> 56.9.
 //
-// The new token's row is scored from k_new itself: the warp that owns its tile writes the K, V and proxy rows and replaces the
-// row in its fragments, so nothing waits for those writes.  The lengths themselves grow in the second half, which reads the old
-// ones before this one ends.
+// The new token's row is scored from k_new itself: the CTA whose share it ends writes the K, V and proxy rows before it streams
+// and keeps the row's channel pairs in shared memory, where the warp that owns its tile takes them for its fragments; nothing waits
+// for those writes.  (Written by that warp in its loop, the row's addresses cost 8 to 40 bytes of spills around it at 64 registers:
+// batch 4, 30-56 K, a set per head, 36.3 us a step, 31.8 without; default sets, batch 8, 60-90 K, 8 FCs 53.6, 46.4.)  What is left: 8 to 72 bytes
+// where one tile fills the registers or the sums of six and more heads do.  The lengths themselves grow in the second half, which
+// reads the old ones before this one ends.
 #include <algorithm>
 #include <type_traits>
 
@@ -123,12 +126,22 @@ score_stream_kernel(const StreamParams p) {
   const int u = blockIdx.y;
   const int b = u / p.n_units, hs = u - b * p.n_units, h = hs / (p.n_units / p.n_kv_heads), kv = b * p.n_kv_heads + h;
   __shared__ __align__(16) uint32_t s_q[HQ * KB][32][4];
+  __shared__ uint32_t s_new[APPEND ? 64 : 1];                 // the appended row's channel pairs
   extern __shared__ uint32_t s_first[];                       // (PAGED) the pool's index of the first tile of each page
   pdl_wait_for_predecessor();
   pdl_release_successor();
   const ProxyGeom pg = proxy_geom(p.chunks);
   const int n_blocks = pg.n16 + pg.n8;
   const int tiles_alloc = (p.max_len + 15) >> 4;
+  // The channel pairs that this thread's words of the query operand take: a thread meets every second block, or the only one.
+  constexpr int NW = KB < 2 ? 1 : KB / 2;
+  const int qe = tid & 3, ql = (tid >> 2) & 31, qkb = KB < 2 ? 0 : tid >> 7;
+  uint32_t chan2[NW];
+#pragma unroll
+  for (int i = 0; i < NW; ++i) {
+    const int w = (qkb + 2 * i) * 8 + (qe >> 1) * 4 + (ql & 3);
+    chan2[i] = w < 4 * p.chunks ? *reinterpret_cast<const uint32_t*>(p.chan + (h * p.chunks * 8 + 2 * w)) : 0xffffffffu;
+  }
   // The unit's tokens are shared out to the CTAs of its row of the grid as its length stands on the device: nothing is read past
   // it, and a short sequence in a long cache takes as many CTAs as it has work for.
   const int old_len = clamp_len(p.seq_lens[b], p.max_len, p.status);
@@ -143,15 +156,6 @@ score_stream_kernel(const StreamParams p) {
 #pragma unroll
     for (int j = 0; j < NT; ++j) load_tile<KB>(a[j], unit + (int64_t)(T + j) * pg.tile_bytes, pg, lane, (T + j) * 16 < row1);
   }
-  // the channel pairs that this thread's words of the query operand take: a thread meets every second block, or the only one
-  constexpr int NW = KB < 2 ? 1 : KB / 2;
-  const int qe = tid & 3, ql = (tid >> 2) & 31, qkb = KB < 2 ? 0 : tid >> 7;
-  uint32_t chan2[NW];
-#pragma unroll
-  for (int i = 0; i < NW; ++i) {
-    const int w = (qkb + 2 * i) * 8 + (qe >> 1) * 4 + (ql & 3);
-    chan2[i] = w < 4 * p.chunks ? *reinterpret_cast<const uint32_t*>(p.chan + (h * p.chunks * 8 + 2 * w)) : 0xffffffffu;
-  }
   const int sh = p.pm.shift - 4, page0 = PAGED ? tile0 >> sh : 0;
   if constexpr (PAGED) {
     for (int i = tid; i <= ((row1 - 1) >> p.pm.shift) - page0; i += kStreamThreads) {
@@ -161,6 +165,35 @@ score_stream_kernel(const StreamParams p) {
         page = 0;
       }
       s_first[i] = (uint32_t)(page * p.n_kv_heads + h) << sh;
+    }
+  }
+  // The appended row is in this CTA's share: its K, V and proxy rows (a CTA of every unit that reads this KV head writes them, the
+  // same bytes), and its channel pairs from their source for the warp that scores its tile.
+  if (APPEND && new_row >= tile0 * 16 && new_row < row1) {    // uniform
+    bool mapped = true;
+    int64_t koff = b * p.ksb + h * p.ksh + (int64_t)new_row * p.kst, voff = b * p.vsb + h * p.vsh + (int64_t)new_row * p.vst;
+    int64_t poff = (int64_t)kv * tiles_alloc * pg.tile_bytes;
+    int prow = new_row;
+    if constexpr (PAGED) {
+      const int page = page_of(p.pm, b, new_row);
+      mapped = page_ok(p.pm, page);
+      if (!mapped && tid == 0) atomicOr(p.status, FASA_DEV_PAGE_CLAMPED);
+      prow = new_row & ((1 << p.pm.shift) - 1);
+      koff = page * p.ksb + h * p.ksh + (int64_t)prow * p.kst;
+      voff = page * p.vsb + h * p.vsh + (int64_t)prow * p.vst;
+      poff = ((int64_t)page * p.n_kv_heads + h) * (1 << sh) * pg.tile_bytes;
+    }
+    if (tid < 4 * p.chunks) {
+      const uint16_t* kn = p.k_new + (int64_t)kv * FASA_HEAD_DIM;
+      const int16_t* ch = p.chan + h * p.chunks * 8;
+      const int c0 = ch[2 * tid], c1 = ch[2 * tid + 1];
+      const uint32_t x = (c0 >= 0 ? (uint32_t)kn[c0] : 0u) | ((c1 >= 0 ? (uint32_t)kn[c1] : 0u) << 16);
+      s_new[tid] = x;
+      if (mapped) *reinterpret_cast<uint32_t*>(p.proxy_w + poff + proxy_word_offset(pg, prow, tid)) = x;
+    } else if (tid >= kStreamThreads - 32 && mapped) {
+      const uint16_t* from = (lane < 16 ? p.k_new : p.v_new) + (int64_t)kv * FASA_HEAD_DIM + (lane & 15) * 8;
+      uint16_t* to = (lane < 16 ? p.k_w + koff : p.v_w + voff) + (lane & 15) * 8;
+      *reinterpret_cast<uint4*>(to) = *reinterpret_cast<const uint4*>(from);
     }
   }
   // The query as operand A: rows 0-7 are the rows of head 2 hp, rows 8-15 those of head 2 hp + 1.
@@ -204,48 +237,19 @@ score_stream_kernel(const StreamParams p) {
   const bool no_head = TREE && p.max_reduce && (four ? g & 3 : g) >= p.heads;
   const bool pairs_ok = ((p.max_len & 1) == 0) && (reinterpret_cast<uintptr_t>(p.scores) & 7) == 0;
 
-  // Channel pair i of the appended row, from its source: the row is scored from there (its tile's fragments take it as they are
-  // used), and nothing waits for the proxy row that is written here.
-  auto new_word = [&](int i) -> uint32_t {
-    const uint16_t* kn = p.k_new + (int64_t)kv * FASA_HEAD_DIM;
-    const int16_t* ch = p.chan + h * p.chunks * 8;
-    const int c0 = ch[2 * i], c1 = ch[2 * i + 1];
-    return (c0 >= 0 ? (uint32_t)kn[c0] : 0u) | ((c1 >= 0 ? (uint32_t)kn[c1] : 0u) << 16);
-  };
+  // The appended row's words in place of its tile's: nothing waits for the proxy row that is written above.
   auto take_new = [&](uint4 (&x)[KB]) {
     const int r = new_row & 15;
     if (g == (r & 7)) {
 #pragma unroll
       for (int kb = 0; kb < KB; ++kb) {
         if (kb < n_blocks) {
-          const uint32_t w0 = new_word(kb * 8 + t), w1 = kb < pg.n16 ? new_word(kb * 8 + t + 4) : 0u;
+          const uint32_t w0 = s_new[kb * 8 + t], w1 = kb < pg.n16 ? s_new[kb * 8 + t + 4] : 0u;
           if (r < 8) { x[kb].x = w0; x[kb].z = w1; }
           else { x[kb].y = w0; x[kb].w = w1; }
         }
       }
     }
-  };
-  // Its K, V and proxy rows (one warp of every unit that reads this KV head writes them, the same bytes).
-  auto store_new = [&]() {
-    int64_t koff = b * p.ksb + h * p.ksh + (int64_t)new_row * p.kst, voff = b * p.vsb + h * p.vsh + (int64_t)new_row * p.vst;
-    int64_t poff = (int64_t)kv * tiles_alloc * pg.tile_bytes;
-    int prow = new_row;
-    if constexpr (PAGED) {
-      const int page = page_of(p.pm, b, new_row);
-      if (!page_ok(p.pm, page)) {
-        if (lane == 0) atomicOr(p.status, FASA_DEV_PAGE_CLAMPED);
-        return;
-      }
-      prow = new_row & ((1 << p.pm.shift) - 1);
-      koff = page * p.ksb + h * p.ksh + (int64_t)prow * p.kst;
-      voff = page * p.vsb + h * p.vsh + (int64_t)prow * p.vst;
-      poff = ((int64_t)page * p.n_kv_heads + h) * (1 << sh) * pg.tile_bytes;
-    }
-    const uint16_t* from = (lane < 16 ? p.k_new : p.v_new) + (int64_t)kv * FASA_HEAD_DIM + (lane & 15) * 8;
-    uint16_t* to = (lane < 16 ? p.k_w + koff : p.v_w + voff) + (lane & 15) * 8;
-    *reinterpret_cast<uint4*>(to) = *reinterpret_cast<const uint4*>(from);
-    for (int i = lane; i < 4 * p.chunks; i += 32)
-      *reinterpret_cast<uint32_t*>(p.proxy_w + poff + proxy_word_offset(pg, prow, i)) = new_word(i);
   };
 
   auto stream = [&](auto exact_tag) {
@@ -259,10 +263,7 @@ score_stream_kernel(const StreamParams p) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
           const int j = (2 * jp + e) % NT;                    // (one register tile: both tiles of a pair go through it)
-          if (APPEND && T + 2 * jp + e == (new_row >> 4)) {     // (-1: none) uniform
-            take_new(a[j]);
-            store_new();
-          }
+          if (APPEND && T + 2 * jp + e == (new_row >> 4)) take_new(a[j]);     // (-1: none) uniform
           float c[HQ][2][4];
 #pragma unroll
           for (int hp = 0; hp < HQ; ++hp) {
@@ -414,7 +415,7 @@ cudaError_t launch_stream(fasa_ctx* ctx, StreamParams& p, cudaStream_t stream) {
   const fasa_config_t& c = ctx->cfg;
   const int units = c.batch * p.n_units, tiles = (c.max_len + 15) / 16;
   // CTAs to a unit: as many as fit in one to eight waves, whichever a full cache is scored in soonest.  A CTA's start costs two
-  // iterations or so, and the last ones end up to a fifth of their time apart.  Measured, one wave against two, three and four: a
+  // iterations or so, and the last ones end up to a fifth of their time apart.  Measured with the spills, one wave against two, three and four: a
   // set per head, batch 4, 30-56 K, 36.5 us a step / 37.1 / 38.9 / 39.6; batch 16, 20-30 K 92.2 / 86.7 / 86.8 / 87.3; default sets, batch
   // 12, 40-60 K 70.0 / 66.1 / 66.9 / 68.3; batch 14, 72 K 126 / 99 / 100 / 99; batch 32, 16-28 K 86.8 / 85.4 / 85.3 / 81.7 (two CTAs to
   // each of 256 units leave a seventh of a wave empty); blocks of three, batch 3, 84-108 K 49.1 / 52.0 / 52.8 / 55.1.
