@@ -286,25 +286,25 @@ extern "C" int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max
 //
 // A set for all heads of a KV head takes two launches where the one-launch step's clusters run in rounds or lie unevenly on the
 // SMs: the score stream shares every sequence's tokens out to all SMs, and all sets are selected at once.  Batch 12, 32 / 8 heads,
-// 40-60 K, 256 rows 83.5 -> 65.5 us, 4 K in caches of 64 K 40.6 -> 23.5; 3-28 K on pages of 64, 512 rows 46.7 -> 40.0; batch 32 at 16-28 K
-// 101 -> 82; batch 16 at 3-7 K 27.5 -> 26.7.  Resident clusters with an SM to each CTA are faster (batch 8 at 57 K 52 / 57, batch 4 at
-// 60-120 K 47 / 53).  The lines are drawn through 14400 pairs of both routes (60 to 600 sets, 1 to 8 heads, 4 to 64 FCs, 2 K to 128 K
+// 40-60 K, 256 rows 83.4 -> 64.2 us, 4 K in caches of 64 K 40.6 -> 22.8; 3-28 K on pages of 64, 512 rows 46.7 -> 38.0; batch 32 at 16-28 K
+// 102 -> 80; batch 16 at 3-7 K 27.3 -> 24.8.  Resident clusters with an SM to each CTA are faster (batch 8 at 57 K 52 / 57, batch 4 at
+// 60-120 K 47 / 53).  The lines are drawn through 12000 pairs of both routes (60 to 400 sets, 1 to 8 heads, 4 to 64 FCs, 2 K to 128 K
 // full and a quarter full, 64 to 1024 rows, contiguous and paged; times of one launch over times of two, mean and worst twentieth):
 //   - Clusters of one CTA end by themselves, two to an SM, and one's attention runs beside the other's stream.  Lists of up to 256
-//     repay the second launch (1.22, 1.02), of 512 where all CTAs are resident (1.14, 0.98); in rounds 512 come to 1.09, 0.93, and
-//     1024 to 1.04, 0.85 and 0.98, 0.81.
-//   - Larger ones: up to 512 rows 1.33, 1.06, and 1024 up to two sets to an SM (1.25, 1.00; beyond 1.01, 0.89).
+//     repay the second launch (1.29, 1.08), of 512 too (1.19, 1.01), of 1024 not (1.07, 0.89; in rounds 0.99, 0.86).
+//   - Larger ones: up to 512 rows 1.41, 1.12, and 1024 up to two sets to an SM (1.30, 1.06; beyond 1.04, 0.92).
 //   - A single round that fills four fifths of the SMs or more leaves little to even out, and the other route attends long lists with
-//     a CTA to a set, of half the threads beyond a set to an SM: 256 sets of 4 K in caches of 16 K, 256 rows 34.0 / 35.5; 144 of 26 K, 512
-//     rows 50 / 57.  From 256 rows and 8 K to each CTA of a cluster 1.03, 0.86; 1.20, 0.98 below.
+//     a CTA to a set, of half the threads beyond a set to an SM: from 256 rows and 8 K to each CTA of a cluster 1.08, 0.90, full caches
+//     alone 1.01, 0.87 (256 sets of 15 K, 512 rows 70 / 82; 136 of 21 K, 1024 rows 60 / 69); 1.26, 1.05 below.  Not so with large
+//     proxies (24 FCs and more 1.10, 0.97), whose stream decides.
 static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, const void* workspace) {
   const fasa_config_t& c = ctx->cfg;
   const long long sets = (long long)c.batch * ctx->n_sets;
   if (workspace == nullptr || !two_launches_possible(ctx) || n_sel_max > (sets <= ctx->n_sm ? 3072 : 2048)) return false;
   if (!set_per_head(ctx)) {
     const int cs = ctx->step_cs;
-    const bool one_round = sets <= ctx->step_resident, full = one_round && 5 * sets >= 4ll * ctx->step_resident;
-    const int most = cs == 1 ? (one_round ? 512 : 256) : (sets <= 2ll * ctx->n_sm ? 1024 : 512);
+    const bool full = sets <= ctx->step_resident && 5 * sets >= 4ll * ctx->step_resident && c.n_dom <= 20;
+    const int most = cs == 1 || sets > 2ll * ctx->n_sm ? 512 : 1024;
     if (n_sel_max > most || 8ll * n_sel_max > c.max_len || (full && n_sel_max >= 256 * cs && c.max_len > 8192 * cs)) return false;
     return !(c.page_size == 0 && fasa_on_host(k_cache));
   }

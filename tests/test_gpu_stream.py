@@ -49,8 +49,8 @@ def test_short_sequences_in_a_long_cache_are_scored_as_in_a_short_one():
     (18, 8, 17408, 256, 2),
     (20, 8, 8704, 512, 2),      # 160 clusters of one: some SMs with two CTAs, others with one
     (20, 8, 8704, 1024, 1),
-    (48, 8, 4352, 512, 1),      # rounds of clusters of one
-    (48, 8, 4352, 256, 2),
+    (48, 8, 8704, 1024, 1),     # rounds of clusters of one
+    (48, 8, 4352, 512, 2),
 ])
 def test_default_sets_take_two_launches_only_where_they_gain(B, H, max_len, n, launches):
     f = binding.Fasa(B, 4 * H, H, max_len, torch.arange(16, dtype=torch.int32).repeat(H, 1))
