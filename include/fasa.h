@@ -147,10 +147,16 @@ int32_t fasa_proxy_row_elems(int32_t n_dom);
  * n_pages * n_kv_heads * page_size * proxy_row_elems * 2 bytes for paged caches. */
 int32_t fasa_proxy_bytes(const fasa_ctx_t* ctx, size_t* out_bytes);
 
-/* Bytes of caller-provided scratch that fasa_topk, the two attention calls and
- * fasa_decode_step need for selections of at most n_sel_max tokens.  The
- * workspace must be 256-byte aligned; its contents need not be preserved
- * between calls, and two calls that overlap on the GPU need separate ones. */
+/* Bytes of caller-provided scratch that fasa_topk, the attention calls, fasa_decode_step and
+ * fasa_append_decode_step, the host-buffer step, and the batched and split-key steps need for
+ * selections of at most n_sel_max tokens.  The workspace must be 256-byte aligned; its contents
+ * need not be preserved between calls, and two calls that overlap on the GPU need separate ones.
+ * What it holds: partial results of the attention (260 bytes or so to a query head and 1000
+ * positions, and about 3 MB); 4 bytes per position (batch * n_kv_heads * max_len) for blocks of
+ * queries, or 4.5 per position and index set where a step can run as two launches (see "whole
+ * step").  The latter two are 1 % of a cache; a paged context whose pool holds less than half of
+ * batch * max_len tokens does without them, but for sets per query head, and takes the other
+ * routes. */
 int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max, size_t* out_bytes);
 
 const char* fasa_status_string(int32_t status);

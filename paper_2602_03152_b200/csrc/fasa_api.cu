@@ -235,7 +235,8 @@ fasa_split_plan fasa_plan_splits(const fasa_ctx* ctx, int n_upper, int units) {
 }
 
 // Workspace: split-K partial results, then (contexts whose steps can run as two launches) what the first half passes to the
-// second, a score row and a row of group maxima per index set.  The partial-result area is sized for the largest
+// second, a score row and a row of group maxima per index set.  A block of queries has its group maxima there before it attends:
+// 4 bytes to a position and KV head.  The partial-result area is sized for the largest
 // split count any call can use (the bound at max_len for the fewest units a launch can have, one per KV head), so
 // nothing here depends on the selection size.
 static bool set_per_head(const fasa_ctx* ctx) { return ctx->sel_heads == 1 && ctx->group > 1; }
@@ -244,11 +245,18 @@ static bool clusters_crowd(const fasa_ctx* ctx) {
   const long long units = (long long)ctx->cfg.batch * ctx->n_sets;
   return ctx->fused_cs > 0 && (units * ctx->step_cs > ctx->n_sm || units > ctx->step_resident);
 }
+// Scratch that grows with batch x max_len is for caches that do: of a page pool, those that hold half of it or more.  (Pages are there
+// to give many long sequences room that they share: 64 sequences of up to 128 K, 8 heads, in a pool of 1 M tokens would have 370 MB
+// of scratch beside 4.8 GB of cache and proxy, and have 68.)
+static bool cache_covers_max_len(const fasa_ctx* ctx) {
+  const fasa_config_t& c = ctx->cfg;
+  return c.page_size == 0 || 2ll * c.n_pages * c.page_size >= (long long)c.batch * c.max_len;
+}
 // Whether any step of this context can run as two launches (see two_launches).
 static bool two_launches_possible(const fasa_ctx* ctx) {
   if (ctx->cfg.max_len < 2048 || !fasa_select_attend_ok(ctx, 1)) return false;
   if (set_per_head(ctx)) return ctx->group >= 4 || (long long)ctx->cfg.batch * ctx->n_sets >= 192;
-  return ctx->sel_heads == ctx->group && clusters_crowd(ctx);
+  return ctx->sel_heads == ctx->group && clusters_crowd(ctx) && cache_covers_max_len(ctx);
 }
 struct fasa_ws {
   size_t scores, gm, total;
@@ -263,7 +271,7 @@ static fasa_ws ws_layout(const fasa_ctx* ctx) {
   w.gm = w.scores + fasa_align_up(rows * (size_t)c.max_len * sizeof(float), 256);
   w.total = w.gm + fasa_align_up(rows * (size_t)fasa_stream_gm_stride(ctx) * sizeof(float), 256);
   // (a block of queries keeps its group maxima here between scoring and selection, before any partial result)
-  w.total = std::max(w.total, fasa_block_maxima_bytes(ctx));
+  if (cache_covers_max_len(ctx)) w.total = std::max(w.total, fasa_block_maxima_bytes(ctx));
   return w;
 }
 extern "C" int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max, size_t* out_bytes) {

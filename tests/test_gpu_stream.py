@@ -61,3 +61,42 @@ def test_default_sets_take_two_launches_only_where_they_gain(B, H, max_len, n, l
     n0 = f.launch_count()
     f.decode_step(q, k, k, f.alloc_proxy(), lens, n, None, idx, n_sel, torch.empty((B, 4 * H, 128), device="cuda"), f.alloc_workspace(n))
     assert f.launch_count() - n0 == launches
+
+
+def test_workspace_of_a_page_pool_goes_by_what_it_holds():
+    # sequences of up to 32 K, 24 of them, in a pool of a quarter of that: partial results alone, not 4 bytes to a position
+    B, H, max_len, page, T, n = 24, 8, 32768, 64, 3, 256
+    dom = torch.arange(16, dtype=torch.int32).repeat(H, 1)
+    f = [binding.Fasa(B, 4 * H, H, max_len, dom, page_size=page, n_pages=p) for p in (B * max_len // page // 4, B * max_len // page)]
+    rows = B * H * max_len * 4
+    small, large = (x.workspace_bytes(n) for x in f)
+    assert small < 2 * B * 4 * H * 130 * 4 * (max_len // 2048) < rows and large >= rows
+    # and what it does without changes no result
+    pages = f[0].n_pages
+    g = torch.Generator(device="cuda").manual_seed(3)
+    k, v = ((0.5 * torch.randn((pages, H, page, 128), generator=g, device="cuda")).to(torch.bfloat16) for _ in range(2))
+    q = torch.randn((B, T, 4 * H, 128), generator=g, device="cuda").to(torch.bfloat16)
+    lens = torch.randint(5000, max_len // 4, (B,), generator=g, device="cuda").to(torch.int32)
+    table = torch.zeros((B, max_len // page), dtype=torch.int32, device="cuda")
+    table[:, :max_len // 4 // page] = torch.randperm(pages, generator=g, device="cuda").to(torch.int32).view(B, -1)
+    got = []
+    for x in f:
+        x.set_block_table(table)
+        proxy = x.alloc_proxy()
+        kk, vv = k, v
+        if x.n_pages > pages:
+            kk, vv = (torch.cat([y, torch.zeros((x.n_pages - pages, H, page, 128), dtype=torch.bfloat16, device="cuda")]) for y in (k, v))
+        x.proxy_build(kk, proxy, lens)
+        ws = x.alloc_workspace(n)
+        o = [torch.zeros((B, T, H, max_len), device="cuda"), torch.zeros((B, T, H, n), dtype=torch.int32, device="cuda"),
+             torch.zeros((B, T, H), dtype=torch.int32, device="cuda"), torch.zeros((B, T, 4 * H, 128), device="cuda")]
+        s = [torch.zeros((B, H, max_len), device="cuda"), torch.zeros((B, H, n), dtype=torch.int32, device="cuda"),
+             torch.zeros((B, H), dtype=torch.int32, device="cuda"), torch.zeros((B, 4 * H, 128), device="cuda")]
+        x.decode_step_batched(q, kk, vv, proxy, lens, n, *o, ws)
+        x.decode_step(q[:, 0].contiguous(), kk, vv, proxy, lens, n, *s, ws)
+        torch.cuda.synchronize()
+        assert x.device_status() == 0
+        got.append(o + s)
+        del kk, vv, proxy
+    for i, (a, b) in enumerate(zip(*got)):
+        assert torch.equal(a, b) if i % 4 < 3 else float((a - b).abs().max()) <= 1e-5
