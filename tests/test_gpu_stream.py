@@ -2,9 +2,13 @@
 import pytest
 import torch
 
-from paper_2602_03152_b200 import binding
+from paper_2602_03152_b200 import binding, synth
+
+from gpu_harness import SENTINEL, Run
 
 pytestmark = pytest.mark.gpu
+
+C = synth.CONFIGS
 
 
 def _device_us(call, n=20, reps=9):
@@ -100,3 +104,79 @@ def test_workspace_of_a_page_pool_goes_by_what_it_holds():
         del kk, vv, proxy
     for i, (a, b) in enumerate(zip(*got)):
         assert torch.equal(a, b) if i % 4 < 3 else float((a - b).abs().max()) <= 1e-5
+
+
+def _score_bounds(r, q, t, T):
+    """Scores of query t in fp64 and the sums of the products' magnitudes, [batch][kv heads][max_len]."""
+    w = r.w
+    B, H, G = w.batch, w.n_kv_heads, w.group
+    ref = torch.empty((B, H, w.max_len), dtype=torch.float64, device="cuda")
+    mag = torch.empty_like(ref)
+    c0 = r.dom.long() if w.pairing == 0 else 2 * r.dom.long()
+    chan = torch.cat([c0, c0 + (64 if w.pairing == 0 else 1)], dim=1).cuda()          # [kv heads][2 F]
+    for b in range(B):
+        for h in range(H):
+            kk = r.k[b, h][:, chan[h]].double()
+            qq = q[b, t, h * G:(h + 1) * G][:, chan[h]].double()
+            s, m = kk @ qq.T, kk.abs() @ qq.abs().T
+            ref[b, h] = s.max(1).values if w.group_reduce else s.sum(1)
+            mag[b, h] = m.max(1).values if w.group_reduce else m.sum(1)
+    return ref, mag
+
+
+# Blocks whose warps take several iterations (a share of 3 to 12), ending anywhere in one; the number of rows and max_len decide
+# the thread block of the selection that takes the stream's maxima: 1024, 512 or 256 threads.
+@pytest.mark.parametrize("kw,T,page", [
+    (dict(batch=24, n_q_heads=16, n_dom=8, max_len=4001, budget=256, n_sink=3, n_recent=13), 3, 0),    # 576 rows, misaligned: eight listed positions to a thread of 256
+    (dict(batch=24, n_q_heads=32, n_dom=16, max_len=4000, budget=100), 5, 0),                          # groups of 8, chunks of 32 at 256 threads
+    (dict(batch=24, n_q_heads=16, n_dom=16, max_len=4096, budget=300, n_sink=40), 8, 64),
+    (dict(batch=20, n_q_heads=48, n_dom=32, max_len=4000, budget=64, group_reduce=1), 2, 0),           # three pairs of heads, max
+    (dict(batch=20, n_q_heads=56, n_dom=28, max_len=4096, budget=64), 4, 16),                          # four pairs, seven chunks, pages of one tile
+    (dict(batch=20, n_q_heads=64, n_dom=64, max_len=4000, budget=3), 3, 0),                            # one tile in registers; groups of 32
+    (dict(batch=24, n_q_heads=24, n_dom=64, max_len=3999, budget=200, n_recent=70), 2, 0),             # odd group
+    (dict(batch=24, n_q_heads=8, n_dom=4, max_len=8000, budget=500, pairing=1), 2, 0),                 # one head to a set
+    (dict(batch=2, n_q_heads=16, n_kv_heads=4, n_dom=16, max_len=20003, budget=700, n_sink=5, n_recent=9), 5, 0),   # 40 rows: 1024 threads
+    (dict(batch=6, n_q_heads=28, n_kv_heads=4, n_dom=8, max_len=20000, budget=512), 6, 0),             # 144 rows
+    (dict(batch=1, n_q_heads=32, n_dom=16, max_len=66003, budget=512, n_sink=4, n_recent=64), 5, 0),   # beyond 65536: groups of 32
+    (dict(batch=5, n_q_heads=32, n_dom=16, max_len=66000, budget=800), 4, 0),                          # 160 rows
+])
+def test_blocks_whose_warps_take_several_iterations(kw, T, page):
+    base = dict(n_kv_heads=8, len_lo=kw["max_len"] // 3, len_hi=kw["max_len"], n_sink=0, n_recent=0)
+    w = C["c1"].replace(**dict(base, **kw))
+    t = synth.make_inputs(w.replace(rope=False), "cuda")
+    t["seq_lens"][0], t["seq_lens"][-1] = w.max_len, T + 1
+    r = Run(w, t)
+    f, k, v = r.fasa, r.k, r.v
+    B, Hs = w.batch, w.n_sets
+    if page:
+        n = w.max_len // page
+        f = binding.Fasa(B, w.n_q_heads, w.n_kv_heads, w.max_len, r.dom, rope_pairing=w.pairing, group_reduce=w.group_reduce,
+                         n_sink=w.n_sink, n_recent=w.n_recent, page_size=page, n_pages=B * n)
+        table = torch.randperm(B * n, generator=torch.Generator(device="cuda").manual_seed(5), device="cuda").to(torch.int32).view(B, n)
+        f.set_block_table(table)
+        pool = [torch.empty((B * n, w.n_kv_heads, page, 128), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+        for p, c in zip(pool, (r.k, r.v)):
+            p[table.reshape(-1).long()] = c.view(B, w.n_kv_heads, n, page, 128).transpose(1, 2).reshape(-1, w.n_kv_heads, page, 128)
+        k, v = pool
+    proxy = f.alloc_proxy()
+    f.proxy_build(k, proxy, r.seq_lens)
+    q = torch.stack([synth.make_step_inputs(w, i, "cuda")["q"] for i in range(T)], dim=1).contiguous()
+    scores = torch.full((B, T, Hs, w.max_len), SENTINEL, dtype=torch.float32, device="cuda")
+    o = [torch.full((B, T, Hs, r.n_sel_max), -7, dtype=torch.int32, device="cuda"), torch.full((B, T, Hs), -7, dtype=torch.int32, device="cuda"),
+         torch.full((B, T, w.n_q_heads, 128), SENTINEL, dtype=torch.float32, device="cuda")]
+    o2 = [x.clone() for x in o]
+    ws = f.alloc_workspace(r.n_sel_max)
+    f.decode_step_batched(q, k, v, proxy, r.seq_lens, w.budget, scores, *o, ws)
+    for i in range(T):
+        lens = (r.seq_lens - (T - 1 - i)).clamp(min=0)
+        seen = torch.arange(w.max_len, device="cuda") < lens.view(B, 1, 1)
+        ref, mag = _score_bounds(r, q, i, T)
+        assert torch.all((scores[:, i] == SENTINEL) == ~seen.expand(B, Hs, -1))
+        # (a sum of at most 2 F bf16 products to a head, then of the heads, each addition rounded in fp32: 136 roundings of 2^-24)
+        assert torch.all(((scores[:, i].double() - ref).abs() <= 1e-5 * mag) | ~seen)
+    # the selection without the stream's maxima, and its attention, from the same scores
+    f.topk_batched(scores, r.seq_lens, w.budget, *o2[:2])
+    f.sparse_decode_attn_batched(q, k, v, *o2[:2], o2[2], ws)
+    for x, y in zip(o, o2):
+        assert torch.equal(x, y)
+    assert f.device_status() == 0
