@@ -418,8 +418,10 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
   // Listed groups of 8 are visited by a thread each where they occupy 128 of 256 threads, or all of more: two 16-byte loads, eight
   // bins kept as 16 bytes, a byte of the masks.  Against positions in chunks of 32 to a warp, 1024 rows a set: batch 4 at 30-56 K, a
   // set per query head 51.8 -> 49.3 us a step, batch 32 at 16-31 K 122 -> 117; calibration, 512 of 8-16 K 80 -> 67.5, 128 of 12-24 K 44.5
-  // -> 42.6.  With fewer groups than threads the chunks are more parallel: 512 threads, 256 of 3-7 K 26.3 / 27.2.
-  const bool octets = gs == 3 && held && (NT == 256 ? 2 : 1) * n_list >= NT;
+  // -> 42.6.  With fewer groups than threads the chunks are more parallel: 512 threads, 256 of 3-7 K 26.3 / 27.2.  So they are for
+  // 1024 threads on rows that are not aligned, whose groups take eight loads of 4 bytes: 128 rows of 43765 after their scoring, 1024
+  // of each: 81.3 / 83.5 us in all (aligned rows of 40960 that have left the caches: 15.8 / 14.8).
+  const bool octets = gs == 3 && held && (NT == 256 ? 2 : 1) * n_list >= NT && (NT < 1024 || r.src.aligned());
   SelBinning second{0.f, 0.f};
   if (listed) {
     second = sel_binning(bound, reach > bound ? reach : top);
@@ -442,19 +444,21 @@ __device__ __forceinline__ void sel_row(const SelRow<Src>& r, int gs, Fill fill,
 #pragma unroll 2
         for (int e = tid; e < n_list; e += NT) {
           const int p = base + ((int)list[e] << 3);
-          float4 x = make_float4(0.f, 0.f, 0.f, 0.f), y = x;
-          const bool plain = whole && p >= r.lo && p + 8 <= r.hi;
-          if (plain) {
-            x = r.src.four(p);
-            y = r.src.four(p + 4);
+          // (all eight are loaded before the first is used, also where a row is not aligned: one after another, 128 rows of 43765
+          // that have left the caches cost 4 us more)
+          float v[8];
+          if (whole && p >= r.lo && p + 8 <= r.hi) {
+            const float4 x = r.src.four(p), y = r.src.four(p + 4);
+            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+            v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+          } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = p + i >= r.lo && p + i < r.hi ? r.src(p + i) : -INFINITY;
           }
-          const float v[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
           uint32_t bin[8];
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            bin[i] = 0u;
-            if (plain) bin[i] = (uint32_t)second.bin(v[i]);
-            else if (p + i >= r.lo && p + i < r.hi) bin[i] = (uint32_t)second.bin(r.src(p + i));
+            bin[i] = p + i >= r.lo && p + i < r.hi ? (uint32_t)second.bin(v[i]) : 0u;
             if (bin[i] > 0u) atomicAdd(&sm.hist[1][bin[i]], 1u);
           }
           *reinterpret_cast<uint4*>(bins16 + e * 8) =

@@ -180,3 +180,25 @@ def test_blocks_whose_warps_take_several_iterations(kw, T, page):
     for x, y in zip(o, o2):
         assert torch.equal(x, y)
     assert f.device_status() == 0
+
+
+# Where a thread takes a listed group of eight: 1024, 512 and 256 threads, rows that are aligned or not, groups that the forced
+# positions cut.
+@pytest.mark.parametrize("B,H,L,k", [(4, 8, 20003, 1500), (4, 8, 20004, 1500), (20, 8, 9001, 700), (20, 8, 9004, 700), (40, 8, 5001, 300), (40, 8, 5004, 300)])
+@pytest.mark.parametrize("n_sink,n_recent", [(0, 0), (3, 13)])
+def test_listed_groups_of_rows_that_are_not_aligned(B, H, L, k, n_sink, n_recent):
+    g = torch.Generator(device="cuda").manual_seed(L)
+    scores = torch.randn((B, H, L), generator=g, device="cuda")
+    f = binding.Fasa(B, H, H, L, torch.arange(4, dtype=torch.int32).repeat(H, 1), n_sink=n_sink, n_recent=n_recent)
+    f.set_step_mode(2)
+    lens = torch.randint(12 * k + 100, L + 1, (B,), generator=g, device="cuda").to(torch.int32)
+    lens[0], lens[1] = L, L - 1
+    n = k + n_sink + n_recent
+    idx, n_sel = torch.empty((B, H, n), dtype=torch.int32, device="cuda"), torch.empty((B, H), dtype=torch.int32, device="cuda")
+    f.topk(scores, lens, k, idx, n_sel)
+    at = torch.arange(L, device="cuda").view(1, 1, L)
+    end = lens.view(B, 1, 1)
+    forced = (at < end) & ((at < n_sink) | (at >= end - n_recent))
+    key = torch.where(at < end, torch.where(forced, torch.inf, scores), -torch.inf)
+    ref = torch.sort(torch.sort(key, dim=2, descending=True, stable=True).indices[:, :, :n], dim=2).values.to(torch.int32)
+    assert torch.equal(idx, ref) and torch.all(n_sel == n)
