@@ -135,13 +135,21 @@ static constexpr int kTopkRowMaxLen = 524288;
 bool fasa_topk_row_ok(const fasa_ctx* ctx) { return ctx->cfg.max_len <= kTopkRowMaxLen; }
 
 // A cluster per row keeps the row's keys in shared memory and selects by their bits, whatever their distribution.  One CTA per
-// row pays for every position that it looks at again: the more, the larger the selection (8 rows: at 16 K 7.6 against 8.2 us at 256,
-// 8.9 / 17.0 at 2048; at 128 K 12 / 16 and 13 / 47) and the more scores are outliers (64 rows at 16 K, 256, one score in 500 an
-// outlier: 18 / 14).  It is the better one for short rows, for small selections of many, and when the clusters have large slices
-// or run in rounds, which is what more than 32 rows beyond 32 K come to (40 rows of 64 K: 15.2 / 12.0 at 256, 15.5 / 14.9 at 1024, 15.6 /
-// 21.2 at 2048; of 128 K 27.6 / 16.4, 29.7 / 30.8, 29.6 / 47.6; 32 rows of 64 K 12.0 / 11.9, 13.8 / 14.8, 13.1 / 21.2; 64 and 72 rows of 32 K, 1024:
-// 12.9 / 14.3 and 19.8 / 14.5), unless nothing narrows a row down (96 rows at 65 K, 12387 of each: 48 / 35; 320 rows: 172 / 102; 320 rows
-// at 16 K, 2048 of each: 42 / 29): then a row held in shared memory is read once, here three times.
+// row pays for every position that it looks at again, the more, the larger the selection.  Measured (us, clusters / one CTA, budgets
+// of 64, 256, 1024, 4096):
+//   8 to 16 rows     of 12 K 7.6 / 7.3, 8.0 / 8.6, 8.4 / 13.5 (of 8 K, after their scoring, 512: 12.9 / 12.2)
+//   32 rows          of 32 K 10.2 / 9.4, 11.3 / 9.8, 11.9 / 14.3, 13.8 / 22.6; of 128 K 15.0 / 13.9, 15.7 / 16.7, 16.6 / 30.8, 17.6 / 69
+//   64 rows          of 32 K 11.7 / 9.4, 13.1 / 9.9, 12.9 / 14.4, 15.2 / 22.7; of 64 K 15 / 12, 16 / 12, 17 / 15, 18 / 31; of 128 K 29 / 14,
+//                    30 / 17, 33 / 31, 33 / 73
+//   74 rows          of 32 K 18 / 10, 19 / 10, 20 / 14, 24 / 23; of 50 K 20 / 11, 22 / 12, 23 / 14, 26 / 31; of 128 K 37 / 14, 40 / 17, 43 / 31, 44 / 73
+// Rows that are not aligned are read 4 bytes at a time by one CTA: scoring and selection of 40 rows of 50001, 256 of each, 33.2 / 34.5,
+// 1024 33.8 / 37.8; 72 of 65535, 2048: 46.2 / 48.4.
+// One CTA's bins are spread evenly over the scores, and outliers can spoil that (they are clamped into the last bin where the rest is
+// far below): one score in 500 thirty times as large, 24 to 32 rows beyond 64 K, 64 of each, 13 / 18 to 14 / 21 us; sums over seven heads
+// with outlier channels do it too (24 rows of 100 K, 64: 13.5 / 21.8), so rows of that length go to clusters although scores that are
+// spread evenly would take 14 / 13.
+// Where nothing narrows a row down (96 rows at 65 K, 12387 of each: 35 / 48 us; 320 rows: 102 / 172; 320 rows at 16 K, 2048 of each:
+// 29 / 42) a row held in shared memory is read once, here three times.
 // block: of a block of queries; given: the scoring pass has left the rows' maxima, which spares the pass over the row (blocks of queries, 64 rows of 120 K,
 // 128: 64 us a block by clusters, 48; 16 rows of 64 K 34.7 / 31.5; 16 K, 1024: 31.4 / 35.5; 32 rows of 120 K, 512: 43.0 / 45.8).
 static bool topk_by_clusters(const fasa_ctx* ctx, long long n_rows, int budget, bool block, bool given) {
@@ -153,10 +161,11 @@ static bool topk_by_clusters(const fasa_ctx* ctx, long long n_rows, int budget, 
   if (ctx->fused_cs <= 1) return false;
   // up to 16, 32, 64 and 74 of 148 SMs' rows
   const bool r16 = n_rows <= 16, r32 = 9 * n_rows <= 2ll * ctx->n_sm, r64 = 9 * n_rows <= 4ll * ctx->n_sm, r74 = 2 * n_rows <= ctx->n_sm;
+  const bool odd = (c.max_len & 3) != 0;
   const bool few = r16 && c.max_len >= 2048 && (c.max_len > 16384 || (k >= 128 && (narrowed || whole) && (n_rows <= 12 || c.max_len > 8192)));
-  const bool large = r32   ? c.max_len > 8192 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || (c.max_len > 65536 && k >= 128))
-                     : r64 ? c.max_len > 8192 && (k >= 2048 || (k >= 1024 && (c.max_len <= 32768 || c.max_len > 65536)))
-                           : r74 && c.max_len > 65536 && k >= 2048;
+  const bool large = r32   ? c.max_len > 8192 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || c.max_len > 65536)
+                     : r64 ? c.max_len > 8192 && (k >= 2048 || (k >= 1024 && (c.max_len <= 32768 || c.max_len > 65536)) || (odd && k >= 256 && c.max_len > 32768 && c.max_len <= 65536))
+                           : r74 && (c.max_len > 65536 ? k >= 2048 : c.max_len > 32768 && k >= (odd ? 2048 : 4096));
   if (given && !(k >= 1024 && (r32 || (r74 && c.max_len <= 32768))) && !(r32 && k >= 512 && c.max_len > 65536)) return false;
   // (a block's rows have smaller clusters of their own)
   return few || large || (block && r74 && k >= 1024 && c.max_len > 8192 && c.max_len <= 32768);
@@ -197,9 +206,9 @@ int32_t fasa_topk_row_launch(fasa_ctx* ctx, const float* scores, const int32_t* 
     FASA_CUDA_TRY(ctx, launch_after_predecessor(kernel, dim3((unsigned)rows), dim3((unsigned)threads), (size_t)p.lay.bytes(), stream, 0, p));
     return FASA_OK;
   };
-  // Threads: a lone row ends soonest with many, a launch of many rows issues fewest instructions with few (every
-  // warp scans the histograms) and needs all of them resident: 320 rows of 64 K took two rounds of 512 threads,
-  // 38 us, and fit in one round of 256.
+  // Threads: a row ends soonest with many where it is long, and all rows should be resident: rows of 128 K, 256 of each, 17 us with
+  // 1024 threads, 20 with 512, 30 with 256; 160 of 32 K 18 / 13 / 13; 320 of 64 K, two rounds of 512 threads 27.5, one of 256 23.9; 512 of
+  // 16 K 33 / 20 / 15.
   if (calib) return go(topk_row_kernel<256, true>, 256);
   if (given) {
     if (rows <= ctx->n_sm && c.max_len > 16384) return go(topk_row_kernel<1024, false, true>, 1024);

@@ -202,3 +202,31 @@ def test_listed_groups_of_rows_that_are_not_aligned(B, H, L, k, n_sink, n_recent
     key = torch.where(at < end, torch.where(forced, torch.inf, scores), -torch.inf)
     ref = torch.sort(torch.sort(key, dim=2, descending=True, stable=True).indices[:, :, :n], dim=2).values.to(torch.int32)
     assert torch.equal(idx, ref) and torch.all(n_sel == n)
+
+
+@pytest.mark.parametrize("rows,L,budgets", [
+    ((4, 8), 65536, (255, 256)),            # a cluster each from here on
+    ((5, 8), 50001, (255, 256)),            # where rows are not aligned
+    ((9, 8), 40001, (2047, 2048)),
+    ((4, 8), 66000, (64, 128)),
+    ((8, 8), 40000, (2047, 2048)),
+    ((9, 8), 40000, (4095, 4096)),
+    ((9, 8), 66000, (2047, 2048)),
+])
+@pytest.mark.parametrize("outliers", [0, 1])
+def test_topk_where_the_route_of_its_rows_changes(rows, L, budgets, outliers):
+    B, H = rows
+    g = torch.Generator(device="cuda").manual_seed(L + B)
+    scores = torch.randn((B, H, L), generator=g, device="cuda")
+    if outliers:                            # one in 500 far above the others
+        scores[torch.rand(scores.shape, generator=g, device="cuda") < 0.002] *= 30
+    f = binding.Fasa(B, H, H, L, torch.arange(4, dtype=torch.int32).repeat(H, 1))
+    lens = torch.full((B,), L, dtype=torch.int32, device="cuda")
+    order = torch.sort(scores, dim=2, descending=True, stable=True).indices
+    for k in budgets:
+        ref = torch.sort(order[:, :, :k], dim=2).values.to(torch.int32)
+        for mode in (1, 2):
+            f.set_step_mode(mode)
+            idx, n_sel = torch.empty((B, H, k), dtype=torch.int32, device="cuda"), torch.empty((B, H), dtype=torch.int32, device="cuda")
+            f.topk(scores, lens, k, idx, n_sel)
+            assert torch.equal(idx, ref) and torch.all(n_sel == k)
