@@ -439,9 +439,13 @@ cudaError_t launch_stream(fasa_ctx* ctx, StreamParams& p, cudaStream_t stream) {
   auto go = [&](auto kernel, size_t smem) { return launch_after_predecessor(kernel, grid, dim3(kStreamThreads), smem, stream, 0, p); };
   if (c.page_size > 0) {
     const size_t smem = (size_t)((stream_share<KB, HP>(tiles, n) >> (p.pm.shift - 4)) + 2) * 4;
-    return p.k_new ? go(score_stream_kernel<KB, HP, true, true>, smem) : go(score_stream_kernel<KB, HP, true, false>, smem);
+    if constexpr (HP <= 1)
+      if (p.k_new) return go(score_stream_kernel<KB, HP, true, true>, smem);
+    return go(score_stream_kernel<KB, HP, true, false>, smem);
   }
-  return p.k_new ? go(score_stream_kernel<KB, HP, false, true>, 0) : go(score_stream_kernel<KB, HP, false, false>, 0);
+  if constexpr (HP <= 1)                             // (a step appends: sets of one row, or of one head)
+    if (p.k_new) return go(score_stream_kernel<KB, HP, false, true>, 0);
+  return go(score_stream_kernel<KB, HP, false, false>, 0);
 }
 
 }  // namespace
