@@ -143,7 +143,7 @@ bool fasa_topk_row_ok(const fasa_ctx* ctx) { return ctx->cfg.max_len <= kTopkRow
 //                    30 / 17, 33 / 31, 33 / 73
 //   74 rows          of 32 K 18 / 10, 19 / 10, 20 / 14, 24 / 23; of 50 K 20 / 11, 22 / 12, 23 / 14, 26 / 31; of 128 K 37 / 14, 40 / 17, 43 / 31, 44 / 73
 // Rows that are not aligned are read 4 bytes at a time by one CTA: scoring and selection of 40 rows of 50001, 256 of each, 33.2 / 34.5,
-// 1024 33.8 / 37.8; 72 of 65535, 2048: 46.2 / 48.4.
+// 1024 33.8 / 37.8; 48 of 119943, 512, with its attention 63.5 / 69.8; 72 of 65535, 2048: 46.2 / 48.4.
 // One CTA's bins are spread evenly over the scores, and outliers can spoil that (they are clamped into the last bin where the rest is
 // far below): one score in 500 thirty times as large, 24 to 32 rows beyond 64 K, 64 of each, 13 / 18 to 14 / 21 us; sums over seven heads
 // with outlier channels do it too (24 rows of 100 K, 64: 13.5 / 21.8), so rows of that length go to clusters although scores that are
@@ -164,7 +164,7 @@ static bool topk_by_clusters(const fasa_ctx* ctx, long long n_rows, int budget, 
   const bool odd = (c.max_len & 3) != 0;
   const bool few = r16 && c.max_len >= 2048 && (c.max_len > 16384 || (k >= 128 && (narrowed || whole) && (n_rows <= 12 || c.max_len > 8192)));
   const bool large = r32   ? c.max_len > 8192 && (k >= 1024 || (c.max_len > 32768 && k >= 256) || c.max_len > 65536)
-                     : r64 ? c.max_len > 8192 && (k >= 2048 || (k >= 1024 && (c.max_len <= 32768 || c.max_len > 65536)) || (odd && k >= 256 && c.max_len > 32768 && c.max_len <= 65536))
+                     : r64 ? c.max_len > 8192 && (k >= 2048 || (k >= 1024 && (c.max_len <= 32768 || c.max_len > 65536)) || (odd && k >= 256 && c.max_len > 32768))
                            : r74 && (c.max_len > 65536 ? k >= 2048 : c.max_len > 32768 && k >= (odd ? 2048 : 4096));
   if (given && !(k >= 1024 && (r32 || (r74 && c.max_len <= 32768))) && !(r32 && k >= 512 && c.max_len > 65536)) return false;
   // (a block's rows have smaller clusters of their own)
