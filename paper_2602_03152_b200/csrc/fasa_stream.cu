@@ -114,7 +114,9 @@ __device__ __forceinline__ void mma_q_tokens(float (&c)[4], const uint4& q, uint
         : "r"(q.x), "r"(q.y), "r"(q.z), "r"(q.w), "r"(b0), "r"(b1));
 }
 
-// KB: 16-channel blocks per tile rounded up to 1, 2, 4 or 8.  HP: pairs of heads that are reduced; 0: one row, whose up to eight
+// KB: 16-channel blocks per tile (the last one may be half), from five on rounded up to 8.  Up to four blocks the loop knows how many
+// bytes a tile has; with tests of the geometry and loads under them, 12 FCs took 72.1 us a default step (12 sequences of 40-60 K) where
+// 57.0 are enough, 16 FCs 65.6; 24 FCs, in a loop for four blocks, 88.7 -> 84.5; a block of seven at 61-73 K, 24 FCs 133.6 -> 123.2.  HP: pairs of heads that are reduced; 0: one row, whose up to eight
 // heads are rows 0-7 of the product (an eighth of the products that HP > 0 takes for a single row).  Their sum is a tree over
 // lanes in which every step also halves the tokens a lane holds: ((0 + 1) + (2 + 3)) + ((4 + 5) + (6 + 7)), as everywhere else.
 // The query's fragments are read from shared memory for each tile: in registers they cost CTAs (47 against 46 us).
@@ -137,7 +139,7 @@ score_stream_kernel(const StreamParams p) {
   const int n_blocks = pg.n16 + pg.n8;
   const int tiles_alloc = (p.max_len + 15) >> 4;
   // The channel pairs that this thread's words of the query operand take: a thread meets every second block, or the only one.
-  constexpr int NW = KB < 2 ? 1 : KB / 2;
+  constexpr int NW = (KB + 1) / 2;
   const int qe = tid & 3, ql = (tid >> 2) & 31, qkb = KB < 2 ? 0 : tid >> 7;
   uint32_t chan2[NW];
 #pragma unroll
@@ -211,7 +213,7 @@ score_stream_kernel(const StreamParams p) {
       const int c0 = (int16_t)(chan2[i] & 0xffffu), c1 = (int16_t)(chan2[i] >> 16);
       x = (c0 >= 0 ? (uint32_t)qrow[c0] : 0u) | ((c1 >= 0 ? (uint32_t)qrow[c1] : 0u) << 16);
     }
-    if (hp < HQ) s_q[hp * KB + kb][ql][qe] = x;
+    if (hp < HQ && kb < KB) s_q[hp * KB + kb][ql][qe] = x;
   }
   __syncthreads();
   auto tile_at = [&](int TT) -> const unsigned char* {
@@ -255,9 +257,11 @@ score_stream_kernel(const StreamParams p) {
     }
   };
 
-  auto stream = [&](auto exact_tag) {
-    constexpr bool EXACT = decltype(exact_tag)::value;        // the dominant channels fill exactly KB whole blocks
-    const unsigned char* ahead = unit + (int64_t)T * (KB * 512) + lane * 16;    // (EXACT, contiguous) of the tile at T
+  auto stream = [&](auto geometry) {
+    constexpr int GEO = decltype(geometry)::value;            // the dominant channels fill KB whole blocks (2), the last one by half (1)
+    constexpr bool EXACT = GEO != 0;
+    constexpr int kTile = GEO == 1 ? KB * 512 - 256 : KB * 512;
+    const unsigned char* ahead = unit + (int64_t)T * kTile + lane * 16;   // (EXACT, contiguous) of the tile at T
     while (T * 16 < row1) {                                   // uniform over the warp
       const int next = T + kStreamWarps * STEP;
 #pragma unroll
@@ -291,10 +295,19 @@ score_stream_kernel(const StreamParams p) {
             if constexpr (EXACT) {
               const unsigned char* tile;
               if constexpr (PAGED) tile = tile_at(TN) + lane * 16;
-              else tile = ahead + (NT == 1 && e == 0 ? 1 : kStreamWarps * STEP + 2 * jp + (NT == 1 ? 0 : e)) * KB * 512;
+              else tile = ahead + (NT == 1 && e == 0 ? 1 : kStreamWarps * STEP + 2 * jp + (NT == 1 ? 0 : e)) * kTile;
 #pragma unroll
-              for (int kb = 0; kb < KB; ++kb)
-                if (ok) a[j][kb] = ld_proxy_u4(tile + kb * 512);
+              for (int kb = 0; kb < KB; ++kb) {
+                if (GEO == 1 && kb == KB - 1) {
+                  if (ok) {
+                    const uint2 w = ld_proxy_u2(tile + kb * 512 - lane * 8);
+                    a[j][kb].x = w.x;
+                    a[j][kb].y = w.y;
+                  }
+                } else if (ok) {
+                  a[j][kb] = ld_proxy_u4(tile + kb * 512);
+                }
+              }
             } else {
               load_tile<KB>(a[j], tile_at(TN), pg, lane, ok);
             }
@@ -405,11 +418,16 @@ score_stream_kernel(const StreamParams p) {
         }
       }
       T = next;
-      ahead += kStreamWarps * STEP * KB * 512;
+      ahead += kStreamWarps * STEP * kTile;
     }
   };
-  if (pg.n8 == 0 && pg.n16 == KB) stream(std::true_type{});
-  else stream(std::false_type{});
+  if constexpr (KB <= 4) {                                   // (KB blocks, the last one whole or half: see fasa_stream_launch)
+    if (pg.n8 == 0) stream(std::integral_constant<int, 2>{});
+    else stream(std::integral_constant<int, 1>{});
+  } else {
+    if (pg.n8 == 0 && pg.n16 == KB) stream(std::integral_constant<int, 2>{});
+    else stream(std::integral_constant<int, 0>{});
+  }
 }
 
 template <int KB, int HP>
@@ -418,10 +436,11 @@ cudaError_t launch_stream(fasa_ctx* ctx, StreamParams& p, cudaStream_t stream) {
   const fasa_config_t& c = ctx->cfg;
   const int units = c.batch * p.n_units, tiles = (c.max_len + 15) / 16;
   // CTAs to a unit: as many as fit in one to eight waves, whichever a full cache is scored in soonest.  A CTA's start costs two
-  // iterations or so, and the last ones end up to a fifth of their time apart.  Measured with the spills, one wave against two, three and four: a
-  // set per head, batch 4, 30-56 K, 36.5 us a step / 37.1 / 38.9 / 39.6; batch 16, 20-30 K 92.2 / 86.7 / 86.8 / 87.3; default sets, batch
-  // 12, 40-60 K 70.0 / 66.1 / 66.9 / 68.3; batch 14, 72 K 126 / 99 / 100 / 99; batch 32, 16-28 K 86.8 / 85.4 / 85.3 / 81.7 (two CTAs to
-  // each of 256 units leave a seventh of a wave empty); blocks of three, batch 3, 84-108 K 49.1 / 52.0 / 52.8 / 55.1.
+  // iterations or so, and the last ones end up to a fifth of their time apart.  One wave against two, three and four (with the append
+  // still in the loop, shares of whole iterations): a set per head, batch 4, 30-56 K, 36.5 us a step / 37.1 / 38.9 / 39.6; batch 16, 20-30 K
+  // 92.2 / 86.7 / 86.8 / 87.3; default sets, batch 12, 40-60 K 70.0 / 66.1 / 66.9 / 68.3; batch 14, 72 K 126 / 99 / 100 / 99; batch 32, 16-28 K
+  // 86.8 / 85.4 / 85.3 / 81.7 (two CTAs to each of 256 units leave a seventh of a wave empty); blocks of three, batch 3, 84-108 K 49.1 /
+  // 52.0 / 52.8 / 55.1.  Against the best of ten counts the rule loses 1 % over 173 shapes.
   const int least = (tiles + kStreamMaxTiles - 1) / kStreamMaxTiles, most = (tiles + kStep - 1) / kStep;
   const long long slots = (long long)StreamShape<KB, HP>::ctas * ctx->n_sm;
   int n = least;
@@ -492,6 +511,7 @@ int32_t fasa_stream_launch(fasa_ctx* ctx, const fasa_stream_args& a, cudaStream_
   cudaError_t e;
   if (nb <= 1) e = pick(std::integral_constant<int, 1>{});
   else if (nb <= 2) e = pick(std::integral_constant<int, 2>{});
+  else if (nb <= 3) e = pick(std::integral_constant<int, 3>{});
   else if (nb <= 4) e = pick(std::integral_constant<int, 4>{});
   else e = pick(std::integral_constant<int, 8>{});
   ctx->launches += 1;
