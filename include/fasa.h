@@ -283,9 +283,17 @@ int32_t fasa_sparse_decode_attn_static(fasa_ctx_t* ctx, const void* q, const voi
  *     four stand alone on their SMs, for 1024 rows or more (64 to 1023 on long slices in the former case);
  *   - for large selections (from 1024 or 2048 rows) of sets that share a KV head, whose rows come from L2;
  *   - for at most 8 units with max_len <= 8192 once n_sel_max * ceil(heads per set / 4) >= 2048.
- * A set per query head (select_heads = 1) with a workspace, rows of at least 2048 positions, many sets and selections of
- * up to a sixteenth of the context (short rows: up to 2048) runs as two launches instead: one stream of the proxy that
- * scores all heads of a KV head, then selection and attention.
+ * With a workspace and max_len from 2048 to 262144 a step may run as two launches of another kind, one stream of the proxy that
+ * scores (and appends) and one kernel that selects and attends:
+ *   - a set per query head (select_heads = 1): many sets and selections of up to a sixteenth of the context (short rows: up
+ *     to 2048);
+ *   - a set for all heads of a KV head: where the cluster kernel's CTAs run in rounds or lie unevenly on the SMs, for n_sel_max
+ *     of up to 512 (clusters of one CTA, or more than two sets to an SM) or 1024, of up to 24 * (index sets of the batch - 8),
+ *     and of up to an eighth of max_len; not where a
+ *     single round fills four fifths of the SMs and lists are long (256 rows and 8192 positions to each CTA of a cluster and
+ *     more, up to 20 dominant FCs), not for caches in host memory, and not for page pools that hold less than half of
+ *     batch * max_len tokens.
+ * fasa_launch_count tells the launches of a call.
  * Mode 0, and every configuration mode 1 cannot take: fasa_fc_score -> fasa_topk ->
  * fasa_sparse_decode_attn; scores and workspace are then required (INVALID_ARG if NULL).
  * Both modes select identical index sets; outputs agree to fp32 rounding, or to 17 bits of each probability where a long
@@ -309,8 +317,8 @@ int32_t fasa_decode_step(fasa_ctx_t* ctx, const void* q, const void* k_cache,
 /* Algorithm 2's order for one new token per sequence: UpdateCache (K, V and the dominant
  * part of the key cache), then the step above on the grown cache; seq_lens[b] += 1 on the
  * device.  k_new, v_new: bf16 [batch][n_kv_heads][1][128], post-RoPE, 16-byte aligned.
- * In mode 1 the append happens inside the same kernel (the CTA whose slice ends the
- * sequence writes the three rows before it scores them), so the whole step is one launch;
+ * In mode 1 the append happens inside the step's first kernel (the CTA whose slice ends the
+ * sequence writes the three rows), so it costs no launch of its own;
  * otherwise it is fasa_kv_append followed by fasa_decode_step.  A full cache drops the
  * token and sets FASA_DEV_APPEND_FULL, as fasa_kv_append does. */
 int32_t fasa_append_decode_step(fasa_ctx_t* ctx, const void* q, const void* k_new,
@@ -446,9 +454,8 @@ int32_t fasa_m_resident_build(fasa_ctx_t* ctx, const void* k_nondom, const void*
  * them in place, across the host link; otherwise one small kernel brings them to the device
  * staging area dev_stage (>= fasa_stage_bytes) first.  Pageable inputs are copied there with
  * three asynchronous copies.  A pinned out_host is written by the step's last kernel itself.
- * The context remembers what the driver said about the last four host pointers it saw, so a
- * loop that passes the same buffers asks once; a buffer must therefore not change its kind
- * (pageable / page-locked) while keeping its address between two calls. */
+ * The driver is asked about each host pointer in every call: a buffer may change its kind
+ * (pageable / page-locked) between two calls. */
 int32_t fasa_stage_bytes(const fasa_ctx_t* ctx, size_t* out_bytes);
 int32_t fasa_decode_step_host(fasa_ctx_t* ctx, const void* q_host, const void* k_new_host,
                               const void* v_new_host, void* dev_stage, void* k_cache,

@@ -301,6 +301,9 @@ extern "C" int32_t fasa_workspace_bytes(const fasa_ctx_t* ctx, int32_t n_sel_max
 //   - Clusters of one CTA end by themselves, two to an SM, and one's attention runs beside the other's stream.  Lists of up to 256
 //     repay the second launch (1.29, 1.08), of 512 too (1.19, 1.01), of 1024 not (1.07, 0.89; in rounds 0.99, 0.86).
 //   - Larger ones: up to 512 rows 1.41, 1.12, and 1024 up to two sets to an SM (1.30, 1.06; beyond 1.04, 0.92).
+//   - Few sets (long rows, whose clusters of eight run in rounds) leave SMs idle while each CTA selects a whole row for itself: 16 sets,
+//     128 rows 1.54, 1.33, 256 1.10, 0.90, 512 0.94, 0.73; 24 sets, 256 rows 1.34, 1.15, 512 1.18, 1.05, 1024 0.90, 0.81; 40 sets, 1024 rows
+//     1.24, 0.94; 48 sets 1.26, 1.03 (3800 pairs of 16 to 72 sets).
 //   - A single round that fills four fifths of the SMs or more leaves little to even out, and the other route attends long lists with
 //     a CTA to a set, of half the threads beyond a set to an SM: from 256 rows and 8 K to each CTA of a cluster 1.08, 0.90, full caches
 //     alone 1.01, 0.87 (256 sets of 15 K, 512 rows 70 / 82; 136 of 21 K, 1024 rows 60 / 69); 1.26, 1.05 below.  Not so with large
@@ -312,7 +315,7 @@ static bool two_launches(fasa_ctx* ctx, const void* k_cache, int n_sel_max, cons
   if (!set_per_head(ctx)) {
     const int cs = ctx->step_cs;
     const bool full = sets <= ctx->step_resident && 5 * sets >= 4ll * ctx->step_resident && c.n_dom <= 20;
-    const int most = cs == 1 || sets > 2ll * ctx->n_sm ? 512 : 1024;
+    const long long most = std::min(cs == 1 || sets > 2ll * ctx->n_sm ? 512ll : 1024ll, 24 * (sets - 8));
     if (n_sel_max > most || 8ll * n_sel_max > c.max_len || (full && n_sel_max >= 256 * cs && c.max_len > 8192 * cs)) return false;
     return !(c.page_size == 0 && fasa_on_host(k_cache));
   }

@@ -204,10 +204,33 @@ def test_listed_groups_of_rows_that_are_not_aligned(B, H, L, k, n_sink, n_recent
     assert torch.equal(idx, ref) and torch.all(n_sel == n)
 
 
+def test_few_sets_of_long_rows_leave_the_selection_to_clusters():
+    # 16 sets of 35 K in caches of 142 K, 512 of each: a step that selects whole rows with one CTA each takes 55 us, the cluster
+    # kernel's selection and the attention of its lists 39
+    B, H, max_len, n = 2, 8, 142710, 512
+    g = torch.Generator(device="cuda").manual_seed(9)
+    f = binding.Fasa(B, 4 * H, H, max_len, torch.arange(8, dtype=torch.int32).repeat(H, 1))
+    k, v = (torch.randn((B, H, max_len, 128), generator=g, device="cuda", dtype=torch.bfloat16) for _ in range(2))
+    q = torch.randn((B, 4 * H, 128), generator=g, device="cuda", dtype=torch.bfloat16)
+    lens = torch.tensor([35000, 34000], dtype=torch.int32, device="cuda")
+    proxy, ws = f.alloc_proxy(), f.alloc_workspace(n)
+    f.proxy_build(k, proxy, lens)
+    idx, n_sel = torch.empty((B, H, n), dtype=torch.int32, device="cuda"), torch.empty((B, H), dtype=torch.int32, device="cuda")
+    out = torch.empty((B, 4 * H, 128), device="cuda")
+    step = _device_us(lambda: f.decode_step(q, k, v, proxy, lens, n, None, idx, n_sel, out, ws))
+
+    def apart():
+        f.select_step(q, k, v, proxy, lens, n, None, idx, n_sel)
+        f.sparse_decode_attn(q, k, v, idx, n_sel, out, ws)
+    apart = _device_us(apart)
+    assert step <= 1.1 * apart, (step, apart)
+
+
 @pytest.mark.parametrize("rows,L,budgets", [
     ((4, 8), 65536, (255, 256)),            # a cluster each from here on
     ((5, 8), 50001, (255, 256)),            # where rows are not aligned
     ((9, 8), 40001, (2047, 2048)),
+    ((6, 8), 66001, (255, 256)),
     ((4, 8), 66000, (64, 128)),
     ((8, 8), 40000, (2047, 2048)),
     ((9, 8), 40000, (4095, 4096)),
