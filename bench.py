@@ -7,8 +7,8 @@ One step = one pass of the whole hot path over one batch: append one token per s
 (K, V and proxy-K rows), score every cached key on the dominant FCs, select the top-budget
 tokens, run exact attention over the selected rows and merge the splits.  The step is one
 call, fasa_append_decode_step (one cluster kernel: append -> score -> select -> attention, or
-that kernel ending after the selection + the split-K attention kernels where the selection is
-large); the stand-alone calls (fasa_kv_append, fasa_fc_score, fasa_topk,
+two: that kernel ending after the selection + the split-K attention, or a stream of the proxy
+that scores + a kernel that selects and attends); the stand-alone calls (fasa_kv_append, fasa_fc_score, fasa_topk,
 fasa_sparse_decode_attn) and the dense path are timed beside it.  The headline workload is
 the largest single-GPU configuration (c2: batch 16, 64K-128K contexts, 8 GiB of K/V); the
 smaller configurations ride along under `other_workloads`, and the budget row of
@@ -18,10 +18,9 @@ line.
 
 Headline metric: effective HBM GB/s = algorithmic bytes of the step (proxy bytes of every
 cached token + K/V rows of the selected tokens + q + out) / device time, summed over ranks;
-`us_per_step`, the dense-path time and the speedup ride along.  `roofline` describes the
-dominant kernel (the cluster kernel: the whole step where it is one launch, scoring +
-selection where attention is handed to the split-K kernel), `kernels` the three calls the
-method names, `cpu_baseline` the fp64 oracle timed on the host, `parity` one unit of the timed
+`us_per_step`, the dense-path time and the speedup ride along.  `roofline` describes the whole
+step, of one launch or two (`select_step` beside it: scoring and selection alone, by the cluster
+kernel in one launch), `kernels` the three calls the method names, `cpu_baseline` the fp64 oracle timed on the host, `parity` one unit of the timed
 configuration checked against that oracle.
 """
 from __future__ import annotations
@@ -314,7 +313,7 @@ def measure(w, K, W, dev, world, step_mode=None, sampler_factory=None, want_e2e=
     by = step_bytes(w, lens_full.cpu().tolist(), n_sel_total)
     Kk = min(K, 200)
 
-    # ---- the dominant kernel alone, where the step is several launches --------------------
+    # ---- scoring and selection alone, where the step is several launches ------------------
     launches_per_step = launches / max(K, 1)
     select_us = None
     if fused and launches_per_step > 1:
@@ -400,7 +399,7 @@ def summarize(m, peak):
         "n_sel_per_unit": m["n_sel_total"] / (w.batch * w.n_sets), "heads_per_index_set": w.heads_per_set,
         "step_mode": ("three kernels" if not m["fused"] else
                       f"one cluster kernel (cluster of {m['cluster_size']})" if m["launches_per_step"] == 1 else
-                      f"cluster kernel (cluster of {m['cluster_size']}, ends after the selection) + split-K tensor-core attention + merge"),
+                      "several launches: scoring (and selection), then (selection and) attention"),
         "launches_per_step": m["launches_per_step"],
         "us_per_step": m["us_per_step"], "us_per_step_median": m["step_us_median"], "step_bytes": by["fasa"],
         "step_gbs": gbs(by["fasa"], m["us_per_step"]), "step_frac_of_peak": gbs(by["fasa"], m["us_per_step"]) / peak,
@@ -495,15 +494,15 @@ def run_fasa(args, w):
                     "bytes_per_launch": by["fasa"], "us_per_launch": us_per_step, "peak_source": peak_src,
                     "cluster_size": m["cluster_size"]}
     elif m["fused"]:
-        # dominant kernel = the cluster kernel ending after the selection (append + scoring + selection
-        # in one launch): it moves the proxy rows of every token, q and the index lists it writes
+        # several kernels: the library picks them (cluster kernel and split-K attention, or score stream and
+        # select-and-attend), so the figure is the whole step's; the cluster kernel ending after the selection moves
+        # the proxy rows of every token, q and the index lists it writes
         kb = by["proxy"] + by["qo"] // 3 + 4 * m["n_sel_total"]
-        us = m["select_us"]
-        tr, tr_src = _traffic(kb, wl.name)
-        roofline = {"kernel": "fused_decode_kernel (append + scoring + selection)", "bound": "hbm",
-                    "achieved": kb / us / 1e3, "peak": peak, "unit": "GB/s", "frac": kb / us / 1e3 / peak,
-                    "traffic": tr, "traffic_source": tr_src, "bytes_per_launch": kb, "us_per_launch": us,
-                    "share_of_step_time": us / us_per_step, "peak_source": peak_src, "cluster_size": m["cluster_size"]}
+        roofline = {"kernel": "the whole step, %g launches" % m["launches_per_step"], "bound": "hbm", "achieved": head["step_gbs"],
+                    "peak": peak, "unit": "GB/s", "frac": head["step_frac_of_peak"], "traffic": None,
+                    "traffic_source": "no counters of a whole step of several launches", "bytes_per_launch": by["fasa"],
+                    "us_per_launch": us_per_step, "peak_source": peak_src, "cluster_size": m["cluster_size"],
+                    "select_step": {"bytes": kb, "us": m["select_us"], "gbs": kb / m["select_us"] / 1e3, "frac": kb / m["select_us"] / 1e3 / peak}}
     else:
         fc_us = m["kern_us"]["fc_score"]
         roofline = {"kernel": "fc_score_kernel", "bound": "hbm", "achieved": by["proxy"] / (fc_us * 1e-6) / 1e9,

@@ -4,11 +4,10 @@
 // q_t), so a block of T queries is T decode steps that happen to read the same cache: query t of
 // the block sits at cache position L - T + t (L = seq_lens[b] counts the block's own keys, already
 // appended), sees the rows up to its own, and gets its own scores, index set and output.  What
-// the T steps share is the proxy-K stream: scoring all of them is ONE pass over it,
-//     S[L x (G T)] = P[L x 2F] . Q[2F x (G T)],
-// a matrix product with up to 64 columns, after which the G columns of each query are reduced.
-//
-// by the kernel of fasa_stream.cu: the block's queries are the rows of its result, the heads of a set are summed.
+// the T steps share is the proxy-K stream: scoring all of them is ONE pass over it, for every head of a set
+//     S[T x L] = Q[T x 2F] . P^T[2F x L],
+// whose heads are then summed (or their maximum taken), by the kernel of fasa_stream.cu: the block's queries are the rows of its
+// products, two heads to one.
 //
 // Selection and attention of the block are those of fasa_topk and fasa_sparse_decode_attn over (sequence, query) pairs.
 #include "fasa_common.cuh"
