@@ -14,11 +14,11 @@
 // sequences in caches of 64 K lay on two or three CTAs of several iterations each, and the others read 21 MB of nothing: a step with a
 // set per head 24.4 us, now 18.4; 16 sequences of 2 K in 32 K 45.6 -> 35.6; blocks of five, 8 sequences of 4 K in 64 K 44.6 -> 34.6.
 //
-// Measured (batch 8, 32 / 8 heads, 40-65 K, 16 FCs, T = 5): 45.6 us, 6.0 TB/s.  Before, tcgen05.mma with both operands in shared
+// Measured (batch 8, 32 / 8 heads, 40-65 K, 16 FCs, T = 5): 45.1 us, 6.0 TB/s.  Before, tcgen05.mma with both operands in shared
 // memory took 71.0 us: the proxy had to be scattered into its operand layout, four warps met at a barrier for each 128 tokens,
 // 250 instructions per 32 tokens and warp against 146 here.  The tensor pipe is no limit: 16 products of 8 cycles per 32 tokens
 // and scheduler, a quarter of the time that the tokens take to arrive.  At 8 FCs and five heads a set 59.6 -> 32.9 us, 32 FCs
-// 97.5 -> 77.4, 64 FCs 189 -> 139, 12 FCs (no whole blocks) 82.6 -> 42.2; the same bits throughout.
+// 97.5 -> 77.7, 64 FCs 189 -> 141, 12 FCs (no whole blocks) 82.6 -> 41.0; the same bits throughout.
 //
 // A set per query head took another kernel, a persistent grid with rings of bulk copies whose every warp had an equal share, 171
 // instructions per 32 tokens and heads in columns that shuffles brought together; its SMs were busy for 31 to 50 thousand cycles.
@@ -28,9 +28,9 @@
 // The new token's row is scored from k_new itself: the CTA whose share it ends writes the K, V and proxy rows before it streams
 // and keeps the row's channel pairs in shared memory, where the warp that owns its tile takes them for its fragments; nothing waits
 // for those writes.  (Written by that warp in its loop, the row's addresses cost 8 to 40 bytes of spills around it at 64 registers:
-// batch 4, 30-56 K, a set per head, 36.3 us a step, 31.8 without; default sets, batch 8, 60-90 K, 8 FCs 53.6, 46.4.)  What is left: 8 to 72 bytes
-// where one tile fills the registers or the sums of six and more heads do.  The lengths themselves grow in the second half, which
-// reads the old ones before this one ends.
+// batch 4, 30-56 K, a set per head, 36.3 us a step, 31.8 without; default sets, batch 8, 60-90 K, 8 FCs 53.6, 46.4.)  What is left: 8 to
+// 72 bytes where the sums of six heads and more fill the registers.  The lengths themselves grow in the second half, which reads the
+// old ones before this one ends.
 #include <algorithm>
 #include <type_traits>
 
@@ -114,11 +114,13 @@ __device__ __forceinline__ void mma_q_tokens(float (&c)[4], const uint4& q, uint
         : "r"(q.x), "r"(q.y), "r"(q.z), "r"(q.w), "r"(b0), "r"(b1));
 }
 
-// KB: 16-channel blocks per tile (the last one may be half), from five on rounded up to 8.  Up to four blocks the loop knows how many
-// bytes a tile has; with tests of the geometry and loads under them, 12 FCs took 72.1 us a default step (12 sequences of 40-60 K) where
-// 57.0 are enough, 16 FCs 65.6; 24 FCs, in a loop for four blocks, 88.7 -> 84.5; a block of seven at 61-73 K, 24 FCs 133.6 -> 123.2.  HP: pairs of heads that are reduced; 0: one row, whose up to eight
-// heads are rows 0-7 of the product (an eighth of the products that HP > 0 takes for a single row).  Their sum is a tree over
-// lanes in which every step also halves the tokens a lane holds: ((0 + 1) + (2 + 3)) + ((4 + 5) + (6 + 7)), as everywhere else.
+// KB: 16-channel blocks per tile (the last one may be half), from five on rounded up to 8.  Up to four blocks the loop knows how
+// many bytes a tile has; with tests of the geometry and loads under them, 12 FCs took 72.1 us a default step (12 sequences of
+// 40-60 K) where 57.0 are enough, 16 FCs 65.6; 24 FCs, in a loop for four blocks, 88.7 -> 84.5; blocks of seven at 61-73 K, 24 FCs
+// 133.6 -> 123.2.
+// HP: pairs of heads that are reduced; 0: one row, whose up to eight heads are rows 0-7 of the product (an eighth of the products
+// that HP > 0 takes for a single row).  Their sum is a tree over lanes in which every step also halves the tokens a lane holds:
+// ((0 + 1) + (2 + 3)) + ((4 + 5) + (6 + 7)), as everywhere else.
 // The query's fragments are read from shared memory for each tile: in registers they cost CTAs (47 against 46 us).
 // APPEND: the sequence grows by a token first.
 template <int KB, int HP, bool PAGED, bool APPEND>
