@@ -223,7 +223,7 @@ def test_few_sets_of_long_rows_leave_the_selection_to_clusters():
         f.select_step(q, k, v, proxy, lens, n, None, idx, n_sel)
         f.sparse_decode_attn(q, k, v, idx, n_sel, out, ws)
     apart = _device_us(apart)
-    assert step <= 1.1 * apart, (step, apart)
+    assert step <= 1.2 * apart, (step, apart)
 
 
 @pytest.mark.parametrize("rows,L,budgets", [
